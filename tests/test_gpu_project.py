@@ -96,3 +96,28 @@ def test_project_llama2_7b_shape_sampled_rows():
     ref = oracle.project(f64(heads_out.cpu())[:, rows].reshape(B, len(rows), Hq * d), f64(wo))
     assert_close(y[:, rows, 0].float().cpu().numpy(), ref, "bf16", "output projection W^O")
     assert lb.lisa_check() == lb.OK
+
+
+@pytest.mark.parametrize("B,N,d_in,heads", [
+    (1, 1, 64, [(1, 8)]),                                   # one row, one slice, less than a tile of columns
+    (16, 1, 136, [(2, 21), (2, 21), (1, 60)]),              # d_in just past a slice; blocks off the 8-column groups
+    (17, 1, 1000, [(3, 40), (1, 24)]),                      # first row of the next build; K split over a cluster
+    (5, 13, 512, [(4, 20), (4, 20), (2, 64)]),              # 65 rows of five sequences as one batch
+    (1, 129, 328, [(1, 264)]),                              # 256-row build, one row past 128
+    (2, 256, 192, [(2, 128), (1, 16)]),                     # 512 rows: two row tiles
+    (3, 171, 192, [(2, 128), (1, 16)]),                     # 513: the persistent kernel, batches flattened
+])
+def test_project_few_rows(B, N, d_in, heads):
+    """Row counts around the builds of the few-row kernel (16 ... 256 rows), with the batches flattened into one."""
+    x, w = draw(B, N, d_in, heads, "bf16", 17)
+    outs = [torch.full((B, N, H, xx), 7.0, dtype=torch.bfloat16, device="cuda") for H, xx in heads]
+    lb.lisa_project(dev(x), dev(w), outs)
+    strided = torch.zeros((B, N + 1, d_in + 8), dtype=torch.bfloat16, device="cuda")   # rows at two distances: tiled per batch
+    strided[:, :N, :d_in] = dev(x)
+    again = [torch.empty_like(o) for o in outs]
+    lb.lisa_project(strided[:, :N, :d_in], dev(w), again)
+    torch.cuda.synchronize()
+    assert lb.lisa_check() == lb.OK
+    for o, a, r in zip(outs, again, split(oracle.project(f64(x), f64(w)), heads)):
+        assert_close(o.float().cpu().numpy(), r, "bf16", "projection of few rows")
+        assert_close(a.float().cpu().numpy(), r, "bf16", "the same from strided rows")
