@@ -135,15 +135,15 @@ cudaError_t launch_tc_align_link(const TcAlignLinkArgs& a, cudaStream_t s);
 // waits before it finishes, completion is transitive.  In a kernel launched the ordinary way both are no-ops.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-template <typename Params>
-cudaError_t launch_chained(void (*kernel)(Params), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const Params& p) {
+template <typename... Params>
+cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const Params&... p) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, p);
+    return cudaLaunchKernelEx(&cfg, kernel, p...);
 }
 
 // Packs Q' or K' ([B,N,H,r], any strides) into zero-padded bf16 [B][H][N][64] rows for the tensor-core kernels.

@@ -1,0 +1,71 @@
+// What the decode kernels share: their parameters and score-row access.
+#pragma once
+#include "common.cuh"
+
+namespace lisa {
+
+constexpr int kDecodeThreads = 256;
+constexpr int kDecodeWarps = kDecodeThreads / 32;
+
+struct DecodeParams {
+    int B, Hq, Hkv, d, L_cap, L_uniform, n_chunks;
+    int chunk;              // cached positions per chunk: 128, or 64 or 32 in the kernels for small batches
+    int heads;              // query heads per CTA where the heads are divided over CTAs
+    int prefetch;           // a CTA asks its part of the caches into L2 when it starts
+    const int32_t* seq_lens;
+    // shared layer
+    const void* prev;       // fp32, or bf16 when row_bf16
+    int64_t prev_sb, prev_sh;
+    TView qp;
+    const void* kpT;
+    int r, m, act, integrate, ffn_layers, w_dtype;
+    const void *w1, *b1, *w2, *b2;
+    int w_vec;              // W1 and W2 are bf16 and 16-byte aligned
+    // standard layer
+    TView q;
+    const void* kcache;
+    // common
+    const void* vcache;
+    int cache_dtype;
+    void* out_scores;       // fp32, or bf16 when row_bf16
+    int64_t sc_sb, sc_sh;
+    int row_bf16;           // the score rows handed between layers are bf16 (Sec. 5.2 counts them at 2 bytes) instead of fp32
+    float *ws_m, *ws_l, *ws_o;
+    TView o;
+};
+
+// Score-row access: RB = rows are bf16.
+template <bool RB>
+__device__ __forceinline__ float ld_row(const void* p, int64_t i) {
+    if constexpr (RB) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p)[i]);
+    else return reinterpret_cast<const float*>(p)[i];
+}
+template <bool RB>
+__device__ __forceinline__ void st_row(void* p, int64_t i, float v) {
+    if constexpr (RB) reinterpret_cast<__nv_bfloat16*>(p)[i] = __float2bfloat16_rn(v);
+    else reinterpret_cast<float*>(p)[i] = v;
+}
+
+__device__ __forceinline__ float ldw(const void* p, int idx, int dtype) { return p ? ld_elem(p, idx, dtype) : 0.f; }
+
+__device__ __forceinline__ uint4 ld_stream16(const void* p) {
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p));
+    return v;
+}
+
+__device__ __forceinline__ void bf16x8_to_f32(const uint4& v, float* f) {
+    f[0] = __uint_as_float(v.x << 16); f[1] = __uint_as_float(v.x & 0xffff0000u);
+    f[2] = __uint_as_float(v.y << 16); f[3] = __uint_as_float(v.y & 0xffff0000u);
+    f[4] = __uint_as_float(v.z << 16); f[5] = __uint_as_float(v.z & 0xffff0000u);
+    f[6] = __uint_as_float(v.w << 16); f[7] = __uint_as_float(v.w & 0xffff0000u);
+}
+
+// Context length of sequence b, never beyond the chunks the launch covers.
+__device__ __forceinline__ int decode_length(const DecodeParams& p, int b) {
+    return p.seq_lens ? min(p.seq_lens[b], p.L_uniform) : p.L_uniform;
+}
+
+}  // namespace lisa
