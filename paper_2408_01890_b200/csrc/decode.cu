@@ -454,11 +454,21 @@ void set_chunk(DecodeParams& p, int ch, void* ws) {
     carve_workspace(p, ws);
 }
 
-template <int HQ, int HG, int CH, int M_C, int ENG, int CTAS = 2>
+// Two or three CTAs per SM: a CTA of the three-per-SM build takes about 1.3 times as long as one of the two-per-SM build runs
+// beside one neighbour (B 64, L 4096, 40 heads: 0.510 against 0.528 ms for the whole grid), and the grid runs in whole waves of
+// CTAs: take the build whose waves cost less.
+bool three_per_sm(int64_t ctas) {
+    const int64_t sms = sm_count();
+    return 1.3 * (double)((ctas + 3 * sms - 1) / (3 * sms)) < (double)((ctas + 2 * sms - 1) / (2 * sms));
+}
+
+template <int HQ, int HG, int CH, int M_C, int ENG>
 cudaError_t launch_shared_fast(DecodeParams& p, cudaStream_t s) {
-    auto kernel = shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, CTAS>;
-    const size_t smem = shared_fast_layout(HQ, HG, CH, ENG, p.m, HQ / p.Hkv).total;
     const int64_t ctas = (int64_t)p.n_chunks * (HQ / HG) * p.B;
+    auto kernel = shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2>;
+    if constexpr (ENG == kEngTf32 && CH == 128)
+        if (three_per_sm(ctas)) kernel = shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3>;
+    const size_t smem = shared_fast_layout(HQ, HG, CH, ENG, p.m, HQ / p.Hkv).total;
     p.prefetch = ctas <= 2 * (int64_t)sm_count();   // a grid that is resident at once
     cudaError_t e = set_smem(kernel, smem);
     return e != cudaSuccess ? e : launch_chained(kernel, dim3(p.n_chunks, HQ / HG, p.B), dim3(kDecodeThreads), smem, s, p);
@@ -476,18 +486,24 @@ cudaError_t shared_fast(DecodeParams& p, void* ws, cudaStream_t s, bool* taken) 
     p.w_vec = bf16_w;
     const int64_t n_ctas = (int64_t)p.B * ((p.L_uniform + kChunk - 1) / kChunk), sms = sm_count();
     if (tf32) {
-        if (8 % G == 0 && n_ctas < 2 * sms) {   // heads divided as well, eight to a CTA
-            set_chunk(p, chunk_length(p.B, p.Hq, p.L_uniform, HQ / 8), ws);
-            if (p.chunk == 128) return launch_shared_fast<HQ, 8, 128, M_C, kEngTf32>(p, s);
-            if (p.chunk == 64) return launch_shared_fast<HQ, 8, 64, M_C, kEngTf32>(p, s);
-            return launch_shared_fast<HQ, 8, 32, M_C, kEngTf32>(p, s);
+        // All heads to a CTA once that gives every SM two CTAs -- one with grouped queries, where the aligner is most of a CTA's work and
+        // each group of heads would repeat half of it.  Else sixteen or eight heads to a CTA, then shorter chunks (7B-shaped, us:
+        // B 64 L 300 55 -> 43 with 16 heads; B 8 L 1111 38 -> 25 with 8; B 4 L 1000 15.3 at 64 positions, 18.2 at 128).
+        const int64_t want = G > 1 ? sms : 2 * sms;
+        const bool full = 8 % G != 0 || n_ctas >= want;
+        if (full) {
+            set_chunk(p, kChunk, ws);
+            return launch_shared_fast<HQ, HQ, 128, M_C, kEngTf32>(p, s);
         }
-        set_chunk(p, kChunk, ws);
-        // Two or three CTAs per SM: a CTA of the three-per-SM build takes about 1.3 times as long as one of the two-per-SM
-        // build runs beside one neighbour (measured at B 64, L 4096, 40 heads: 0.534 against 0.566 ms for the whole grid), and the
-        // grid runs in whole waves of CTAs: take the build whose waves cost less.
-        const bool three = kv_group(G) == 1 && 1.3 * (double)((n_ctas + 3 * sms - 1) / (3 * sms)) < (double)((n_ctas + 2 * sms - 1) / (2 * sms));
-        return three ? launch_shared_fast<HQ, HQ, 128, M_C, kEngTf32, 3>(p, s) : launch_shared_fast<HQ, HQ, 128, M_C, kEngTf32>(p, s);
+        if constexpr (HQ % 16 == 0)
+            if (n_ctas * (HQ / 16) >= want) {
+                set_chunk(p, kChunk, ws);
+                return launch_shared_fast<HQ, 16, 128, M_C, kEngTf32>(p, s);
+            }
+        set_chunk(p, chunk_length(p.B, p.Hq, p.L_uniform, HQ / 8), ws);
+        if (p.chunk == 128) return launch_shared_fast<HQ, 8, 128, M_C, kEngTf32>(p, s);
+        if (p.chunk == 64) return launch_shared_fast<HQ, 8, 64, M_C, kEngTf32>(p, s);
+        return launch_shared_fast<HQ, 8, 32, M_C, kEngTf32>(p, s);
     }
     set_chunk(p, chunk_length(p.B, p.Hq, p.L_uniform, 1), ws);
     if (p.integrate == LISA_INTEGRATE_ADD) {
@@ -565,13 +581,16 @@ cudaError_t launch_anchor_decode(const lisa_anchor_args& a, void* ws, cudaStream
     const TView& q = p.q;
     cudaError_t e;
     if (p.cache_dtype == LISA_BF16 && p.d == 128 && q.dtype == LISA_BF16 && vec16(q.ptr) && q.sb % 8 == 0 && q.sh % 8 == 0) {
-        // all heads to a CTA; fewer (down to one KV head), then shorter chunks, where that does not give two CTAs per SM
-        const int64_t want = 2 * (int64_t)sm_count(), chunks = (int64_t)p.B * ((a.L + kChunk - 1) / kChunk);
-        int kv = p.Hkv;
+        // Eight KV heads to a CTA, one per warp: CTAs small enough for even waves, nothing computed twice (40 heads, us: B 12 L 3500
+        // 178 -> 138 against all heads to a CTA, B 64 L 4096 803 -> 790).  Fewer, then shorter chunks, where that does not give
+        // every SM a CTA.
+        const int64_t want = sm_count(), chunks = (int64_t)p.B * ((a.L + kChunk - 1) / kChunk);
+        int kv = std::min(8, p.Hkv);
+        while (p.Hkv % kv) --kv;
         while (kv % 2 == 0 && chunks * (p.Hkv / kv) < want) kv /= 2;
         p.heads = kv * G;
         set_chunk(p, chunk_length(p.B, p.Hq, a.L, p.Hkv / kv), ws);
-        p.prefetch = (int64_t)p.n_chunks * p.B * (p.Hkv / kv) <= want;   // a grid that is resident at once
+        p.prefetch = (int64_t)p.n_chunks * p.B * (p.Hkv / kv) <= 2 * want;   // a grid that is resident at once
         const size_t smem = anchor_fast_smem(p.heads, p.chunk, G);
         auto kernel = p.chunk == 128 ? anchor_decode_fast_kernel<128> : p.chunk == 64 ? anchor_decode_fast_kernel<64> : anchor_decode_fast_kernel<32>;
         if ((e = set_smem(kernel, smem)) != cudaSuccess) return e;

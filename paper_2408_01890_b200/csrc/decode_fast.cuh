@@ -42,10 +42,37 @@ struct Rows {
 // Streams the rows of nv virtual KV heads (vper of them on each KV head) through body(regs, v, row0): one warp per head, or per (head,
 // range of rows); two register sets of U 16-byte loads per lane alternate, across heads too.  A lane holds the 16 bytes `lane % 16` of
 // rows row0 + 2 u + lane / 16.  done(v, part) is called behind a head's (or range's) last body.
-template <int U, typename Body, typename Done>
+template <int CH, int U, typename Body, typename Done>
 __device__ __forceinline__ void stream_rows(const Rows& r, int nv, int vper, int ps, Body body, Done done) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane & 15, rsel = lane >> 4;
-    constexpr int ROWS = 2 * U;
+    constexpr int ROWS = 2 * U, NB = CH / ROWS;
+    if (r.nrows == CH && ps == 1) {   // a full chunk: every offset a compile-time constant off one pointer
+        if (warp >= nv) return;
+        auto head_ptr = [&](int v) { return r.base + (size_t)(v / vper) * r.head_stride + rsel * 16 + sub; };
+        auto load = [&](uint4* q, const uint4* hp, int bt) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) q[u] = ld_stream16(hp + (bt * ROWS + 2 * u) * 16);
+        };
+        const uint4* hp = head_ptr(warp);
+        uint4 qa[U], qb[U];
+        load(qa, hp, 0);
+        for (int v = warp; v < nv; v += kDecodeWarps) {
+            const bool has_next = v + kDecodeWarps < nv;
+            const uint4* np = has_next ? head_ptr(v + kDecodeWarps) : hp;
+            // (groups of four heads: the unrolled code would not stay in the instruction cache, 188 instead of 184 us at B 32, L 8192)
+#pragma unroll(U == 8 ? NB / 2 : 1)
+            for (int bt = 0; bt < NB; bt += 2) {
+                load(qb, hp, bt + 1);
+                body(qa, v, bt * ROWS);
+                if (bt + 2 < NB) load(qa, hp, bt + 2);
+                else if (has_next) load(qa, np, 0);
+                body(qb, v, (bt + 1) * ROWS);
+            }
+            done(v, 0);
+            hp = np;
+        }
+        return;
+    }
     const int part = warp / nv * (ps > 1), first = ps > 1 ? warp % nv : warp;
     if (first >= nv || part >= ps) return;
     const int nb_all = (r.nrows + ROWS - 1) / ROWS, b0 = nb_all * part / ps, b1 = nb_all * (part + 1) / ps;
@@ -83,10 +110,10 @@ __device__ __forceinline__ void stream_rows(const Rows& r, int nv, int vper, int
 
 // Partial P.V of a chunk: s_s[head][ld] holds the exponentials (zero past the sequence's end), red scratch for position ranges beyond
 // the first ((ps - 1) x HG x 128 floats); results go to out[head][128].
-template <int GV>
-__device__ __forceinline__ void pv_stream(const Rows& r, int nv, int vper, int ch, const float* s_s, int ld, float* red, float* out) {
+template <int CH, int GV>
+__device__ __forceinline__ void pv_stream(const Rows& r, int nv, int vper, const float* s_s, int ld, float* red, float* out) {
     constexpr int U = stream_loads(GV);
-    const int lane = threadIdx.x & 31, sub = lane & 15, rsel = lane >> 4, ps = row_parts(nv, ch, GV);
+    const int lane = threadIdx.x & 31, sub = lane & 15, rsel = lane >> 4, ps = row_parts(nv, CH, GV);
     float acc[GV][8];
 #pragma unroll
     for (int q = 0; q < GV; ++q)
@@ -120,7 +147,7 @@ __device__ __forceinline__ void pv_stream(const Rows& r, int nv, int vper, int c
             for (int t = 0; t < 8; ++t) acc[q][t] = 0.f;
         }
     };
-    stream_rows<U>(r, nv, vper, ps, body, done);
+    stream_rows<CH, U>(r, nv, vper, ps, body, done);
     if (ps > 1) {   // add the ranges, in order; a range without rows wrote nothing
         __syncthreads();
         const int nb = (r.nrows + 2 * U - 1) / (2 * U);
@@ -139,8 +166,8 @@ __device__ __forceinline__ void pv_stream(const Rows& r, int nv, int vper, int c
 // Scores of a chunk: s_s[head][j] = scale * q_head . K_j; q_s [head][128] fp32.  A lane holds the partial dot products of U rows and GV
 // heads over its 8 of the 128 dimensions; the sum over the 16 lanes of a row is a butterfly that halves the number of live values
 // at every step.
-template <int GV>
-__device__ __forceinline__ void qk_stream(const Rows& r, int nv, int vper, int ch, const float* q_s, float* s_s, int ld, float scale) {
+template <int CH, int GV>
+__device__ __forceinline__ void qk_stream(const Rows& r, int nv, int vper, const float* q_s, float* s_s, int ld, float scale) {
     constexpr int U = stream_loads(GV), NV = GV * U;   // 8 or 16 values
     const int lane = threadIdx.x & 31, sub = lane & 15, rsel = lane >> 4;
     auto body = [&](const uint4* regs, int v, int row0) {
@@ -177,7 +204,7 @@ __device__ __forceinline__ void qk_stream(const Rows& r, int nv, int vper, int c
         }
         if (NV == 16 || (sub & 1) == 0) s_s[(v * GV + idx / U) * ld + row0 + 2 * (idx % U) + rsel] = dot[0] * scale;
     };
-    stream_rows<U>(r, nv, vper, row_parts(nv, ch, GV), body, [](int, int) {});
+    stream_rows<CH, U>(r, nv, vper, row_parts(nv, CH, GV), body, [](int, int) {});
 }
 
 // Softmax of a chunk per head, in place: s_s[head][CH] scores (add_s), plus HS partial sums y_s[hs][head][CH] where y_s is given,
@@ -226,14 +253,13 @@ __device__ __forceinline__ void finish_scores(const DecodeParams& p, float* s_s,
     }
 }
 
-// MOST: the largest group of query heads the build is for.
-template <int MOST>
-__device__ __forceinline__ void pv_chunk(const DecodeParams& p, const float* s_s, int ch, float* red, int b, int kv0, int HG, int j0, int nrows, float* out) {
+template <int CH>
+__device__ __forceinline__ void pv_chunk(const DecodeParams& p, const float* s_s, float* red, int b, int kv0, int HG, int j0, int nrows, float* out) {
     const int G = p.Hq / p.Hkv, gv = kv_group(G);
     const Rows rows{reinterpret_cast<const uint4*>(p.vcache) + (((size_t)b * p.Hkv + kv0) * p.L_cap + j0) * 16, (size_t)p.L_cap * 16, nrows};
-    if (MOST == 1 || gv == 1) pv_stream<1>(rows, HG, G, ch, s_s, ch, red, out);
-    else if (gv == 2) pv_stream<2>(rows, HG / 2, G / 2, ch, s_s, ch, red, out);
-    else pv_stream<4>(rows, HG / 4, G / 4, ch, s_s, ch, red, out);
+    if (gv == 1) pv_stream<CH, 1>(rows, HG, G, s_s, CH, red, out);
+    else if (gv == 2) pv_stream<CH, 2>(rows, HG / 2, G / 2, s_s, CH, red, out);
+    else pv_stream<CH, 4>(rows, HG / 4, G / 4, s_s, CH, red, out);
 }
 
 // The caches of this CTA's chunk on their way into L2, before the wait for the preceding kernel: a hint (the length may be read before
@@ -288,14 +314,14 @@ __global__ void __launch_bounds__(kDecodeThreads, 2) anchor_decode_fast_kernel(c
     __syncthreads();
     const Rows rows{reinterpret_cast<const uint4*>(p.kcache) + (((size_t)b * p.Hkv + kv0) * p.L_cap + j0) * 16, (size_t)p.L_cap * 16, nrows};
     const float scale = rsqrtf(128.f);
-    if (gv == 1) qk_stream<1>(rows, HG, G, CH, q_s, s_s, CH, scale);
-    else if (gv == 2) qk_stream<2>(rows, HG / 2, G / 2, CH, q_s, s_s, CH, scale);
-    else qk_stream<4>(rows, HG / 4, G / 4, CH, q_s, s_s, CH, scale);
+    if (gv == 1) qk_stream<CH, 1>(rows, HG, G, q_s, s_s, CH, scale);
+    else if (gv == 2) qk_stream<CH, 2>(rows, HG / 2, G / 2, q_s, s_s, CH, scale);
+    else qk_stream<CH, 4>(rows, HG / 4, G / 4, q_s, s_s, CH, scale);
     __syncthreads();
     const size_t part = ((size_t)b * p.n_chunks + chunk) * p.Hq + h0;
     finish_scores<CH, 1>(p, s_s, nullptr, true, HG, h0, b, j0, nrows, part);
     __syncthreads();
-    pv_chunk<4>(p, s_s, CH, red, b, kv0, HG, j0, nrows, p.ws_o + part * 128);
+    pv_chunk<CH>(p, s_s, red, b, kv0, HG, j0, nrows, p.ws_o + part * 128);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -416,12 +442,11 @@ __host__ __device__ inline SharedFastLayout shared_fast_layout(int HQ, int HG, i
 }
 
 // CTAS: CTAs per SM the kernel is compiled for.  Three hide the FFN phase (no loads in flight from the CTA that is in it) better than
-// two, at 80 instead of 128 registers (no room for groups of query heads); which one a launch takes depends on how its grid fills
-// the waves.
+// two, at 80 instead of 128 registers; which one a launch takes depends on how its grid fills the waves.
 template <int HQ, int HG, int CH, int M_C, int ENG, int CTAS>
 __global__ void __launch_bounds__(kDecodeThreads, CTAS) shared_decode_fast_kernel(const __grid_constant__ DecodeParams p) {
     static_assert(ENG == kEngTf32 ? M_C > 0 : HG == HQ, "the split forms run with all heads");
-    constexpr int HS = 128 / CH, NT2 = HG / 8, MOST = CTAS == 3 ? 1 : 4;
+    constexpr int HS = 128 / CH, NT2 = HG / 8;
     extern __shared__ __align__(16) uint8_t smem_b[];
     const int b = blockIdx.z, chunk = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int h0 = blockIdx.y * HG, G = HQ / p.Hkv, kv0 = h0 / G, j0 = chunk * CH;
@@ -490,7 +515,7 @@ __global__ void __launch_bounds__(kDecodeThreads, CTAS) shared_decode_fast_kerne
     __syncthreads();
     {
         const int gv = kv_group(G);
-        if (MOST == 1 || gv == 1) delta_chunk<CH, 1>(p, s_s, qp_s, b, kv0, HG, j0);
+        if (gv == 1) delta_chunk<CH, 1>(p, s_s, qp_s, b, kv0, HG, j0);
         else if (gv == 2) delta_chunk<CH, 2>(p, s_s, qp_s, b, kv0, HG, j0);
         else delta_chunk<CH, 4>(p, s_s, qp_s, b, kv0, HG, j0);
     }
@@ -628,7 +653,7 @@ __global__ void __launch_bounds__(kDecodeThreads, CTAS) shared_decode_fast_kerne
     const size_t part = ((size_t)b * p.n_chunks + chunk) * HQ + h0;
     finish_scores<CH, HS>(p, s_s, (HS > 1 || ENG == kEngConcat) ? y_s : nullptr, ENG != kEngConcat, HG, h0, b, j0, nrows, part);
     __syncthreads();
-    pv_chunk<MOST>(p, s_s, CH, reinterpret_cast<float*>(smem_b + lay.w1), b, kv0, HG, j0, nrows, p.ws_o + part * 128);
+    pv_chunk<CH>(p, s_s, reinterpret_cast<float*>(smem_b + lay.w1), b, kv0, HG, j0, nrows, p.ws_o + part * 128);
 }
 
 }  // namespace lisa

@@ -79,6 +79,38 @@ def test_shared_decode_three_ctas_per_sm(Hq, Hkv, m, B, L):
     run_shared_decode(w, B, L, lens=lens, seed=6)
 
 
+@pytest.mark.parametrize("Hq,Hkv,m,act,integrate,B,L", [
+    (32, 32, 64, "relu", lb.INTEGRATE_ADD, 1, 31), (32, 16, 64, "silu", lb.INTEGRATE_ADD, 2, 33), (40, 40, 80, "relu", lb.INTEGRATE_ADD, 3, 65),
+    (32, 4, 64, "relu", lb.INTEGRATE_ADD, 1, 1000),          # eight query heads to a KV head, chunks of 32 and 64 positions
+    (32, 8, 64, "relu", lb.INTEGRATE_ADD, 9, 1100),          # heads in groups, chunks of 128
+    (32, 32, 64, "relu", lb.INTEGRATE_ADD, 50, 385),         # sixteen heads to a CTA
+    (32, 32, 256, "relu", lb.INTEGRATE_CONCAT, 2, 257), (32, 8, 72, "silu", lb.INTEGRATE_CONCAT, 30, 640), (40, 8, 128, "relu", lb.INTEGRATE_CONCAT, 2, 130),
+    (32, 8, 256, "relu", lb.INTEGRATE_ADD, 1, 97), (40, 40, 24, "silu", lb.INTEGRATE_ADD, 3, 700)])
+def test_shared_decode_small_and_grouped(Hq, Hkv, m, act, integrate, B, L):
+    """Every way a launch is cut: chunk lengths, groups of heads, query heads that share a KV head, FFN widths off the compiled ones."""
+    w = synth.Workload("dcut", "bf16", B, L, Hq, Hkv, 128, 21, m, act, 1, True)
+    lens = [max(1, (L * (b + 1)) // B - b % 3) for b in range(B)]
+    run_shared_decode(w, B, L, lens=lens, seed=8, integrate=integrate, bias=True)
+
+
+@pytest.mark.parametrize("Hq,Hkv,B,L", [(32, 32, 1, 31), (32, 16, 2, 65), (32, 8, 3, 129), (32, 4, 20, 1030), (40, 8, 2, 300), (2, 1, 1, 17)])
+def test_anchor_decode_cuts(Hq, Hkv, B, L):
+    """The standard layer's chunk lengths, groups of KV heads and shared KV heads, sequences that end inside a chunk."""
+    w = synth.Workload("acut", "bf16", B, L, Hq, Hkv, 128, 8, 16, "relu", 1, True)
+    t = synth.decode_inputs(w, 7, B=B, L=L)
+    cache = lb.KVCacheLayer(lb.CACHE_STANDARD, B, Hkv, (L + 7) // 8 * 8, 128)
+    lb.lisa_kvcache_append(cache, dev(t["k"]), dev(t["v"]))
+    lens = np.array([max(1, (L * (b + 1)) // B - b % 3) for b in range(B)], dtype=np.int32)
+    row = torch.full((B, Hq, cache.L_cap), -7.0, dtype=torch.float32, device="cuda")
+    out = lb.lisa_attn_anchor(dev(t["q0"]), cache=cache, L=L, seq_lens=torch.from_numpy(lens).cuda(), out_scores=row)
+    O, R = oracle.decode_anchor(f64(t["q0"])[:, 0], f64(t["k"]), f64(t["v"]), lens)
+    assert_close(out[:, 0].float().cpu().numpy(), O, "bf16", "anchor decode O")
+    row_h = row.cpu().numpy()
+    for b in range(B):
+        assert_close(row_h[b, :, :lens[b]], R[b, :, :lens[b]], "f32", "anchor score row")
+        assert np.all(row_h[b, :, lens[b]:] == -7.0)
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("Hq,Hkv,d,L", [(40, 40, 128, 600), (32, 8, 128, 257), (6, 3, 64, 130), (4, 4, 32, 7)])
 def test_anchor_decode(dtype, Hq, Hkv, d, L):
