@@ -3,7 +3,8 @@
 Every function here has the name of the C entry point it calls and does nothing but build the
 descriptor structs from torch tensors (device pointers, strides, dtypes), allocate outputs and scratch
 with torch, and pass torch's current CUDA stream.  All arithmetic runs in the library's kernels; if the
-library is missing, importing works but the first call raises.
+library is missing, importing works but the first call raises.  The entry points of a model's inner loop (attention, cache
+append, projections) are marshalled by the native module _lisa_binding (csrc/binding_ext.cpp), the others by ctypes.
 """
 from __future__ import annotations
 
@@ -113,14 +114,19 @@ class SharedDecodeArgs(C.Structure):
 
 
 _lib = None
+_ext = None
 
 
 def load():
     """Loads liblisa_b200.so (built by paper_2408_01890_b200.build). Raises if it is missing."""
-    global _lib
+    global _lib, _ext
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError("CUDA library not built: %s is missing (run python -m paper_2408_01890_b200.build)" % LIB_PATH)
+        try:
+            from . import _lisa_binding as ext
+        except ImportError as e:
+            raise RuntimeError("binding not built: run python -m paper_2408_01890_b200.build (%s)" % e)
         lib = C.CDLL(LIB_PATH)
         lib.lisa_status_string.restype = C.c_char_p
         lib.lisa_status_string.argtypes = [C.c_int]
@@ -152,8 +158,17 @@ def load():
         lib.lisa_check.argtypes = [C.c_void_p]
         lib.lisa_kernel_launches.restype = C.c_uint64
         lib.lisa_debug_wait_timeout.argtypes = [C.c_int64, C.c_void_p]
-        _lib = lib
+        ext.bind(*[C.cast(getattr(lib, n), C.c_void_p).value for n in (
+            "lisa_attn_anchor", "lisa_attn_shared_prefill", "lisa_attn_shared_prefill_carry", "lisa_attn_shared_decode",
+            "lisa_kvcache_append", "lisa_kvcache_append_layer", "lisa_project", "lisa_workspace_bytes")])
+        _lib, _ext = lib, ext
     return _lib
+
+
+def _native():
+    if _ext is None:
+        load()
+    return _ext
 
 
 def _check(status: int, where: str):
@@ -264,9 +279,7 @@ class KVCache:
         return self.layers[l]
 
     def append(self, l: int, k_or_kp: torch.Tensor, v: torch.Tensor, seq_lens_before: Optional[torch.Tensor] = None):
-        kt, vt = _tensor4(k_or_kp), _tensor4(v)
-        _check(load().lisa_kvcache_append_layer(C.byref(self.c), int(l), C.byref(kt), C.byref(vt), _ptr(seq_lens_before),
-                                                int(v.shape[1]), _stream()), "lisa_kvcache_append_layer")
+        _check(_native().append_layer(C.addressof(self.c), int(l), k_or_kp, v, seq_lens_before), "lisa_kvcache_append_layer")
 
 
 def lisa_kvcache_bytes(kind: int, B: int, Hkv: int, L_cap: int, d: int, r: int = 0, dtype: int = BF16):
@@ -279,25 +292,13 @@ def lisa_kvcache_bytes(kind: int, B: int, Hkv: int, L_cap: int, d: int, r: int =
 def lisa_kvcache_append(cache: KVCacheLayer, k_or_kp: torch.Tensor, v: torch.Tensor,
                         seq_lens_before: Optional[torch.Tensor] = None):
     """k_or_kp [B,n_new,Hkv,d|r], v [B,n_new,Hkv,d]; seq_lens_before int32 [B] on the device or None (= 0)."""
-    kt, vt = _tensor4(k_or_kp), _tensor4(v)
-    _check(load().lisa_kvcache_append(C.byref(cache.desc), C.byref(kt), C.byref(vt), _ptr(seq_lens_before),
-                                      int(v.shape[1]), _stream()), "lisa_kvcache_append")
+    _check(_native().append(C.addressof(cache.desc), k_or_kp, v, seq_lens_before), "lisa_kvcache_append")
 
 
 def lisa_project(x: torch.Tensor, w: torch.Tensor, outs: Sequence[torch.Tensor]) -> Sequence[torch.Tensor]:
     """C = x . w scattered into outs: x [B,N,d_in] (rows contiguous), w [d_in, n_out] row-major, outs[o] a [B,N,H_o,x_o] tensor
     (any strides, innermost contiguous) that receives the next H_o*x_o columns of C."""
-    B, N, d_in = x.shape
-    assert x.stride(2) == 1 and w.is_contiguous() and w.shape[0] == d_in and w.shape[1] == sum(o.shape[2] * o.shape[3] for o in outs)
-    assert 1 <= len(outs) <= 4
-    a = ProjectArgs()
-    a.struct_size = C.sizeof(ProjectArgs)
-    a.B, a.N, a.d_in, a.n_outputs = B, N, d_in, len(outs)
-    a.x = Tensor(x.data_ptr(), _dt(x), 0, x.stride(0), x.stride(1), 0)
-    a.w, a.w_dtype = w.data_ptr(), _dt(w)
-    for i, o in enumerate(outs):
-        a.outputs[i] = CProjectOutput(_tensor4(o), int(o.shape[2]), int(o.shape[3]))
-    _check(load().lisa_project(C.byref(a), _stream()), "lisa_project")
+    _check(_native().project(x, w, outs), "lisa_project")
     return outs
 
 
@@ -329,26 +330,9 @@ def lisa_attn_anchor(q: torch.Tensor, k: Optional[torch.Tensor] = None, v: Optio
                      out: Optional[torch.Tensor] = None, out_scores: Optional[torch.Tensor] = None,
                      workspace: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Standard causal attention. Prefill: q,k,v [B,N,H,d]. Decode: q [B,1,Hq,d] against a STANDARD cache."""
-    B, Nq, Hq, d = q.shape
     out = torch.empty_like(q) if out is None else out
-    a = AnchorArgs()
-    a.struct_size = C.sizeof(AnchorArgs)
-    a.B, a.Nq, a.Hq, a.d, a.L = B, Nq, Hq, d, int(L)
-    a.q, a.o = _tensor4(q), _tensor4(out)
-    if cache is None:
-        a.Hkv = k.shape[2]
-        a.k, a.v = _tensor4(k), _tensor4(v)
-    else:
-        a.Hkv = cache.Hkv
-        a.cache = C.pointer(cache.desc)
-        a.seq_lens = _ptr(seq_lens)
-        if out_scores is not None:
-            assert out_scores.stride(2) == 1
-            a.out_scores, a.scores_stride_b, a.scores_stride_h = out_scores.data_ptr(), out_scores.stride(0), out_scores.stride(1)
-            a.scores_dtype = _dt(out_scores)
-    ws = workspace if workspace is not None else _workspace(OP_ANCHOR, a)
-    a.workspace, a.workspace_bytes = _ptr(ws), (ws.numel() if ws is not None else 0)
-    _check(load().lisa_attn_anchor(C.byref(a), _stream()), "lisa_attn_anchor")
+    _check(_native().anchor(q, k, v, 0 if cache is None else C.addressof(cache.desc), int(L), seq_lens, out, out_scores, workspace),
+           "lisa_attn_anchor")
     return out
 
 
@@ -367,10 +351,7 @@ def lisa_attn_shared_prefill(q0: torch.Tensor, k0: torch.Tensor, links: Sequence
                              out: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None) -> torch.Tensor:
     """A shared layer at chain depth len(links) over a whole prompt; links[-1] is the layer's own."""
     out = torch.empty_like(q0) if out is None else out
-    a, keep = _prefill_args(q0, k0, links, v, out)
-    ws = workspace if workspace is not None else _workspace(OP_SHARED_PREFILL, a)
-    a.workspace, a.workspace_bytes = _ptr(ws), (ws.numel() if ws is not None else 0)
-    _check(load().lisa_attn_shared_prefill(C.byref(a), _stream()), "lisa_attn_shared_prefill")
+    _check(_native().prefill(q0, k0, links, v, out, workspace), "lisa_attn_shared_prefill")
     return out
 
 
@@ -405,10 +386,7 @@ def lisa_attn_shared_prefill_carry(q0: Optional[torch.Tensor], k0: Optional[torc
     when keep, leaves its own there for the next one.  q0, k0 may be None unless first (then pass `out`)."""
     if out is None:
         out = torch.empty_like(q0)
-    c, keepalive = _carry_args(q0, k0, link, v, out, scores, first, keep)
-    ws = workspace if workspace is not None else _workspace(OP_SHARED_PREFILL_CARRY, c)
-    c.layer.workspace, c.layer.workspace_bytes = _ptr(ws), (ws.numel() if ws is not None else 0)
-    _check(load().lisa_attn_shared_prefill_carry(C.byref(c), _stream()), "lisa_attn_shared_prefill_carry")
+    _check(_native().carry(q0, k0, link, v, out, scores, int(first), int(keep), workspace), "lisa_attn_shared_prefill_carry")
     return out
 
 
@@ -494,24 +472,10 @@ def lisa_attn_shared_decode(prev_scores: torch.Tensor, link: Link, cache: KVCach
                             workspace: Optional[torch.Tensor] = None) -> torch.Tensor:
     """One decode step of a shared layer. prev_scores [B,Hq,>=L] fp32 or bf16 (out_scores then has the same type);
     link.qp [B,1,Hq,r]; returns o [B,1,Hq,d]."""
-    B, Hq = prev_scores.shape[0], prev_scores.shape[1]
-    assert prev_scores.stride(2) == 1
     if out is None:
-        out = torch.empty((B, 1, Hq, cache.d), dtype=cache.v.dtype, device=prev_scores.device)
-    a = SharedDecodeArgs()
-    a.struct_size = C.sizeof(SharedDecodeArgs)
-    a.B, a.Hq, a.L, a.scores_dtype = B, Hq, int(L), _dt(prev_scores)
-    a.prev_scores, a.prev_stride_b, a.prev_stride_h = prev_scores.data_ptr(), prev_scores.stride(0), prev_scores.stride(1)
-    a.link = link.to_c()
-    a.cache = C.pointer(cache.desc)
-    a.seq_lens = _ptr(seq_lens)
-    a.o = _tensor4(out)
-    if out_scores is not None:
-        assert out_scores.dtype == prev_scores.dtype and out_scores.stride(2) == 1
-        a.out_scores, a.scores_stride_b, a.scores_stride_h = out_scores.data_ptr(), out_scores.stride(0), out_scores.stride(1)
-    ws = workspace if workspace is not None else _workspace(OP_SHARED_DECODE, a)
-    a.workspace, a.workspace_bytes = _ptr(ws), (ws.numel() if ws is not None else 0)
-    _check(load().lisa_attn_shared_decode(C.byref(a), _stream()), "lisa_attn_shared_decode")
+        out = torch.empty((prev_scores.shape[0], 1, prev_scores.shape[1], cache.d), dtype=cache.v.dtype, device=prev_scores.device)
+    _check(_native().decode(prev_scores, link, C.addressof(cache.desc), int(L), seq_lens, out, out_scores, workspace),
+           "lisa_attn_shared_decode")
     return out
 
 

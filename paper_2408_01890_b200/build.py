@@ -1,6 +1,7 @@
 """Builds the CUDA library in-tree: `python -m paper_2408_01890_b200.build [--verbose]`.
 
-One shared object, sm_100a only, no relocatable device code: liblisa_b200.so next to this file.
+Two shared objects next to this file: liblisa_b200.so, the library (sm_100a only, no relocatable device code), and
+_lisa_binding.so, the native half of binding.py (a CPython extension against torch's headers, no device code).
 """
 from __future__ import annotations
 
@@ -12,6 +13,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "liblisa_b200.so")
+EXT = os.path.join(HERE, "_lisa_binding.so")
+EXT_SOURCE = os.path.join(HERE, "csrc", "binding_ext.cpp")
 
 
 def sources():
@@ -26,7 +29,28 @@ def _stale():
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def build_binding(force: bool = False) -> str:
+    deps = [EXT_SOURCE] + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    if not force and os.path.exists(EXT) and all(os.path.getmtime(p) <= os.path.getmtime(EXT) for p in deps):
+        return EXT
+    import sysconfig
+
+    import torch
+    tdir = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = EXT + ".%d.tmp" % os.getpid()
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+                           "-I", os.path.join(tdir, "include"), "-I", os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
+                           "-I", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
+                           EXT_SOURCE, "-o", tmp, "-L", os.path.join(tdir, "lib"),
+                           "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
+    os.replace(tmp, EXT)
+    return EXT
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_binding(force)
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -146,9 +146,6 @@ cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&cfg, kernel, p...);
 }
 
-// Packs Q' or K' ([B,N,H,r], any strides) into zero-padded bf16 [B][H][N][64] rows for the tensor-core kernels.
-cudaError_t launch_pack_lowrank(const lisa_tensor& src, int B, int N, int H, int r, void* dst, cudaStream_t s);
-
 // Tensor-core prefill of a shared layer (tc_prefill.cu): emit planes -> align -> attention, wave by wave.
 bool tc_shared_prefill_supported(const lisa_shared_prefill_args& a);
 size_t tc_shared_prefill_workspace(const lisa_shared_prefill_args& a);

@@ -19,7 +19,7 @@ namespace {
 
 constexpr int kTile = 128;
 constexpr int kPadRank = 64;
-constexpr int kMaxPackLinks = 4;   // links whose Q', K' one call packs (the aligner takes chains of up to three)
+constexpr int kMaxPackLinks = kMaxChain;   // links whose Q', K' one call packs
 // A wave takes query tiles until its head-partitioned kernels have at least kWaveCtasPerSm CTAs per SM (with
 // fewer, the grids do not fill the GPU and launch and tail costs dominate) and then further tiles while the causal
 // part of its score planes stays within kWaveBytes.  Measured on B200: grid fill matters far more than keeping
@@ -34,25 +34,42 @@ struct PackJobs {
     int H[2 * kMaxPackLinks], r[2 * kMaxPackLinks];
 };
 
-__global__ void pack_lowrank_kernel(const __grid_constant__ PackJobs jobs, int B, int N) {
+// A CTA packs kPackPos positions of one sequence: the rows of H x r values are read as they lie (one warp per position) into shared
+// memory and leave as whole 128-byte rows.  Bound by HBM where it runs alone; beside a flash kernel, by the shared memory that leaves free.
+constexpr int kPackPos = 8, kPackThreads = kPackPos * 32;
+__global__ void __launch_bounds__(kPackThreads) pack_lowrank_kernel(const __grid_constant__ PackJobs jobs, int B, int N) {
+    __shared__ __align__(16) __nv_bfloat16 rows[kPackPos][kMaxHeads * kMaxRank];
     const TView src = jobs.src[blockIdx.y];
-    const int H = jobs.H[blockIdx.y], r = jobs.r[blockIdx.y];
-    __nv_bfloat16* dst = jobs.dst[blockIdx.y];
-    const int64_t total = (int64_t)B * H * N * (kPadRank / 8);
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int chunk = (int)(e % (kPadRank / 8));
-        int64_t rest = e / (kPadRank / 8);
-        const int n = (int)(rest % N); rest /= N;
-        const int h = (int)(rest % H);
-        const int b = (int)(rest / H);
-        const __nv_bfloat16* sp = reinterpret_cast<const __nv_bfloat16*>(src.ptr) + b * src.sb + (int64_t)n * src.sn + h * src.sh;
-        __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int x = chunk * 8 + j;
-            v[j] = x < r ? sp[x] : __float2bfloat16_rn(0.f);
+    const int H = jobs.H[blockIdx.y], r = jobs.r[blockIdx.y], n0 = blockIdx.x * kPackPos;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, vals = H * r;
+    for (int b = blockIdx.z; b < B; b += gridDim.z) {
+        if (n0 + warp < N) {
+            const __nv_bfloat16* sp = reinterpret_cast<const __nv_bfloat16*>(src.ptr) + b * src.sb + (int64_t)(n0 + warp) * src.sn;
+            if (src.sh == r && (vals & 1) == 0 && (reinterpret_cast<uintptr_t>(sp) & 3u) == 0) {
+                const uint32_t* wp = reinterpret_cast<const uint32_t*>(sp);
+#pragma unroll 8
+                for (int e = lane; e < vals / 2; e += 32) reinterpret_cast<uint32_t*>(rows[warp])[e] = wp[e];
+            } else {
+                for (int e = lane; e < vals; e += 32) rows[warp][e] = sp[(e / r) * src.sh + e % r];
+            }
         }
-        *reinterpret_cast<uint4*>(dst + e * 8) = *reinterpret_cast<const uint4*>(v);
+        __syncthreads();
+        __nv_bfloat16* dst = jobs.dst[blockIdx.y] + ((int64_t)b * H * N + n0) * kPadRank;
+        constexpr int CH = kPadRank / 8;   // 16-byte pieces of a row
+        for (int e = threadIdx.x; e < H * kPackPos * CH; e += kPackThreads) {
+            const int c = e % CH, n = e / CH % kPackPos, h = e / (CH * kPackPos);
+            if (n0 + n >= N) continue;
+            uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int x = c * 8 + 2 * j;
+                const uint16_t* v = reinterpret_cast<const uint16_t*>(rows[n]) + h * r + x;
+                if (x < r) w[j] = v[0];
+                if (x + 1 < r) w[j] |= (uint32_t)v[1] << 16;
+            }
+            *reinterpret_cast<uint4*>(dst + ((int64_t)h * N + n) * kPadRank + c * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        __syncthreads();
     }
 }
 
@@ -167,16 +184,6 @@ lisa_tensor packed_view(void* ptr, int H, int N) {
 }
 
 }  // namespace
-
-cudaError_t launch_pack_lowrank(const lisa_tensor& src, int B, int N, int H, int r, void* dst, cudaStream_t s) {
-    PackJobs jobs{};
-    jobs.src[0] = make_view(src); jobs.dst[0] = reinterpret_cast<__nv_bfloat16*>(dst); jobs.H[0] = H; jobs.r[0] = r;
-    const int64_t total = (int64_t)B * H * N * (kPadRank / 8);
-    const int blocks = (int)std::min<int64_t>((total + 255) / 256, sm_count() * 32);
-    pack_lowrank_kernel<<<dim3(blocks, 1), 256, 0, s>>>(jobs, B, N);
-    count_launches(1);
-    return cudaGetLastError();
-}
 
 bool tc_shared_prefill_supported(const lisa_shared_prefill_args& a) {
     if (a.d != 128 || a.chain_len < 1 || a.N > kTile * 1024) return false;
@@ -340,8 +347,7 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
             jobs.src[2 * k + 1] = make_view(a.links[k].kp); jobs.dst[2 * k + 1] = reinterpret_cast<__nv_bfloat16*>(base + l.kp_off[k]);
             jobs.H[2 * k + 1] = a.Hkv; jobs.r[2 * k + 1] = a.links[k].r;
         }
-        const int64_t total = (int64_t)a.B * a.Hq * a.N * (kPadRank / 8);
-        const int blocks = (int)std::min<int64_t>((total + 255) / 256, sm_count() * 16);
+        const dim3 grid((a.N + kPackPos - 1) / kPackPos, 2 * c, std::min(a.B, 65535));
         // beside the first emit, unless the per-kernel timing is on (then every kernel is timed on the caller's stream)
         if (!g_pt.on) {
             std::lock_guard<std::mutex> lock(g_side_mutex);
@@ -349,12 +355,12 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
             if (side) {
                 if ((e = cudaEventRecord(side->fork, s)) != cudaSuccess) return e;
                 if ((e = cudaStreamWaitEvent(side->stream, side->fork, 0)) != cudaSuccess) return e;
-                pack_lowrank_kernel<<<dim3(blocks, 2 * c), 256, 0, side->stream>>>(jobs, a.B, a.N);
+                pack_lowrank_kernel<<<grid, kPackThreads, 0, side->stream>>>(jobs, a.B, a.N);
                 if ((e = cudaGetLastError()) != cudaSuccess) return e;
                 if ((e = cudaEventRecord(side->join, side->stream)) != cudaSuccess) return e;
             }
         }
-        if (!side) pack_lowrank_kernel<<<dim3(blocks, 2 * c), 256, 0, s>>>(jobs, a.B, a.N);
+        if (!side) pack_lowrank_kernel<<<grid, kPackThreads, 0, s>>>(jobs, a.B, a.N);
         count_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

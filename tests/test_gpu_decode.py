@@ -157,6 +157,25 @@ def test_append_layouts_bit_exact(dtype):
     assert torch.equal(st.k.cpu()[:, :, :20], k1.permute(0, 2, 1, 3)) and torch.equal(st.v.cpu()[:, :, :20], v1.permute(0, 2, 1, 3))
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("B,n,Hkv,r,d,before", [(2, 64, 3, 21, 128, 0), (1, 130, 2, 32, 64, 5), (3, 63, 5, 1, 32, 3), (2, 200, 1, 20, 128, 41)])
+def test_append_prompt_layouts(dtype, B, n, Hkv, r, d, before):
+    """Prompts around the 64-position tiles of the transposed copy, odd start positions, one run past the capacity."""
+    g = torch.Generator().manual_seed(1)
+    kp, v = torch.randn(B, n, Hkv, r, generator=g).to(dtype), torch.randn(B, n, Hkv, d, generator=g).to(dtype)
+    L_cap = (before + n + 7) // 8 * 8
+    sh = lb.KVCacheLayer(lb.CACHE_SHARED, B, Hkv, L_cap, d, r, dtype=dtype)
+    lens = torch.tensor([before + (2 * b if b + 1 == B else 0) for b in range(B)], dtype=torch.int32)
+    lb.lisa_kvcache_append(sh, kp.cuda(), v.cuda(), lens.cuda())
+    exp_k, exp_v = torch.zeros(B, Hkv, r, L_cap, dtype=dtype), torch.zeros(B, Hkv, L_cap, d, dtype=dtype)
+    for b, s in enumerate(lens.tolist()):
+        m = min(n, L_cap - s)
+        exp_k[b, :, :, s:s + m] = kp[b, :m].permute(1, 2, 0)
+        exp_v[b, :, s:s + m] = v[b, :m].permute(1, 0, 2)
+    assert torch.equal(sh.k.cpu(), exp_k) and torch.equal(sh.v.cpu(), exp_v)
+    lb.lisa_check()   # (a run past the capacity was counted)
+
+
 def test_append_beyond_capacity_is_dropped_and_reported():
     B, Hkv, d, r, L_cap = 1, 1, 32, 4, 8
     sh = lb.KVCacheLayer(lb.CACHE_SHARED, B, Hkv, L_cap, d, r)
