@@ -1,80 +1,217 @@
 // General SIMT prefill of a LiSA shared layer (and, with chain_len == 0, of a standard layer).
 //
-// One CTA per query row (b, i).  Keys are visited in chunks of 128; thread t of a chunk owns key
-// j and rebuilds the whole score chain for that position in fp32: the anchor score q0.k0/sqrt(d) for
-// every head (Eq. 2), then per link the low-rank difference q'.k'/sqrt(r) (Eq. 3), the head-axis FFN
-// and the integration (Sec. 5.1, Eq. 4).  The chunk's final scores go to shared memory, get the causal
-// mask (keys j > i are never visited), an online softmax per head, and the product with V (Eq. 1).
-// The N x N x Hq scores are never stored.  Every integrate mode, activation, FFN depth, dtype and
-// shape in the supported range runs here; the tensor-core kernels cover the fast cases.
+// One CTA per query row (b, i).  Keys are visited in chunks of 128, whose score chain is rebuilt in fp32: the anchor score
+// q0.k0/sqrt(d) for every head (Eq. 2), then per link the low-rank difference q'.k'/sqrt(r) (Eq. 3), the head-axis FFN and the
+// integration (Sec. 5.1, Eq. 4).  The chunk's final scores get the causal mask (keys j > i are never visited), an online softmax
+// per head, and the product with V (Eq. 1).  The N x N x Hq scores are never stored.  Every integrate mode, activation, FFN depth,
+// dtype and shape in the supported range runs here; the tensor-core kernels cover the fast cases.
+//
+// A small prompt is bound by the latency of one CTA, so every phase spreads over all threads with its loads in flight together: the dot
+// products over (head, key, part of the row), the FFN over keys (weights in shared memory, registers for up to eight heads), the softmax over heads, the
+// product with V over (head, column) and, where these are few, ranges of keys.  4 heads of 32, N 128: 31 us with a thread per key
+// doing all of it, 10 now.
 #include "common.cuh"
 
 namespace lisa {
 namespace {
 
 constexpr int kChunk = 128;
-constexpr int kThreads = 128;
+constexpr int kMaxThreads = 512;   // a grid that leaves SMs idle runs with twice the threads of a larger one
 
 struct PrefillParams {
     int B, N, Hq, Hkv, d, c;
     TView q0, k0, v, o;
     LinkDev links[kMaxChain];
+    int vec_k0, vec_kp[kMaxChain];   // rows start on 16 bytes (fp32 and bf16 builds)
+    int w_off[kMaxChain], w_floats[kMaxChain];   // where a link's weights are staged in shared memory (floats; -1: read from memory), how many
 };
 
-__device__ __forceinline__ float ldw(const void* p, int idx, int dtype) { return p ? ld_elem(p, idx, dtype) : 0.f; }
+// DT: 0 = fp32, 1 = bf16, 2 = any mix, decided per access
+template <int DT>
+__device__ __forceinline__ float ld(const TView& t, int64_t i) {
+    if constexpr (DT == 0) return reinterpret_cast<const float*>(t.ptr)[i];
+    else if constexpr (DT == 1) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(t.ptr)[i]);
+    else return ld_elem(t.ptr, i, t.dtype);
+}
 
-// Sec. 5.1 at one position: a <- Integrate(Align(a), dl).  hid is scratch of kMaxHidden floats.
-__device__ void align_integrate(float* a, const float* dl, int Hq, const LinkDev& lk, float* hid) {
+// out[h][jj] = scale * (q[h] . row of key jj in KV head h / G) for the chunk's nk keys: neighbouring lanes take neighbouring V values of a
+// row (V values are 16 bytes, or one where rows do not start on 16 bytes), four rows of a lane are in flight, shuffles add up a row.
+template <int DT, int V>
+__device__ __forceinline__ void dots(float* out, const float* q, int q_ld, const TView& t, int64_t at, int Hq, int G, int nk, int n, float scale) {
+    constexpr int U = 4;
+    const int lanes = (n + V - 1) / V;
+    const int lpr = lanes <= 1 ? 1 : lanes >= 32 ? 32 : 1 << (32 - __clz(lanes - 1));   // lanes per row
+    const int sub = threadIdx.x & (lpr - 1), grp = threadIdx.x / lpr, groups = blockDim.x / lpr, total = Hq * kChunk;
+    for (int r0 = 0; r0 < total; r0 += U * groups) {
+        float part[U];
+        int64_t row[U];
+        const float* qh[U];
+        bool ok[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int rr = r0 + u * groups + grp, h = rr / kChunk, jj = rr % kChunk;
+            ok[u] = rr < total && jj < nk;
+            row[u] = at + jj * t.sn + (G == 1 ? h : h / G) * t.sh;
+            qh[u] = q + h * q_ld;
+            part[u] = 0.f;
+        }
+        for (int x = sub * V; x < n; x += lpr * V) {   // (once, unless rows of more than 32 values are read one by one)
+            if constexpr (V == 4) {
+                float4 v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) v[u] = ok[u] ? *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(t.ptr) + row[u] + x) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (!ok[u]) continue;
+                    const float4 w = *reinterpret_cast<const float4*>(qh[u] + x);
+                    part[u] = fmaf(w.x, v[u].x, part[u]); part[u] = fmaf(w.y, v[u].y, part[u]);
+                    part[u] = fmaf(w.z, v[u].z, part[u]); part[u] = fmaf(w.w, v[u].w, part[u]);
+                }
+            } else if constexpr (V == 8) {
+                uint4 v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) v[u] = ok[u] ? *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(t.ptr) + row[u] + x) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (!ok[u]) continue;
+                    const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        part[u] = fmaf(qh[u][x + 2 * j], __uint_as_float(w[j] << 16), part[u]);
+                        part[u] = fmaf(qh[u][x + 2 * j + 1], __uint_as_float(w[j] & 0xffff0000u), part[u]);
+                    }
+                }
+            } else {
+                float v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) v[u] = ok[u] ? ld<DT>(t, row[u] + x) : 0.f;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (ok[u]) part[u] = fmaf(qh[u][x], v[u], part[u]);
+            }
+        }
+        for (int off = lpr >> 1; off > 0; off >>= 1)
+#pragma unroll
+            for (int u = 0; u < U; ++u) part[u] += __shfl_xor_sync(0xffffffffu, part[u], off);
+        if (sub == 0)
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (ok[u]) out[r0 + u * groups + grp] = part[u] * scale;
+    }
+}
+template <int DT>
+__device__ __forceinline__ void dots_any(float* out, const float* q, int q_ld, const TView& t, int64_t at, int Hq, int G, int nk, int n, float scale, int vec) {
+    if (DT == 0 && vec && n % 4 == 0) dots<DT, DT == 0 ? 4 : 1>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
+    else if (DT == 1 && vec && n % 8 == 0) dots<DT, DT == 1 ? 8 : 1>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
+    else dots<DT, 1>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
+}
+
+// A link's FFN weights: fp32 in shared memory (SM; w1, b1, w2, b2 one after the other), or where the model keeps them.
+template <bool SM>
+struct Weights {
+    const float *p1, *pb1, *p2, *pb2;
+    const LinkDev& l;
+    __device__ Weights(const float* s, const LinkDev& link, int h_in, int Hq) : p1(s), pb1(s + h_in * link.m), p2(pb1 + link.m), pb2(p2 + link.m * Hq), l(link) {}
+    __device__ __forceinline__ float w1(int i) const { return SM ? p1[i] : ld_elem(l.w1, i, l.w_dtype); }
+    __device__ __forceinline__ float b1(int i) const { return SM ? pb1[i] : l.b1 ? ld_elem(l.b1, i, l.w_dtype) : 0.f; }
+    __device__ __forceinline__ float w2(int i) const { return SM ? p2[i] : ld_elem(l.w2, i, l.w_dtype); }
+    __device__ __forceinline__ float b2(int i) const { return SM ? pb2[i] : l.b2 ? ld_elem(l.b2, i, l.w_dtype) : 0.f; }
+};
+
+// Sec. 5.1 at one position: a <- Integrate(Align(a), dl); a and dl are columns of shared memory, one head every kChunk floats.  HQ > 0: that
+// many heads, in registers.
+template <int HQ, bool SM>
+__device__ __forceinline__ void align_integrate(float* a, const float* dl, int n_heads, const Weights<SM>& w) {
+    const int Hq = HQ ? HQ : n_heads;
+    const LinkDev& lk = w.l;
     if (lk.integrate == LISA_INTEGRATE_PLUS) {
-        for (int g = 0; g < Hq; ++g) a[g] += dl[g];
+        for (int g = 0; g < Hq; ++g) a[g * kChunk] += dl[g * kChunk];
         return;
     }
     const int m = lk.m;
-    for (int u = 0; u < m; ++u) {
-        float s = ldw(lk.b1, u, lk.w_dtype);
-        for (int x = 0; x < Hq; ++x) s = fmaf(a[x], ld_elem(lk.w1, (int64_t)x * m + u, lk.w_dtype), s);
-        if (lk.integrate == LISA_INTEGRATE_CONCAT)
-            for (int x = 0; x < Hq; ++x) s = fmaf(dl[x], ld_elem(lk.w1, (int64_t)(Hq + x) * m + u, lk.w_dtype), s);
-        hid[u] = s;
+    const bool concat = lk.integrate == LISA_INTEGRATE_CONCAT, two = lk.ffn_layers == 2;
+    const int act = lk.act;
+    constexpr int CAP = HQ ? HQ : kMaxHeads;
+    float x[CAP], y[CAP];
+#pragma unroll(HQ ? HQ : 1)
+    for (int h = 0; h < Hq; ++h) {
+        x[h] = a[h * kChunk];
+        y[h] = two ? w.b2(h) : 0.f;
     }
-    if (lk.ffn_layers == 1) {
-        for (int g = 0; g < Hq; ++g) a[g] = hid[g];
-    } else {
-        for (int u = 0; u < m; ++u) hid[u] = act_apply(hid[u], lk.act);
-        for (int g = 0; g < Hq; ++g) {
-            float s = ldw(lk.b2, g, lk.w_dtype);
-            for (int u = 0; u < m; ++u) s = fmaf(hid[u], ld_elem(lk.w2, (int64_t)u * Hq + g, lk.w_dtype), s);
-            a[g] = s;
+    auto units = [&](auto activate) {
+#pragma unroll(HQ ? 4 : 1)
+        for (int u = 0; u < m; ++u) {
+            float s = w.b1(u);
+#pragma unroll(HQ ? HQ : 4)
+            for (int h = 0; h < Hq; ++h) s = fmaf(x[h], w.w1(h * m + u), s);
+            if (concat)
+#pragma unroll(HQ ? HQ : 4)
+                for (int h = 0; h < Hq; ++h) s = fmaf(dl[h * kChunk], w.w1((Hq + h) * m + u), s);
+            if (two) {
+                s = activate(s);
+#pragma unroll(HQ ? HQ : 4)
+                for (int g = 0; g < Hq; ++g) y[g] = fmaf(s, w.w2(u * Hq + g), y[g]);
+            } else if constexpr (HQ > 0) {
+#pragma unroll
+                for (int g = 0; g < HQ; ++g) y[g] = g == u ? s : y[g];
+            } else {
+                y[u] = s;   // one layer: m == Hq
+            }
         }
-    }
-    if (lk.integrate == LISA_INTEGRATE_ADD)
-        for (int g = 0; g < Hq; ++g) a[g] += dl[g];
+    };
+    const float floor = act == LISA_ACT_RELU ? 0.f : -INFINITY;
+    if (act == LISA_ACT_SILU) units([](float s) { return act_apply(s, LISA_ACT_SILU); });
+    else units([floor](float s) { return fmaxf(s, floor); });
+#pragma unroll(HQ ? HQ : 1)
+    for (int g = 0; g < Hq; ++g) a[g * kChunk] = lk.integrate == LISA_INTEGRATE_ADD ? y[g] + dl[g * kChunk] : y[g];
 }
 
-__global__ void __launch_bounds__(kThreads) generic_prefill_kernel(const __grid_constant__ PrefillParams p) {
-    extern __shared__ float smem[];
-    const int b = blockIdx.y, i = blockIdx.x, tid = threadIdx.x;
-    const int Hq = p.Hq, d = p.d, G = p.Hq / p.Hkv;
-    float* q0_s = smem;                       // [Hq*d]
-    float* o_s = q0_s + Hq * d;               // [Hq*d]
-    float* s_s = o_s + Hq * d;                // [Hq*kChunk]
-    float* m_s = s_s + Hq * kChunk;           // [Hq]
+template <int DT, int HQ>
+__global__ void __launch_bounds__(kMaxThreads) generic_prefill_kernel(const __grid_constant__ PrefillParams p) {
+    extern __shared__ __align__(16) float smem[];
+    const int b = blockIdx.y, i = (int)(gridDim.x - 1 - blockIdx.x), tid = threadIdx.x;   // the longest rows first
+    const int Hq = HQ ? HQ : p.Hq, d = p.d, G = Hq / p.Hkv;
+    const int warp = tid >> 5, lane = tid & 31, kThreads = blockDim.x, kWarps = kThreads / 32;
+    float* q0_s = smem;                       // [Hq][d]
+    float* o_s = q0_s + Hq * d;               // [Hq][d]
+    float* s_s = o_s + Hq * d;                // [Hq][kChunk] scores of the chunk
+    float* d_s = s_s + Hq * kChunk;           // [Hq][kChunk] a link's difference; then partial sums of the product with V
+    float* m_s = d_s + Hq * kChunk;           // [Hq]
     float* l_s = m_s + Hq;                    // [Hq]
     float* sc_s = l_s + Hq;                   // [Hq]
-    float* qp_s = sc_s + Hq;                  // [c][Hq*kMaxRank]
+    float* qp_s = sc_s + Hq;                  // [c][Hq][kMaxRank]
 
-    for (int e = tid; e < Hq * d; e += kThreads) {
-        const int h = e / d, x = e % d;
-        q0_s[e] = ld_elem(p.q0.ptr, b * p.q0.sb + i * p.q0.sn + h * p.q0.sh + x, p.q0.dtype);
-        o_s[e] = 0.f;
-    }
-    for (int k = 0; k < p.c; ++k) {
-        const LinkDev& lk = p.links[k];
-        for (int e = tid; e < Hq * lk.r; e += kThreads) {
-            const int h = e / lk.r, x = e % lk.r;
-            qp_s[k * Hq * kMaxRank + h * kMaxRank + x] =
-                ld_elem(lk.qp.ptr, b * lk.qp.sb + i * lk.qp.sn + h * lk.qp.sh + x, lk.qp.dtype);
+    // everything a CTA reads once, as one flat range: one round of loads for a small layer, not one per tensor
+    chain_release();
+    chain_wait();
+    const int n_q0 = Hq * d;
+    int total = n_q0;
+    for (int k = 0; k < p.c; ++k) total += Hq * p.links[k].r + p.w_floats[k];
+    for (int e0 = tid; e0 < total; e0 += kThreads) {
+        int e = e0;
+        if (e < n_q0) {
+            const int h = e / d, x = e % d;
+            q0_s[e] = ld<DT>(p.q0, b * p.q0.sb + i * p.q0.sn + h * p.q0.sh + x);
+            o_s[e] = 0.f;
+            continue;
         }
+        e -= n_q0;
+        int k = 0;
+        while (e >= Hq * p.links[k].r + p.w_floats[k]) e -= Hq * p.links[k].r + p.w_floats[k++];
+        const LinkDev& lk = p.links[k];
+        if (e < Hq * lk.r) {
+            const int h = e / lk.r, x = e % lk.r;
+            qp_s[k * Hq * kMaxRank + h * kMaxRank + x] = ld<DT>(lk.qp, b * lk.qp.sb + i * lk.qp.sn + h * lk.qp.sh + x);
+            continue;
+        }
+        e -= Hq * lk.r;   // w1, b1, w2, b2 one after the other
+        const int n1 = (lk.integrate == LISA_INTEGRATE_CONCAT ? 2 : 1) * Hq * lk.m, n2 = lk.m * Hq;
+        float v;
+        if (e < n1) v = ld_elem(lk.w1, e, lk.w_dtype);
+        else if (e < n1 + lk.m) v = lk.b1 ? ld_elem(lk.b1, e - n1, lk.w_dtype) : 0.f;
+        else if (e < n1 + lk.m + n2) v = ld_elem(lk.w2, e - n1 - lk.m, lk.w_dtype);
+        else v = lk.b2 ? ld_elem(lk.b2, e - n1 - lk.m - n2, lk.w_dtype) : 0.f;
+        smem[p.w_off[k] + e] = v;
     }
     for (int h = tid; h < Hq; h += kThreads) {
         m_s[h] = -INFINITY;
@@ -82,42 +219,30 @@ __global__ void __launch_bounds__(kThreads) generic_prefill_kernel(const __grid_
     }
     __syncthreads();
 
-    float a[kMaxHeads], dl[kMaxHeads], hid[kMaxHidden];
     const float inv_sqrt_d = rsqrtf((float)d);
-    const int warp = tid >> 5, lane = tid & 31;
-
+    // the product with V: a thread owns output columns, or, where there are fewer of these than threads, one column and a range of keys
+    const int cols = Hq * d, splits = cols < kThreads ? min(kThreads / cols, max(1, Hq * kChunk / cols)) : 1;
     for (int j0 = 0; j0 <= i; j0 += kChunk) {
-        const int j = j0 + tid;
-        if (j <= i) {
-            for (int h = 0; h < Hq; ++h) {
-                const int64_t kb = b * p.k0.sb + (int64_t)j * p.k0.sn + (h / G) * p.k0.sh;
-                float s = 0.f;
-                for (int x = 0; x < d; ++x) s = fmaf(q0_s[h * d + x], ld_elem(p.k0.ptr, kb + x, p.k0.dtype), s);
-                a[h] = s * inv_sqrt_d;
+        const int nk = min(kChunk, i + 1 - j0);
+        dots_any<DT>(s_s, q0_s, d, p.k0, b * p.k0.sb + (int64_t)j0 * p.k0.sn, Hq, G, nk, d, inv_sqrt_d, p.vec_k0);
+        for (int k = 0; k < p.c; ++k) {
+            const LinkDev& lk = p.links[k];
+            dots_any<DT>(d_s, qp_s + k * Hq * kMaxRank, kMaxRank, lk.kp, b * lk.kp.sb + (int64_t)j0 * lk.kp.sn, Hq, G, nk, lk.r, rsqrtf((float)lk.r), p.vec_kp[k]);
+            __syncthreads();
+            const int h_in = (lk.integrate == LISA_INTEGRATE_CONCAT ? 2 : 1) * Hq;
+            if (tid < nk) {
+                if (p.w_off[k] >= 0) align_integrate<HQ>(s_s + tid, d_s + tid, Hq, Weights<true>(smem + p.w_off[k], lk, h_in, Hq));
+                else align_integrate<HQ>(s_s + tid, d_s + tid, Hq, Weights<false>(nullptr, lk, h_in, Hq));
             }
-            for (int k = 0; k < p.c; ++k) {
-                const LinkDev& lk = p.links[k];
-                const float inv_sqrt_r = rsqrtf((float)lk.r);
-                for (int h = 0; h < Hq; ++h) {
-                    const int64_t kb = b * lk.kp.sb + (int64_t)j * lk.kp.sn + (h / G) * lk.kp.sh;
-                    const float* qrow = qp_s + k * Hq * kMaxRank + h * kMaxRank;
-                    float s = 0.f;
-                    for (int x = 0; x < lk.r; ++x) s = fmaf(qrow[x], ld_elem(lk.kp.ptr, kb + x, lk.kp.dtype), s);
-                    dl[h] = s * inv_sqrt_r;
-                }
-                align_integrate(a, dl, Hq, lk, hid);
-            }
-            for (int h = 0; h < Hq; ++h) s_s[h * kChunk + tid] = a[h];
-        } else {
-            for (int h = 0; h < Hq; ++h) s_s[h * kChunk + tid] = -INFINITY;  // causal mask, after the chain
+            __syncthreads();
         }
-        __syncthreads();
-        for (int h = warp; h < Hq; h += kThreads / 32) {
+        if (p.c == 0) __syncthreads();
+        for (int h = warp; h < Hq; h += kWarps) {
             float v[kChunk / 32];
             float cmax = -INFINITY;
 #pragma unroll
             for (int t = 0; t < kChunk / 32; ++t) {
-                v[t] = s_s[h * kChunk + lane + 32 * t];
+                v[t] = lane + 32 * t < nk ? s_s[h * kChunk + lane + 32 * t] : -INFINITY;   // causal mask, after the chain
                 cmax = fmaxf(cmax, v[t]);
             }
 #pragma unroll
@@ -133,6 +258,7 @@ __global__ void __launch_bounds__(kThreads) generic_prefill_kernel(const __grid_
             }
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            __syncwarp();
             if (lane == 0) {
                 const float sc = __expf(m_old - m_new);
                 sc_s[h] = sc;
@@ -141,26 +267,48 @@ __global__ void __launch_bounds__(kThreads) generic_prefill_kernel(const __grid_
             }
         }
         __syncthreads();
-        if (tid < d) {
-            const int nk = min(kChunk, i + 1 - j0);
-            for (int h = 0; h < Hq; ++h) {
-                float acc = o_s[h * d + tid] * sc_s[h];
-                const int64_t vb = b * p.v.sb + (int64_t)j0 * p.v.sn + (h / G) * p.v.sh + tid;
-                for (int jj = 0; jj < nk; ++jj)
-                    acc = fmaf(s_s[h * kChunk + jj], ld_elem(p.v.ptr, vb + (int64_t)jj * p.v.sn, p.v.dtype), acc);
-                o_s[h * d + tid] = acc;
-            }
+        for (int e = tid; e < cols * splits; e += kThreads) {
+            const int part = e / cols, col = e % cols, h = col / d, x = col % d;
+            const int k0 = nk * part / splits, k1 = nk * (part + 1) / splits;
+            const int64_t vb = b * p.v.sb + (int64_t)j0 * p.v.sn + (h / G) * p.v.sh + x;
+            float acc = 0.f;
+#pragma unroll 16
+            for (int jj = k0; jj < k1; ++jj) acc = fmaf(s_s[h * kChunk + jj], ld<DT>(p.v, vb + (int64_t)jj * p.v.sn), acc);
+            if (splits == 1) o_s[col] = o_s[col] * sc_s[h] + acc;
+            else d_s[e] = acc;
         }
         __syncthreads();
+        if (splits > 1) {
+            if (tid < cols) {
+                float acc = o_s[tid] * sc_s[tid / d];
+                for (int q = 0; q < splits; ++q) acc += d_s[q * cols + tid];
+                o_s[tid] = acc;
+            }
+            __syncthreads();
+        }
     }
-    if (tid < d)
-        for (int h = 0; h < Hq; ++h)
-            st_elem(const_cast<void*>(p.o.ptr), b * p.o.sb + i * p.o.sn + h * p.o.sh + tid, p.o.dtype,
-                    o_s[h * d + tid] / l_s[h]);
+    for (int e = tid; e < cols; e += kThreads) {
+        const int h = e / d, x = e % d;
+        st_elem(const_cast<void*>(p.o.ptr), b * p.o.sb + i * p.o.sn + h * p.o.sh + x, p.o.dtype, o_s[e] / l_s[h]);
+    }
 }
 
-size_t smem_bytes(int Hq, int d, int c) {
-    return sizeof(float) * ((size_t)2 * Hq * d + (size_t)Hq * kChunk + 3 * (size_t)Hq + (size_t)c * Hq * kMaxRank);
+size_t smem_floats(int Hq, int d, int c) {
+    return (size_t)2 * Hq * d + (size_t)2 * Hq * kChunk + 3 * (size_t)Hq + (size_t)c * Hq * kMaxRank;
+}
+constexpr size_t kMaxSmemFloats = 232448 / sizeof(float);
+
+bool vec_rows(const lisa_tensor& t) {
+    const int64_t n = t.dtype == LISA_BF16 ? 8 : 4;
+    return t.stride_b % n == 0 && t.stride_n % n == 0 && t.stride_h % n == 0;   // (the pointer is: checked by the entry points)
+}
+
+template <int DT>
+void* pick(int Hq) {
+    return Hq == 2   ? reinterpret_cast<void*>(generic_prefill_kernel<DT, 2>)
+           : Hq == 4 ? reinterpret_cast<void*>(generic_prefill_kernel<DT, 4>)
+           : Hq == 8 ? reinterpret_cast<void*>(generic_prefill_kernel<DT, 8>)
+                     : reinterpret_cast<void*>(generic_prefill_kernel<DT, 0>);
 }
 
 }  // namespace
@@ -169,14 +317,31 @@ cudaError_t launch_generic_prefill(const lisa_shared_prefill_args& a, cudaStream
     PrefillParams p;
     p.B = a.B; p.N = a.N; p.Hq = a.Hq; p.Hkv = a.Hkv; p.d = a.d; p.c = a.chain_len;
     p.q0 = make_view(a.q0); p.k0 = make_view(a.k0); p.v = make_view(a.v); p.o = make_view(a.o);
-    for (int k = 0; k < a.chain_len; ++k) p.links[k] = make_link(a.links[k]);
-    const size_t smem = smem_bytes(a.Hq, a.d, a.chain_len);
-    cudaError_t e = cudaFuncSetAttribute(generic_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    p.vec_k0 = vec_rows(a.k0);
+    int dt = a.q0.dtype;
+    bool same = a.k0.dtype == dt && a.v.dtype == dt;
+    size_t floats = smem_floats(a.Hq, a.d, a.chain_len);
+    for (int k = 0; k < a.chain_len; ++k) {
+        const lisa_link& l = a.links[k];
+        p.links[k] = make_link(l);
+        p.vec_kp[k] = vec_rows(l.kp);
+        same = same && l.qp.dtype == dt && l.kp.dtype == dt;
+        p.w_off[k] = -1;
+        p.w_floats[k] = 0;
+        if (l.integrate == LISA_INTEGRATE_PLUS) continue;
+        // staged while a CTA keeps to half an SM's shared memory (or is beyond that anyway)
+        const size_t n = (size_t)(l.integrate == LISA_INTEGRATE_CONCAT ? 2 : 1) * a.Hq * l.m + l.m + (l.ffn_layers == 2 ? (size_t)l.m * a.Hq + a.Hq : 0);
+        const size_t room = floats > kMaxSmemFloats / 2 - 512 ? kMaxSmemFloats : kMaxSmemFloats / 2 - 512;
+        if (floats + n <= room) { p.w_off[k] = (int)floats; p.w_floats[k] = (int)n; floats += n; }
+    }
+    const void* kernel = !same ? pick<2>(a.Hq) : dt == LISA_BF16 ? pick<1>(a.Hq) : pick<0>(a.Hq);
+    const size_t smem = floats * sizeof(float);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.N, a.B);
-    generic_prefill_kernel<<<grid, kThreads, smem, s>>>(p);
+    const int threads = (int64_t)a.N * a.B <= 2 * (int64_t)sm_count() ? kMaxThreads : kMaxThreads / 2;
+    e = launch_chained(reinterpret_cast<void (*)(PrefillParams)>(const_cast<void*>(kernel)), dim3(a.N, a.B), dim3(threads), smem, s, p);
     count_launches(1);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace lisa
