@@ -60,6 +60,12 @@ int* status_words();
 // Streaming multiprocessors of the current device (cached per device; 1 if the query fails).
 int sm_count();
 
+// Opts a kernel into `bytes` of dynamic shared memory on the current device (and, with all_shared, into the largest carveout); what has been
+// set before is remembered, per device, so that a repeated launch does not pay for the runtime call.
+cudaError_t allow_smem(const void* kernel, size_t bytes, bool all_shared = false);
+template <typename K>
+cudaError_t allow_smem(K* kernel, size_t bytes, bool all_shared = false) { return allow_smem(reinterpret_cast<const void*>(kernel), bytes, all_shared); }
+
 // Adds n to the process-wide count of kernels enqueued by the library.
 void count_launches(int n);
 
@@ -90,6 +96,7 @@ struct TcFlashArgs {
     // after it was read).
     void* carry = nullptr;
     int plane_row0 = -1;  // first query row the plane / emit_plane / carry buffers hold (-1: qt_begin * 128)
+    bool chained = false; // launch as part of a programmatic chain (see launch_kernel)
 };
 bool tc_flash_supported(const TcFlashArgs& a);
 cudaError_t launch_tc_flash(const TcFlashArgs& a, cudaStream_t s);
@@ -103,6 +110,7 @@ struct TcAlignArgs {
     const lisa_link* links;
     int ctas = 0;  // grid size (0 = three per SM)
     int row0 = -1;  // first query row the planes hold (-1: qt_begin * 128)
+    bool chained = false;    // launch as part of a programmatic chain
     bool store_all = false;  // every link's output is stored (times log2 e): link k (0-based) into planes[k]
 };
 bool tc_align_supported(int Hq, const lisa_link* links, int chain);
@@ -122,6 +130,7 @@ struct TcAlignLinkArgs {
     // plane_d with a geometry of its own (0 / -1: the same as plane_x): carried scores as plane_x, a wave's plane as plane_d
     int64_t d_plane_rows = 0, d_plane_cols = 0;
     int d_row0 = -1;
+    bool chained = false;   // launch as part of a programmatic chain
 };
 bool tc_align_concat_supported(int Hq, const lisa_link* links, int chain);
 bool tc_align_link_supported(int Hq, const lisa_link* links, int chain);
@@ -136,14 +145,18 @@ cudaError_t launch_tc_align_link(const TcAlignLinkArgs& a, cudaStream_t s);
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... Params>
-cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const Params&... p) {
+cudaError_t launch_kernel(bool chained, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const Params&... p) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr; cfg.numAttrs = 1;
+    cfg.attrs = &attr; cfg.numAttrs = chained ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, p...);
+}
+template <typename... Params>
+cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const Params&... p) {
+    return launch_kernel(true, kernel, grid, block, smem, s, p...);
 }
 
 // Tensor-core prefill of a shared layer (tc_prefill.cu): emit planes -> align -> attention, wave by wave.

@@ -423,11 +423,6 @@ void carve_workspace(DecodeParams& p, void* ws) {
     p.ws_o = p.ws_l + npad;
 }
 
-template <typename K>
-cudaError_t set_smem(K kernel, size_t smem) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 // Partial results (chunks over all sequences) a call may produce: one per 128 positions, or, for small batches, whose chunks
 // are cut finer, one per 32 as long as the scratch stays below kSmallScratch.  Grows with B and L, so that a buffer sized for the
 // largest step serves every smaller one.
@@ -470,7 +465,7 @@ cudaError_t launch_shared_fast(DecodeParams& p, cudaStream_t s) {
         if (three_per_sm(ctas)) kernel = shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3>;
     const size_t smem = shared_fast_layout(HQ, HG, CH, ENG, p.m, HQ / p.Hkv).total;
     p.prefetch = ctas <= 2 * (int64_t)sm_count();   // a grid that is resident at once
-    cudaError_t e = set_smem(kernel, smem);
+    cudaError_t e = allow_smem(kernel, smem);
     return e != cudaSuccess ? e : launch_chained(kernel, dim3(p.n_chunks, HQ / HG, p.B), dim3(kDecodeThreads), smem, s, p);
 }
 
@@ -561,7 +556,7 @@ cudaError_t launch_shared_decode(const lisa_shared_decode_args& a, void* ws, cud
         set_chunk(p, kChunk, ws);
         const size_t smem = shared_decode_smem(p.Hq, p.m, p.integrate);
         auto kernel = p.row_bf16 ? shared_decode_chunk_kernel<true> : shared_decode_chunk_kernel<false>;
-        if ((e = set_smem(kernel, smem)) != cudaSuccess) return e;
+        if ((e = allow_smem(kernel, smem)) != cudaSuccess) return e;
         e = launch_chained(kernel, dim3(p.n_chunks, p.B), dim3(kThreads), smem, s, p);
     }
     return e == cudaSuccess ? launch_merge(p, s) : e;
@@ -593,12 +588,12 @@ cudaError_t launch_anchor_decode(const lisa_anchor_args& a, void* ws, cudaStream
         p.prefetch = (int64_t)p.n_chunks * p.B * (p.Hkv / kv) <= 2 * want;   // a grid that is resident at once
         const size_t smem = anchor_fast_smem(p.heads, p.chunk, G);
         auto kernel = p.chunk == 128 ? anchor_decode_fast_kernel<128> : p.chunk == 64 ? anchor_decode_fast_kernel<64> : anchor_decode_fast_kernel<32>;
-        if ((e = set_smem(kernel, smem)) != cudaSuccess) return e;
+        if ((e = allow_smem(kernel, smem)) != cudaSuccess) return e;
         e = launch_chained(kernel, dim3(p.n_chunks, p.Hkv / kv, p.B), dim3(kDecodeThreads), smem, s, p);
     } else {
         set_chunk(p, kChunk, ws);
         const size_t smem = sizeof(float) * ((size_t)p.Hq * kChunk + (size_t)p.Hq * p.d);
-        if ((e = set_smem(anchor_decode_chunk_kernel, smem)) != cudaSuccess) return e;
+        if ((e = allow_smem(anchor_decode_chunk_kernel, smem)) != cudaSuccess) return e;
         e = launch_chained(anchor_decode_chunk_kernel, dim3(p.n_chunks, p.B), dim3(kThreads), smem, s, p);
     }
     return e == cudaSuccess ? launch_merge(p, s) : e;

@@ -336,7 +336,7 @@ cudaError_t launch_generic_prefill(const lisa_shared_prefill_args& a, cudaStream
     }
     const void* kernel = !same ? pick<2>(a.Hq) : dt == LISA_BF16 ? pick<1>(a.Hq) : pick<0>(a.Hq);
     const size_t smem = floats * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kernel, smem);
     if (e != cudaSuccess) return e;
     const int threads = (int64_t)a.N * a.B <= 2 * (int64_t)sm_count() ? kMaxThreads : kMaxThreads / 2;
     e = launch_chained(reinterpret_cast<void (*)(PrefillParams)>(const_cast<void*>(kernel)), dim3(a.N, a.B), dim3(threads), smem, s, p);

@@ -2,6 +2,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 
 #include "common.cuh"
 
@@ -36,6 +37,32 @@ int sm_count() {
         cached[dev] = n;
     }
     return cached[dev];
+}
+
+cudaError_t allow_smem(const void* kernel, size_t bytes, bool all_shared) {
+    struct Entry { std::atomic<const void*> kernel{nullptr}; std::atomic<size_t> bytes{0}; };
+    constexpr int kSlots = 256, kDevices = 16;
+    static Entry table[kDevices][kSlots];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    Entry* slot = nullptr;
+    if (dev >= 0 && dev < kDevices) {
+        size_t h = (reinterpret_cast<uintptr_t>(kernel) >> 4) * 0x9e3779b97f4a7c15ull >> 56;
+        for (int i = 0; i < kSlots && !slot; ++i, h = (h + 1) % kSlots) {
+            const void* have = table[dev][h].kernel.load(std::memory_order_acquire);
+            if (!have && !table[dev][h].kernel.compare_exchange_strong(have, kernel)) { if (have != kernel) continue; }
+            if (!have || have == kernel) slot = &table[dev][h];
+        }
+        if (slot && slot->bytes.load(std::memory_order_acquire) >= bytes + 1) return cudaSuccess;
+    }
+    static std::mutex mutex;   // the limit only ever grows, whatever sizes several threads ask for
+    std::lock_guard<std::mutex> lock(mutex);
+    if (slot && slot->bytes.load(std::memory_order_relaxed) >= bytes + 1) return cudaSuccess;
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)) != cudaSuccess) return e;
+    if (all_shared && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
+    if (slot) slot->bytes.store(bytes + 1, std::memory_order_release);
+    return cudaSuccess;
 }
 
 namespace {
@@ -314,6 +341,7 @@ static lisa_status_t shared_prefill_impl(const lisa_shared_prefill_args* a, lisa
     if (!g_force_general.load() && a->d == 128 && a->chain_len == 0) {
         TcFlashArgs f{a->B, a->N, a->Hq, a->Hkv, 128, a->q0, a->k0, a->v, a->o, 1.0f / sqrtf((float)a->d), nullptr, 0, 0,
                       0, (a->N + 127) / 128};
+        f.chained = (int64_t)a->B * a->Hq * f.qt_count <= 2 * (int64_t)sm_count();
         if (tc_flash_supported(f)) {
             cudaError_t e = launch_tc_flash(f, s);
             return e == cudaSuccess ? LISA_OK : cuda_fail(e);

@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(NT, MIN_CTAS)
 tc_align_kernel(const __grid_constant__ AlignParams p) {
     extern __shared__ __align__(16) uint8_t smem[];
     const int c = p.chain;
+    chain_release();
     uint8_t* sW = smem;                               // per link: W1 fragments, W2 fragments, b1[64], b2[32]
     uint8_t* sScr = sW + c * LINK_BYTES;              // per warp: STAGES buffers of c planes x [32 heads][64 B]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -75,6 +76,7 @@ tc_align_kernel(const __grid_constant__ AlignParams p) {
         stage_link_fragments(sW + k * LINK_BYTES, p.w1[k], p.b1[k], p.w2[k], p.b2[k], p.w_dtype[k], p.kind[k], out_scale, tid, NT);
     }
     __syncthreads();
+    chain_wait();   // from here on: the planes, which earlier kernels of the stream produce
 
     // Parameter fields of the main loop, read once into registers: behind the asm statements (memory clobbers) the
     // compiler would re-read them from the parameter bank every time, the per-link ones through a run-time index.
@@ -413,18 +415,15 @@ cudaError_t launch_tc_align(const TcAlignArgs& a, cudaStream_t stream) {
         kernel = act == LISA_ACT_RELU ? LISA_ALIGN_REGW(LISA_ACT_RELU) : act == LISA_ACT_SILU ? LISA_ALIGN_REGW(LISA_ACT_SILU) : LISA_ALIGN_REGW(LISA_ACT_NONE);
 #undef LISA_ALIGN_REGW
     }
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kernel, smem);
     if (e != cudaSuccess) return e;
     const int64_t total_units = (int64_t)p.units_per_batch * a.B;
     if (total_units <= 0 || total_units > 0x7fffffff) return cudaErrorInvalidValue;
-    int dev = 0, sms = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int max_ctas = a.ctas > 0 ? a.ctas : sms * ctas_per_sm;
+    const int max_ctas = a.ctas > 0 ? a.ctas : sm_count() * ctas_per_sm;
     dim3 grid((unsigned)std::min<int64_t>((total_units + 3) / 4, max_ctas));  // at least a unit per warp
-    kernel<<<grid, threads, smem, stream>>>(p);
+    e = launch_kernel(a.chained, kernel, grid, dim3(threads), smem, stream, p);
     count_launches(1);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace lisa

@@ -324,7 +324,7 @@ cudaError_t launch_shape(const LinkParams& p, int act, unsigned grid, cudaStream
     auto kernel = act == LISA_ACT_RELU   ? tc_align_link_kernel<NH, CONCAT, CHUNK, NCHUNK, LISA_ACT_RELU, NTHREADS>
                   : act == LISA_ACT_SILU ? tc_align_link_kernel<NH, CONCAT, CHUNK, NCHUNK, LISA_ACT_SILU, NTHREADS>
                                          : tc_align_link_kernel<NH, CONCAT, CHUNK, NCHUNK, LISA_ACT_NONE, NTHREADS>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kernel, smem);
     if (e != cudaSuccess) return e;
     kernel<<<grid, NTHREADS, smem, stream>>>(p);
     return cudaGetLastError();

@@ -161,6 +161,10 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // What comes before -- barriers, tensor memory -- overlaps the tail of the kernel before this one.  The release comes second, so that a
+    // kernel further down the chain starts only after everything that preceded the call, weights it reads before its own wait included.
+    chain_wait();
+    chain_release();
     const uint32_t tmem_base = *tmem_slot;
     const uint32_t tmem_O = tmem_base + 128;
 
@@ -599,11 +603,8 @@ cudaError_t launch_tc_flash(const TcFlashArgs& a, cudaStream_t stream) {
 #define LISA_LAUNCH_FLASH(KD_, PL_)                                                                                       \
     do {                                                                                                                   \
         auto kern = tc_flash_kernel<KD_, PL_>;                                                                             \
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<KD_, PL_>::TOTAL)) != cudaSuccess) \
-            return e;                                                                                                      \
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) \
-            return e;                                                                                                      \
-        kern<<<grid, kThreads, Smem<KD_, PL_>::TOTAL, stream>>>(p, tmQ, tmK, tmV, tmY, tmC);                                    \
+        if ((e = allow_smem(kern, Smem<KD_, PL_>::TOTAL, true)) != cudaSuccess) return e;                                  \
+        e = launch_kernel(a.chained, kern, grid, dim3(kThreads), Smem<KD_, PL_>::TOTAL, stream, p, tmQ, tmK, tmV, tmY, tmC); \
     } while (0)
     if (a.emit_plane) {
         if (a.kd == 128) LISA_LAUNCH_FLASH(128, MODE_EMIT);
@@ -615,7 +616,7 @@ cudaError_t launch_tc_flash(const TcFlashArgs& a, cudaStream_t stream) {
     else return cudaErrorInvalidValue;  // 128-wide scores plus a plane do not fit shared memory
 #undef LISA_LAUNCH_FLASH
     count_launches(1);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace lisa

@@ -39,6 +39,8 @@ struct PackJobs {
 constexpr int kPackPos = 8, kPackThreads = kPackPos * 32;
 __global__ void __launch_bounds__(kPackThreads) pack_lowrank_kernel(const __grid_constant__ PackJobs jobs, int B, int N) {
     __shared__ __align__(16) __nv_bfloat16 rows[kPackPos][kMaxHeads * kMaxRank];
+    chain_release();
+    chain_wait();
     const TView src = jobs.src[blockIdx.y];
     const int H = jobs.H[blockIdx.y], r = jobs.r[blockIdx.y], n0 = blockIdx.x * kPackPos;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, vals = H * r;
@@ -338,6 +340,7 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
     const int c = a.chain_len;
     cudaError_t e;
     SideStream* side = nullptr;
+    const bool small = !ho && (int64_t)a.B * a.Hq * ((a.N + kTile - 1) / kTile) <= 2 * (int64_t)sm_count();   // one wave of CTAs that are resident at once: its kernels go out as a programmatic chain
     {
         PhaseMark mark(0, s);
         PackJobs jobs{};
@@ -360,9 +363,8 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
                 if ((e = cudaEventRecord(side->join, side->stream)) != cudaSuccess) return e;
             }
         }
-        if (!side) pack_lowrank_kernel<<<grid, kPackThreads, 0, s>>>(jobs, a.B, a.N);
+        if (!side && (e = launch_kernel(false, pack_lowrank_kernel, grid, dim3(kPackThreads), 0, s, jobs, a.B, a.N)) != cudaSuccess) return e;
         count_launches(1);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     bool joined = side == nullptr;
     auto join_pack = [&]() -> cudaError_t {   // before the first kernel that reads the packed Q'/K'
@@ -410,8 +412,9 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
         const size_t* po = l.plane_off[set];
         if (stream_in && (e = copy_in(wv, st)) != cudaSuccess) return e;
         // 1. anchor scores and the differences of the links below the top one
-        const TcFlashArgs fw{a.B, a.N, a.Hq, a.Hkv, 128, a.q0, a.k0, a.v, a.o, 1.f / sqrtf((float)a.d), nullptr, l.plane_rows, l.plane_cols,
+        TcFlashArgs fw{a.B, a.N, a.Hq, a.Hkv, 128, a.q0, a.k0, a.v, a.o, 1.f / sqrtf((float)a.d), nullptr, l.plane_rows, l.plane_cols,
                              wv.begin, wv.count};                 // the wave's own planes
+        fw.chained = small;
         TcFlashArgs f = fw;                                       // the plane of the running scores
         f.plane_rows = x_rows; f.plane_cols = x_cols; f.plane_row0 = row0;
         char* const x_plane = cy ? plane_base : base + po[0];
@@ -480,6 +483,7 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
         al.links = a.links;
         al.row0 = row0;
         al.store_all = all_layers;
+        al.chained = small;
         if (!per_link) {
             PhaseMark mark(2, st);
             if ((e = launch_tc_align(al, st)) != cudaSuccess) return e;

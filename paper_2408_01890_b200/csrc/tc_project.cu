@@ -454,9 +454,7 @@ bool tc_project_supported(const lisa_project_args& a) {
 namespace {
 template <int NR>
 cudaError_t prepare_narrow() {   // the default carveout leaves room for one CTA per SM only
-    cudaError_t e = cudaFuncSetAttribute(tc_project_narrow_kernel<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, Narrow<NR>::TOTAL);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(tc_project_narrow_kernel<NR>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    return allow_smem(tc_project_narrow_kernel<NR>, Narrow<NR>::TOTAL, true);
 }
 template <int NR>
 cudaError_t launch_narrow_nr(const ProjParams& p, int split, int n_tiles, int row_tiles, const CUtensorMap& tmX, const CUtensorMap& tmW, cudaStream_t s) {
@@ -544,7 +542,7 @@ cudaError_t launch_tc_project(const lisa_project_args& a, cudaStream_t stream) {
         if (!make_tensor_map_bf16(&tmW, a.w, 2, dims, str, box)) return cudaErrorInvalidValue;
     }
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(tc_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_TOTAL)) != cudaSuccess) return e;
+    if ((e = allow_smem(tc_project_kernel, SMEM_TOTAL)) != cudaSuccess) return e;
     const unsigned grid = (unsigned)std::min<long long>(p.tiles_total, sm_count());
     tc_project_kernel<<<grid, kThreads, SMEM_TOTAL, stream>>>(p, tmX, tmW);
     count_launches(1);

@@ -402,3 +402,33 @@ def test_carried_scores_single_layer_keeps_nothing():
     assert torch.equal(got, rec)
     ref = oracle.prefill_full(f64(t["q0"]), f64(t["k0"]), f64(t["v1"]), ol)
     assert_close(got.float().cpu().numpy(), ref, "bf16", "carried call, single layer")
+
+
+def test_small_prompt_chain_replayed_from_a_graph():
+    """A prompt whose kernels are launched as a programmatic chain, with the packing on a stream of its own: captured and replayed, the
+    results are those of the plain calls."""
+    B, N, Hkv, chain = 1, 200, 8, 2
+    w = synth.Workload("graph", "bf16", B, N, 32, Hkv, 128, 21, 64, "relu", chain)
+    t = synth.prefill_inputs(w, 12)
+    dl, _ = make_links(t, chain, "relu")
+    q0, k0 = dev(t["q0"]), dev(t["k0"])
+    vs = [dev(t[f"v{k}"]) for k in range(1, chain + 1)]
+    outs = [torch.zeros_like(q0) for _ in range(chain)]
+    scores = torch.empty(lb.lisa_prefill_scores_bytes(B, N, 32), dtype=torch.uint8, device="cuda")
+    ws = lb.prefill_carry_workspace(q0, k0, dl[0], vs[0], outs[0], scores)
+
+    def layers():
+        for k in range(chain):
+            lb.lisa_attn_shared_prefill_carry(q0, k0, dl[k], vs[k], scores, first=k == 0, keep=k + 1 < chain, out=outs[k], workspace=ws)
+    layers()
+    torch.cuda.synchronize()
+    ref = [o.clone() for o in outs]
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        layers()
+    for o in outs:
+        o.zero_()
+    g.replay()
+    g.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(outs, ref)) and lb.lisa_check() == lb.OK
