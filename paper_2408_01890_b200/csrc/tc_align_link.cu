@@ -1,5 +1,5 @@
-// Head-axis aligner (Sec. 5.1), one link per launch, on warp-level tensor-core MMAs, for the shapes and Integrate modes
-// the chain kernel of tc_align.cu does not take:
+// Head-axis aligner (Sec. 5.1), one link per launch, on tcgen05, for the shapes and Integrate modes the chain kernel of
+// tc_align.cu does not take:
 //   CONCAT  (32 heads)        A_k = W2^T act(W1^T [A_{k-1}; D_k] + b1) + b2    W1 [64, m], W2 [m, 32], m <= 256: the paper's
 //                             complete model (Sec. 5.1, "An overview of LiSA": 64 x 256 and 256 x 32), and its one-layer
 //                             form A_k = W1^T [A_{k-1}; D_k] + b1 with W1 [64, 32]
@@ -14,9 +14,14 @@
 // Outputs go over the inputs, which are dead once the launch has read them: the scores for the next link (unscaled) and
 // log2(e) times the FFN output for the attention kernel (which works in the exp2 domain), each over plane_x or plane_d
 // as the caller says.
-// A warp owns pieces of 32 key positions of one query row; per 16-position strip the A fragments come from ldmatrix.trans,
-// the hidden layer is computed CHUNK units at a time with fp16 accumulators whose registers are the A fragments of the
-// second layer (see tc_align_mma.cuh), the output accumulates in fp32 over the chunks.
+//
+// A tile is 64 key positions of two query rows: 128 positions, the M of both MMAs.  In a plane the positions of a head are
+// 128 contiguous bytes, so the TMA-loaded tile is the first layer's A operand as it stands (M-major, K = heads); its fp32
+// result goes from tensor memory through the registers (bias, activation, rounding to fp16) back into tensor memory, where
+// it is the second layer's A operand.  Nothing but the planes and the weights (B operands, in shared memory for the whole
+// launch) touches shared memory.  Roles: one warp loads, one issues each layer's MMAs, WGS warpgroups take the tiles in
+// turn, each with 512 / WGS columns of tensor memory of its own, so that the waits of one tile (two MMAs, four barriers)
+// hide behind the arithmetic of the others.
 #include <algorithm>
 
 #include "tc_align_mma.cuh"
@@ -30,304 +35,419 @@ using alignmma::KIND_FFN;
 using alignmma::KIND_PLUS;
 using alignmma::KIND_SINGLE;
 using alignmma::kLog2e;
-using alignmma::ldmatrix_x4_trans;
 using alignmma::ldw;
-using alignmma::mma_f16;
-using alignmma::mma_f16acc;
-using alignmma::stmatrix_x4_trans;
 
-constexpr int UNIT = 128, PP = 32;
-constexpr int kStages = 2;
+constexpr int UNIT = 128;
+constexpr int kMaxStages = 8;
 
 struct LinkParams {
-    int B, N, row0, qt_begin, qt_count, units_per_batch;
-    int64_t plane_cols;
-    int d_row0;                         // geometry of plane_d where it differs from plane_x's
-    int64_t d_plane_cols;
-    __half *plane_x, *plane_d;          // plane_d == nullptr: no difference plane (ADD, top link)
+    int N, row0, d_row0;                // first query row of plane_x / plane_d
+    int row_begin, row_end;             // query rows of the launch
+    int tiles_per_batch, total;         // tiles: (row pair, 64-column block up to the diagonal)
+    int has_d;                          // a difference plane is read (always with CONCAT)
     int dst_next, dst_scaled;           // where the next link's input / the attention kernel's plane go: -1 nowhere, 0 plane_x, 1 plane_d
     const void *w1, *b1, *w2, *b2;
     int w_dtype, m, kind;               // kind: KIND_FFN (hidden width m) / KIND_SINGLE / KIND_PLUS
+    int hid;                            // hidden units of the MMAs: m (or the inputs, without a hidden layer) rounded up to 16
+    int stages;
+    int* status;
 };
 
-// NH heads; CONCAT: the difference plane is the second half of the FFN's input; the hidden layer is CHUNK * NCHUNK wide
-template <int NH, bool CONCAT, int CHUNK, int NCHUNK>
+// Shared memory of a launch: [stages][plane x, plane d][2 rows][heads, padded][128 B], weights, staging, biases, barriers.
+template <int NH, bool CONCAT, int WGS>
 struct Shape {
-    static constexpr int HB = (NH + 15) / 16;                 // 16-head blocks of a plane (the last one zero-padded)
-    static constexpr int KS_IN = CONCAT ? 2 * HB : HB;        // k-steps of the first layer
+    static constexpr int HK = (NH + 15) / 16 * 16;            // heads as an MMA's K (or N): zero-padded to 16
     static constexpr int H_IN = CONCAT ? 2 * NH : NH;
-    static constexpr int MHID = CHUNK * NCHUNK;
-    static constexpr int NT_OUT = NH / 8;                     // 8-head n-tiles of the output
-    static constexpr int PLANE_SCR = HB * 16 * PP * 2;        // [heads, padded][32 positions] fp16
-    static constexpr int W1F = KS_IN * (MHID / 8) * 32 * 8;
-    static constexpr int W2F = (MHID / 16) * NT_OUT * 32 * 8;
-    static constexpr int WEIGHTS = W1F + W2F + (MHID / 2 + HB * 16) * 4;
-    static_assert(NH % 8 == 0 && CHUNK % 16 == 0 && (!CONCAT || NH % 16 == 0), "fragment shapes");
+    static constexpr int K1 = CONCAT ? 2 * HK : HK;
+    static constexpr int SLOT = HK * 128;                     // one query row of a tile
+    static constexpr int TILE = 2 * SLOT;
+    static constexpr int STG = NH * 64;                       // a warp's 32 positions on the way out
+    static constexpr int STRIDE = 512 / WGS, D_OFF = STRIDE / 2;   // tensor-memory columns of a warpgroup; its second-layer result
+    static constexpr int CHUNK = WGS > 2 ? 32 : 64;           // hidden units a thread holds at a time (registers)
+    static constexpr int THREADS = WGS * 128 + 96;            // + loader, two MMA issuers
+    static_assert(K1 <= 64 && (!CONCAT || HK == NH) && D_OFF + HK <= STRIDE, "layout");
+    static __host__ __device__ int stage_bytes(bool has_d) { return TILE * (has_d ? 2 : 1); }
+    static __host__ __device__ int w1_off(int stages, bool has_d) { return stages * stage_bytes(has_d); }
+    static __host__ __device__ int w2_off(int w1, int hid) { return w1 + hid * 128; }
+    static __host__ __device__ int stg_off(int w2, int hid) { return w2 + (hid + 63) / 64 * (HK * 128); }
+    static __host__ __device__ int bias_off(int stg) { return stg + WGS * 4 * 2 * STG; }
+    static __host__ __device__ int bar_off(int bias, int hid) { return bias + hid * 2 + HK * 4; }
+    static __host__ int total(int stages, bool has_d, int hid) {
+        return bar_off(bias_off(stg_off(w2_off(w1_off(stages, has_d), hid), hid)), hid) + (2 * kMaxStages + 4 * 4) * 8 + 16;
+    }
 };
 
-template <int NH, bool CONCAT, int CHUNK, int NCHUNK, int ACT, int NTHREADS>
-__global__ void __launch_bounds__(NTHREADS, 1) tc_align_link_kernel(const __grid_constant__ LinkParams p) {
-    using S = Shape<NH, CONCAT, CHUNK, NCHUNK>;
-    constexpr int HB = S::HB, KS_IN = S::KS_IN, MHID = S::MHID, NT_OUT = S::NT_OUT, PLANE_SCR = S::PLANE_SCR;
-    extern __shared__ __align__(16) uint8_t smem[];
-    uint2* w1f = reinterpret_cast<uint2*>(smem);                               // [k-step KS_IN][n-tile MHID/8][lane]
-    uint2* w2f = reinterpret_cast<uint2*>(smem + S::W1F);                      // [k-step MHID/16][n-tile NT_OUT][lane]
-    uint32_t* b1h = reinterpret_cast<uint32_t*>(smem + S::W1F + S::W2F);       // [MHID/2] packed fp16 pairs
-    float* b2 = reinterpret_cast<float*>(b1h + MHID / 2);                      // [HB * 16]
-    uint8_t* sScr = smem + S::WEIGHTS;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m = p.m, wd = p.w_dtype, kind = p.kind;
+__host__ __device__ constexpr uint32_t umma_idesc_f16(int M, int N, int a_mn_major, int b_mn_major) {
+    return (1u << 4) | ((uint32_t)a_mn_major << 15) | ((uint32_t)b_mn_major << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+// D[tmem] (+)= A[tmem] * B[smem]: A holds row i in lane i, two K elements per column
+__device__ __forceinline__ void umma_ts_if(uint32_t issue, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(issue)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+                 "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
 
-    // ---- weights as ready-made B fragments; inputs beyond the heads and hidden units beyond m are zero rows / columns ----
+// Two hidden units: the MMA's sums rounded to fp16, plus the bias, through the activation.
+template <int ACT>
+__device__ __forceinline__ uint32_t hidden_pair(float lo, float hi, uint32_t bias) {
+    const uint32_t x = pack_f16(lo, hi);
+    uint32_t r;
+    if constexpr (ACT == LISA_ACT_RELU) {
+        asm("fma.rn.relu.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(0x3c003c00u), "r"(bias));
+        return r;
+    } else {
+        asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(bias));
+        return act_h2<ACT>(r);
+    }
+}
+
+// Position of a tile in the launch: (sequence, first of two query rows, 64-column block)
+struct Cursor {
+    int b, r, jb;
+    __device__ __forceinline__ void seek(const LinkParams& p, int t) {
+        b = t / p.tiles_per_batch;
+        int rem = t - b * p.tiles_per_batch;
+        r = p.row_begin;
+        for (;;) {   // blocks of 64 query rows
+            const int pairs = (min(p.row_end - r, 64) + 1) / 2, cols = (r >> 6) + 1;
+            if (rem < pairs * cols) {
+                r += rem / cols * 2;
+                jb = rem % cols;
+                return;
+            }
+            rem -= pairs * cols;
+            r += 64;
+        }
+    }
+    __device__ __forceinline__ void step(const LinkParams& p) {
+        if (++jb <= (r >> 6)) return;
+        jb = 0;
+        if ((r += 2) < p.row_end) return;
+        r = p.row_begin;
+        ++b;
+    }
+};
+
+template <int NH, bool CONCAT, int ACT, int WGS>
+__global__ void __launch_bounds__(Shape<NH, CONCAT, WGS>::THREADS, 1)
+tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD,
+                     const __grid_constant__ CUtensorMap tmXs, const __grid_constant__ CUtensorMap tmDs) {
+    using S = Shape<NH, CONCAT, WGS>;
+    constexpr int HK = S::HK, K1 = S::K1, SLOT = S::SLOT, TILE = S::TILE, STG = S::STG;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    if ((smem_u32(smem) & 1023u) != 0) {   // the swizzled tiles' bases: refuse loudly instead of computing garbage
+        if (threadIdx.x == 0) atomicAdd(p.status + 1, 1);
+        return;
+    }
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int hid = p.hid, stages = p.stages, kind = p.kind, m = p.m, wd = p.w_dtype;
+    const bool has_d = p.has_d != 0;
+    const int stage_bytes = S::stage_bytes(has_d);
+    const int w1_off = S::w1_off(stages, has_d), w2_off = S::w2_off(w1_off, hid), stg_off = S::stg_off(w2_off, hid);
+    const int bias_off = S::bias_off(stg_off), bar_off = S::bar_off(bias_off, hid);
+    uint8_t* sW1 = smem + w1_off;                                      // [hidden][64 inputs], swizzled
+    uint8_t* sW2 = smem + w2_off;                                      // [64 hidden units][heads, padded][64], swizzled
+    uint32_t* b1h = reinterpret_cast<uint32_t*>(smem + bias_off);      // [hid / 2] packed fp16 pairs
+    float* b2 = reinterpret_cast<float*>(b1h + hid / 2);               // [HK]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + bar_off);
+    uint64_t* full = bars;                       // [stages]
+    uint64_t* empty = bars + kMaxStages;         // [stages] first layer done (and, where it is added later, plane d read)
+    uint64_t* s_full = bars + 2 * kMaxStages;    // [WGS] first layer's sums
+    uint64_t* h_full = s_full + 4;               // [WGS] hidden layer written back
+    uint64_t* o_full = s_full + 8;               // [WGS] second layer's sums
+    uint64_t* b_free = s_full + 12;              // [WGS] ... read: the columns are free
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_full + 16);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    // this CTA's contiguous range of tiles
+    const int per = (p.total + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int t_begin = min(p.total, (int)blockIdx.x * per), n_tiles = min(p.total, t_begin + per) - t_begin;
+
+    // ---- weights as fp16 B operands; inputs beyond the heads and hidden units beyond m are zero ----
     auto first = [&](int k, int n) -> float {      // [inputs][hidden]
         if (k >= S::H_IN) return 0.f;
         if (kind != KIND_FFN) return k == n ? 1.f : 0.f;
         return n < m ? ld_elem(p.w1, k * m + n, wd) : 0.f;
     };
     auto second = [&](int k, int n) -> float {     // [hidden][heads]
+        if (n >= NH) return 0.f;
         if (kind == KIND_FFN) return k < m ? ld_elem(p.w2, k * NH + n, wd) : 0.f;
         if (kind == KIND_SINGLE) return k < S::H_IN ? ld_elem(p.w1, k * NH + n, wd) : 0.f;
         return k == n ? 1.f : 0.f;
     };
-    // input index of row kk of the first layer's K dimension: with CONCAT the difference plane's heads follow the padded block of the scores
-    auto in_index = [&](int kk) -> int {
-        if (!CONCAT) return kk < NH ? kk : 1 << 20;
-        const int half = kk / (HB * 16), h = kk % (HB * 16);
-        return h < NH ? half * NH + h : 1 << 20;
-    };
-    for (int e = tid; e < KS_IN * (MHID / 8) * 32; e += NTHREADS) {
-        const int ln = e & 31, j = (e >> 5) % (MHID / 8), ks = (e >> 5) / (MHID / 8), g = ln >> 2, t = ln & 3;
-        const int k0 = ks * 16 + 2 * t, n = j * 8 + g;
-        w1f[e] = make_uint2(pack_f16(first(in_index(k0), n), first(in_index(k0 + 1), n)), pack_f16(first(in_index(k0 + 8), n), first(in_index(k0 + 9), n)));
+    for (int e = tid; e < hid * (K1 / 8); e += S::THREADS) {
+        const int n = e % hid, k = e / hid * 8;
+        uint4 v;
+        v.x = pack_f16(first(k, n), first(k + 1, n)); v.y = pack_f16(first(k + 2, n), first(k + 3, n));
+        v.z = pack_f16(first(k + 4, n), first(k + 5, n)); v.w = pack_f16(first(k + 6, n), first(k + 7, n));
+        *reinterpret_cast<uint4*>(sW1 + sw128_offset(n, k >> 3)) = v;
     }
-    for (int e = tid; e < (MHID / 16) * NT_OUT * 32; e += NTHREADS) {
-        const int ln = e & 31, j2 = (e >> 5) % NT_OUT, s2 = (e >> 5) / NT_OUT, g = ln >> 2, t = ln & 3;
-        const int k0 = s2 * 16 + 2 * t, n = j2 * 8 + g;
-        w2f[e] = make_uint2(pack_f16(second(k0, n), second(k0 + 1, n)), pack_f16(second(k0 + 8, n), second(k0 + 9, n)));
+    for (int e = tid; e < HK * (hid / 8); e += S::THREADS) {
+        const int n = e % HK, k = e / HK * 8;
+        uint4 v;
+        v.x = pack_f16(second(k, n), second(k + 1, n)); v.y = pack_f16(second(k + 2, n), second(k + 3, n));
+        v.z = pack_f16(second(k + 4, n), second(k + 5, n)); v.w = pack_f16(second(k + 6, n), second(k + 7, n));
+        *reinterpret_cast<uint4*>(sW2 + (k >> 6) * (HK * 128) + sw128_offset(n, (k >> 3) & 7)) = v;
     }
-    for (int e = tid; e < MHID / 2; e += NTHREADS)
+    for (int e = tid; e < hid / 2; e += S::THREADS)
         b1h[e] = (kind != KIND_FFN || 2 * e >= m) ? 0u : pack_f16(ldw(p.b1, 2 * e, wd), 2 * e + 1 < m ? ldw(p.b1, 2 * e + 1, wd) : 0.f);
-    for (int e = tid; e < HB * 16; e += NTHREADS)
+    for (int e = tid; e < HK; e += S::THREADS)
         b2[e] = e >= NH ? 0.f : (kind == KIND_FFN ? ldw(p.b2, e, wd) : (kind == KIND_SINGLE ? ldw(p.b1, e, wd) : 0.f));
-    // the scratch rows of the padding heads stay zero for the whole launch (copies only touch real heads)
-    for (int e = tid; e < (NTHREADS / 32) * kStages * 2 * PLANE_SCR / 16; e += NTHREADS) reinterpret_cast<uint4*>(sScr)[e] = make_uint4(0u, 0u, 0u, 0u);
-    __syncthreads();
-
-    // ---- this warp's contiguous range of pieces: (batch, query tile, row, 64-key block, half) ----
-    const int pB = p.B, pN = p.N, p_row0 = p.row0, p_qt0 = p.qt_begin, p_qt1 = p.qt_begin + p.qt_count;
-    const int p_ncb = (int)(p.plane_cols >> 6);
-    const int p_row0_d = p.d_row0, p_ncb_d = (int)(p.d_plane_cols >> 6);
-    constexpr int PPU = UNIT / PP;
-    const long long n_pieces = (long long)p.units_per_batch * pB * PPU;
-    const long long n_warps = (long long)gridDim.x * (NTHREADS / 32);
-    const long long per_warp = (n_pieces + n_warps - 1) / n_warps;
-    const long long s_begin = min(n_pieces, ((long long)blockIdx.x * (NTHREADS / 32) + warp) * per_warp);
-    const long long s_end = min(n_pieces, s_begin + per_warp);
-    if (s_begin >= s_end) return;
-    struct Cursor { int b, t, row, jb, sub; };
-    Cursor cu;
-    {
-        const long long u = s_begin / PPU;
-        cu.sub = (int)(s_begin % PPU);
-        cu.b = (int)(u / p.units_per_batch);
-        int rem = (int)(u - (long long)cu.b * p.units_per_batch);
-        cu.t = p_qt0;
-        for (;; ++cu.t) {
-            const int n_t = min(UNIT, pN - cu.t * UNIT) * (cu.t + 1);
-            if (rem < n_t || cu.t + 1 >= p_qt1) break;
-            rem -= n_t;
-        }
-        cu.row = rem / (cu.t + 1);
-        cu.jb = rem - cu.row * (cu.t + 1);
+    if constexpr (HK != NH) {   // the padding heads of the tiles stay zero: copies only touch real heads
+        constexpr int PAD = (HK - NH) * 8;   // 16-byte pieces per slot
+        for (int e = tid; e < stages * (stage_bytes / SLOT) * PAD; e += S::THREADS)
+            *reinterpret_cast<uint4*>(smem + e / PAD * SLOT + NH * 128 + e % PAD * 16) = make_uint4(0u, 0u, 0u, 0u);
     }
-    auto advance = [&](Cursor& x) {
-        if (++x.sub < PPU) return;
-        x.sub = 0;
-        if (++x.jb <= x.t) return;
-        x.jb = 0;
-        if (++x.row < min(UNIT, pN - x.t * UNIT)) return;
-        x.row = 0;
-        if (++x.t < p_qt1) return;
-        x.t = p_qt0;
-        ++x.b;
-    };
-    // four lanes cover the 64 bytes [head][32 positions] of one head: a warp-wide access moves 8 heads
-    constexpr int CPR = PP / 8, HPA = 32 / CPR, NACC = NH / HPA;
-    const int l_head = lane / CPR, l_chunk = lane % CPR;
-    auto piece_off = [&](const Cursor& x, int which) {   // which: 0 = plane_x's geometry, 1 = plane_d's
-        const int r = x.t * UNIT + x.row - (which ? p_row0_d : p_row0);
-        const int col = x.sub * PP;
-        const int64_t blk = (int64_t)(r >> 7) * (which ? p_ncb_d : p_ncb) + (x.jb * 2 + (col >> 6));
-        return ((blk * 128 + (r & 127)) * (pB * NH) + (x.b * NH + l_head)) * 64 + (col & 63) + l_chunk * 8;
-    };
-    auto scr_off = [&](int head, int chunk) { return (uint32_t)(head * (PP * 2) + ((chunk ^ ((head >> 1) & 3)) << 4)); };
-    uint8_t* scr = sScr + warp * (kStages * 2 * PLANE_SCR);   // [stage][plane x, plane d][heads][64 B]
-    __half* const gx = p.plane_x;
-    __half* const gd = p.plane_d;
-    const bool has_d = gd != nullptr;
-    auto fetch = [&](const Cursor& x, int buf) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            if (k == 1 && !has_d) break;
-            const int64_t off = piece_off(x, k);
-            const __half* src = k == 0 ? gx : gd;
-#pragma unroll
-            for (int i = 0; i < NACC; ++i) {
-                const uint32_t dst = smem_u32(scr + (buf * 2 + k) * PLANE_SCR) + scr_off(l_head + HPA * i, l_chunk);
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + off + i * (HPA * 64)) : "memory");
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    const int mi = lane >> 3, lr = lane & 7, t4 = lane & 3;
-    auto frag_off = [&](int s2, int x) { return scr_off(x * 16 + 8 * (mi >> 1) + lr, 2 * s2 + (mi & 1)); };
-    const int dst_next = p.dst_next, dst_scaled = p.dst_scaled;
+    if (tid == 0) {
+        for (int i = 0; i < stages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, (!CONCAT && has_d) ? 5 : 1); }
+        for (int i = 0; i < WGS; ++i) { mbar_init(s_full + i, 1); mbar_init(h_full + i, 4); mbar_init(o_full + i, 1); mbar_init(b_free + i, 4); }
+        *abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp == 0) tmem_alloc(tmem_slot, 512);
+    fence_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    chain_wait();
+    chain_release();
+    const uint32_t tmem_base = *tmem_slot;
 
-    fetch(cu, 0);
-    Cursor ahead = cu;
-    advance(ahead);
-    int buf = 0;
-    for (long long sidx = s_begin; sidx < s_end; ++sidx) {
-        const Cursor here = cu;
-        advance(cu);
-        if (sidx + 1 < s_end) { fetch(ahead, buf ^ 1); advance(ahead); }
-        else asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-        __syncwarp();
-        const uint32_t base_x = smem_u32(scr + (buf * 2) * PLANE_SCR), base_d = base_x + PLANE_SCR;
-        // both 16-position strips of the piece go through the FFN together: every weight fragment read from shared memory
-        // feeds two MMAs (with one, the shared-memory pipe moves 256 bytes per MMA, about all it delivers at the MMA rate)
-        constexpr int NS = PP / 16;
-        {
-            uint32_t afr[NS][KS_IN][4];      // CONCAT: the first HB k-steps are the heads of the scores, the others the heads of D_k
-#pragma unroll
-            for (int s2 = 0; s2 < NS; ++s2)
-#pragma unroll
-                for (int x = 0; x < HB; ++x) {
-                    ldmatrix_x4_trans(afr[s2][x], base_x + frag_off(s2, x));
-                    if constexpr (CONCAT) ldmatrix_x4_trans(afr[s2][HB + x], base_d + frag_off(s2, x));
-                }
-            float y[NS][2 * HB][4];
-#pragma unroll
-            for (int j2 = 0; j2 < 2 * HB; ++j2) {
-                const float2 bb = *reinterpret_cast<const float2*>(b2 + j2 * 8 + 2 * t4);
-#pragma unroll
-                for (int s2 = 0; s2 < NS; ++s2) { y[s2][j2][0] = bb.x; y[s2][j2][1] = bb.y; y[s2][j2][2] = bb.x; y[s2][j2][3] = bb.y; }
+    if (warp == WGS * 4) {
+        // ------------------------------ loader ------------------------------
+        Cursor cu;
+        if (n_tiles > 0) cu.seek(p, t_begin);
+        int s = 0;
+        uint32_t par = 1;
+        if (lane == 0) { tma_prefetch_desc(&tmX); if (has_d) tma_prefetch_desc(&tmD); }
+        for (int i = 0; i < n_tiles; ++i) {
+            bool ok = true;
+            if (lane == 0) {
+                ok = mbar_wait(empty + s, par, abort_flag);
+                if (ok) mbar_expect_tx(full + s, (has_d ? 4 : 2) * NH * 128);
             }
-#pragma unroll 1
-            for (int q = 0; q < NCHUNK; ++q) {
-                uint32_t h[NS][CHUNK / 8][2];
-#pragma unroll
-                for (int j = 0; j < CHUNK / 8; ++j) {
-                    const uint32_t bb = b1h[(q * (CHUNK / 8) + j) * 4 + t4];
-                    const uint2 w = w1f[(q * (CHUNK / 8) + j) * 32 + lane];
-#pragma unroll
-                    for (int s2 = 0; s2 < NS; ++s2) mma_f16acc(h[s2][j], afr[s2][0], w.x, w.y, bb, bb);
-                }
-#pragma unroll
-                for (int ks = 1; ks < KS_IN; ++ks)
-#pragma unroll
-                    for (int j = 0; j < CHUNK / 8; ++j) {
-                        const uint2 w = w1f[(ks * (MHID / 8) + q * (CHUNK / 8) + j) * 32 + lane];
-#pragma unroll
-                        for (int s2 = 0; s2 < NS; ++s2) mma_f16acc(h[s2][j], afr[s2][ks], w.x, w.y, h[s2][j][0], h[s2][j][1]);
-                    }
-#pragma unroll
-                for (int s2 = 0; s2 < NS; ++s2)
-#pragma unroll
-                    for (int j = 0; j < CHUNK / 8; ++j) {
-                        h[s2][j][0] = act_h2<ACT>(h[s2][j][0]);
-                        h[s2][j][1] = act_h2<ACT>(h[s2][j][1]);
-                    }
-#pragma unroll
-                for (int s = 0; s < CHUNK / 16; ++s)
-#pragma unroll
-                    for (int j2 = 0; j2 < NT_OUT; ++j2) {
-                        const uint2 w = w2f[((q * (CHUNK / 16) + s) * NT_OUT + j2) * 32 + lane];
-#pragma unroll
-                        for (int s2 = 0; s2 < NS; ++s2) {
-                            const uint32_t hfr[4] = {h[s2][2 * s][0], h[s2][2 * s][1], h[s2][2 * s + 1][0], h[s2][2 * s + 1][1]};
-                            mma_f16(y[s2][j2], hfr, w.x, w.y);
-                        }
-                    }
-            }
-            // every lane has read its fragments of the scores (the MMAs that consumed them have completed): results go back transposed
+            if (!__shfl_sync(0xffffffffu, ok, 0)) break;
+            uint8_t* dst = smem + s * stage_bytes + lane * SLOT;
+            const int rx = cu.r + lane - p.row0;
+            if (lane < 2) tma_load_5d(dst, &tmX, full + s, 0, cu.b * NH, rx & 127, cu.jb, rx >> 7);
             __syncwarp();
+            if (has_d) {
+                const int rd = cu.r + lane - p.d_row0;
+                if (lane < 2) tma_load_5d(dst + TILE, &tmD, full + s, 0, cu.b * NH, rd & 127, cu.jb, rd >> 7);
+                __syncwarp();
+            }
+            cu.step(p);
+            if (++s == stages) { s = 0; par ^= 1; }
+        }
+    } else if (warp == WGS * 4 + 1) {
+        // ------------------------------ MMA issuer: first layer ------------------------------
+        const uint32_t issue = lane == 0;
+        const uint32_t idesc = umma_idesc_f16(128, hid, 1, 0);
+        const uint64_t da0 = umma_desc_sw128(smem_u32(smem), SLOT, 1024), db0 = umma_desc_sw128(smem_u32(sW1), 16, 1024);
+        auto desc_off = [](uint64_t d, uint32_t bytes) -> uint64_t { return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4)); };
+        int s = 0, w = 0;
+        uint32_t par = 0, wpar = 1;
+        for (int i = 0; i < n_tiles; ++i) {
+            bool ok = mbar_wait(full + s, par, abort_flag) && mbar_wait(b_free + w, wpar, abort_flag);
+            if (!(ok = __all_sync(0xffffffffu, ok))) break;
+            tc_fence_after();
+            const uint64_t da = desc_off(da0, s * stage_bytes);
+#pragma unroll
+            for (int ks = 0; ks < K1 / 16; ++ks) {   // 16 heads = two groups of 8 rows; the second half of K lies in plane d's tile
+                const uint32_t a_off = ks < HK / 16 ? ks * 2048 : TILE + (ks - HK / 16) * 2048;
+                umma_ss_if(issue, tmem_base + w * S::STRIDE, desc_off(da, a_off), desc_off(db0, ks * 32), idesc, ks > 0);
+            }
+            umma_commit_if(issue, empty + s);
+            umma_commit_if(issue, s_full + w);
+            if (++s == stages) { s = 0; par ^= 1; }
+            if (++w == WGS) { w = 0; wpar ^= 1; }
+        }
+    } else if (warp == WGS * 4 + 2) {
+        // ------------------------------ MMA issuer: second layer ------------------------------
+        const uint32_t issue = lane == 0;
+        constexpr uint32_t idesc = umma_idesc_f16(128, HK, 0, 0);
+        const uint64_t db0 = umma_desc_sw128(smem_u32(sW2), 16, 1024);
+        auto desc_off = [](uint64_t d, uint32_t bytes) -> uint64_t { return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4)); };
+        int w = 0;
+        uint32_t wpar = 0;
+        for (int i = 0; i < n_tiles; ++i) {
+            bool ok = mbar_wait(h_full + w, wpar, abort_flag);
+            if (!(ok = __all_sync(0xffffffffu, ok))) break;
+            tc_fence_after();
+            const uint32_t buf = tmem_base + w * S::STRIDE;
+            for (int ks = 0; ks < hid / 16; ++ks)
+                umma_ts_if(issue, buf + S::D_OFF, buf + ks * 8, desc_off(db0, (ks >> 2) * (HK * 128) + (ks & 3) * 32), idesc, ks > 0);
+            umma_commit_if(issue, o_full + w);
+            if (++w == WGS) { w = 0; wpar ^= 1; }
+        }
+    } else {
+        // ------------------------------ warpgroups: hidden layer and results (thread = position) ------------------------------
+        const int w = warp >> 2, q = warp & 3;
+        const uint32_t buf = tmem_base + w * S::STRIDE + ((uint32_t)(q * 32) << 16);
+        const int dst_next = p.dst_next, dst_scaled = p.dst_scaled;
+        uint8_t* stg = smem + stg_off + warp * (2 * STG);
+        // this position's first head in plane d's tile: 128-byte rows, 16-byte chunks swizzled by the head
+        const int pos = (q & 1) * 32 + lane;
+        const uint32_t d_chunk = (uint32_t)(pos >> 3), d_in = TILE + (q >> 1) * SLOT + (pos & 7) * 2;
+        Cursor cu;
+        if (w < n_tiles) cu.seek(p, t_begin + w);
+        int s = w % stages;
+        uint32_t spar = (w / stages) & 1, wpar = 0;
+        for (int i = w; i < n_tiles; i += WGS) {
+            if (!__all_sync(0xffffffffu, mbar_wait(s_full + w, wpar, abort_flag))) break;
+            tc_fence_after();
+            int c = 0;
+            for (; c + S::CHUNK <= hid; c += S::CHUNK) {
+                uint32_t f[S::CHUNK], h[S::CHUNK / 2];
+#pragma unroll
+                for (int k = 0; k < S::CHUNK; k += 32) tmem_ld32(buf + c + k, f + k);
+                tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < S::CHUNK / 8; ++j) {
+                    const uint4 bb = *reinterpret_cast<const uint4*>(b1h + c / 2 + 4 * j);
+                    h[4 * j + 0] = hidden_pair<ACT>(__uint_as_float(f[8 * j + 0]), __uint_as_float(f[8 * j + 1]), bb.x);
+                    h[4 * j + 1] = hidden_pair<ACT>(__uint_as_float(f[8 * j + 2]), __uint_as_float(f[8 * j + 3]), bb.y);
+                    h[4 * j + 2] = hidden_pair<ACT>(__uint_as_float(f[8 * j + 4]), __uint_as_float(f[8 * j + 5]), bb.z);
+                    h[4 * j + 3] = hidden_pair<ACT>(__uint_as_float(f[8 * j + 6]), __uint_as_float(f[8 * j + 7]), bb.w);
+                }
+#pragma unroll
+                for (int k = 0; k < S::CHUNK / 2; k += 16) tmem_st16(buf + c / 2 + k, h + k);
+            }
+            for (; c < hid; c += 16) {
+                uint32_t f[16], h[8];
+                tmem_ld16(buf + c, f);
+                tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < 8; ++j) h[j] = hidden_pair<ACT>(__uint_as_float(f[2 * j]), __uint_as_float(f[2 * j + 1]), b1h[c / 2 + j]);
+                tmem_st8(buf + c / 2, h);
+            }
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(h_full + w);
+
+            if (!__all_sync(0xffffffffu, mbar_wait(o_full + w, wpar, abort_flag))) break;
+            wpar ^= 1;
+            tc_fence_after();
+            uint32_t yr[HK];
+            tmem_ld32(buf + S::D_OFF, yr);
+            if constexpr (HK > 32) tmem_ld16(buf + S::D_OFF + 32, yr + 32);
+            tmem_wait_ld();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(b_free + w);
+                tma_store_wait_read<0>();   // the previous tile's stores have read the staging buffers
+            }
+            __syncwarp();
+            float* y = reinterpret_cast<float*>(yr);
+#pragma unroll
+            for (int h = 0; h < NH; h += 4) {
+                const float4 bb = *reinterpret_cast<const float4*>(b2 + h);
+                y[h] += bb.x; y[h + 1] += bb.y; y[h + 2] += bb.z; y[h + 3] += bb.w;
+            }
             if (dst_scaled >= 0) {
-                const uint32_t base = dst_scaled == 0 ? base_x : base_d;
 #pragma unroll
-                for (int s2 = 0; s2 < NS; ++s2)
+                for (int h = 0; h < NH; ++h) *reinterpret_cast<__half*>(stg + h * 64 + lane * 2) = __float2half_rn(y[h] * kLog2e);
+            }
+            if (!CONCAT && has_d) {   // A_k = FFN(A_{k-1}) + D_k
+                if (!__all_sync(0xffffffffu, mbar_wait(full + s, spar, abort_flag))) break;
+                const uint8_t* db = smem + s * stage_bytes + d_in;
 #pragma unroll
-                    for (int x = 0; x < HB; ++x) {
-                        uint32_t r[4];
-                        r[0] = pack_f16(y[s2][2 * x][0] * kLog2e, y[s2][2 * x][1] * kLog2e);
-                        r[1] = pack_f16(y[s2][2 * x][2] * kLog2e, y[s2][2 * x][3] * kLog2e);
-                        r[2] = pack_f16(y[s2][2 * x + 1][0] * kLog2e, y[s2][2 * x + 1][1] * kLog2e);
-                        r[3] = pack_f16(y[s2][2 * x + 1][2] * kLog2e, y[s2][2 * x + 1][3] * kLog2e);
-                        stmatrix_x4_trans(base + frag_off(s2, x), r);
-                    }
+                for (int h = 0; h < NH; ++h) y[h] += __half2float(*reinterpret_cast<const __half*>(db + h * 128 + ((d_chunk ^ (h & 7)) << 4)));
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty + s);
             }
             if (dst_next >= 0) {
-                if constexpr (!CONCAT) {
-                    if (has_d) {   // A_k = FFN(A_{k-1}) + D_k: the difference in the fragment arrangement the scores came in
 #pragma unroll
-                        for (int s2 = 0; s2 < NS; ++s2)
+                for (int h = 0; h < NH; ++h) *reinterpret_cast<__half*>(stg + STG + h * 64 + lane * 2) = __float2half_rn(y[h]);
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                const int row = cu.r + (q >> 1), x = (q & 1) * 32;
 #pragma unroll
-                            for (int x = 0; x < HB; ++x) {
-                                uint32_t dfr[4];
-                                ldmatrix_x4_trans(dfr, base_d + frag_off(s2, x));
-#pragma unroll
-                                for (int qq = 0; qq < 4; ++qq) {
-                                    const float2 dv = unpack_f16(dfr[qq]);
-                                    y[s2][2 * x + (qq >> 1)][2 * (qq & 1)] += dv.x;
-                                    y[s2][2 * x + (qq >> 1)][2 * (qq & 1) + 1] += dv.y;
-                                }
-                            }
-                        __syncwarp();   // all lanes hold their part of D_k before it is overwritten
-                    }
+                for (int k = 0; k < 2; ++k) {
+                    const int rel = row - (k ? p.d_row0 : p.row0);
+                    const CUtensorMap* map = k ? &tmDs : &tmXs;
+                    if (dst_scaled == k) tma_store_5d(map, stg, x, cu.b * NH, rel & 127, cu.jb, rel >> 7);
+                    if (dst_next == k) tma_store_5d(map, stg + STG, x, cu.b * NH, rel & 127, cu.jb, rel >> 7);
                 }
-                const uint32_t base = dst_next == 0 ? base_x : base_d;
+                tma_store_commit();
+            }
 #pragma unroll
-                for (int s2 = 0; s2 < NS; ++s2)
-#pragma unroll
-                    for (int x = 0; x < HB; ++x) {
-                        uint32_t r[4];
-                        r[0] = pack_f16(y[s2][2 * x][0], y[s2][2 * x][1]);
-                        r[1] = pack_f16(y[s2][2 * x][2], y[s2][2 * x][3]);
-                        r[2] = pack_f16(y[s2][2 * x + 1][0], y[s2][2 * x + 1][1]);
-                        r[3] = pack_f16(y[s2][2 * x + 1][2], y[s2][2 * x + 1][3]);
-                        stmatrix_x4_trans(base + frag_off(s2, x), r);
-                    }
+            for (int k = 0; k < WGS; ++k) {
+                cu.step(p);
+                if (++s == stages) { s = 0; spar ^= 1; }
             }
         }
+        if (lane == 0) tma_store_wait_all<0>();
+    }
+    // ------------------------------ teardown ------------------------------
+    tc_fence_before();
+    __syncthreads();
+    if (*abort_flag) {
+        // a wait ran out: give copies and MMAs still in flight time to land before the memory is released
+        if (tid == 0) atomicAdd(p.status + 1, 1);
+        const long long t0 = clock64();
+        while (clock64() - t0 < 4000000ll) __nanosleep(1000);
+        __syncthreads();
+    }
+    if (warp == 0) {
         __syncwarp();
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            if (dst_next != k && dst_scaled != k) continue;
-            const int64_t here_off = piece_off(here, k);
-            __half* dst = k == 0 ? gx : gd;
-#pragma unroll
-            for (int i = 0; i < NACC; ++i)
-                *reinterpret_cast<uint4*>(dst + here_off + i * (HPA * 64)) =
-                    *reinterpret_cast<const uint4*>(scr + (buf * 2 + k) * PLANE_SCR + scr_off(l_head + HPA * i, l_chunk));
-        }
-        __syncwarp();   // the next iteration's fetch refills the other buffer; this one is refilled an iteration later
-        buf ^= 1;
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 512);
     }
 }
 
-template <int NH, bool CONCAT, int CHUNK, int NCHUNK, int NTHREADS>
-cudaError_t launch_shape(const LinkParams& p, int act, unsigned grid, cudaStream_t stream) {
-    using S = Shape<NH, CONCAT, CHUNK, NCHUNK>;
-    const size_t smem = (size_t)S::WEIGHTS + (size_t)(NTHREADS / 32) * kStages * 2 * S::PLANE_SCR;
-    static_assert(S::WEIGHTS + (NTHREADS / 32) * kStages * 2 * S::PLANE_SCR <= 232448, "one CTA's shared memory");
-    auto kernel = act == LISA_ACT_RELU   ? tc_align_link_kernel<NH, CONCAT, CHUNK, NCHUNK, LISA_ACT_RELU, NTHREADS>
-                  : act == LISA_ACT_SILU ? tc_align_link_kernel<NH, CONCAT, CHUNK, NCHUNK, LISA_ACT_SILU, NTHREADS>
-                                         : tc_align_link_kernel<NH, CONCAT, CHUNK, NCHUNK, LISA_ACT_NONE, NTHREADS>;
-    cudaError_t e = allow_smem(kernel, smem);
+// One plane as the loads see it (a query row's 64 columns x the heads, swizzled) and as the stores do (a warp's 32 columns).
+bool plane_maps(CUtensorMap* load, CUtensorMap* store, const void* plane, int B, int NH, int64_t rows, int64_t cols) {
+    const uint64_t bh = (uint64_t)B * NH, ncb = (uint64_t)cols / 64, nrb = (uint64_t)rows / UNIT;
+    const uint64_t dims[5] = {64, bh, (uint64_t)UNIT, ncb, nrb};
+    const uint64_t str[4] = {128, bh * 128, UNIT * bh * 128, ncb * UNIT * bh * 128};
+    const uint32_t in[5] = {64, (uint32_t)NH, 1, 1, 1}, out[5] = {32, (uint32_t)NH, 1, 1, 1};
+    return make_tensor_map_bf16(load, plane, 5, dims, str, in, true) && make_tensor_map_bf16(store, plane, 5, dims, str, out, true, false);
+}
+
+template <int NH, bool CONCAT, int WGS>
+cudaError_t launch_shape(LinkParams p, int act, const CUtensorMap* maps, bool chained, cudaStream_t stream) {
+    using S = Shape<NH, CONCAT, WGS>;
+    constexpr int kSmem = 232448;   // one CTA's shared memory
+    p.stages = kMaxStages;
+    while (p.stages > 2 && S::total(p.stages, p.has_d != 0, p.hid) > kSmem) --p.stages;
+    const size_t smem = std::max(S::total(p.stages, p.has_d != 0, p.hid), kSmem / 2 + 1);   // one CTA per SM: it takes all of the tensor memory
+    if (smem > kSmem) return cudaErrorInvalidValue;
+    auto kernel = act == LISA_ACT_RELU   ? tc_align_link_kernel<NH, CONCAT, LISA_ACT_RELU, WGS>
+                  : act == LISA_ACT_SILU ? tc_align_link_kernel<NH, CONCAT, LISA_ACT_SILU, WGS>
+                                         : tc_align_link_kernel<NH, CONCAT, LISA_ACT_NONE, WGS>;
+    cudaError_t e = allow_smem(kernel, smem, true);
     if (e != cudaSuccess) return e;
-    kernel<<<grid, NTHREADS, smem, stream>>>(p);
-    return cudaGetLastError();
+    // two tiles per CTA at least: half of a CTA's time on a single tile would be the weights
+    const unsigned grid = (unsigned)std::min<int64_t>((p.total + 1) / 2, sm_count());
+    return launch_kernel(chained, kernel, dim3(grid), dim3(S::THREADS), smem, stream, p, maps[0], maps[1], maps[2], maps[3]);
 }
 
 bool link_ok(int Hq, const lisa_link& l) {
@@ -364,30 +484,40 @@ cudaError_t launch_tc_align_link(const TcAlignLinkArgs& a, cudaStream_t stream) 
     const bool concat = l.integrate == LISA_INTEGRATE_CONCAT;
     if (concat && !a.plane_d) return cudaErrorInvalidValue;
     LinkParams p{};
-    p.B = a.B; p.N = a.N; p.row0 = a.row0 >= 0 ? a.row0 : a.qt_begin * UNIT; p.qt_begin = a.qt_begin; p.qt_count = a.qt_count;
+    p.N = a.N; p.row0 = a.row0 >= 0 ? a.row0 : a.qt_begin * UNIT;
     if (p.row0 % UNIT != 0 || p.row0 > a.qt_begin * UNIT) return cudaErrorInvalidValue;
-    p.plane_cols = a.plane_cols;
-    p.d_plane_cols = a.d_plane_cols > 0 ? a.d_plane_cols : a.plane_cols;
+    const int64_t d_cols = a.d_plane_cols > 0 ? a.d_plane_cols : a.plane_cols;
     p.d_row0 = a.d_plane_cols > 0 ? (a.d_row0 >= 0 ? a.d_row0 : a.qt_begin * UNIT) : p.row0;
-    if (p.d_plane_cols % 64 != 0 || p.d_row0 % UNIT != 0 || p.d_row0 > a.qt_begin * UNIT || (a.d_plane_cols > 0 && a.d_plane_rows % 128 != 0))
+    if (d_cols % 64 != 0 || p.d_row0 % UNIT != 0 || p.d_row0 > a.qt_begin * UNIT || (a.d_plane_cols > 0 && a.d_plane_rows % 128 != 0))
         return cudaErrorInvalidValue;
-    for (int t = a.qt_begin; t < a.qt_begin + a.qt_count; ++t) p.units_per_batch += std::min(UNIT, a.N - t * UNIT) * (t + 1);
-    p.plane_x = reinterpret_cast<__half*>(a.plane_x); p.plane_d = reinterpret_cast<__half*>(a.plane_d);
+    p.row_begin = a.qt_begin * UNIT;
+    p.row_end = std::min(a.N, (a.qt_begin + a.qt_count) * UNIT);
+    if (p.row_end <= p.row_begin) return cudaErrorInvalidValue;
+    int64_t tiles = 0;
+    for (int r = p.row_begin; r < p.row_end; r += 64) tiles += (int64_t)((std::min(p.row_end - r, 64) + 1) / 2) * (r / 64 + 1);
+    if (tiles * a.B > 0x3fffffff) return cudaErrorInvalidValue;
+    p.tiles_per_batch = (int)tiles;
+    p.total = (int)tiles * a.B;
+    CUtensorMap maps[4];
+    if (!plane_maps(maps, maps + 2, a.plane_x, a.B, a.Hq, a.plane_rows, a.plane_cols)) return cudaErrorInvalidValue;
+    maps[1] = maps[0]; maps[3] = maps[2];
+    p.has_d = a.plane_d != nullptr;
+    if (a.plane_d && !plane_maps(maps + 1, maps + 3, a.plane_d, a.B, a.Hq, a.d_plane_cols > 0 ? a.d_plane_rows : a.plane_rows, d_cols))
+        return cudaErrorInvalidValue;
+    p.status = status_words();
+    if (!p.status) return cudaErrorUnknown;
     p.dst_next = a.dst_next; p.dst_scaled = a.dst_scaled;
     p.w1 = l.w1; p.b1 = l.b1; p.w2 = l.w2; p.b2 = l.b2; p.w_dtype = l.w_dtype;
     p.kind = alignmma::link_kind(l.integrate, l.ffn_layers);
     p.m = l.m;
     const int act = p.kind == KIND_FFN ? l.act : LISA_ACT_NONE;
-    const int64_t total_units = (int64_t)p.units_per_batch * a.B;
-    if (total_units <= 0 || total_units > 0x7fffffff) return cudaErrorInvalidValue;
-    const unsigned grid = (unsigned)std::min<int64_t>((total_units + 3) / 4, sm_count());
-    const bool narrow = p.kind != KIND_FFN || l.m <= 64;   // hidden layer (or identity) within 64 units
+    const int inputs = concat ? 2 * a.Hq : a.Hq;
+    p.hid = ((p.kind == KIND_FFN ? l.m : inputs) + 15) / 16 * 16;
+    // Four warpgroups in turn as long as a quarter of the tensor memory holds a tile's hidden layer (128 units), two above.
     cudaError_t e;
-    if (concat) e = narrow ? launch_shape<32, true, 64, 1, 512>(p, act, grid, stream) : launch_shape<32, true, 64, 4, 512>(p, act, grid, stream);
-    else if (a.Hq == 32) e = narrow ? launch_shape<32, false, 64, 1, 512>(p, act, grid, stream) : launch_shape<32, false, 64, 4, 512>(p, act, grid, stream);
-    else if (narrow) e = launch_shape<40, false, 64, 1, 384>(p, act, grid, stream);
-    else if (l.m <= 80) e = launch_shape<40, false, 80, 1, 384>(p, act, grid, stream);
-    else e = launch_shape<40, false, 64, 4, 384>(p, act, grid, stream);
+    if (concat) e = p.hid <= 128 ? launch_shape<32, true, 4>(p, act, maps, a.chained, stream) : launch_shape<32, true, 2>(p, act, maps, a.chained, stream);
+    else if (a.Hq == 32) e = p.hid <= 128 ? launch_shape<32, false, 4>(p, act, maps, a.chained, stream) : launch_shape<32, false, 2>(p, act, maps, a.chained, stream);
+    else e = p.hid <= 128 ? launch_shape<40, false, 4>(p, act, maps, a.chained, stream) : launch_shape<40, false, 2>(p, act, maps, a.chained, stream);
     count_launches(1);
     return e;
 }

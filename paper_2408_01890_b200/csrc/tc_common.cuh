@@ -205,9 +205,9 @@ __device__ __forceinline__ uint32_t sw128_offset(uint32_t row, uint32_t chunk) {
 
 }  // namespace tc
 
-// Host: builds a tiled tensor map for a bf16 (or, with fp16 = true, fp16) tensor (driver entry point looked up at run time, no libcuda link).
+// Host: builds a tiled tensor map for a bf16 (or, with fp16 = true, fp16) tensor, with the 128-byte swizzle or none (driver entry point looked up at run time, no libcuda link).
 // dims/strides innermost first; strides_bytes[i] is the stride of dim i+1.  Returns false if the driver refuses.
 bool make_tensor_map_bf16(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
-                          const uint32_t* box, bool fp16 = false);
+                          const uint32_t* box, bool fp16 = false, bool swizzle = true);
 
 }  // namespace lisa

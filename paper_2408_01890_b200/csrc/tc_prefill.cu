@@ -444,6 +444,7 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
                                    &a.links[k], (k + 1 < c || (cy && cy->keep)) ? 0 : -1, (all_layers || k == c - 1) ? 1 : -1, row0,
                                    l.plane_rows, l.plane_cols, -1};
                 PhaseMark mark(2, st);
+                ac.chained = small;
                 if ((e = launch_tc_align_link(ac, st)) != cudaSuccess) return e;
             }
             // 3c. softmax and .V on the finished scores: the attention kernel's own difference is switched off (scale 0)
@@ -472,6 +473,7 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
                                    k + 1 < c ? base + po[k + 1] : nullptr, &a.links[k], k + 1 < c ? 1 : -1,
                                    (all_layers || k == c - 1) ? 0 : -1, row0};
                 PhaseMark mark(2, st);
+                al.chained = small;
                 if ((e = launch_tc_align_link(al, st)) != cudaSuccess) return e;
             }
         }
