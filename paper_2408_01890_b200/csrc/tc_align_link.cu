@@ -35,7 +35,9 @@ using alignmma::KIND_FFN;
 using alignmma::KIND_PLUS;
 using alignmma::KIND_SINGLE;
 using alignmma::kLog2e;
+using alignmma::ldmatrix_x4_trans;
 using alignmma::ldw;
+using alignmma::stmatrix_x4_trans;
 
 constexpr int UNIT = 128;
 constexpr int kMaxStages = 8;
@@ -53,21 +55,22 @@ struct LinkParams {
     int* status;
 };
 
-// Shared memory of a launch: [stages][plane x, plane d][2 rows][heads, padded][128 B], weights, staging, biases, barriers.
+// Shared memory of a launch: [stages][plane x, plane d][2 rows][heads][128 B], zero rows, weights, staging, biases, barriers.
 template <int NH, bool CONCAT, int WGS>
 struct Shape {
     static constexpr int HK = (NH + 15) / 16 * 16;            // heads as an MMA's K (or N): zero-padded to 16
     static constexpr int H_IN = CONCAT ? 2 * NH : NH;
     static constexpr int K1 = CONCAT ? 2 * HK : HK;
-    static constexpr int SLOT = HK * 128;                     // one query row of a tile
+    static constexpr int SLOT = NH * 128;                     // one query row of a tile
     static constexpr int TILE = 2 * SLOT;
+    static constexpr int ZERO = HK == NH ? 0 : SLOT + 1024;   // the padding heads of both rows (see the first layer's issuer)
     static constexpr int STG = NH * 64;                       // a warp's 32 positions on the way out
     static constexpr int STRIDE = 512 / WGS, D_OFF = STRIDE / 2;   // tensor-memory columns of a warpgroup; its second-layer result
     static constexpr int CHUNK = WGS > 2 ? 32 : 64;           // hidden units a thread holds at a time (registers)
     static constexpr int THREADS = WGS * 128 + 96;            // + loader, two MMA issuers
     static_assert(K1 <= 64 && (!CONCAT || HK == NH) && D_OFF + HK <= STRIDE, "layout");
     static __host__ __device__ int stage_bytes(bool has_d) { return TILE * (has_d ? 2 : 1); }
-    static __host__ __device__ int w1_off(int stages, bool has_d) { return stages * stage_bytes(has_d); }
+    static __host__ __device__ int w1_off(int stages, bool has_d) { return stages * stage_bytes(has_d) + ZERO; }
     static __host__ __device__ int w2_off(int w1, int hid) { return w1 + hid * 128; }
     static __host__ __device__ int stg_off(int w2, int hid) { return w2 + (hid + 63) / 64 * (HK * 128); }
     static __host__ __device__ int bias_off(int stg) { return stg + WGS * 4 * 2 * STG; }
@@ -108,6 +111,34 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                  ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                  : "memory");
+}
+
+// 16 lanes x 8 columns as an MMA accumulator fragment: thread t gets columns 2(t % 4), + 1 of lanes t / 4 and t / 4 + 8
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float* r) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];" : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void stmatrix_x2_trans(uint32_t saddr, uint32_t r0, uint32_t r1) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x2.trans.shared.b16 [%0], {%1,%2};" ::"r"(saddr), "r"(r0), "r"(r1) : "memory");
+}
+// A warp's results, times `scale`, as [head][32 positions] rows of 64 bytes whose 16-byte chunks carry the copy engine's 64-byte swizzle.
+template <int NH>
+__device__ __forceinline__ void put_frags(uint32_t stg, int lane, const float (*y)[NH / 8][4], float scale) {
+    constexpr int NG = NH / 8;
+#pragma unroll
+    for (int s2 = 0; s2 < 2; ++s2)
+#pragma unroll
+        for (int g = 0; g < NG; g += 2) {
+            const int head = (g + (lane >> 4)) * 8 + (lane & 7), chunk = 2 * s2 + ((lane >> 3) & 1);   // x2 reads lanes 0-15 only
+            const uint32_t addr = stg + head * 64 + ((chunk ^ ((head >> 1) & 3)) << 4);
+            uint32_t r[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float* v = y[s2][min(g + (k >> 1), NG - 1)] + 2 * (k & 1);
+                r[k] = pack_f16(v[0] * scale, v[1] * scale);
+            }
+            if (g + 1 < NG) stmatrix_x4_trans(addr, r);
+            else stmatrix_x2_trans(addr, r[0], r[1]);
+        }
 }
 
 // Two hidden units: the MMA's sums rounded to fp16, plus the bias, through the activation.
@@ -162,7 +193,7 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
         if (threadIdx.x == 0) atomicAdd(p.status + 1, 1);
         return;
     }
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
     const int hid = p.hid, stages = p.stages, kind = p.kind, m = p.m, wd = p.w_dtype;
     const bool has_d = p.has_d != 0;
     const int stage_bytes = S::stage_bytes(has_d);
@@ -216,11 +247,8 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
         b1h[e] = (kind != KIND_FFN || 2 * e >= m) ? 0u : pack_f16(ldw(p.b1, 2 * e, wd), 2 * e + 1 < m ? ldw(p.b1, 2 * e + 1, wd) : 0.f);
     for (int e = tid; e < HK; e += S::THREADS)
         b2[e] = e >= NH ? 0.f : (kind == KIND_FFN ? ldw(p.b2, e, wd) : (kind == KIND_SINGLE ? ldw(p.b1, e, wd) : 0.f));
-    if constexpr (HK != NH) {   // the padding heads of the tiles stay zero: copies only touch real heads
-        constexpr int PAD = (HK - NH) * 8;   // 16-byte pieces per slot
-        for (int e = tid; e < stages * (stage_bytes / SLOT) * PAD; e += S::THREADS)
-            *reinterpret_cast<uint4*>(smem + e / PAD * SLOT + NH * 128 + e % PAD * 16) = make_uint4(0u, 0u, 0u, 0u);
-    }
+    for (int e = tid; e < S::ZERO / 16; e += S::THREADS)
+        *reinterpret_cast<uint4*>(smem + stages * stage_bytes + e * 16) = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) {
         for (int i = 0; i < stages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, (!CONCAT && has_d) ? 5 : 1); }
         for (int i = 0; i < WGS; ++i) { mbar_init(s_full + i, 1); mbar_init(h_full + i, 4); mbar_init(o_full + i, 1); mbar_init(b_free + i, 4); }
@@ -234,39 +262,35 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
     tc_fence_after();
     chain_wait();
     chain_release();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     if (warp == WGS * 4) {
-        // ------------------------------ loader ------------------------------
-        Cursor cu;
-        if (n_tiles > 0) cu.seek(p, t_begin);
-        int s = 0;
-        uint32_t par = 1;
-        if (lane == 0) { tma_prefetch_desc(&tmX); if (has_d) tma_prefetch_desc(&tmD); }
-        for (int i = 0; i < n_tiles; ++i) {
-            bool ok = true;
-            if (lane == 0) {
-                ok = mbar_wait(empty + s, par, abort_flag);
-                if (ok) mbar_expect_tx(full + s, (has_d ? 4 : 2) * NH * 128);
+        // ------------------------------ loader: one thread, one copy per plane and tile ------------------------------
+        // (a copy per query row, issued by two lanes of a converged warp, took 1300 cycles a tile: more than the tile's arithmetic)
+        if (lane == 0) {
+            Cursor cu;
+            if (n_tiles > 0) cu.seek(p, t_begin);
+            int s = 0;
+            uint32_t par = 1;
+            tma_prefetch_desc(&tmX);
+            if (has_d) tma_prefetch_desc(&tmD);
+            for (int i = 0; i < n_tiles; ++i) {
+                if (!mbar_wait(empty + s, par, abort_flag)) break;
+                mbar_expect_tx(full + s, (has_d ? 2 : 1) * TILE);
+                uint8_t* dst = smem + s * stage_bytes;
+                const int rx = cu.r - p.row0, rd = cu.r - p.d_row0;
+                tma_load_5d(dst, &tmX, full + s, 0, cu.b * NH, rx & 127, cu.jb, rx >> 7);
+                if (has_d) tma_load_5d(dst + TILE, &tmD, full + s, 0, cu.b * NH, rd & 127, cu.jb, rd >> 7);
+                cu.step(p);
+                if (++s == stages) { s = 0; par ^= 1; }
             }
-            if (!__shfl_sync(0xffffffffu, ok, 0)) break;
-            uint8_t* dst = smem + s * stage_bytes + lane * SLOT;
-            const int rx = cu.r + lane - p.row0;
-            if (lane < 2) tma_load_5d(dst, &tmX, full + s, 0, cu.b * NH, rx & 127, cu.jb, rx >> 7);
-            __syncwarp();
-            if (has_d) {
-                const int rd = cu.r + lane - p.d_row0;
-                if (lane < 2) tma_load_5d(dst + TILE, &tmD, full + s, 0, cu.b * NH, rd & 127, cu.jb, rd >> 7);
-                __syncwarp();
-            }
-            cu.step(p);
-            if (++s == stages) { s = 0; par ^= 1; }
         }
+        __syncwarp();
     } else if (warp == WGS * 4 + 1) {
         // ------------------------------ MMA issuer: first layer ------------------------------
         const uint32_t issue = lane == 0;
         const uint32_t idesc = umma_idesc_f16(128, hid, 1, 0);
-        const uint64_t da0 = umma_desc_sw128(smem_u32(smem), SLOT, 1024), db0 = umma_desc_sw128(smem_u32(sW1), 16, 1024);
+        const uint64_t db0 = umma_desc_sw128(smem_u32(sW1), 16, 1024);
         auto desc_off = [](uint64_t d, uint32_t bytes) -> uint64_t { return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4)); };
         int s = 0, w = 0;
         uint32_t par = 0, wpar = 1;
@@ -274,11 +298,15 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
             bool ok = mbar_wait(full + s, par, abort_flag) && mbar_wait(b_free + w, wpar, abort_flag);
             if (!(ok = __all_sync(0xffffffffu, ok))) break;
             tc_fence_after();
-            const uint64_t da = desc_off(da0, s * stage_bytes);
+            const uint32_t st = smem_u32(smem) + s * stage_bytes;
+            const uint64_t da = umma_desc_sw128(st, SLOT, 1024);
 #pragma unroll
             for (int ks = 0; ks < K1 / 16; ++ks) {   // 16 heads = two groups of 8 rows; the second half of K lies in plane d's tile
                 const uint32_t a_off = ks < HK / 16 ? ks * 2048 : TILE + (ks - HK / 16) * 2048;
-                umma_ss_if(issue, tmem_base + w * S::STRIDE, desc_off(da, a_off), desc_off(db0, ks * 32), idesc, ks > 0);
+                uint64_t a = desc_off(da, a_off);
+                // 40 heads: the last group's partner is eight zero rows behind the stages (for the tile's second row SLOT further on)
+                if (HK != NH && ks == HK / 16 - 1) a = umma_desc_sw128(st + a_off, SLOT, smem_u32(smem) + stages * stage_bytes - (st + a_off));
+                umma_ss_if(issue, tmem_base + w * S::STRIDE, a, desc_off(db0, ks * 32), idesc, ks > 0);
             }
             umma_commit_if(issue, empty + s);
             umma_commit_if(issue, s_full + w);
@@ -298,7 +326,13 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
             if (!(ok = __all_sync(0xffffffffu, ok))) break;
             tc_fence_after();
             const uint32_t buf = tmem_base + w * S::STRIDE;
-            for (int ks = 0; ks < hid / 16; ++ks)
+            int ks = 0;
+            for (; ks + 4 <= hid / 16; ks += 4) {
+                const uint64_t db = desc_off(db0, (ks >> 2) * (HK * 128));
+#pragma unroll
+                for (int k = 0; k < 4; ++k) umma_ts_if(issue, buf + S::D_OFF, buf + (ks + k) * 8, desc_off(db, k * 32), idesc, ks + k > 0);
+            }
+            for (; ks < hid / 16; ++ks)
                 umma_ts_if(issue, buf + S::D_OFF, buf + ks * 8, desc_off(db0, (ks >> 2) * (HK * 128) + (ks & 3) * 32), idesc, ks > 0);
             umma_commit_if(issue, o_full + w);
             if (++w == WGS) { w = 0; wpar ^= 1; }
@@ -309,9 +343,11 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
         const uint32_t buf = tmem_base + w * S::STRIDE + ((uint32_t)(q * 32) << 16);
         const int dst_next = p.dst_next, dst_scaled = p.dst_scaled;
         uint8_t* stg = smem + stg_off + warp * (2 * STG);
-        // this position's first head in plane d's tile: 128-byte rows, 16-byte chunks swizzled by the head
-        const int pos = (q & 1) * 32 + lane;
-        const uint32_t d_chunk = (uint32_t)(pos >> 3), d_in = TILE + (q >> 1) * SLOT + (pos & 7) * 2;
+        const uint32_t stg_u32 = smem_u32(stg);
+        constexpr int NG = NH / 8;
+        float2 bias2[NG];
+#pragma unroll
+        for (int g = 0; g < NG; ++g) bias2[g] = *reinterpret_cast<const float2*>(b2 + g * 8 + 2 * (lane & 3));
         Cursor cu;
         if (w < n_tiles) cu.seek(p, t_begin + w);
         int s = w % stages;
@@ -352,9 +388,13 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
             if (!__all_sync(0xffffffffu, mbar_wait(o_full + w, wpar, abort_flag))) break;
             wpar ^= 1;
             tc_fence_after();
-            uint32_t yr[HK];
-            tmem_ld32(buf + S::D_OFF, yr);
-            if constexpr (HK > 32) tmem_ld16(buf + S::D_OFF + 32, yr + 32);
+            // a warp's 32 positions as two strips of 16, eight heads at a time: lane holds heads 2(lane % 4), + 1 of positions lane / 4, + 8,
+            // the fragment arrangement stmatrix and ldmatrix transpose from and to [head][position] rows
+            float y[2][NG][4];
+#pragma unroll
+            for (int s2 = 0; s2 < 2; ++s2)
+#pragma unroll
+                for (int g = 0; g < NG; ++g) tmem_ld_frag(buf + S::D_OFF + ((uint32_t)(s2 * 16) << 16) + g * 8, y[s2][g]);
             tmem_wait_ld();
             tc_fence_before();
             __syncwarp();
@@ -363,28 +403,37 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
                 tma_store_wait_read<0>();   // the previous tile's stores have read the staging buffers
             }
             __syncwarp();
-            float* y = reinterpret_cast<float*>(yr);
 #pragma unroll
-            for (int h = 0; h < NH; h += 4) {
-                const float4 bb = *reinterpret_cast<const float4*>(b2 + h);
-                y[h] += bb.x; y[h + 1] += bb.y; y[h + 2] += bb.z; y[h + 3] += bb.w;
-            }
-            if (dst_scaled >= 0) {
+            for (int s2 = 0; s2 < 2; ++s2)
 #pragma unroll
-                for (int h = 0; h < NH; ++h) *reinterpret_cast<__half*>(stg + h * 64 + lane * 2) = __float2half_rn(y[h] * kLog2e);
-            }
+                for (int g = 0; g < NG; ++g) {
+                    y[s2][g][0] += bias2[g].x; y[s2][g][1] += bias2[g].y;
+                    y[s2][g][2] += bias2[g].x; y[s2][g][3] += bias2[g].y;
+                }
+            if (dst_scaled >= 0) put_frags<NH>(stg_u32, lane, y, kLog2e);
             if (!CONCAT && has_d) {   // A_k = FFN(A_{k-1}) + D_k
                 if (!__all_sync(0xffffffffu, mbar_wait(full + s, spar, abort_flag))) break;
-                const uint8_t* db = smem + s * stage_bytes + d_in;
+                const uint32_t db = smem_u32(smem) + s * stage_bytes + TILE + (q >> 1) * SLOT;
 #pragma unroll
-                for (int h = 0; h < NH; ++h) y[h] += __half2float(*reinterpret_cast<const __half*>(db + h * 128 + ((d_chunk ^ (h & 7)) << 4)));
+                for (int s2 = 0; s2 < 2; ++s2)
+#pragma unroll
+                    for (int g = 0; g < NG; g += 2) {
+                        // four 8 x 8 blocks: (heads g, positions 0-7), (g, 8-15), (g + 1, 0-7), (g + 1, 8-15); beyond the last head: g again
+                        const int head = min(g + (lane >> 4), NG - 1) * 8 + (lane & 7), chunk = (q & 1) * 4 + 2 * s2 + ((lane >> 3) & 1);
+                        uint32_t dfr[4];
+                        ldmatrix_x4_trans(dfr, db + sw128_offset(head, chunk));
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if (g + (k >> 1) >= NG) break;
+                            const float2 dv = unpack_f16(dfr[k]);
+                            y[s2][g + (k >> 1)][2 * (k & 1)] += dv.x;
+                            y[s2][g + (k >> 1)][2 * (k & 1) + 1] += dv.y;
+                        }
+                    }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty + s);
             }
-            if (dst_next >= 0) {
-#pragma unroll
-                for (int h = 0; h < NH; ++h) *reinterpret_cast<__half*>(stg + STG + h * 64 + lane * 2) = __float2half_rn(y[h]);
-            }
+            if (dst_next >= 0) put_frags<NH>(stg_u32 + STG, lane, y, 1.f);
             fence_async_smem();
             __syncwarp();
             if (lane == 0) {
@@ -423,13 +472,13 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
     }
 }
 
-// One plane as the loads see it (a query row's 64 columns x the heads, swizzled) and as the stores do (a warp's 32 columns).
+// One plane as the loads see it (64 columns x the heads of two query rows) and as the stores do (a warp's 32 columns of one).
 bool plane_maps(CUtensorMap* load, CUtensorMap* store, const void* plane, int B, int NH, int64_t rows, int64_t cols) {
     const uint64_t bh = (uint64_t)B * NH, ncb = (uint64_t)cols / 64, nrb = (uint64_t)rows / UNIT;
     const uint64_t dims[5] = {64, bh, (uint64_t)UNIT, ncb, nrb};
     const uint64_t str[4] = {128, bh * 128, UNIT * bh * 128, ncb * UNIT * bh * 128};
-    const uint32_t in[5] = {64, (uint32_t)NH, 1, 1, 1}, out[5] = {32, (uint32_t)NH, 1, 1, 1};
-    return make_tensor_map_bf16(load, plane, 5, dims, str, in, true) && make_tensor_map_bf16(store, plane, 5, dims, str, out, true, false);
+    const uint32_t in[5] = {64, (uint32_t)NH, 2, 1, 1}, out[5] = {32, (uint32_t)NH, 1, 1, 1};
+    return make_tensor_map_bf16(load, plane, 5, dims, str, in, true) && make_tensor_map_bf16(store, plane, 5, dims, str, out, true, 64);
 }
 
 template <int NH, bool CONCAT, int WGS>

@@ -12,6 +12,10 @@ namespace tc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// The warp's index, read through a shuffle so that the compiler knows it to be the same in all lanes: the code of a warp's role is then
+// warp-uniform, and descriptors and loop counters stay in uniform registers instead of being moved there before every MMA.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ uint64_t global_timer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -205,9 +209,9 @@ __device__ __forceinline__ uint32_t sw128_offset(uint32_t row, uint32_t chunk) {
 
 }  // namespace tc
 
-// Host: builds a tiled tensor map for a bf16 (or, with fp16 = true, fp16) tensor, with the 128-byte swizzle or none (driver entry point looked up at run time, no libcuda link).
+// Host: builds a tiled tensor map for a bf16 (or, with fp16 = true, fp16) tensor, with a 128- or 64-byte swizzle (driver entry point looked up at run time, no libcuda link).
 // dims/strides innermost first; strides_bytes[i] is the stride of dim i+1.  Returns false if the driver refuses.
 bool make_tensor_map_bf16(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
-                          const uint32_t* box, bool fp16 = false, bool swizzle = true);
+                          const uint32_t* box, bool fp16 = false, int swizzle = 128);
 
 }  // namespace lisa

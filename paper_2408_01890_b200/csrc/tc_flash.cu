@@ -133,7 +133,7 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
         else return sP + (t & 1) * L::P_BYTES;
     };
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
     // blockIdx.x (the fastest-dispatched index) runs over (batch, head), blockIdx.y over query tiles from the last one
     // down: every CTA of the heaviest tile is handed out before any lighter one, so the SMs finish close together
     // With keys and values too large for L2 to hold for all heads at once, the order is turned round: blockIdx.x runs over the
@@ -165,7 +165,7 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
     // kernel further down the chain starts only after everything that preceded the call, weights it reads before its own wait included.
     chain_wait();
     chain_release();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     const uint32_t tmem_O = tmem_base + 128;
 
     // The kernel is compiled for 128 registers per thread (two CTAs of 256 threads per SM).  The three single-thread
@@ -516,7 +516,7 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
 }  // namespace
 
 bool make_tensor_map_bf16(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
-                          const uint32_t* box, bool fp16, bool swizzle) {
+                          const uint32_t* box, bool fp16, int swizzle) {
     typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -534,7 +534,7 @@ bool make_tensor_map_bf16(CUtensorMap* map, const void* base, int rank, const ui
     for (int i = 0; i < rank; ++i) { gdims[i] = dims[i]; gbox[i] = box[i]; estr[i] = 1; }
     for (int i = 0; i + 1 < rank; ++i) gstr[i] = strides_bytes[i];
     return encode(map, fp16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), gdims, gstr, gbox, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

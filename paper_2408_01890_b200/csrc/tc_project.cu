@@ -85,7 +85,7 @@ tc_project_kernel(const __grid_constant__ ProjParams p, const __grid_constant__ 
     uint64_t* acc_empty = bars + 2 * STAGES + 2;   // [2]
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * STAGES + 5);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
     if (tid == 0) {
         for (int i = 0; i < STAGES; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(acc_full + i, 1); mbar_init(acc_empty + i, 128); }
@@ -96,7 +96,7 @@ tc_project_kernel(const __grid_constant__ ProjParams p, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     const int k_slices = (p.K + BK - 1) / BK;
     // tile index -> (batch, row tile, column tile); column tiles vary fastest so that concurrent CTAs share their X rows in L2
     auto tile_coord = [&](long long tile, int& b, int& mt, int& nt) {
@@ -258,7 +258,7 @@ tc_project_narrow_kernel(const __grid_constant__ ProjParams p, const __grid_cons
     uint64_t* acc_full = bars + 2 * S::ST;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S::ST + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * S::ST + 2);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
     const int split = gridDim.x, rank = blockIdx.x;             // the cluster spans grid dimension x
     const int nt = blockIdx.y, rt = blockIdx.z;
     const int rows = p.rows_per_batch;
@@ -284,7 +284,7 @@ tc_project_narrow_kernel(const __grid_constant__ ProjParams p, const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     chain_wait();
     bool have = false;   // epilogue warps: the accumulator holds the CTA's share
     if (warp == 4) {
