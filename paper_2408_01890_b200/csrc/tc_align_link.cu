@@ -84,13 +84,12 @@ __host__ __device__ constexpr uint32_t umma_idesc_f16(int M, int N, int a_mn_maj
     return (1u << 4) | ((uint32_t)a_mn_major << 15) | ((uint32_t)b_mn_major << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 // D[tmem] (+)= A[tmem] * B[smem]: A holds row i in lane i, two K elements per column
-__device__ __forceinline__ void umma_ts_if(uint32_t issue, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
+        "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "setp.ne.b32 q, %5, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(issue)
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
@@ -267,7 +266,7 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
     if (warp == WGS * 4) {
         // ------------------------------ loader: one thread, one copy per plane and tile ------------------------------
         // (a copy per query row, issued by two lanes of a converged warp, took 1300 cycles a tile: more than the tile's arithmetic)
-        if (lane == 0) {
+        if (elect_one()) {
             Cursor cu;
             if (n_tiles > 0) cu.seek(p, t_begin);
             int s = 0;
@@ -288,7 +287,6 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
         __syncwarp();
     } else if (warp == WGS * 4 + 1) {
         // ------------------------------ MMA issuer: first layer ------------------------------
-        const uint32_t issue = lane == 0;
         const uint32_t idesc = umma_idesc_f16(128, hid, 1, 0);
         const uint64_t db0 = umma_desc_sw128(smem_u32(sW1), 16, 1024);
         auto desc_off = [](uint64_t d, uint32_t bytes) -> uint64_t { return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4)); };
@@ -298,24 +296,26 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
             bool ok = mbar_wait(full + s, par, abort_flag) && mbar_wait(b_free + w, wpar, abort_flag);
             if (!(ok = __all_sync(0xffffffffu, ok))) break;
             tc_fence_after();
-            const uint32_t st = smem_u32(smem) + s * stage_bytes;
-            const uint64_t da = umma_desc_sw128(st, SLOT, 1024);
+            if (elect_one()) {
+                const uint32_t st = smem_u32(smem) + s * stage_bytes;
+                const uint64_t da = umma_desc_sw128(st, SLOT, 1024);
 #pragma unroll
-            for (int ks = 0; ks < K1 / 16; ++ks) {   // 16 heads = two groups of 8 rows; the second half of K lies in plane d's tile
-                const uint32_t a_off = ks < HK / 16 ? ks * 2048 : TILE + (ks - HK / 16) * 2048;
-                uint64_t a = desc_off(da, a_off);
-                // 40 heads: the last group's partner is eight zero rows behind the stages (for the tile's second row SLOT further on)
-                if (HK != NH && ks == HK / 16 - 1) a = umma_desc_sw128(st + a_off, SLOT, smem_u32(smem) + stages * stage_bytes - (st + a_off));
-                umma_ss_if(issue, tmem_base + w * S::STRIDE, a, desc_off(db0, ks * 32), idesc, ks > 0);
+                for (int ks = 0; ks < K1 / 16; ++ks) {   // 16 heads = two groups of 8 rows; the second half of K lies in plane d's tile
+                    const uint32_t a_off = ks < HK / 16 ? ks * 2048 : TILE + (ks - HK / 16) * 2048;
+                    uint64_t a = desc_off(da, a_off);
+                    // 40 heads: the last group's partner is eight zero rows behind the stages (for the tile's second row SLOT further on)
+                    if (HK != NH && ks == HK / 16 - 1) a = umma_desc_sw128(st + a_off, SLOT, smem_u32(smem) + stages * stage_bytes - (st + a_off));
+                    umma_ss(tmem_base + w * S::STRIDE, a, desc_off(db0, ks * 32), idesc, ks > 0);
+                }
+                umma_commit(empty + s);
+                umma_commit(s_full + w);
             }
-            umma_commit_if(issue, empty + s);
-            umma_commit_if(issue, s_full + w);
+            __syncwarp();
             if (++s == stages) { s = 0; par ^= 1; }
             if (++w == WGS) { w = 0; wpar ^= 1; }
         }
     } else if (warp == WGS * 4 + 2) {
         // ------------------------------ MMA issuer: second layer ------------------------------
-        const uint32_t issue = lane == 0;
         constexpr uint32_t idesc = umma_idesc_f16(128, HK, 0, 0);
         const uint64_t db0 = umma_desc_sw128(smem_u32(sW2), 16, 1024);
         auto desc_off = [](uint64_t d, uint32_t bytes) -> uint64_t { return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4)); };
@@ -326,15 +326,18 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
             if (!(ok = __all_sync(0xffffffffu, ok))) break;
             tc_fence_after();
             const uint32_t buf = tmem_base + w * S::STRIDE;
-            int ks = 0;
-            for (; ks + 4 <= hid / 16; ks += 4) {
-                const uint64_t db = desc_off(db0, (ks >> 2) * (HK * 128));
+            if (elect_one()) {
+                int ks = 0;
+                for (; ks + 4 <= hid / 16; ks += 4) {
+                    const uint64_t db = desc_off(db0, (ks >> 2) * (HK * 128));
 #pragma unroll
-                for (int k = 0; k < 4; ++k) umma_ts_if(issue, buf + S::D_OFF, buf + (ks + k) * 8, desc_off(db, k * 32), idesc, ks + k > 0);
+                    for (int k = 0; k < 4; ++k) umma_ts(buf + S::D_OFF, buf + (ks + k) * 8, desc_off(db, k * 32), idesc, ks + k > 0);
+                }
+                for (; ks < hid / 16; ++ks)
+                    umma_ts(buf + S::D_OFF, buf + ks * 8, desc_off(db0, (ks >> 2) * (HK * 128) + (ks & 3) * 32), idesc, ks > 0);
+                umma_commit(o_full + w);
             }
-            for (; ks < hid / 16; ++ks)
-                umma_ts_if(issue, buf + S::D_OFF, buf + ks * 8, desc_off(db0, (ks >> 2) * (HK * 128) + (ks & 3) * 32), idesc, ks > 0);
-            umma_commit_if(issue, o_full + w);
+            __syncwarp();
             if (++w == WGS) { w = 0; wpar ^= 1; }
         }
     } else {

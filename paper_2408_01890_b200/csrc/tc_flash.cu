@@ -175,25 +175,19 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     if (warp == 4) {
         // ------------------------------ TMA producer ------------------------------
-        // The two single-thread roles (this one and the MMA issuer) share their scheduler with busy softmax warps and
-        // get an instruction slot every several cycles, so their loops are kept to a few dozen instructions per tile:
-        // running stage counters instead of divisions, one wait/arm section by lane 0 per tile, then every copy of
-        // the tile issued by different lanes (one 64-column box each).
         // V(t) (with Y(t)) travels together with K(t+1): both wait for the P.V of tile t-2 at the latest.
         constexpr int NQ = KD / 64, NK = KD / 64, NV = EMIT ? 0 : D / 64;
-        if (lane == 0) {
+        if (elect_one()) {
             tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK);
             if (!EMIT) tma_prefetch_desc(&tmV);
             if (PLANE) tma_prefetch_desc(&tmY);
             mbar_expect_tx(q_full, L::Q_BYTES);
             mbar_expect_tx(k_full, L::K_BYTES);
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) tma_load_4d(sQ + i * (BM * 128), &tmQ, q_full, i * 64, h, q0, b);
+#pragma unroll
+            for (int i = 0; i < NK; ++i) tma_load_4d(sK + i * (BN * 128), &tmK, k_full, i * 64, g, 0, b);
         }
-        __syncwarp();
-        // One call site per tensor map, each reached with the map and the barrier uniform over the warp and only the
-        // lane-dependent box differing, and a reconvergence point between sites.
-        if (lane < NQ) tma_load_4d(sQ + lane * (BM * 128), &tmQ, q_full, lane * 64, h, q0, b);
-        __syncwarp();
-        if (lane < NK) tma_load_4d(sK + lane * (BN * 128), &tmK, k_full, lane * 64, g, 0, b);
         __syncwarp();
         int ks_next = 1 % KST;              // K stage of tile t+1
         uint32_t kpar_next = 1;             // parity to wait for on its "empty" barrier (first pass: passes at once)
@@ -201,42 +195,37 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
             const int sv = t & 1;
             const bool more_k = t + 1 < nt;
             bool okp = true;
-            if (lane == 0) {
-                if constexpr (!EMIT) {
-                    okp = mbar_wait(v_empty + sv, ((t >> 1) & 1) ^ 1, abort_flag);
-                    if (okp) mbar_expect_tx(v_full + sv, L::V_BYTES + L::Y_BYTES);
-                }
-                if (okp && more_k) {
-                    okp = mbar_wait(k_empty + ks_next, kpar_next, abort_flag);
-                    if (okp) mbar_expect_tx(k_full + ks_next, L::K_BYTES);
-                }
-            }
-            okp = __shfl_sync(0xffffffffu, okp, 0);
-            if (!okp) break;
             if constexpr (!EMIT) {
-                if (lane < NV) tma_load_4d(sV + sv * L::V_BYTES + lane * (BN * 128), &tmV, v_full + sv, lane * 64, g, t * BN, b);
-                __syncwarp();
-            }
-            if constexpr (PLANE) {
-                if (lane == 0) tma_load_5d(sY + sv * L::Y_BYTES, &tmY, v_full + sv, 0, b * p.Hq + h, 0, t, (q0 - p.plane_row0) / BM);
+                okp = mbar_wait(v_empty + sv, ((t >> 1) & 1) ^ 1, abort_flag);
+                if (!__all_sync(0xffffffffu, okp)) break;
+                if (elect_one()) {
+                    mbar_expect_tx(v_full + sv, L::V_BYTES + L::Y_BYTES);
+#pragma unroll
+                    for (int i = 0; i < NV; ++i) tma_load_4d(sV + sv * L::V_BYTES + i * (BN * 128), &tmV, v_full + sv, i * 64, g, t * BN, b);
+                    if constexpr (PLANE) tma_load_5d(sY + sv * L::Y_BYTES, &tmY, v_full + sv, 0, b * p.Hq + h, 0, t, (q0 - p.plane_row0) / BM);
+                }
                 __syncwarp();
             }
             if (more_k) {
-                if (lane < NK) tma_load_4d(sK + ks_next * L::K_BYTES + lane * (BN * 128), &tmK, k_full + ks_next, lane * 64, g, (t + 1) * BN, b);
+                okp = mbar_wait(k_empty + ks_next, kpar_next, abort_flag);
+                if (!__all_sync(0xffffffffu, okp)) break;
+                if (elect_one()) {
+                    mbar_expect_tx(k_full + ks_next, L::K_BYTES);
+#pragma unroll
+                    for (int i = 0; i < NK; ++i) tma_load_4d(sK + ks_next * L::K_BYTES + i * (BN * 128), &tmK, k_full + ks_next, i * 64, g, (t + 1) * BN, b);
+                }
                 __syncwarp();
             }
             // The V and Y stages of a tile cannot be refilled before the P.V of the tile two before it has run, one softmax pass
             // before they are needed -- less than a trip to HBM under load.  Their tiles are therefore asked into L2 earlier,
             // kPrefetchAhead tiles ahead of the one just issued.
             if constexpr (kPrefetchAhead > 0 && !EMIT) {
-                if (t + kPrefetchAhead < nt) {
-                    if (lane < NV) tma_prefetch_l2_4d(&tmV, lane * 64, g, (t + kPrefetchAhead) * BN, b);
-                    __syncwarp();
-                    if constexpr (PLANE) {
-                        if (lane == 0) tma_prefetch_l2_5d(&tmY, 0, b * p.Hq + h, 0, t + kPrefetchAhead, (q0 - p.plane_row0) / BM);
-                        __syncwarp();
-                    }
+                if (t + kPrefetchAhead < nt && elect_one()) {
+#pragma unroll
+                    for (int i = 0; i < NV; ++i) tma_prefetch_l2_4d(&tmV, i * 64, g, (t + kPrefetchAhead) * BN, b);
+                    if constexpr (PLANE) tma_prefetch_l2_5d(&tmY, 0, b * p.Hq + h, 0, t + kPrefetchAhead, (q0 - p.plane_row0) / BM);
                 }
+                __syncwarp();
             }
             if (++ks_next == KST) { ks_next = 0; kpar_next ^= 1; }
         }
@@ -246,8 +235,7 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
         // the score MMAs and the P.V MMAs are issued by two different warps: each waits for its own operands and the
         // two hold-ups overlap instead of adding up.  Every lane of an issuing warp runs the loop (waits, stage
         // counters, descriptor arithmetic: all warp-uniform); only the MMA and commit instructions themselves are
-        // predicated on lane 0.
-        const uint32_t issue = lane == 0;
+        // issued by one elected lane.
         constexpr uint32_t IDESC_QK = umma_idesc_bf16(BM, BN, 0, 0);
         const int ksteps = p.ksteps;
         // Descriptors are built once; per MMA only the start-address field (bits 0-13 of the low word, in
@@ -268,21 +256,21 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
             tc_fence_after();
             const uint64_t dk = desc_off(dk0, sk * L::K_BYTES);
             const uint32_t dst = tmem_base + s * BN;
+            if (elect_one()) {
 #pragma unroll
-            for (int ks = 0; ks < KD / 16; ++ks) {
-                if (ks < ksteps) {
-                    umma_ss_if(issue, dst, desc_off(dq0, (ks >> 2) * (BM * 128) + (ks & 3) * 32), desc_off(dk, (ks >> 2) * (BN * 128) + (ks & 3) * 32),
-                               IDESC_QK, ks > 0);
+                for (int ks = 0; ks < KD / 16; ++ks) {
+                    if (ks < ksteps)
+                        umma_ss(dst, desc_off(dq0, (ks >> 2) * (BM * 128) + (ks & 3) * 32), desc_off(dk, (ks >> 2) * (BN * 128) + (ks & 3) * 32), IDESC_QK, ks > 0);
                 }
+                umma_commit(s_full + s);
+                if (!L::P_IN_K && t + KST < nt) umma_commit(k_empty + sk);  // nobody waits for the last ones: do not arm them
             }
-            umma_commit_if(issue, s_full + s);
-            if (!L::P_IN_K && t + KST < nt) umma_commit_if(issue, k_empty + sk);  // nobody waits for the last ones: do not arm them
+            __syncwarp();
             if (++sk == KST) { sk = 0; kpar ^= 1; }
         }
     } else if (warp == 6) {
         // ------------------------------ MMA issuer: P.V ------------------------------
         if constexpr (!EMIT) {
-            const uint32_t issue = lane == 0;
             constexpr uint32_t IDESC_PV = umma_idesc_bf16(BM, D, 0, 1);
             auto desc_off = [](uint64_t d, uint32_t bytes) -> uint64_t {
                 return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4));
@@ -299,15 +287,18 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                 tc_fence_after();
                 const uint64_t dp = desc_off(dp0, (L::P_IN_K ? pk : s) * P_STRIDE);
                 const uint64_t dv = desc_off(dv0, s * L::V_BYTES);
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < BN / 16; ++ks) {
-                    // P: K-major, 64 keys per 128-byte row; V: 16 keys = two 8-row groups, the next 64 d-columns
-                    // BN * 128 bytes further on
-                    umma_ss_if(issue, tmem_O, desc_off(dp, ks * 32), desc_off(dv, ks * 2048), IDESC_PV, (t > 0) || (ks > 0));
+                    for (int ks = 0; ks < BN / 16; ++ks) {
+                        // P: K-major, 64 keys per 128-byte row; V: 16 keys = two 8-row groups, the next 64 d-columns
+                        // BN * 128 bytes further on
+                        umma_ss(tmem_O, desc_off(dp, ks * 32), desc_off(dv, ks * 2048), IDESC_PV, (t > 0) || (ks > 0));
+                    }
+                    umma_commit(pv_done + s);
+                    if (t + 2 < nt) umma_commit(v_empty + s);
+                    if (L::P_IN_K && t + KST < nt) umma_commit(k_empty + pk);
                 }
-                umma_commit_if(issue, pv_done + s);
-                if (t + 2 < nt) umma_commit_if(issue, v_empty + s);
-                if (L::P_IN_K && t + KST < nt) umma_commit_if(issue, k_empty + pk);
+                __syncwarp();
                 if (++pk == KST) pk = 0;
             }
         }

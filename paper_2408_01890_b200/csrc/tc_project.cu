@@ -116,30 +116,25 @@ tc_project_kernel(const __grid_constant__ ProjParams p, const __grid_constant__ 
             tile_coord(tile, b, mt, nt);
             for (int ks = 0; ks < k_slices; ++ks, ++it) {
                 const int s = (int)(it % STAGES);
-                if (lane == 0) {
-                    ok = mbar_wait(empty + s, (uint32_t)((it / STAGES) & 1) ^ 1u, abort_flag);
-                    if (ok) mbar_expect_tx(full + s, STAGE_BYTES);
-                }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) break;
+                ok = mbar_wait(empty + s, (uint32_t)((it / STAGES) & 1) ^ 1u, abort_flag);
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
                 uint8_t* sa = smem + s * STAGE_BYTES;
                 uint8_t* sb = sa + A_BYTES;
                 // X slice: [128 rows][64 k]; W slice: four [64 k][64 n] quarters
-                if (lane == 0) {
+                if (elect_one()) {
+                    mbar_expect_tx(full + s, STAGE_BYTES);
                     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
                                  ::"r"(smem_u32(sa)), "l"(&tmX), "r"(smem_u32(full + s)), "r"(ks * BK), "r"(mt * BM), "r"(b) : "memory");
-                }
-                __syncwarp();
-                if (lane < BN / 64) {
-                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                                 ::"r"(smem_u32(sb + lane * (BK * 128))), "l"(&tmW), "r"(smem_u32(full + s)), "r"(nt * BN + lane * 64), "r"(ks * BK) : "memory");
+#pragma unroll
+                    for (int i = 0; i < BN / 64; ++i)
+                        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+                                     ::"r"(smem_u32(sb + i * (BK * 128))), "l"(&tmW), "r"(smem_u32(full + s)), "r"(nt * BN + i * 64), "r"(ks * BK) : "memory");
                 }
                 __syncwarp();
             }
         }
     } else if (warp == 1) {
-        // ------------------------------ MMA issuer (warp-uniform control flow, lane 0 issues) ------------------------------
-        const uint32_t issue = lane == 0;
+        // ------------------------------ MMA issuer (warp-uniform control flow, one elected lane issues) ------------------------------
         constexpr uint32_t IDESC = umma_idesc_bf16(BM, BN, 0, 1);   // X: K contiguous; W: N contiguous
         auto desc_off = [](uint64_t d, uint32_t bytes) -> uint64_t { return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4)); };
         const uint64_t da0 = umma_desc_sw128(smem_u32(smem), 16, 1024);
@@ -159,13 +154,14 @@ tc_project_kernel(const __grid_constant__ ProjParams p, const __grid_constant__ 
                 if (!(ok = __all_sync(0xffffffffu, ok))) break;
                 tc_fence_after();
                 const uint64_t da = desc_off(da0, s * STAGE_BYTES), db = desc_off(db0, s * STAGE_BYTES);
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk)
-                    umma_ss_if(issue, dst, desc_off(da, kk * 32), desc_off(db, kk * 2048), IDESC, (ks > 0) || (kk > 0));
-                umma_commit_if(issue, empty + s);
+                    for (int kk = 0; kk < BK / 16; ++kk) umma_ss(dst, desc_off(da, kk * 32), desc_off(db, kk * 2048), IDESC, (ks > 0) || (kk > 0));
+                    umma_commit(empty + s);
+                    if (ks + 1 == k_slices) umma_commit(acc_full + a);
+                }
+                __syncwarp();
             }
-            if (!ok) break;
-            umma_commit_if(issue, acc_full + a);
         }
     } else if (warp >= 4) {
         // ------------------------------ epilogue (thread = output row) ------------------------------
@@ -292,25 +288,24 @@ tc_project_narrow_kernel(const __grid_constant__ ProjParams p, const __grid_cons
         bool ok = aligned;
         for (int i = 0; ok && i < n_slices; ++i) {
             const int s = i % S::ST;
-            if (lane == 0) {
-                ok = mbar_wait(empty + s, (uint32_t)((i / S::ST) & 1) ^ 1u, abort_flag);
-                if (ok) mbar_expect_tx(full + s, S::STAGE);
-            }
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (!ok) break;
+            ok = mbar_wait(empty + s, (uint32_t)((i / S::ST) & 1) ^ 1u, abort_flag);
+            if (!(ok = __all_sync(0xffffffffu, ok))) break;
             uint8_t* sw = smem + s * S::STAGE;
             const int k0 = (k_begin + i) * S::KS;
-            if (lane < WB)
-                asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                             ::"r"(smem_u32(sw + lane * (S::KS * 128))), "l"(&tmW), "r"(smem_u32(full + s)), "r"(nt * S::BN_ + lane * 64), "r"(k0) : "memory");
-            __syncwarp();
-            if (lane < S::KS / 64)
-                asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                             ::"r"(smem_u32(sw + S::W_BYTES + lane * (NR * 128))), "l"(&tmX), "r"(smem_u32(full + s)), "r"(k0 + lane * 64), "r"(rt * NR) : "memory");
+            if (elect_one()) {
+                mbar_expect_tx(full + s, S::STAGE);
+#pragma unroll
+                for (int c = 0; c < WB; ++c)
+                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+                                 ::"r"(smem_u32(sw + c * (S::KS * 128))), "l"(&tmW), "r"(smem_u32(full + s)), "r"(nt * S::BN_ + c * 64), "r"(k0) : "memory");
+#pragma unroll
+                for (int c = 0; c < S::KS / 64; ++c)
+                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+                                 ::"r"(smem_u32(sw + S::W_BYTES + c * (NR * 128))), "l"(&tmX), "r"(smem_u32(full + s)), "r"(k0 + c * 64), "r"(rt * NR) : "memory");
+            }
             __syncwarp();
         }
     } else if (warp == 5) {
-        const uint32_t issue = lane == 0;
         constexpr uint32_t IDESC = umma_idesc_bf16(S::BN_, NR, 1, 0);   // W^T: columns contiguous (MN-major); X: K contiguous
         auto desc_off = [](uint64_t d, uint32_t bytes) -> uint64_t { return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4)); };
         const uint64_t da0 = umma_desc_sw128(smem_u32(smem), S::KS * 128, 1024);
@@ -322,12 +317,15 @@ tc_project_narrow_kernel(const __grid_constant__ ProjParams p, const __grid_cons
             if (!(ok = __all_sync(0xffffffffu, ok))) break;
             tc_fence_after();
             const uint64_t da = desc_off(da0, s * S::STAGE), db = desc_off(db0, s * S::STAGE);
+            if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < S::KS / 16; ++kk)
-                umma_ss_if(issue, tmem_base, desc_off(da, kk * 2048), desc_off(db, (kk >> 2) * (NR * 128) + (kk & 3) * 32), IDESC, (i > 0) || (kk > 0));
-            if (i + S::ST < n_slices) umma_commit_if(issue, empty + s);
+                for (int kk = 0; kk < S::KS / 16; ++kk)
+                    umma_ss(tmem_base, desc_off(da, kk * 2048), desc_off(db, (kk >> 2) * (NR * 128) + (kk & 3) * 32), IDESC, (i > 0) || (kk > 0));
+                if (i + S::ST < n_slices) umma_commit(empty + s);
+                if (i + 1 == n_slices) umma_commit(acc_full);
+            }
+            __syncwarp();
         }
-        if (ok) umma_commit_if(issue, acc_full);
     } else {
         // thread = column of the tile; fp32 partial tile [row][columns] over the drained stages.  Tensor-memory lane of a column:
         // the column itself with 128 of them; with 64, sixteen per warp's quarter
