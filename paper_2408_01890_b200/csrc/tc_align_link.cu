@@ -19,9 +19,12 @@
 // 128 contiguous bytes, so the TMA-loaded tile is the first layer's A operand as it stands (M-major, K = heads); its fp32
 // result goes from tensor memory through the registers (bias, activation, rounding to fp16) back into tensor memory, where
 // it is the second layer's A operand.  Nothing but the planes and the weights (B operands, in shared memory for the whole
-// launch) touches shared memory.  Roles: one warp loads, one issues each layer's MMAs, WGS warpgroups take the tiles in
-// turn, each with 512 / WGS columns of tensor memory of its own, so that the waits of one tile (two MMAs, four barriers)
-// hide behind the arithmetic of the others.
+// launch) touches shared memory.  Roles: one warp loads, one issues each layer's MMAs, and BUFS tiles are in flight, each with
+// 512 / BUFS columns of tensor memory, so that the waits of one tile (two MMAs, four barriers) hide behind the arithmetic of
+// the others.  There are always four warpgroups: with two tiles in flight, two share a tile, half of the hidden layer and half
+// of the heads each.
+// Measured: 64 -> 256 -> 32 on 2048 tokens of 32 heads 272 us with warp-level MMAs (their fragments came through shared
+// memory), 120 us now, where the planes' 415 MB take 63; 40 -> 80 -> 40 on 2 x 1777 tokens 138 us before, 97 now (80).
 #include <algorithm>
 
 #include "tc_align_mma.cuh"
@@ -56,7 +59,7 @@ struct LinkParams {
 };
 
 // Shared memory of a launch: [stages][plane x, plane d][2 rows][heads][128 B], zero rows, weights, staging, biases, barriers.
-template <int NH, bool CONCAT, int WGS>
+template <int NH, bool CONCAT, int BUFS>
 struct Shape {
     static constexpr int HK = (NH + 15) / 16 * 16;            // heads as an MMA's K (or N): zero-padded to 16
     static constexpr int H_IN = CONCAT ? 2 * NH : NH;
@@ -64,16 +67,22 @@ struct Shape {
     static constexpr int SLOT = NH * 128;                     // one query row of a tile
     static constexpr int TILE = 2 * SLOT;
     static constexpr int ZERO = HK == NH ? 0 : SLOT + 1024;   // the padding heads of both rows (see the first layer's issuer)
-    static constexpr int STG = NH * 64;                       // a warp's 32 positions on the way out
-    static constexpr int STRIDE = 512 / WGS, D_OFF = STRIDE / 2;   // tensor-memory columns of a warpgroup; its second-layer result
-    static constexpr int CHUNK = WGS > 2 ? 32 : 64;           // hidden units a thread holds at a time (registers)
-    static constexpr int THREADS = WGS * 128 + 96;            // + loader, two MMA issuers
-    static_assert(K1 <= 64 && (!CONCAT || HK == NH) && D_OFF + HK <= STRIDE, "layout");
+    static constexpr int TW = 4 / BUFS;                       // warpgroups that share a tile
+    static constexpr int STRIDE = 512 / BUFS;                 // tensor-memory columns of a tile in flight
+    // Hidden units HALF * i .. of warpgroup i of a tile.  Their sums are read from columns HALF * i and written back, half as wide, from
+    // the same column on, so that the two never touch what the other has not read; the second layer's result follows the first's.
+    static constexpr int HALF = STRIDE / TW, D_OFF = HALF / 2;
+    static constexpr int NG = NH / 8, GW = (NG + TW - 1) / TW;   // groups of 8 heads; of a warpgroup
+    static constexpr int BOX = NG % TW == 0 ? GW * 8 : 8;     // heads of one copy out
+    static constexpr int STG = GW * 8 * 64;                   // a warp's 32 positions of its heads on the way out
+    static constexpr int CHUNK = 32;                          // hidden units a thread holds at a time (registers)
+    static constexpr int THREADS = 4 * 128 + 96;              // + loader, two MMA issuers
+    static_assert(K1 <= 64 && (!CONCAT || HK == NH) && D_OFF + HK <= HALF, "layout");
     static __host__ __device__ int stage_bytes(bool has_d) { return TILE * (has_d ? 2 : 1); }
     static __host__ __device__ int w1_off(int stages, bool has_d) { return stages * stage_bytes(has_d) + ZERO; }
     static __host__ __device__ int w2_off(int w1, int hid) { return w1 + hid * 128; }
     static __host__ __device__ int stg_off(int w2, int hid) { return w2 + (hid + 63) / 64 * (HK * 128); }
-    static __host__ __device__ int bias_off(int stg) { return stg + WGS * 4 * 2 * STG; }
+    static __host__ __device__ int bias_off(int stg) { return stg + 16 * 2 * STG; }
     static __host__ __device__ int bar_off(int bias, int hid) { return bias + hid * 2 + HK * 4; }
     static __host__ int total(int stages, bool has_d, int hid) {
         return bar_off(bias_off(stg_off(w2_off(w1_off(stages, has_d), hid), hid)), hid) + (2 * kMaxStages + 4 * 4) * 8 + 16;
@@ -120,9 +129,8 @@ __device__ __forceinline__ void stmatrix_x2_trans(uint32_t saddr, uint32_t r0, u
     asm volatile("stmatrix.sync.aligned.m8n8.x2.trans.shared.b16 [%0], {%1,%2};" ::"r"(saddr), "r"(r0), "r"(r1) : "memory");
 }
 // A warp's results, times `scale`, as [head][32 positions] rows of 64 bytes whose 16-byte chunks carry the copy engine's 64-byte swizzle.
-template <int NH>
-__device__ __forceinline__ void put_frags(uint32_t stg, int lane, const float (*y)[NH / 8][4], float scale) {
-    constexpr int NG = NH / 8;
+template <int NG>
+__device__ __forceinline__ void put_frags(uint32_t stg, int lane, const float (*y)[NG][4], float scale) {
 #pragma unroll
     for (int s2 = 0; s2 < 2; ++s2)
 #pragma unroll
@@ -181,11 +189,11 @@ struct Cursor {
     }
 };
 
-template <int NH, bool CONCAT, int ACT, int WGS>
-__global__ void __launch_bounds__(Shape<NH, CONCAT, WGS>::THREADS, 1)
+template <int NH, bool CONCAT, int ACT, int BUFS>
+__global__ void __launch_bounds__(Shape<NH, CONCAT, BUFS>::THREADS, 1)
 tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD,
                      const __grid_constant__ CUtensorMap tmXs, const __grid_constant__ CUtensorMap tmDs) {
-    using S = Shape<NH, CONCAT, WGS>;
+    using S = Shape<NH, CONCAT, BUFS>;
     constexpr int HK = S::HK, K1 = S::K1, SLOT = S::SLOT, TILE = S::TILE, STG = S::STG;
     extern __shared__ __align__(1024) uint8_t smem[];
     if ((smem_u32(smem) & 1023u) != 0) {   // the swizzled tiles' bases: refuse loudly instead of computing garbage
@@ -205,10 +213,10 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + bar_off);
     uint64_t* full = bars;                       // [stages]
     uint64_t* empty = bars + kMaxStages;         // [stages] first layer done (and, where it is added later, plane d read)
-    uint64_t* s_full = bars + 2 * kMaxStages;    // [WGS] first layer's sums
-    uint64_t* h_full = s_full + 4;               // [WGS] hidden layer written back
-    uint64_t* o_full = s_full + 8;               // [WGS] second layer's sums
-    uint64_t* b_free = s_full + 12;              // [WGS] ... read: the columns are free
+    uint64_t* s_full = bars + 2 * kMaxStages;    // [BUFS] first layer's sums
+    uint64_t* h_full = s_full + 4;               // [BUFS] hidden layer written back
+    uint64_t* o_full = s_full + 8;               // [BUFS] second layer's sums
+    uint64_t* b_free = s_full + 12;              // [BUFS] ... read: the columns are free
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_full + 16);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -249,8 +257,8 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
     for (int e = tid; e < S::ZERO / 16; e += S::THREADS)
         *reinterpret_cast<uint4*>(smem + stages * stage_bytes + e * 16) = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) {
-        for (int i = 0; i < stages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, (!CONCAT && has_d) ? 5 : 1); }
-        for (int i = 0; i < WGS; ++i) { mbar_init(s_full + i, 1); mbar_init(h_full + i, 4); mbar_init(o_full + i, 1); mbar_init(b_free + i, 4); }
+        for (int i = 0; i < stages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, (!CONCAT && has_d) ? 1 + 4 * S::TW : 1); }
+        for (int i = 0; i < BUFS; ++i) { mbar_init(s_full + i, 1); mbar_init(h_full + i, 4 * S::TW); mbar_init(o_full + i, 1); mbar_init(b_free + i, 4 * S::TW); }
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -263,7 +271,7 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
     chain_release();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
-    if (warp == WGS * 4) {
+    if (warp == 16) {
         // ------------------------------ loader: one thread, one copy per plane and tile ------------------------------
         // (a copy per query row, issued by two lanes of a converged warp, took 1300 cycles a tile: more than the tile's arithmetic)
         if (elect_one()) {
@@ -285,7 +293,7 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
             }
         }
         __syncwarp();
-    } else if (warp == WGS * 4 + 1) {
+    } else if (warp == 17) {
         // ------------------------------ MMA issuer: first layer ------------------------------
         const uint32_t idesc = umma_idesc_f16(128, hid, 1, 0);
         const uint64_t db0 = umma_desc_sw128(smem_u32(sW1), 16, 1024);
@@ -312,9 +320,9 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
             }
             __syncwarp();
             if (++s == stages) { s = 0; par ^= 1; }
-            if (++w == WGS) { w = 0; wpar ^= 1; }
+            if (++w == BUFS) { w = 0; wpar ^= 1; }
         }
-    } else if (warp == WGS * 4 + 2) {
+    } else if (warp == 18) {
         // ------------------------------ MMA issuer: second layer ------------------------------
         constexpr uint32_t idesc = umma_idesc_f16(128, HK, 0, 0);
         const uint64_t db0 = umma_desc_sw128(smem_u32(sW2), 16, 1024);
@@ -327,61 +335,70 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
             tc_fence_after();
             const uint32_t buf = tmem_base + w * S::STRIDE;
             if (elect_one()) {
-                int ks = 0;
-                for (; ks + 4 <= hid / 16; ks += 4) {
-                    const uint64_t db = desc_off(db0, (ks >> 2) * (HK * 128));
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) umma_ts(buf + S::D_OFF, buf + (ks + k) * 8, desc_off(db, k * 32), idesc, ks + k > 0);
+                for (int i2 = 0; i2 < S::TW; ++i2) {
+                    const int n_ks = min(hid - i2 * S::HALF, S::HALF) / 16;   // k-steps of this warpgroup's hidden units
+                    const uint32_t a = buf + i2 * S::HALF, b_ks = i2 * (S::HALF / 16);
+                    int ks = 0;
+                    for (; ks + 4 <= n_ks; ks += 4) {
+                        const uint64_t db = desc_off(db0, ((b_ks + ks) >> 2) * (HK * 128));
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) umma_ts(buf + S::D_OFF, a + (ks + k) * 8, desc_off(db, k * 32), idesc, b_ks + ks + k > 0);
+                    }
+                    for (; ks < n_ks; ++ks)
+                        umma_ts(buf + S::D_OFF, a + ks * 8, desc_off(db0, ((b_ks + ks) >> 2) * (HK * 128) + (ks & 3) * 32), idesc, b_ks + ks > 0);
                 }
-                for (; ks < hid / 16; ++ks)
-                    umma_ts(buf + S::D_OFF, buf + ks * 8, desc_off(db0, (ks >> 2) * (HK * 128) + (ks & 3) * 32), idesc, ks > 0);
                 umma_commit(o_full + w);
             }
             __syncwarp();
-            if (++w == WGS) { w = 0; wpar ^= 1; }
+            if (++w == BUFS) { w = 0; wpar ^= 1; }
         }
     } else {
         // ------------------------------ warpgroups: hidden layer and results (thread = position) ------------------------------
-        const int w = warp >> 2, q = warp & 3;
+        const int w = (warp >> 2) / S::TW, hf = (warp >> 2) % S::TW, q = warp & 3;   // tile in flight, share of it, quarter of the positions
         const uint32_t buf = tmem_base + w * S::STRIDE + ((uint32_t)(q * 32) << 16);
         const int dst_next = p.dst_next, dst_scaled = p.dst_scaled;
         uint8_t* stg = smem + stg_off + warp * (2 * STG);
         const uint32_t stg_u32 = smem_u32(stg);
-        constexpr int NG = NH / 8;
-        float2 bias2[NG];
+        constexpr int NG = S::NG, GW = S::GW;
+        const int g0 = hf * GW;   // this warpgroup's first group of heads; groups beyond the last are computed as the last and not stored
+        float2 bias2[GW];
 #pragma unroll
-        for (int g = 0; g < NG; ++g) bias2[g] = *reinterpret_cast<const float2*>(b2 + g * 8 + 2 * (lane & 3));
+        for (int g = 0; g < GW; ++g) bias2[g] = *reinterpret_cast<const float2*>(b2 + min(g0 + g, NG - 1) * 8 + 2 * (lane & 3));
         Cursor cu;
         if (w < n_tiles) cu.seek(p, t_begin + w);
         int s = w % stages;
         uint32_t spar = (w / stages) & 1, wpar = 0;
-        for (int i = w; i < n_tiles; i += WGS) {
+        for (int i = w; i < n_tiles; i += BUFS) {
             if (!__all_sync(0xffffffffu, mbar_wait(s_full + w, wpar, abort_flag))) break;
             tc_fence_after();
+            const uint32_t col = buf + hf * S::HALF;
+            const uint32_t* bias1 = b1h + hf * (S::HALF / 2);
+            const int units = min(hid - hf * S::HALF, S::HALF);
             int c = 0;
-            for (; c + S::CHUNK <= hid; c += S::CHUNK) {
+            for (; c + S::CHUNK <= units; c += S::CHUNK) {
                 uint32_t f[S::CHUNK], h[S::CHUNK / 2];
 #pragma unroll
-                for (int k = 0; k < S::CHUNK; k += 32) tmem_ld32(buf + c + k, f + k);
+                for (int k = 0; k < S::CHUNK; k += 32) tmem_ld32(col + c + k, f + k);
                 tmem_wait_ld();
 #pragma unroll
                 for (int j = 0; j < S::CHUNK / 8; ++j) {
-                    const uint4 bb = *reinterpret_cast<const uint4*>(b1h + c / 2 + 4 * j);
+                    const uint4 bb = *reinterpret_cast<const uint4*>(bias1 + c / 2 + 4 * j);
                     h[4 * j + 0] = hidden_pair<ACT>(__uint_as_float(f[8 * j + 0]), __uint_as_float(f[8 * j + 1]), bb.x);
                     h[4 * j + 1] = hidden_pair<ACT>(__uint_as_float(f[8 * j + 2]), __uint_as_float(f[8 * j + 3]), bb.y);
                     h[4 * j + 2] = hidden_pair<ACT>(__uint_as_float(f[8 * j + 4]), __uint_as_float(f[8 * j + 5]), bb.z);
                     h[4 * j + 3] = hidden_pair<ACT>(__uint_as_float(f[8 * j + 6]), __uint_as_float(f[8 * j + 7]), bb.w);
                 }
 #pragma unroll
-                for (int k = 0; k < S::CHUNK / 2; k += 16) tmem_st16(buf + c / 2 + k, h + k);
+                for (int k = 0; k < S::CHUNK / 2; k += 16) tmem_st16(col + c / 2 + k, h + k);
             }
-            for (; c < hid; c += 16) {
+            for (; c < units; c += 16) {
                 uint32_t f[16], h[8];
-                tmem_ld16(buf + c, f);
+                tmem_ld16(col + c, f);
                 tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 8; ++j) h[j] = hidden_pair<ACT>(__uint_as_float(f[2 * j]), __uint_as_float(f[2 * j + 1]), b1h[c / 2 + j]);
-                tmem_st8(buf + c / 2, h);
+                for (int j = 0; j < 8; ++j) h[j] = hidden_pair<ACT>(__uint_as_float(f[2 * j]), __uint_as_float(f[2 * j + 1]), bias1[c / 2 + j]);
+                tmem_st8(col + c / 2, h);
             }
             tmem_wait_st();
             tc_fence_before();
@@ -393,15 +410,15 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
             tc_fence_after();
             // a warp's 32 positions as two strips of 16, eight heads at a time: lane holds heads 2(lane % 4), + 1 of positions lane / 4, + 8,
             // the fragment arrangement stmatrix and ldmatrix transpose from and to [head][position] rows
-            float y[2][NG][4];
+            float y[2][GW][4];
 #pragma unroll
             for (int s2 = 0; s2 < 2; ++s2)
 #pragma unroll
-                for (int g = 0; g < NG; ++g) tmem_ld_frag(buf + S::D_OFF + ((uint32_t)(s2 * 16) << 16) + g * 8, y[s2][g]);
+                for (int g = 0; g < GW; ++g) tmem_ld_frag(buf + S::D_OFF + ((uint32_t)(s2 * 16) << 16) + min(g0 + g, NG - 1) * 8, y[s2][g]);
             tmem_wait_ld();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) {
+            if (elect_one()) {
                 mbar_arrive(b_free + w);
                 tma_store_wait_read<0>();   // the previous tile's stores have read the staging buffers
             }
@@ -409,25 +426,25 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
 #pragma unroll
             for (int s2 = 0; s2 < 2; ++s2)
 #pragma unroll
-                for (int g = 0; g < NG; ++g) {
+                for (int g = 0; g < GW; ++g) {
                     y[s2][g][0] += bias2[g].x; y[s2][g][1] += bias2[g].y;
                     y[s2][g][2] += bias2[g].x; y[s2][g][3] += bias2[g].y;
                 }
-            if (dst_scaled >= 0) put_frags<NH>(stg_u32, lane, y, kLog2e);
+            if (dst_scaled >= 0) put_frags<GW>(stg_u32, lane, y, kLog2e);
             if (!CONCAT && has_d) {   // A_k = FFN(A_{k-1}) + D_k
                 if (!__all_sync(0xffffffffu, mbar_wait(full + s, spar, abort_flag))) break;
                 const uint32_t db = smem_u32(smem) + s * stage_bytes + TILE + (q >> 1) * SLOT;
 #pragma unroll
                 for (int s2 = 0; s2 < 2; ++s2)
 #pragma unroll
-                    for (int g = 0; g < NG; g += 2) {
+                    for (int g = 0; g < GW; g += 2) {
                         // four 8 x 8 blocks: (heads g, positions 0-7), (g, 8-15), (g + 1, 0-7), (g + 1, 8-15); beyond the last head: g again
-                        const int head = min(g + (lane >> 4), NG - 1) * 8 + (lane & 7), chunk = (q & 1) * 4 + 2 * s2 + ((lane >> 3) & 1);
+                        const int head = min(g0 + g + (lane >> 4), NG - 1) * 8 + (lane & 7), chunk = (q & 1) * 4 + 2 * s2 + ((lane >> 3) & 1);
                         uint32_t dfr[4];
                         ldmatrix_x4_trans(dfr, db + sw128_offset(head, chunk));
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
-                            if (g + (k >> 1) >= NG) break;
+                            if (g + (k >> 1) >= GW) break;
                             const float2 dv = unpack_f16(dfr[k]);
                             y[s2][g + (k >> 1)][2 * (k & 1)] += dv.x;
                             y[s2][g + (k >> 1)][2 * (k & 1) + 1] += dv.y;
@@ -436,27 +453,33 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty + s);
             }
-            if (dst_next >= 0) put_frags<NH>(stg_u32 + STG, lane, y, 1.f);
+            if (dst_next >= 0) put_frags<GW>(stg_u32 + STG, lane, y, 1.f);
             fence_async_smem();
             __syncwarp();
-            if (lane == 0) {
+            if (elect_one()) {
                 const int row = cu.r + (q >> 1), x = (q & 1) * 32;
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     const int rel = row - (k ? p.d_row0 : p.row0);
                     const CUtensorMap* map = k ? &tmDs : &tmXs;
-                    if (dst_scaled == k) tma_store_5d(map, stg, x, cu.b * NH, rel & 127, cu.jb, rel >> 7);
-                    if (dst_next == k) tma_store_5d(map, stg + STG, x, cu.b * NH, rel & 127, cu.jb, rel >> 7);
+#pragma unroll
+                    for (int g = 0; g < GW; g += S::BOX / 8) {
+                        if (g0 + g >= NG) break;
+                        const int head = cu.b * NH + (g0 + g) * 8;
+                        if (dst_scaled == k) tma_store_5d(map, stg + g * 512, x, head, rel & 127, cu.jb, rel >> 7);
+                        if (dst_next == k) tma_store_5d(map, stg + STG + g * 512, x, head, rel & 127, cu.jb, rel >> 7);
+                    }
                 }
                 tma_store_commit();
             }
 #pragma unroll
-            for (int k = 0; k < WGS; ++k) {
+            for (int k = 0; k < BUFS; ++k) {
                 cu.step(p);
                 if (++s == stages) { s = 0; spar ^= 1; }
             }
         }
-        if (lane == 0) tma_store_wait_all<0>();
+        if (elect_one()) tma_store_wait_all<0>();
+        __syncwarp();
     }
     // ------------------------------ teardown ------------------------------
     tc_fence_before();
@@ -476,30 +499,34 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
 }
 
 // One plane as the loads see it (64 columns x the heads of two query rows) and as the stores do (a warp's 32 columns of one).
-bool plane_maps(CUtensorMap* load, CUtensorMap* store, const void* plane, int B, int NH, int64_t rows, int64_t cols) {
+bool plane_maps(CUtensorMap* load, CUtensorMap* store, const void* plane, int B, int NH, int out_heads, int64_t rows, int64_t cols) {
     const uint64_t bh = (uint64_t)B * NH, ncb = (uint64_t)cols / 64, nrb = (uint64_t)rows / UNIT;
     const uint64_t dims[5] = {64, bh, (uint64_t)UNIT, ncb, nrb};
     const uint64_t str[4] = {128, bh * 128, UNIT * bh * 128, ncb * UNIT * bh * 128};
-    const uint32_t in[5] = {64, (uint32_t)NH, 2, 1, 1}, out[5] = {32, (uint32_t)NH, 1, 1, 1};
+    const uint32_t in[5] = {64, (uint32_t)NH, 2, 1, 1}, out[5] = {32, (uint32_t)out_heads, 1, 1, 1};
     return make_tensor_map_bf16(load, plane, 5, dims, str, in, true) && make_tensor_map_bf16(store, plane, 5, dims, str, out, true, 64);
 }
 
-template <int NH, bool CONCAT, int WGS>
-cudaError_t launch_shape(LinkParams p, int act, const CUtensorMap* maps, bool chained, cudaStream_t stream) {
-    using S = Shape<NH, CONCAT, WGS>;
+template <int NH, bool CONCAT, int BUFS>
+cudaError_t launch_shape(LinkParams p, int act, const TcAlignLinkArgs& a, int64_t d_rows, int64_t d_cols, cudaStream_t stream) {
+    using S = Shape<NH, CONCAT, BUFS>;
     constexpr int kSmem = 232448;   // one CTA's shared memory
+    CUtensorMap maps[4];
+    if (!plane_maps(maps, maps + 2, a.plane_x, a.B, NH, S::BOX, a.plane_rows, a.plane_cols)) return cudaErrorInvalidValue;
+    maps[1] = maps[0]; maps[3] = maps[2];
+    if (a.plane_d && !plane_maps(maps + 1, maps + 3, a.plane_d, a.B, NH, S::BOX, d_rows, d_cols)) return cudaErrorInvalidValue;
     p.stages = kMaxStages;
     while (p.stages > 2 && S::total(p.stages, p.has_d != 0, p.hid) > kSmem) --p.stages;
     const size_t smem = std::max(S::total(p.stages, p.has_d != 0, p.hid), kSmem / 2 + 1);   // one CTA per SM: it takes all of the tensor memory
     if (smem > kSmem) return cudaErrorInvalidValue;
-    auto kernel = act == LISA_ACT_RELU   ? tc_align_link_kernel<NH, CONCAT, LISA_ACT_RELU, WGS>
-                  : act == LISA_ACT_SILU ? tc_align_link_kernel<NH, CONCAT, LISA_ACT_SILU, WGS>
-                                         : tc_align_link_kernel<NH, CONCAT, LISA_ACT_NONE, WGS>;
+    auto kernel = act == LISA_ACT_RELU   ? tc_align_link_kernel<NH, CONCAT, LISA_ACT_RELU, BUFS>
+                  : act == LISA_ACT_SILU ? tc_align_link_kernel<NH, CONCAT, LISA_ACT_SILU, BUFS>
+                                         : tc_align_link_kernel<NH, CONCAT, LISA_ACT_NONE, BUFS>;
     cudaError_t e = allow_smem(kernel, smem, true);
     if (e != cudaSuccess) return e;
     // two tiles per CTA at least: half of a CTA's time on a single tile would be the weights
     const unsigned grid = (unsigned)std::min<int64_t>((p.total + 1) / 2, sm_count());
-    return launch_kernel(chained, kernel, dim3(grid), dim3(S::THREADS), smem, stream, p, maps[0], maps[1], maps[2], maps[3]);
+    return launch_kernel(a.chained, kernel, dim3(grid), dim3(S::THREADS), smem, stream, p, maps[0], maps[1], maps[2], maps[3]);
 }
 
 bool link_ok(int Hq, const lisa_link& l) {
@@ -550,12 +577,8 @@ cudaError_t launch_tc_align_link(const TcAlignLinkArgs& a, cudaStream_t stream) 
     if (tiles * a.B > 0x3fffffff) return cudaErrorInvalidValue;
     p.tiles_per_batch = (int)tiles;
     p.total = (int)tiles * a.B;
-    CUtensorMap maps[4];
-    if (!plane_maps(maps, maps + 2, a.plane_x, a.B, a.Hq, a.plane_rows, a.plane_cols)) return cudaErrorInvalidValue;
-    maps[1] = maps[0]; maps[3] = maps[2];
     p.has_d = a.plane_d != nullptr;
-    if (a.plane_d && !plane_maps(maps + 1, maps + 3, a.plane_d, a.B, a.Hq, a.d_plane_cols > 0 ? a.d_plane_rows : a.plane_rows, d_cols))
-        return cudaErrorInvalidValue;
+    const int64_t d_rows = a.d_plane_cols > 0 ? a.d_plane_rows : a.plane_rows;
     p.status = status_words();
     if (!p.status) return cudaErrorUnknown;
     p.dst_next = a.dst_next; p.dst_scaled = a.dst_scaled;
@@ -565,11 +588,11 @@ cudaError_t launch_tc_align_link(const TcAlignLinkArgs& a, cudaStream_t stream) 
     const int act = p.kind == KIND_FFN ? l.act : LISA_ACT_NONE;
     const int inputs = concat ? 2 * a.Hq : a.Hq;
     p.hid = ((p.kind == KIND_FFN ? l.m : inputs) + 15) / 16 * 16;
-    // Four warpgroups in turn as long as a quarter of the tensor memory holds a tile's hidden layer (128 units), two above.
+    // Four tiles in flight as long as a quarter of the tensor memory holds a tile's hidden layer (128 units), two above.
     cudaError_t e;
-    if (concat) e = p.hid <= 128 ? launch_shape<32, true, 4>(p, act, maps, a.chained, stream) : launch_shape<32, true, 2>(p, act, maps, a.chained, stream);
-    else if (a.Hq == 32) e = p.hid <= 128 ? launch_shape<32, false, 4>(p, act, maps, a.chained, stream) : launch_shape<32, false, 2>(p, act, maps, a.chained, stream);
-    else e = p.hid <= 128 ? launch_shape<40, false, 4>(p, act, maps, a.chained, stream) : launch_shape<40, false, 2>(p, act, maps, a.chained, stream);
+    if (concat) e = p.hid <= 128 ? launch_shape<32, true, 4>(p, act, a, d_rows, d_cols, stream) : launch_shape<32, true, 2>(p, act, a, d_rows, d_cols, stream);
+    else if (a.Hq == 32) e = p.hid <= 128 ? launch_shape<32, false, 4>(p, act, a, d_rows, d_cols, stream) : launch_shape<32, false, 2>(p, act, a, d_rows, d_cols, stream);
+    else e = p.hid <= 128 ? launch_shape<40, false, 4>(p, act, a, d_rows, d_cols, stream) : launch_shape<40, false, 2>(p, act, a, d_rows, d_cols, stream);
     count_launches(1);
     return e;
 }
