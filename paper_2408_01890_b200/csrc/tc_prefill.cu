@@ -340,7 +340,8 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
     const int c = a.chain_len;
     cudaError_t e;
     SideStream* side = nullptr;
-    const bool small = !ho && (int64_t)a.B * a.Hq * ((a.N + kTile - 1) / kTile) <= 2 * (int64_t)sm_count();   // one wave of CTAs that are resident at once: its kernels go out as a programmatic chain
+    // one wave of CTAs that are resident at once: the call's kernels go out as a programmatic chain
+    const bool one_wave = (int64_t)a.B * a.Hq * ((a.N + kTile - 1) / kTile) <= 2 * (int64_t)sm_count(), small = one_wave && !ho;
     {
         PhaseMark mark(0, s);
         PackJobs jobs{};
@@ -463,7 +464,10 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
             if (stream_out && (e = copy_out(wv, st)) != cudaSuccess) return e;
             continue;
         }
-        const bool per_link = !tc_align_supported(a.Hq, a.links, c);
+        // A single link also goes to the link kernel, where tcgen05 gains more than its longer set-up costs: from prompts of a few waves on
+        // (2048 tokens of 32 heads 68 -> 65 us, 4 x 8192 730 -> 420 us a wave; 197 tokens 6.6 -> 8.6 us, hence the limit).  Longer chains in one pass stay with the
+        // chain kernel, which reads and writes the planes once for all links.
+        const bool per_link = !tc_align_supported(a.Hq, a.links, c) || (c == 1 && !one_wave);
         if (per_link) {
             // 2l. shapes the chain kernel does not take (40 heads, wider hidden layers): one launch per link.  Link k reads
             // plane k, writes A_k = FFN_k(A_{k-1}) + D_k over plane k + 1 (which held D_k) and, where a layer's attention
