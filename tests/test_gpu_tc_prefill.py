@@ -432,3 +432,25 @@ def test_small_prompt_chain_replayed_from_a_graph():
     g.replay()
     torch.cuda.synchronize()
     assert all(torch.equal(a, b) for a, b in zip(outs, ref)) and lb.lisa_check() == lb.OK
+
+
+@pytest.mark.parametrize("B,N,Hq,Hkv,m,act,bias", [
+    (3, 385, 32, 8, 64, "relu", True),     # 32 -> 64 -> 32 above one wave of CTAs; odd row count: a tile's second row lies past the prompt
+    (3, 447, 32, 32, 1, "silu", True),     # one hidden unit in a padded k-step
+    (3, 385, 32, 8, 33, "none", False),    # 48 hidden units of the MMAs, the last 15 zero
+    (3, 512, 32, 32, 112, "silu", True),   # remainder of the 32-unit chunks
+    (3, 385, 32, 8, 129, "relu", True),    # the second warpgroup of a tile has one k-step
+    (3, 386, 40, 40, 129, "relu", True)])  # 40 heads over two warpgroups: three groups and two
+def test_single_links_of_several_waves_take_the_link_kernel(B, N, Hq, Hkv, m, act, bias):
+    """One-link calls of more than one wave of CTAs: recomputed, and as two layers that carry the scores."""
+    t = link_inputs(B, N, Hq, Hkv, 2, m, act, 2, 21, 41, bias)
+    dl, ol = make_links(t, 2, act, lb.INTEGRATE_ADD, 2, bias)
+    q0, k0 = dev(t["q0"]), dev(t["k0"])
+    ref = [oracle.prefill_full(f64(t["q0"]), f64(t["k0"]), f64(t[f"v{k + 1}"]), ol[:k + 1]) for k in range(2)]
+    got = lb.lisa_attn_shared_prefill(q0, k0, dl[:1], dev(t["v1"]))
+    assert_close(got.float().cpu().numpy(), ref[0], "bf16", "one link, recomputed")
+    scores = torch.full((lb.lisa_prefill_scores_bytes(B, N, Hq),), 0xFF, dtype=torch.uint8, device="cuda")
+    for k in range(2):
+        got = lb.lisa_attn_shared_prefill_carry(q0, k0, dl[k], dev(t[f"v{k + 1}"]), scores, first=k == 0, keep=k == 0)
+        assert_close(got.float().cpu().numpy(), ref[k], "bf16", "one link a call, layer %d" % (k + 1))
+    assert lb.lisa_check() == lb.OK
