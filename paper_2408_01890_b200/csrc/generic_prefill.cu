@@ -26,6 +26,30 @@ struct PrefillParams {
     int w_off[kMaxChain], w_floats[kMaxChain];   // where a link's weights are staged in shared memory (floats; -1: read from memory), how many
 };
 
+// A CTA's shared memory, in floats from its start; the staged weights follow.  q0, and q' of every link, are read as float4 (dots<0, 4>) at
+// h * d and h * kMaxRank, so both must start on 16 bytes whatever the head count: they come before the arrays of Hq values.
+struct SmemLayout {
+    int q0, o, s, d, qp, m, l, sc, total;
+    __host__ __device__ constexpr SmemLayout(int Hq, int width, int c)
+        : q0(0),                          // [Hq][d]
+          o(q0 + Hq * width),             // [Hq][d]
+          s(o + Hq * width),              // [Hq][kChunk] scores of the chunk
+          d(s + Hq * kChunk),             // [Hq][kChunk] a link's difference; then partial sums of the product with V
+          qp(d + Hq * kChunk),            // [c][Hq][kMaxRank]
+          m(qp + c * Hq * kMaxRank),      // [Hq]
+          l(m + Hq),                      // [Hq]
+          sc(l + Hq),                     // [Hq]
+          total(sc + Hq) {}
+};
+constexpr bool vectors_aligned() {
+    for (int Hq = 1; Hq <= kMaxHeads; ++Hq)
+        for (int width = 32; width <= 128; width *= 2)
+            for (int c = 0; c <= kMaxChain; ++c)
+                if (SmemLayout(Hq, width, c).q0 % 4 != 0 || SmemLayout(Hq, width, c).qp % 4 != 0) return false;
+    return kMaxRank % 4 == 0;
+}
+static_assert(vectors_aligned(), "float4 reads of q0 and q' need 16-byte aligned rows");
+
 // DT: 0 = fp32, 1 = bf16, 2 = any mix, decided per access
 template <int DT>
 __device__ __forceinline__ float ld(const TView& t, int64_t i) {
@@ -172,14 +196,9 @@ __global__ void __launch_bounds__(kMaxThreads) generic_prefill_kernel(const __gr
     const int b = blockIdx.y, i = (int)(gridDim.x - 1 - blockIdx.x), tid = threadIdx.x;   // the longest rows first
     const int Hq = HQ ? HQ : p.Hq, d = p.d, G = Hq / p.Hkv;
     const int warp = tid >> 5, lane = tid & 31, kThreads = blockDim.x, kWarps = kThreads / 32;
-    float* q0_s = smem;                       // [Hq][d]
-    float* o_s = q0_s + Hq * d;               // [Hq][d]
-    float* s_s = o_s + Hq * d;                // [Hq][kChunk] scores of the chunk
-    float* d_s = s_s + Hq * kChunk;           // [Hq][kChunk] a link's difference; then partial sums of the product with V
-    float* m_s = d_s + Hq * kChunk;           // [Hq]
-    float* l_s = m_s + Hq;                    // [Hq]
-    float* sc_s = l_s + Hq;                   // [Hq]
-    float* qp_s = sc_s + Hq;                  // [c][Hq][kMaxRank]
+    const SmemLayout at(Hq, d, p.c);
+    float *q0_s = smem + at.q0, *o_s = smem + at.o, *s_s = smem + at.s, *d_s = smem + at.d, *qp_s = smem + at.qp;
+    float *m_s = smem + at.m, *l_s = smem + at.l, *sc_s = smem + at.sc;
 
     // everything a CTA reads once, as one flat range: one round of loads for a small layer, not one per tensor
     chain_release();
@@ -293,9 +312,6 @@ __global__ void __launch_bounds__(kMaxThreads) generic_prefill_kernel(const __gr
     }
 }
 
-size_t smem_floats(int Hq, int d, int c) {
-    return (size_t)2 * Hq * d + (size_t)2 * Hq * kChunk + 3 * (size_t)Hq + (size_t)c * Hq * kMaxRank;
-}
 constexpr size_t kMaxSmemFloats = 232448 / sizeof(float);
 
 bool vec_rows(const lisa_tensor& t) {
@@ -320,7 +336,7 @@ cudaError_t launch_generic_prefill(const lisa_shared_prefill_args& a, cudaStream
     p.vec_k0 = vec_rows(a.k0);
     int dt = a.q0.dtype;
     bool same = a.k0.dtype == dt && a.v.dtype == dt;
-    size_t floats = smem_floats(a.Hq, a.d, a.chain_len);
+    size_t floats = SmemLayout(a.Hq, a.d, a.chain_len).total;
     for (int k = 0; k < a.chain_len; ++k) {
         const lisa_link& l = a.links[k];
         p.links[k] = make_link(l);

@@ -65,6 +65,15 @@ def test_shapes(B, N, Hq, Hkv, d, r, m):
     run_prefill_case(w, seed=5, chain=2)
 
 
+@pytest.mark.parametrize("r", [4, 8])
+@pytest.mark.parametrize("Hq,Hkv", [(1, 1), (2, 2), (2, 1), (3, 3), (6, 2)])
+def test_fp32_head_counts_that_are_not_multiples_of_four(Hq, Hkv, r):
+    """Ranks of whole 16-byte vectors, so that q' is read as float4 from shared memory, where it follows arrays sized by the head count."""
+    w = synth.Workload("heads", "f32", 1, 150, Hq, Hkv, 32, r, 4 * Hq, "relu", 2)
+    for c in (1, 2):
+        run_prefill_case(w, seed=13, chain=c)
+
+
 def test_strided_inputs_and_output():
     """Views with padding between heads and rows: strides are honoured."""
     w = synth.Workload("strided", "bf16", 2, 70, 4, 2, 32, 8, 8, "relu", 1)
