@@ -142,6 +142,9 @@ cudaError_t launch_tc_align_link(const TcAlignLinkArgs& a, cudaStream_t s);
 // weights -- overlaps the predecessor's tail), and calls chain_release() early so that its own successor can be set up.
 // chain_wait() returns once the predecessor has completed and its writes are visible; as every kernel of such a chain
 // waits before it finishes, completion is transitive.  In a kernel launched the ordinary way both are no-ops.
+// A kernel that allocates tensor memory calls chain_release() behind the __syncthreads() that follows its allocation.  The successor may
+// hold all of an SM's tensor memory while it waits for this kernel; a CTA of this kernel that came to its allocation later would wait
+// for it in turn, and tcgen05.alloc has no limit.  Once every CTA has released, every CTA has its columns.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... Params>

@@ -258,7 +258,6 @@ tc_project_narrow_kernel(const __grid_constant__ ProjParams p, const __grid_cons
     const int split = gridDim.x, rank = blockIdx.x;             // the cluster spans grid dimension x
     const int nt = blockIdx.y, rt = blockIdx.z;
     const int rows = p.rows_per_batch;
-    chain_release();
     const bool aligned = (smem_u32(smem) & 1023u) == 0;           // uniform over the grid; a false one reports and computes nothing
     const int k_all = (p.K + S::KS - 1) / S::KS;
     const int k_begin = (int)((long long)k_all * rank / split), k_end = (int)((long long)k_all * (rank + 1) / split);
@@ -280,6 +279,7 @@ tc_project_narrow_kernel(const __grid_constant__ ProjParams p, const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    chain_release();   // not before every CTA holds its tensor memory (see common.cuh)
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     chain_wait();
     bool have = false;   // epilogue warps: the accumulator holds the CTA's share
