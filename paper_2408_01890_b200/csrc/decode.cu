@@ -427,6 +427,9 @@ void carve_workspace(DecodeParams& p, void* ws) {
 // are cut finer, one per 32 as long as the scratch stays below kSmallScratch.  Grows with B and L, so that a buffer sized for the
 // largest step serves every smaller one.
 constexpr size_t kSmallScratch = (size_t)15 << 19;
+// lisa_attn_shared_decode_static refuses a step whose scratch is larger than its array, so what finer chunks ask for has to fit with the
+// padding of decode_workspace (the m and l arrays to whole float4, the whole to 256 bytes): no step of 128-position chunks that fits may be lost.
+static_assert(kSmallScratch + 2 * 3 * sizeof(float) + 255 <= LISA_STATIC_SCRATCH_BYTES, "finer chunks must fit the scratch of the static call");
 int64_t max_parts(int B, int Hq, int d, int L) {
     const int64_t coarse = (int64_t)B * ((L + kChunk - 1) / kChunk), fine = (int64_t)B * ((L + 31) / 32);
     if (d != 128) return coarse;

@@ -129,6 +129,21 @@ def test_decode_workspace_query(lib):
     assert n.value >= 64 * 32 * 40 * (128 + 2) * 4 and n.value % 256 == 0
 
 
+def test_finer_chunks_lose_no_static_decode_step(lib):
+    """lisa_attn_shared_decode_static takes every step whose partial results of 128-position chunks fit its array: the finer chunks of
+    small batches may ask for more scratch than those, but not for more than the array."""
+    up = lambda x, n: (x + n - 1) // n * n
+    for Hq in (1, 2, 8, 32, 40, 64):
+        for d in (32, 64, 128):
+            for B in (1, 2, 3, 8, 31, 64, 500):
+                for L in (1, 31, 33, 128, 129, 333, 1111, 4096, 8191, 40000):
+                    n = B * up(L, 128) // 128 * Hq
+                    coarse = up((2 * up(n, 4) + n * d) * 4, 256)
+                    need = lb.decode_workspace_bytes(B, Hq, d, L)
+                    assert need >= coarse
+                    assert need <= max(coarse, lb.STATIC_SCRATCH_BYTES), (Hq, d, B, L)
+
+
 def test_multi_layer_cache_is_carved_from_one_buffer(lib):
     """lisa_kvcache_init (host-only): per-layer descriptors at 256-byte aligned, non-overlapping offsets of one base, sizes as
     lisa_kvcache_bytes gives them; a shared layer's k region is smaller by the factor d/r (Sec. 5.2)."""
