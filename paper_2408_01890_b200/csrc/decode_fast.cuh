@@ -6,9 +6,9 @@
 // nothing computed twice) and the heads are divided as well (the first FFN layer, which every head needs, is then computed by
 // each group again).  All 8 warps work in every phase whatever CH is: with fewer than 8 strips of 16 positions the FFN's
 // hidden units are divided over HS = 128 / CH warps per strip and their partial sums added in a fixed order.
-// K and V rows are read once for all query heads of a group of up to four (GV) that share them.  A chunk's last rows, where the
-// sequence ends inside it, are read again in place of rows past the end, with probability zero, so that every chunk runs the
-// pipelined code (a loop with one row in flight took 120 us over a last chunk).
+// K and V rows are read once for all query heads of a group of up to four (GV) that share them.  Where the sequence ends inside a chunk,
+// rows past its end count as zeros, with probability zero (any other stand-in would turn into NaN where it holds an infinity), so that
+// every chunk runs the pipelined code (a loop with one row in flight took 120 us over a last chunk).
 #pragma once
 #include <type_traits>
 
@@ -78,15 +78,10 @@ __device__ __forceinline__ void stream_rows(const Rows& r, int nv, int vper, int
     const int nb_all = (r.nrows + ROWS - 1) / ROWS, b0 = nb_all * part / ps, b1 = nb_all * (part + 1) / ps;
     if (b0 == b1) return;
     auto load = [&](uint4* q, int v, int bt) {
-        const uint4* p = r.base + (size_t)(v / vper) * r.head_stride + sub;
-        if ((bt + 1) * ROWS <= r.nrows) {
-            p += (bt * ROWS + rsel) * 16;
+        const uint4* p = r.base + (size_t)(v / vper) * r.head_stride + (bt * ROWS + rsel) * 16 + sub;
+        const int left = r.nrows - bt * ROWS - rsel;
 #pragma unroll
-            for (int u = 0; u < U; ++u) q[u] = ld_stream16(p + u * 32);
-        } else {
-#pragma unroll
-            for (int u = 0; u < U; ++u) q[u] = ld_stream16(p + (size_t)min(bt * ROWS + 2 * u + rsel, r.nrows - 1) * 16);
-        }
+        for (int u = 0; u < U; ++u) q[u] = ld_stream16_or_zero(p + u * 32, 2 * u < left);
     };
     uint4 qa[U], qb[U];
     int lv = first, lb = b0;      // next batch to load

@@ -111,6 +111,31 @@ def test_anchor_decode_cuts(Hq, Hkv, B, L):
         assert np.all(row_h[b, :, lens[b]:] == -7.0)
 
 
+@pytest.mark.parametrize("Hq,Hkv,L", [(32, 32, 333), (32, 16, 45), (32, 8, 1111), (40, 40, 7)])
+def test_an_infinity_in_the_last_row_stays_one(Hq, Hkv, L):
+    """A sequence that ends inside a chunk, its last V row holding an infinity: that column of the output is infinite, as softmax times V
+    is, and no other column is touched."""
+    w = synth.Workload("inf", "bf16", 1, L, Hq, Hkv, 128, 21, 2 * Hq, "relu", 1, True)
+    t = synth.decode_inputs(w, 9, B=1, L=L)
+    clean = t["v"].clone()
+    t["v"][0, L - 1, :, 5] = float("inf")
+    L_cap = (L + 7) // 8 * 8
+    shared = fill_shared_cache(w, t, 1, L, L_cap, torch.bfloat16)
+    standard = lb.KVCacheLayer(lb.CACHE_STANDARD, 1, Hkv, L_cap, 128)
+    lb.lisa_kvcache_append(standard, dev(t["k"]), dev(t["v"]))
+    got = [lb.lisa_attn_shared_decode(dev(t["prev"]), lb.Link(dev(t["qp"]), None, dev(t["w1"]), dev(t["w2"])), shared, L=L),
+           lb.lisa_attn_anchor(dev(t["q0"]), cache=standard, L=L)]
+    olink = oracle.Link(None, None, f64(t["w1"]), f64(t["w2"]), r=w.r, act=ACT["relu"][1])
+    lens = np.array([L], dtype=np.int32)
+    ref = [oracle.decode_shared(f64(t["prev"]), f64(t["qp"])[:, 0], f64(t["kp"]), f64(clean), olink, lens)[0],
+           oracle.decode_anchor(f64(t["q0"])[:, 0], f64(t["k"]), f64(clean), lens)[0]]
+    others = [x for x in range(128) if x != 5]
+    for o, r in zip(got, ref):
+        o = o[:, 0].float().cpu().numpy()
+        assert np.all(np.isposinf(o[:, :, 5]))
+        assert_close(o[:, :, others], r[:, :, others], "bf16", "columns without an infinity")
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("Hq,Hkv,d,L", [(40, 40, 128, 600), (32, 8, 128, 257), (6, 3, 64, 130), (4, 4, 32, 7)])
 def test_anchor_decode(dtype, Hq, Hkv, d, L):
