@@ -401,9 +401,10 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&v);
 }
-// Two fp32 values as three packed bf16 pairs that add up to them (24 mantissa bits in three times 8)
+// Two fp32 values as three packed bf16 pairs that add up to them (24 mantissa bits in three times 8).  The first term's rounding saturates:
+// otherwise it would take the largest finite scores, a mask's for instance, to infinity.
 __device__ __forceinline__ void split3(float x, float y, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-    hi = pack2(x, y);
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(y), "f"(x));
     x -= __uint_as_float(hi << 16); y -= __uint_as_float(hi & 0xffff0000u);
     mid = pack2(x, y);
     x -= __uint_as_float(mid << 16); y -= __uint_as_float(mid & 0xffff0000u);

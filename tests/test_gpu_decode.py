@@ -136,6 +136,33 @@ def test_an_infinity_in_the_last_row_stays_one(Hq, Hkv, L):
         assert_close(o[:, :, others], r[:, :, others], "bf16", "columns without an infinity")
 
 
+@pytest.mark.parametrize("Hq,m,integrate", [(32, 256, lb.INTEGRATE_CONCAT), (32, 72, lb.INTEGRATE_ADD), (40, 24, lb.INTEGRATE_ADD)])
+def test_the_lowest_score_stays_finite(Hq, m, integrate):
+    """Previous scores of the type's lowest value at some positions, through an FFN whose weights keep its sums below the type's largest:
+    results stay finite and are the oracle's, as with any other scores."""
+    B, L = 2, 77
+    w = synth.Workload("lowest", "bf16", B, L, Hq, Hq, 128, 21, m, "relu", 1, True)
+    t = synth.decode_inputs(w, 10, B=B, L=L)
+    at = [3, 40, 76]
+    t["prev"][:, :, at] = torch.finfo(torch.float32).min
+    h_in = Hq * (2 if integrate == lb.INTEGRATE_CONCAT else 1)
+    w1 = synth.as_dtype(synth.normal("w1", (h_in, m), 10, std=0.02), "bf16")
+    w2 = synth.as_dtype(synth.normal("w2", (m, Hq), 10, std=0.02), "bf16")
+    cache = fill_shared_cache(w, t, B, L, (L + 7) // 8 * 8, torch.bfloat16)
+    row = torch.zeros((B, Hq, L), dtype=torch.float32, device="cuda")
+    out = lb.lisa_attn_shared_decode(dev(t["prev"]), lb.Link(dev(t["qp"]), None, dev(w1), dev(w2), act=lb.ACT_RELU, integrate=integrate),
+                                     cache, L=L, out_scores=row)
+    O, R = oracle.decode_shared(f64(t["prev"]), f64(t["qp"])[:, 0], f64(t["kp"]), f64(t["v"]),
+                                oracle.Link(None, None, f64(w1), f64(w2), r=w.r, act=ACT["relu"][1], integrate=integrate), np.full(B, L, np.int32))
+    row_h = row.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(R[:, :, at]) < 3e38) and np.abs(R[:, :, at]).max() > 1e36
+    # sums of a few hundred products at 24 bits, whose terms are a few times larger than the result
+    assert np.abs(row_h[:, :, at] - R[:, :, at]).max() <= 1e-5 * np.abs(R[:, :, at]).max()
+    others = [j for j in range(L) if j not in at]
+    assert_close(row_h[:, :, others], R[:, :, others], "f32", "row")
+    assert_close(out[:, 0].float().cpu().numpy(), O, "bf16", "O")
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("Hq,Hkv,d,L", [(40, 40, 128, 600), (32, 8, 128, 257), (6, 3, 64, 130), (4, 4, 32, 7)])
 def test_anchor_decode(dtype, Hq, Hkv, d, L):
