@@ -521,8 +521,9 @@ cudaError_t launch_tc_project(const lisa_project_args& a, cudaStream_t stream) {
     if (!p.status) return cudaErrorUnknown;
     // The narrow kernel as long as its CTAs fit the SMs; beyond, the persistent kernel's 256-column tiles fill them as well
     // (4096 x 5440, 512 rows: 37 us against 40; 4096 x 12288, 512 rows: 77 against 76, and 40 against 51 at 256 rows).
+    // Its column tiles are a grid dimension of at most 65535.
     const int narrow_tiles = ((p.n_out + 127) / 128) * ((p.rows_per_batch + 255) / 256);
-    if (flat && (p.rows_per_batch <= 128 || (p.rows_per_batch <= 512 && narrow_tiles <= sm_count()))) return launch_narrow(a, p, row_stride, stream);
+    if (flat && (p.n_out + 63) / 64 <= 65535 && (p.rows_per_batch <= 128 || (p.rows_per_batch <= 512 && narrow_tiles <= sm_count()))) return launch_narrow(a, p, row_stride, stream);
     p.m_tiles_per_batch = (p.rows_per_batch + BM - 1) / BM;
     p.n_tiles = (p.n_out + BN - 1) / BN;
     p.tiles_total = (long long)p.tiled_b * p.m_tiles_per_batch * p.n_tiles;

@@ -121,3 +121,13 @@ def test_project_few_rows(B, N, d_in, heads):
     for o, a, r in zip(outs, again, split(oracle.project(f64(x), f64(w)), heads)):
         assert_close(o.float().cpu().numpy(), r, "bf16", "projection of few rows")
         assert_close(a.float().cpu().numpy(), r, "bf16", "the same from strided rows")
+
+
+def test_project_more_columns_than_a_grid_dimension_of_tiles():
+    """Few rows, but more 64-column tiles than the 65535 of a grid dimension: the persistent kernel takes the call."""
+    n_out = 64 * 65535 + 8
+    x, w = draw(1, 3, 8, [(1, n_out)], "bf16", 19)
+    out = torch.full((1, 3, 1, n_out), 7.0, dtype=torch.bfloat16, device="cuda")
+    lb.lisa_project(dev(x), dev(w), [out])
+    assert lb.lisa_check() == lb.OK
+    assert_close(out[0, :, 0].float().cpu().numpy(), f64(x)[0] @ f64(w), "bf16", "columns past the narrow kernel's grid")
