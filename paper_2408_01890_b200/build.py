@@ -14,6 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "liblisa_b200.so")
 EXT = os.path.join(HERE, "_lisa_binding.so")
+EXT_KEY = os.path.join(HERE, "_lisa_binding.key")   # what the extension was built against
 EXT_SOURCE = os.path.join(HERE, "csrc", "binding_ext.cpp")
 
 
@@ -29,9 +30,25 @@ def _stale():
     return any(os.path.getmtime(p) > t for p in deps)
 
 
-def build_binding(force: bool = False) -> str:
+def _binding_key() -> str:
+    """What _lisa_binding.so is built against besides its sources: torch's C++ interface and the interpreter's."""
+    import torch
+    return "torch %s (cxx11 abi %d), python %s\n" % (torch.__version__, int(torch._C._GLIBCXX_USE_CXX11_ABI), sys.version)
+
+
+def binding_stale() -> bool:
     deps = [EXT_SOURCE] + glob.glob(os.path.join(ROOT, "include", "*.h"))
-    if not force and os.path.exists(EXT) and all(os.path.getmtime(p) <= os.path.getmtime(EXT) for p in deps):
+    if not os.path.exists(EXT) or any(os.path.getmtime(p) > os.path.getmtime(EXT) for p in deps):
+        return True
+    try:
+        with open(EXT_KEY) as f:
+            return f.read() != _binding_key()
+    except OSError:
+        return True
+
+
+def build_binding(force: bool = False) -> str:
+    if not force and not binding_stale():
         return EXT
     import sysconfig
 
@@ -46,6 +63,9 @@ def build_binding(force: bool = False) -> str:
                            EXT_SOURCE, "-o", tmp, "-L", os.path.join(tdir, "lib"),
                            "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
     os.replace(tmp, EXT)
+    with open(tmp, "w") as f:
+        f.write(_binding_key())
+    os.replace(tmp, EXT_KEY)
     return EXT
 
 

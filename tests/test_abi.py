@@ -46,6 +46,14 @@ def test_library_exports_every_declared_symbol(lib):
     assert lib.lisa_status_string(0) == b"ok"
 
 
+def test_binding_is_rebuilt_for_another_torch(lib, monkeypatch):
+    """The native half of the binding is compiled against torch's C++ interface: another torch makes it stale."""
+    import torch
+    assert not lbuild.binding_stale()
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert lbuild.binding_stale()
+
+
 def test_struct_sizes_are_checked(lib):
     a = lb.SharedPrefillArgs()
     a.struct_size = 3
