@@ -3,6 +3,7 @@ rejects malformed calls before touching the device, and its cache accounting mat
 import ctypes as C
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -61,6 +62,30 @@ def test_struct_sizes_are_checked(lib):
     d = lb.SharedDecodeArgs()
     assert lib.lisa_attn_shared_decode(C.byref(d), None) == lb.ERR_INVALID_ARG
     assert lib.lisa_attn_anchor(None, None) == lb.ERR_INVALID_ARG
+
+
+STRUCTS = [(lb.Tensor, "lisa_tensor"), (lb.CLink, "lisa_link"), (lb.CCacheLayer, "lisa_kvcache_layer"), (lb.CCacheDesc, "lisa_kvcache_desc"),
+           (lb.CCache, "lisa_kvcache"), (lb.AnchorArgs, "lisa_anchor_args"), (lb.SharedPrefillArgs, "lisa_shared_prefill_args"),
+           (lb.SharedPrefillChainArgs, "lisa_shared_prefill_chain_args"), (lb.SharedPrefillCarryArgs, "lisa_shared_prefill_carry_args"),
+           (lb.SharedDecodeArgs, "lisa_shared_decode_args"), (lb.CProjectOutput, "lisa_project_output"), (lb.ProjectArgs, "lisa_project_args")]
+
+
+def test_ctypes_structs_are_the_headers(tmp_path):
+    """The native half of the binding is compiled against include/lisa.h; the ctypes structs of the calls that stay on ctypes must have
+    the same fields at the same places, or the two would drift apart."""
+    lines = ['#include <stddef.h>', '#include <stdio.h>', '#include "lisa.h"', "int main(void) {"]
+    for cls, name in STRUCTS:
+        lines.append('printf("%s %%zu\\n", sizeof(%s));' % (name, name))
+        for f in cls._fields_:
+            lines.append('printf("%s.%s %%zu %%zu\\n", offsetof(%s, %s), sizeof(((%s*)0)->%s));' % (name, f[0], name, f[0], name, f[0]))
+    (tmp_path / "layout.c").write_text("\n".join(lines + ["return 0; }"]))
+    subprocess.check_call(["gcc", "-std=c11", "-I", os.path.join(ROOT, "include"), str(tmp_path / "layout.c"), "-o", str(tmp_path / "layout")])
+    header = subprocess.check_output([str(tmp_path / "layout")], text=True).split("\n")[:-1]
+    binding = []
+    for cls, name in STRUCTS:
+        binding.append("%s %d" % (name, C.sizeof(cls)))
+        binding += ["%s.%s %d %d" % (name, f[0], getattr(cls, f[0]).offset, getattr(cls, f[0]).size) for f in cls._fields_]
+    assert binding == header
 
 
 def test_validation_rejects_before_launch(lib):
