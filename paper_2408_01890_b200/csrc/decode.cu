@@ -487,6 +487,9 @@ cudaError_t shared_fast(DecodeParams& p, void* ws, cudaStream_t s, bool* taken) 
         // All heads to a CTA once that gives every SM two CTAs -- one with grouped queries, where the aligner is most of a CTA's work and
         // each group of heads would repeat half of it.  Else sixteen or eight heads to a CTA, then shorter chunks (7B-shaped, us:
         // B 64 L 300 55 -> 43 with 16 heads; B 8 L 1111 38 -> 25 with 8; B 4 L 1000 15.3 at 64 positions, 18.2 at 128).
+        // CTAs are counted as if every sequence had L_uniform positions: the lengths of a ragged batch are on the device, where the host
+        // cannot read them.  Spread over [L / 8, L], little more than half of the CTAs have positions, so such a batch gets longer chunks
+        // than one of that size would.
         const int64_t want = G > 1 ? sms : 2 * sms;
         const bool full = 8 % G != 0 || n_ctas >= want;
         if (full) {
@@ -581,7 +584,7 @@ cudaError_t launch_anchor_decode(const lisa_anchor_args& a, void* ws, cudaStream
     if (p.cache_dtype == LISA_BF16 && p.d == 128 && q.dtype == LISA_BF16 && vec16(q.ptr) && q.sb % 8 == 0 && q.sh % 8 == 0) {
         // Eight KV heads to a CTA, one per warp: CTAs small enough for even waves, nothing computed twice (40 heads, us: B 12 L 3500
         // 178 -> 138 against all heads to a CTA, B 64 L 4096 803 -> 790).  Fewer, then shorter chunks, where that does not give
-        // every SM a CTA.
+        // every SM a CTA (counted as in shared_fast, ragged batches as if they were uniform).
         const int64_t want = sm_count(), chunks = (int64_t)p.B * ((a.L + kChunk - 1) / kChunk);
         int kv = std::min(8, p.Hkv);
         while (p.Hkv % kv) --kv;

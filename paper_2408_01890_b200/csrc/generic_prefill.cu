@@ -7,7 +7,7 @@
 // dtype and shape in the supported range runs here; the tensor-core kernels cover the fast cases.
 //
 // A small prompt is bound by the latency of one CTA, so every phase spreads over all threads with its loads in flight together: the dot
-// products over (head, key, part of the row), the FFN over keys (weights in shared memory, registers for up to eight heads), the softmax over heads, the
+// products over (head, key, part of the row), the FFN over keys (weights in shared memory; 2, 4 or 8 heads in registers), the softmax over heads, the
 // product with V over (head, column) and, where these are few, ranges of keys.  4 heads of 32, N 128: 31 us with a thread per key
 // doing all of it, 10 now.
 #include "common.cuh"
@@ -319,6 +319,9 @@ bool vec_rows(const lisa_tensor& t) {
     return t.stride_b % n == 0 && t.stride_n % n == 0 && t.stride_h % n == 0;   // (the pointer is: checked by the entry points)
 }
 
+// Head counts a compile-time constant keeps a position's scores in registers for; every other count runs the loops over local memory.
+// One link, heads of 32, fp32, 128 positions: 2 heads 8.9 us (loops 10.3), 4 heads 11.9 (13.0), 8 heads 15.9 (21.9); two
+// sequences of 1000, 8 heads: 525 (720).  Counts of tiny test and draft models; beyond eight, larger models are the tensor-core kernels'.
 template <int DT>
 void* pick(int Hq) {
     return Hq == 2   ? reinterpret_cast<void*>(generic_prefill_kernel<DT, 2>)

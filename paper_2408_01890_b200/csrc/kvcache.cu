@@ -57,7 +57,9 @@ template <typename T>
 __device__ __forceinline__ void append_kp_transposed(const AppendParams& p) {
     const int64_t total = (int64_t)p.B * p.n_new * p.Hkv * p.r;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t row = total >> 31 ? (uint32_t)(e / p.r) : (uint32_t)e / (uint32_t)p.r, x = (uint32_t)(e - (int64_t)row * p.r), tb = row / (uint32_t)p.Hkv, g = row - tb * p.Hkv, b = tb / (uint32_t)p.n_new, t = tb - b * p.n_new;
+        const uint32_t row = total >> 31 ? (uint32_t)(e / p.r) : (uint32_t)e / (uint32_t)p.r;   // 64-bit division only where it must be
+        const uint32_t x = (uint32_t)(e - (int64_t)row * p.r), tb = row / (uint32_t)p.Hkv, g = row - tb * p.Hkv;
+        const uint32_t b = tb / (uint32_t)p.n_new, t = tb - b * p.n_new;
         const int64_t pos = (int64_t)(p.lens_before ? p.lens_before[b] : 0) + t;
         if (pos >= p.L_cap || pos < 0) continue;  // counted by the V rows
         reinterpret_cast<T*>(p.kc)[(((int64_t)b * p.Hkv + g) * p.r + x) * p.L_cap + pos] =
@@ -127,7 +129,7 @@ cudaError_t launch_kvcache_append(const lisa_kvcache_layer& c, const lisa_tensor
     if (!p.status) return cudaErrorUnknown;
     const int threads = kAppendThreads;
     const int64_t rows = (int64_t)c.B * n_new * c.Hkv;
-    if (rows > 0x7fffffff) return cudaErrorInvalidValue;   // (half a TB of V rows)
+    if (rows > 0x7fffffff) return cudaErrorInvalidValue;   // (137 GB of V at the narrowest width, and as much again in the cache)
     auto blocks_for = [&](int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + threads - 1) / threads, sm_count() * 16)); };
     cudaError_t e;
     const int64_t k_vals = c.kind == LISA_CACHE_SHARED && n_new < kTilePos ? rows * c.r : 0;
