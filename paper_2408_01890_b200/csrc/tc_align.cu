@@ -22,7 +22,9 @@
 // version spent ~13 clocks per position and link (tensor pipe 5% busy).  mma.sync runs at a quarter of the tcgen05
 // rate (measured 555 TFLOP/s) but nothing leaves the registers.  Every warp is independent: no block-wide barrier
 // after set-up, no mbarrier, no wait that could hang.  The kernel is bound by the planes it moves (4 bytes per
-// position and head for one link), not by its arithmetic.
+// position and head for one link), not by its arithmetic.  That holds for chains, which stay in registers from link to link, and for
+// prompts of one wave; single links of longer prompts are faster on tc_align_link.cu, whose hidden layer stays in tensor memory (4 x 8192
+// positions, 32 heads: 420 us a wave against 730).
 #include <algorithm>
 
 #include "tc_align_mma.cuh"

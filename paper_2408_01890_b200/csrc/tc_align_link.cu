@@ -1,5 +1,5 @@
-// Head-axis aligner (Sec. 5.1), one link per launch, on tcgen05, for the shapes and Integrate modes the chain kernel of
-// tc_align.cu does not take:
+// Head-axis aligner (Sec. 5.1), one link per launch, on tcgen05: single links of prompts above one wave, and the shapes and Integrate
+// modes the chain kernel of tc_align.cu does not take:
 //   CONCAT  (32 heads)        A_k = W2^T act(W1^T [A_{k-1}; D_k] + b1) + b2    W1 [64, m], W2 [m, 32], m <= 256: the paper's
 //                             complete model (Sec. 5.1, "An overview of LiSA": 64 x 256 and 256 x 32), and its one-layer
 //                             form A_k = W1^T [A_{k-1}; D_k] + b1 with W1 [64, 32]
