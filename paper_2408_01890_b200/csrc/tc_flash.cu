@@ -1,8 +1,7 @@
 // Tensor-core flash kernel (tcgen05 + TMEM + TMA) for head width 128, bf16.
 //
 // One CTA per (batch b, query head h, 128-row query tile).  For every 64-key tile j up to the diagonal:
-//   scores  S = QA . KA^T            tcgen05.mma (M 128, N 64), fp32 accumulator in tensor memory (two buffers, so
-//                                    S(t+1) is computed while the softmax of tile t runs)
+//   scores  S = QA . KA^T            tcgen05.mma (M 128, N 64), fp32 accumulator in tensor memory, two buffers
 //   logits  A = S * scale (+ Y)      Y: optional fp16 tile of pre-computed scores (the aligned part of a
 //                                    shared layer, Eq. 4; then QA/KA are the layer's low-rank Q'/K', Eq. 3)
 //   causal mask (tiles that reach past the first query row), online softmax in registers (one thread per query
@@ -13,12 +12,15 @@
 // attention also writes its finished pre-softmax logits A = S * scale + Y (unmasked, Eq. 4's A_n) back as fp16 tiles: the
 // next shared layer of a chain aligns those instead of recomputing the chain from the anchor's scores.
 //
-// Warp roles: warps 0-3 softmax/epilogue (thread = query row = TMEM lane), warp 4 TMA producer,
-// warp 5 issuer of the score MMAs and TMEM owner, warp 6 issuer of the P.V MMAs (warp 7 only completes the warpgroup).  K and V(/Y) have their own rings: a K stage is free again as soon as its
-// score MMA has run, a V stage after its P.V MMA.
-// Sizing: the softmax warps are the slow stage (one exp2 per score on the 16-lane transcendental unit) and every
-// hand-off between the roles costs a few hundred cycles of latency, so TWO CTAs share an SM and fill each other's
-// gaps, prologues and epilogues: 64-key tiles keep a CTA at 112 KB of shared memory and 256 tensor-memory columns.
+// Warp roles: warps 0-3 and 4-7 softmax/epilogue (thread = query row = TMEM lane; the two warpgroups take the key tiles in turn), warp 8
+// TMA producer, warp 9 issuer of the score MMAs and TMEM owner, warp 10 issuer of the P.V MMAs (warp 11 only completes the warpgroup).
+// P stays in tensor memory, over the scores it came from, as the A operand of P.V: a K stage is free again as soon as its score MMA has
+// run, a Y stage once its rows are read, a V stage and a score buffer after the P.V MMA.
+// Sizing: a softmax warp spends as long on waits (tensor memory, barriers, the next scores behind P.V) as on its 64 exponentials a row (16
+// lanes a cycle and SM: 512 cycles a tile), so an SM partition needs four of them in different phases: TWO CTAs share an SM (64-key tiles
+// keep a CTA at 112 KB of shared memory and 256 tensor-memory columns), each with two warpgroups on alternate tiles.  One warpgroup
+// per CTA took 1010 cycles a tile and SM, two warpgroups on halves of the same tile as long (in step, they wait for the same unit at the
+// same time), alternate tiles 845 (attention with plane, 2048 tokens of 32 heads 51 -> 47 us, 4 x 8192 tokens 3.6 -> 3.1 ms).
 // Every wait is bounded; on expiry the CTA records it in the status word, drains and exits.
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -37,7 +39,8 @@ __device__ __forceinline__ float fast_exp2(float x) {
 }
 
 constexpr int kPrefetchAhead = 2;   // tiles (0: no L2 prefetch)
-constexpr int kThreads = 256;   // warpgroup 0: softmax/epilogue; warpgroup 1: producer, two MMA issuers, one idle warp
+constexpr int kSoftmaxWarps = 8;
+constexpr int kThreads = 384;   // warpgroups 0 and 1: softmax/epilogue; warpgroup 2: producer, two MMA issuers, one idle warp
 
 struct FlashParams {
     int B, N, Hq, Hkv;
@@ -62,35 +65,23 @@ struct Smem {
     static constexpr bool PLANE = MODE == MODE_ATTN_PLANE || MODE == MODE_ATTN_CARRY;
     static constexpr bool EMIT = MODE == MODE_EMIT;
     static constexpr bool CARRY = MODE == MODE_ATTN_CARRY;
-    // P (the bf16 probabilities, A operand of P.V) is double-buffered so that the softmax of tile t+1 never waits
-    // for the P.V of tile t.  To stay inside half an SM's shared memory it borrows a buffer whose content is dead
-    // by then: with a plane, the Y tile of the same stage (each thread has read its own row of Y and overwrites just
-    // that row); with 128-wide keys, the K tile of the same stage (its score MMA has completed before the softmax
-    // starts), which is then released by the P.V MMA instead of the score MMA -- hence three K stages.  64-wide
-    // keys without a plane leave room for two buffers of their own.
-    static constexpr bool P_IN_Y = PLANE;
-    static constexpr bool P_IN_K = !EMIT && !PLANE && KD == 128;
-    static constexpr bool P_OWN = !EMIT && !P_IN_Y && !P_IN_K;
-    static constexpr int KST = (EMIT || P_IN_K) ? 3 : 2;  // K ring depth (V/Y: two stages)
+    static constexpr int KST = KD == 128 ? 3 : 2;  // K ring depth (V: two stages)
+    static constexpr int YST = PLANE ? 3 : 0;      // Y ring depth
     static constexpr int Q_BYTES = BM * KD * 2;
     static constexpr int K_BYTES = BN * KD * 2;
     static constexpr int V_BYTES = EMIT ? 0 : BN * D * 2;
-    static constexpr int P_BYTES = BM * BN * 2;
-    static constexpr int P_OWN_BYTES = P_OWN ? 2 * P_BYTES : 0;
     static constexpr int Y_BYTES = PLANE ? BM * BN * 2 : 0;
-    // per epilogue warp: two buffers of [32 rows][128 B] (emit), one (carry)
-    static constexpr int STG_BYTES = EMIT ? 4 * 2 * 4096 : (CARRY ? 4 * 4096 : 0);
+    static constexpr int STG_BYTES = EMIT ? kSoftmaxWarps * 4096 : 0;   // emit: [32 rows][128 B] per epilogue warp
     static constexpr int OFF_Q = 0;
     static constexpr int OFF_K = OFF_Q + Q_BYTES;
     static constexpr int OFF_V = OFF_K + KST * K_BYTES;
-    static constexpr int OFF_P = OFF_V + 2 * V_BYTES;
-    static constexpr int OFF_Y = OFF_P + P_OWN_BYTES;
-    static constexpr int OFF_STG = OFF_Y + 2 * Y_BYTES;
-    static constexpr int OFF_BAR = OFF_STG + STG_BYTES;
-    static constexpr int TOTAL = OFF_BAR + 256;
+    static constexpr int OFF_Y = OFF_V + 2 * V_BYTES;
+    static constexpr int OFF_STG = OFF_Y + YST * Y_BYTES;
+    static constexpr int OFF_M = OFF_STG + STG_BYTES;      // reference maximum of each row: [128] fp32
+    static constexpr int OFF_BAR = OFF_M + (EMIT ? 0 : BM * 4);
+    static constexpr int TOTAL = OFF_BAR + 288;
     static constexpr uint32_t TMEM_COLS = EMIT ? 128 : 256;   // S[2]: [0,128), O: [128,256)
     static_assert(TOTAL <= 115712, "two CTAs must fit one SM's shared memory");
-    static_assert(!P_IN_K || K_BYTES >= P_BYTES, "P must fit the K stage it borrows");
 };
 
 template <int KD, int MODE>
@@ -111,27 +102,23 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
     uint8_t* sQ = smem + L::OFF_Q;
     uint8_t* sK = smem + L::OFF_K;
     uint8_t* sV = smem + L::OFF_V;
-    uint8_t* sP = smem + L::OFF_P;
     uint8_t* sY = smem + L::OFF_Y;
     uint8_t* sStg = smem + L::OFF_STG;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);
     uint64_t* q_full = bars + 0;
     uint64_t* k_full = bars + 1;    // [KST <= 3]
     uint64_t* k_empty = bars + 4;   // [KST <= 3]
-    uint64_t* v_full = bars + 7;    // [2] V and Y of a stage
-    uint64_t* v_empty = bars + 9;   // [2]
-    uint64_t* s_full = bars + 11;   // [2] score buffer written by the MMA
-    uint64_t* s_free = bars + 13;   // [2] score buffer copied to registers by all 128 rows
-    uint64_t* p_full = bars + 15;   // [2]
-    uint64_t* pv_done = bars + 17;  // [2]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 19);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 20);
-    // P of tile t
-    auto p_buf = [&](int t) -> uint8_t* {
-        if constexpr (L::P_IN_Y) return sY + (t & 1) * L::Y_BYTES;
-        else if constexpr (L::P_IN_K) return sK + (t % KST) * L::K_BYTES;
-        else return sP + (t & 1) * L::P_BYTES;
-    };
+    uint64_t* v_full = bars + 7;    // [2]
+    uint64_t* y_full = bars + 9;    // [YST <= 3]
+    uint64_t* y_empty = bars + 12;  // [YST <= 3] Y rows read (carry: and the logits that went over them stored)
+    uint64_t* s_full = bars + 15;   // [2] score buffer written by the MMA
+    uint64_t* s_free = bars + 17;   // [2] emit: score buffer copied to registers (attention: free with pv_done)
+    uint64_t* p_full = bars + 19;   // [2] P in tensor memory
+    uint64_t* pv_done = bars + 21;  // [2] P.V has run: its V stage and its score buffer, which held P, are free
+    uint64_t* m_set = bars + 23;    // [2][4] the rows of a quarter have their reference maximum for a tile
+    uint64_t* o_full = bars + 31;   // the last P.V has run (a barrier of its own: pv_done tells only neighbouring phases apart)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 32);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 33);
 
     const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
     // blockIdx.x (the fastest-dispatched index) runs over (batch, head), blockIdx.y over query tiles from the last one
@@ -150,14 +137,17 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
         mbar_init(q_full, 1);
         for (int i = 0; i < KST; ++i) { mbar_init(k_full + i, 1); mbar_init(k_empty + i, 1); }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(v_full + i, 1); mbar_init(v_empty + i, 1);
-            mbar_init(s_full + i, 1); mbar_init(s_free + i, 128);
-            mbar_init(p_full + i, 128); mbar_init(pv_done + i, 1);
+            mbar_init(v_full + i, 1);
+            mbar_init(s_full + i, 1); mbar_init(s_free + i, 4);
+            mbar_init(p_full + i, 4); mbar_init(pv_done + i, 1);
         }
+        for (int i = 0; i < L::YST; ++i) { mbar_init(y_full + i, 1); mbar_init(y_empty + i, 4); }
+        for (int i = 0; i < 8; ++i) mbar_init(m_set + i, 1);
+        mbar_init(o_full, 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
-    if (warp == 5) tmem_alloc(tmem_slot, L::TMEM_COLS);
+    if (warp == kSoftmaxWarps + 1) tmem_alloc(tmem_slot, L::TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -168,57 +158,62 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     const uint32_t tmem_O = tmem_base + 128;
 
-    // The kernel is compiled for 128 registers per thread (two CTAs of 256 threads per SM).  The three single-thread
-    // roles need few, the softmax threads (64 scores, their exponentials and a row of the accumulator in flight) more:
-    // warpgroup 1 hands registers back and warpgroup 0 takes them (2 x (128 x 72 + 128 x 184) = 64 K).
-    if (warp >= 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
-    if (warp == 4) {
+    // The kernel is compiled for 80 registers per thread (two CTAs of 384 threads per SM).  A softmax thread holds 64 scores; the
+    // single-thread roles need few: warpgroup 2 hands registers back and the softmax warpgroups take them (256 x 104 + 128 x 32 = 384 x 80).
+    if (warp >= kSoftmaxWarps) {
+    if constexpr (!EMIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+    if (warp == kSoftmaxWarps) {
         // ------------------------------ TMA producer ------------------------------
-        // V(t) (with Y(t)) travels together with K(t+1): both wait for the P.V of tile t-2 at the latest.
+        // Round t brings K(t) and Y(t), then V(t - 1): V is needed a softmax pass later than the others, and asked for in its own round
+        // its stage, which waits for the P.V two tiles before, would hold up the Y of the next.
         constexpr int NQ = KD / 64, NK = KD / 64, NV = EMIT ? 0 : D / 64;
         if (elect_one()) {
             tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK);
             if (!EMIT) tma_prefetch_desc(&tmV);
             if (PLANE) tma_prefetch_desc(&tmY);
             mbar_expect_tx(q_full, L::Q_BYTES);
-            mbar_expect_tx(k_full, L::K_BYTES);
 #pragma unroll
             for (int i = 0; i < NQ; ++i) tma_load_4d(sQ + i * (BM * 128), &tmQ, q_full, i * 64, h, q0, b);
-#pragma unroll
-            for (int i = 0; i < NK; ++i) tma_load_4d(sK + i * (BN * 128), &tmK, k_full, i * 64, g, 0, b);
         }
         __syncwarp();
-        int ks_next = 1 % KST;              // K stage of tile t+1
-        uint32_t kpar_next = 1;             // parity to wait for on its "empty" barrier (first pass: passes at once)
-        for (int t = 0; t < nt; ++t) {
-            const int sv = t & 1;
-            const bool more_k = t + 1 < nt;
+        int ks = 0, ys = 0;              // K and Y stage of tile t
+        uint32_t kpar = 1, ypar = 1;     // parity to wait for on their "empty" barriers (first pass: passes at once)
+        for (int t = 0; t < nt + (EMIT ? 0 : 1); ++t) {
             bool okp = true;
+            if (t < nt) {
+                okp = mbar_wait(k_empty + ks, kpar, abort_flag);
+                if (!__all_sync(0xffffffffu, okp)) break;
+                if (elect_one()) {
+                    mbar_expect_tx(k_full + ks, L::K_BYTES);
+#pragma unroll
+                    for (int i = 0; i < NK; ++i) tma_load_4d(sK + ks * L::K_BYTES + i * (BN * 128), &tmK, k_full + ks, i * 64, g, t * BN, b);
+                }
+                __syncwarp();
+                if constexpr (PLANE) {
+                    okp = mbar_wait(y_empty + ys, ypar, abort_flag);
+                    if (!__all_sync(0xffffffffu, okp)) break;
+                    if (elect_one()) {
+                        mbar_expect_tx(y_full + ys, L::Y_BYTES);
+                        tma_load_5d(sY + ys * L::Y_BYTES, &tmY, y_full + ys, 0, b * p.Hq + h, 0, t, (q0 - p.plane_row0) / BM);
+                    }
+                    __syncwarp();
+                }
+            }
             if constexpr (!EMIT) {
-                okp = mbar_wait(v_empty + sv, ((t >> 1) & 1) ^ 1, abort_flag);
-                if (!__all_sync(0xffffffffu, okp)) break;
-                if (elect_one()) {
-                    mbar_expect_tx(v_full + sv, L::V_BYTES + L::Y_BYTES);
+                if (t > 0) {
+                    const int tv = t - 1, s2 = tv & 1;
+                    okp = mbar_wait(pv_done + s2, ((tv >> 1) & 1) ^ 1, abort_flag);
+                    if (!__all_sync(0xffffffffu, okp)) break;
+                    if (elect_one()) {
+                        mbar_expect_tx(v_full + s2, L::V_BYTES);
 #pragma unroll
-                    for (int i = 0; i < NV; ++i) tma_load_4d(sV + sv * L::V_BYTES + i * (BN * 128), &tmV, v_full + sv, i * 64, g, t * BN, b);
-                    if constexpr (PLANE) tma_load_5d(sY + sv * L::Y_BYTES, &tmY, v_full + sv, 0, b * p.Hq + h, 0, t, (q0 - p.plane_row0) / BM);
+                        for (int i = 0; i < NV; ++i) tma_load_4d(sV + s2 * L::V_BYTES + i * (BN * 128), &tmV, v_full + s2, i * 64, g, tv * BN, b);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
             }
-            if (more_k) {
-                okp = mbar_wait(k_empty + ks_next, kpar_next, abort_flag);
-                if (!__all_sync(0xffffffffu, okp)) break;
-                if (elect_one()) {
-                    mbar_expect_tx(k_full + ks_next, L::K_BYTES);
-#pragma unroll
-                    for (int i = 0; i < NK; ++i) tma_load_4d(sK + ks_next * L::K_BYTES + i * (BN * 128), &tmK, k_full + ks_next, i * 64, g, (t + 1) * BN, b);
-                }
-                __syncwarp();
-            }
-            // The V and Y stages of a tile cannot be refilled before the P.V of the tile two before it has run, one softmax pass
-            // before they are needed -- less than a trip to HBM under load.  Their tiles are therefore asked into L2 earlier,
-            // kPrefetchAhead tiles ahead of the one just issued.
+            // The V and Y stages can be refilled at most two softmax passes before they are needed, under load less than a trip to HBM.
+            // Their tiles are therefore asked into L2 earlier, kPrefetchAhead tiles ahead of the one just issued.
             if constexpr (kPrefetchAhead > 0 && !EMIT) {
                 if (t + kPrefetchAhead < nt && elect_one()) {
 #pragma unroll
@@ -227,9 +222,10 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                 }
                 __syncwarp();
             }
-            if (++ks_next == KST) { ks_next = 0; kpar_next ^= 1; }
+            if (++ks == KST) { ks = 0; kpar ^= 1; }
+            if (PLANE && ++ys == L::YST) { ys = 0; ypar ^= 1; }
         }
-    } else if (warp == 5) {
+    } else if (warp == kSoftmaxWarps + 1) {
         // ------------------------------ MMA issuer: scores ------------------------------
         // Issuing a tcgen05.mma holds the issuing thread for about as long as the MMAs queued before it take to run, so
         // the score MMAs and the P.V MMAs are issued by two different warps: each waits for its own operands and the
@@ -245,13 +241,15 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
         };
         const uint64_t dq0 = umma_desc_sw128(smem_u32(sQ), 16, 1024);
         const uint64_t dk0 = umma_desc_sw128(smem_u32(sK), 16, 1024);
-        // scores of tile t into buffer t&1; needs K(t) loaded and (t >= 2) the buffer read by the softmax of t-2
+        // scores of tile t into buffer t&1; needs K(t) loaded and (t >= 2) the buffer: P(t-2), which lies there, multiplied (emit: the
+        // scores read)
+        uint64_t* buf_free = EMIT ? s_free : pv_done;
         int sk = 0;
         uint32_t kpar = 0;
         bool ok = __all_sync(0xffffffffu, mbar_wait(q_full, 0, abort_flag));
         for (int t = 0; ok && t < nt; ++t) {
             const int s = t & 1;
-            ok = mbar_wait(k_full + sk, kpar, abort_flag) && mbar_wait(s_free + s, ((t >> 1) & 1) ^ 1, abort_flag);
+            ok = mbar_wait(k_full + sk, kpar, abort_flag) && mbar_wait(buf_free + s, ((t >> 1) & 1) ^ 1, abort_flag);
             if (!(ok = __all_sync(0xffffffffu, ok))) break;   // one verdict for the whole warp
             tc_fence_after();
             const uint64_t dk = desc_off(dk0, sk * L::K_BYTES);
@@ -263,12 +261,12 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                         umma_ss(dst, desc_off(dq0, (ks >> 2) * (BM * 128) + (ks & 3) * 32), desc_off(dk, (ks >> 2) * (BN * 128) + (ks & 3) * 32), IDESC_QK, ks > 0);
                 }
                 umma_commit(s_full + s);
-                if (!L::P_IN_K && t + KST < nt) umma_commit(k_empty + sk);  // nobody waits for the last ones: do not arm them
+                if (t + KST < nt) umma_commit(k_empty + sk);  // nobody waits for the last ones: do not arm them
             }
             __syncwarp();
             if (++sk == KST) { sk = 0; kpar ^= 1; }
         }
-    } else if (warp == 6) {
+    } else if (warp == kSoftmaxWarps + 2) {
         // ------------------------------ MMA issuer: P.V ------------------------------
         if constexpr (!EMIT) {
             constexpr uint32_t IDESC_PV = umma_idesc_bf16(BM, D, 0, 1);
@@ -276,79 +274,90 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                 return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4));
             };
             const uint64_t dv0 = umma_desc_sw128(smem_u32(sV), BN * 128, 1024);
-            const uint64_t dp0 = umma_desc_sw128(smem_u32(p_buf(0)), 16, 1024);
-            constexpr uint32_t P_STRIDE = L::P_IN_Y ? L::Y_BYTES : (L::P_IN_K ? L::K_BYTES : L::P_BYTES);
-            int pk = 0;   // P_IN_K: K stage that holds P(t)
             bool ok = true;
             for (int t = 0; ok && t < nt; ++t) {
                 const int s = t & 1;
                 ok = mbar_wait(v_full + s, (t >> 1) & 1, abort_flag) && mbar_wait(p_full + s, (t >> 1) & 1, abort_flag);
                 if (!(ok = __all_sync(0xffffffffu, ok))) break;
                 tc_fence_after();
-                const uint64_t dp = desc_off(dp0, (L::P_IN_K ? pk : s) * P_STRIDE);
                 const uint64_t dv = desc_off(dv0, s * L::V_BYTES);
                 if (elect_one()) {
 #pragma unroll
                     for (int ks = 0; ks < BN / 16; ++ks) {
-                        // P: K-major, 64 keys per 128-byte row; V: 16 keys = two 8-row groups, the next 64 d-columns
-                        // BN * 128 bytes further on
-                        umma_ss(tmem_O, desc_off(dp, ks * 32), desc_off(dv, ks * 2048), IDESC_PV, (t > 0) || (ks > 0));
+                        // P: two keys a column; V: 16 keys = two 8-row groups, the next 64 d-columns BN * 128 bytes further on
+                        umma_ts(tmem_O, tmem_base + s * BN + ks * 8, desc_off(dv, ks * 2048), IDESC_PV, (t > 0) || (ks > 0));
                     }
                     umma_commit(pv_done + s);
-                    if (t + 2 < nt) umma_commit(v_empty + s);
-                    if (L::P_IN_K && t + KST < nt) umma_commit(k_empty + pk);
+                    if (t + 1 == nt) umma_commit(o_full);
                 }
                 __syncwarp();
-                if (++pk == KST) pk = 0;
             }
         }
     }
-    } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 184;");
-        // ------------------------------ softmax / epilogue (thread = query row) ------------------------------
-        const int row = tid;                       // 0..127, TMEM lane
-        const int qi = q0 + row;                   // global query index
-        const uint32_t lane_sel = (uint32_t)(warp * 32) << 16;
-        const float scale_log2 = p.scale_log2, emit_scale = p.scale;
-        float m_ref = -INFINITY, l_sum = 0.f;
-        bool ok = true;
-        for (int t = 0; t < nt; ++t) {
-            const int s = t & 1;
-            if (!(ok = mbar_wait(s_full + s, (t >> 1) & 1, abort_flag))) break;
+    } else if constexpr (EMIT) {
+        // ------------------------------ epilogue: warps 0-3 even tiles, 4-7 odd ones (thread = query row) ------------------------------
+        const int q = warp & 3, s = warp >> 2;
+        const uint32_t lane_sel = (uint32_t)(q * 32) << 16;
+        const float emit_scale = p.scale;
+        uint8_t* stg = sStg + warp * 4096;
+        for (int t = s; t < nt; t += 2) {
+            if (!__all_sync(0xffffffffu, mbar_wait(s_full + s, (t >> 1) & 1, abort_flag))) break;
             tc_fence_after();
             uint32_t sr[BN];
 #pragma unroll
             for (int c = 0; c < BN / 32; ++c) tmem_ld32(tmem_base + s * BN + lane_sel + c * 32, sr + c * 32);
             tmem_wait_ld();
             tc_fence_before();
-            mbar_arrive(s_free + s);
-            float* sf = reinterpret_cast<float*>(sr);
-            if constexpr (EMIT) {
-                // this warp's 32 rows x 64 columns as fp16 into its staging buffer (swizzled like any other tile),
-                // then lane 0 stores it with TMA
-                uint8_t* stg = sStg + (warp * 2 + s) * 4096;
-                if (t >= 2 && lane == 0) tma_store_wait_read<1>();  // the store of tile t-2 has read this buffer
-                __syncwarp();
+            if (lane == 0) tma_store_wait_read<0>();  // the store of tile t-2 has read this buffer
+            __syncwarp();
+            if (lane == 0) mbar_arrive(s_free + s);
+            const float2* sf = reinterpret_cast<const float2*>(sr);
+            // this warp's 32 rows x 64 columns as fp16 into its staging buffer (swizzled like any other tile), then lane 0 stores it
 #pragma unroll
-                for (int c = 0; c < BN / 8; ++c) {
-                    uint4 v;
-                    { const float2 t2 = __fmul2_rn(reinterpret_cast<const float2*>(sf)[c * 4 + 0], make_float2(emit_scale, emit_scale)); v.x = pack_f16(t2.x, t2.y); }
-                    { const float2 t2 = __fmul2_rn(reinterpret_cast<const float2*>(sf)[c * 4 + 1], make_float2(emit_scale, emit_scale)); v.y = pack_f16(t2.x, t2.y); }
-                    { const float2 t2 = __fmul2_rn(reinterpret_cast<const float2*>(sf)[c * 4 + 2], make_float2(emit_scale, emit_scale)); v.z = pack_f16(t2.x, t2.y); }
-                    { const float2 t2 = __fmul2_rn(reinterpret_cast<const float2*>(sf)[c * 4 + 3], make_float2(emit_scale, emit_scale)); v.w = pack_f16(t2.x, t2.y); }
-                    *reinterpret_cast<uint4*>(stg + sw128_offset(lane, c)) = v;
+            for (int c = 0; c < BN / 8; ++c) {
+                uint32_t v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 x = __fmul2_rn(sf[c * 4 + e], make_float2(emit_scale, emit_scale));
+                    v[e] = pack_f16(x.x, x.y);
                 }
-                fence_async_smem();
-                __syncwarp();
-                if (lane == 0) {
-                    tma_store_5d(&tmY, stg, 0, b * p.Hq + h, warp * 32, t, (q0 - p.plane_row0) / BM);
-                    tma_store_commit();
-                }
-                continue;
+                *reinterpret_cast<uint4*>(stg + sw128_offset(lane, c)) = make_uint4(v[0], v[1], v[2], v[3]);
             }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                tma_store_5d(&tmY, stg, 0, b * p.Hq + h, q * 32, t, (q0 - p.plane_row0) / BM);
+                tma_store_commit();
+            }
+        }
+        if (lane == 0) tma_store_wait_all<0>();
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+        // ------------------------------ softmax / epilogue (thread = query row = TMEM lane) ------------------------------
+        // The two warpgroups take the key tiles in turn, so that the four softmax warps of an SM partition (two CTAs) are in different
+        // phases: one waits for tensor memory or for its next scores while another keeps the transcendental unit busy.
+        const int q = warp & 3, wg = warp >> 2;
+        const int row = q * 32 + lane;             // 0..127
+        const int qi = q0 + row;                   // global query index
+        const uint32_t lane_sel = (uint32_t)(q * 32) << 16;
+        const float scale_log2 = p.scale_log2;
+        volatile float* m_row = reinterpret_cast<float*>(smem + L::OFF_M) + row;
+        float m_ref = -INFINITY, l_sum = 0.f;
+        bool ok = true;
+        int ys = wg;                               // Y stage and the parity of its barrier
+        uint32_t ypar = 0;
+        for (int t = wg; t < nt; t += 2) {
+            const int s = wg;
+            if (!(ok = __all_sync(0xffffffffu, mbar_wait(s_full + s, (t >> 1) & 1, abort_flag)))) break;
+            tc_fence_after();
+            uint32_t sr[BN];
+#pragma unroll
+            for (int c = 0; c < BN / 32; ++c) tmem_ld32(tmem_base + s * BN + lane_sel + c * 32, sr + c * 32);
+            float* sf = reinterpret_cast<float*>(sr);
             if constexpr (PLANE) {
-                if (!(ok = mbar_wait(v_full + s, (t >> 1) & 1, abort_flag))) break;  // Y of this stage has landed
-                const uint8_t* yb = sY + s * L::Y_BYTES;
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait(y_full + ys, ypar, abort_flag)))) break;
+                uint8_t* yb = sY + ys * L::Y_BYTES;
+                tmem_wait_ld();
 #pragma unroll
                 for (int c = 0; c < BN / 8; ++c) {
                     const uint4 y = *reinterpret_cast<const uint4*>(yb + sw128_offset(row, c));
@@ -358,30 +367,31 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                         float2* s2 = reinterpret_cast<float2*>(sf) + c * 4 + e;
                         *s2 = __ffma2_rn(*s2, make_float2(scale_log2, scale_log2), unpack_f16(w[e]));
                     }
-                }
-            }
-            if constexpr (CARRY) {
-                // the finished logits of this warp's 32 rows x 64 columns leave as fp16 (back in the natural-log domain,
-                // before the mask: the next layer's aligner sees finite values everywhere) through the warp's staging buffer
-                uint8_t* stg = sStg + warp * 4096;
-                if (t >= 1 && lane == 0) tma_store_wait_read<0>();  // the store of the previous tile has read the buffer
-                __syncwarp();
-                constexpr float kLn2 = 0.6931471805599453f;
+                    if constexpr (CARRY) {
+                        // the finished logits go over the row's Y as fp16 (back in the natural-log domain, before the mask: the next
+                        // layer's aligner sees finite values everywhere) and from there to the scores buffer
+                        constexpr float kLn2 = 0.6931471805599453f;
+                        uint32_t v[4];
 #pragma unroll
-                for (int c = 0; c < BN / 8; ++c) {
-                    uint4 v;
-                    { const float2 t2 = __fmul2_rn(reinterpret_cast<const float2*>(sf)[c * 4 + 0], make_float2(kLn2, kLn2)); v.x = pack_f16(t2.x, t2.y); }
-                    { const float2 t2 = __fmul2_rn(reinterpret_cast<const float2*>(sf)[c * 4 + 1], make_float2(kLn2, kLn2)); v.y = pack_f16(t2.x, t2.y); }
-                    { const float2 t2 = __fmul2_rn(reinterpret_cast<const float2*>(sf)[c * 4 + 2], make_float2(kLn2, kLn2)); v.z = pack_f16(t2.x, t2.y); }
-                    { const float2 t2 = __fmul2_rn(reinterpret_cast<const float2*>(sf)[c * 4 + 3], make_float2(kLn2, kLn2)); v.w = pack_f16(t2.x, t2.y); }
-                    *reinterpret_cast<uint4*>(stg + sw128_offset(lane, c)) = v;
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 x = __fmul2_rn(reinterpret_cast<const float2*>(sf)[c * 4 + e], make_float2(kLn2, kLn2));
+                            v[e] = pack_f16(x.x, x.y);
+                        }
+                        *reinterpret_cast<uint4*>(yb + sw128_offset(row, c)) = make_uint4(v[0], v[1], v[2], v[3]);
+                    }
                 }
-                fence_async_smem();
+                if constexpr (CARRY) fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    tma_store_5d(&tmC, stg, 0, b * p.Hq + h, warp * 32, t, (q0 - p.plane_row0) / BM);
-                    tma_store_commit();
+                    if constexpr (CARRY) {
+                        tma_store_5d(&tmC, yb + q * 4096, 0, b * p.Hq + h, q * 32, t, (q0 - p.plane_row0) / BM);
+                        tma_store_commit();
+                    } else {
+                        mbar_arrive(y_empty + ys);
+                    }
                 }
+            } else {
+                tmem_wait_ld();
             }
             // from here on: PLANE -> sf holds log2-domain logits; otherwise raw scores, scaled inside the exp
             if (t * BN + BN - 1 > q0) {   // the tile reaches past the CTA's first query row: mask keys after each row
@@ -399,89 +409,100 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
             mx[2] = fmaxf(mx[2], sf[BN - 2]); mx[3] = fmaxf(mx[3], sf[BN - 1]);
             float m_t = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
             if constexpr (!PLANE) m_t *= scale_log2;
-            // lazy rescale: move the reference maximum only when some row of the warp outgrew it by 2^8
-            // (a row with every key of this tile masked has m_t = -inf and never asks for it)
-            const bool grow = m_t > m_ref + 8.f;
-            const bool rescale = __any_sync(0xffffffffu, grow) || t == 0;
-            float factor = 1.f;
-            if (rescale) {
-                const float m_new = fmaxf(m_ref, m_t);
-                factor = fast_exp2(m_ref - m_new);
-                m_ref = m_new;
+            // The reference maximum of a row goes from tile to tile, that is from one warpgroup to the other, through shared memory.  Lazy
+            // rescale: it moves only when some row of the warp outgrew it by 2^8 (a row with every key of this tile masked has m_t = -inf
+            // and never asks for it); then the accumulator is rescaled, after every P.V issued so far has landed in it.
+            float m_new = -INFINITY;
+            if (t > 0) {
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait(m_set + (wg ^ 1) * 4 + q, ((t - 1) >> 1) & 1, abort_flag)))) break;
+                m_new = *m_row;
             }
-            if (t > 0 && rescale) {   // the accumulator is touched only after every P.V issued so far has landed in it
-                if (!(ok = mbar_wait(pv_done + ((t - 1) & 1), ((t - 1) >> 1) & 1, abort_flag))) break;
-                {
-                    tc_fence_after();
+            const float m_old = m_new;
+            const bool rescale = __any_sync(0xffffffffu, m_t > m_new + 8.f) || t == 0;
+            if (rescale) {
+                m_new = fmaxf(m_new, m_t);
+                *m_row = m_new;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(m_set + wg * 4 + q);
+            const float mine = fast_exp2(m_ref - m_new);   // this warpgroup's sum so far: 1 unless the reference has moved since
+            m_ref = m_new;
+            if (t > 0 && rescale) {
+                const float factor = fast_exp2(m_old - m_new);
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait(pv_done + (wg ^ 1), ((t - 1) >> 1) & 1, abort_flag)))) break;
+                tc_fence_after();
+#pragma unroll 1
+                for (int c = 0; c < D / 16; ++c) {
+                    uint32_t orr[16];
+                    tmem_ld16(tmem_O + lane_sel + c * 16, orr);
+                    tmem_wait_ld();
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t orr[32];
-                        tmem_ld32(tmem_O + lane_sel + c * 32, orr);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            float2* o2 = reinterpret_cast<float2*>(orr) + j;
-                            *o2 = __fmul2_rn(*o2, make_float2(factor, factor));
-                        }
-                        tmem_st32(tmem_O + lane_sel + c * 32, orr);
+                    for (int j = 0; j < 8; ++j) {
+                        float2* o2 = reinterpret_cast<float2*>(orr) + j;
+                        *o2 = __fmul2_rn(*o2, make_float2(factor, factor));
                     }
-                    tmem_wait_st();
+                    tmem_st16(tmem_O + lane_sel + c * 16, orr);
                 }
             }
-            // P(t) is announced on p_full[t & 1], a barrier whose phases the P.V warp tells apart by parity alone.  Since the
-            // score MMAs no longer wait for the P.V MMAs, the softmax could finish tile t while P.V(t-2) has not even been
-            // picked up: the barrier would then run two phases ahead and the waiting warp would never see its phase end.
-            // So tile t's announcement waits until P.V(t-2) has completed (which also frees a P buffer of its own,
-            // where the layout has one); two tiles back, this has nearly always happened already.
-            if (t >= 2 && !(ok = mbar_wait(pv_done + s, ((t - 2) >> 1) & 1, abort_flag))) break;
-            uint8_t* pb = p_buf(t);
-            // The softmax warps are bound by the length of their own instruction chain, so the fp32 arithmetic around
-            // the exponentials runs two values per instruction (packed fp32 pairs; the scores of a thread sit in
-            // consecutive registers).
+            // The fp32 arithmetic around the exponentials runs two values per instruction (packed fp32 pairs; the scores of a thread sit in
+            // consecutive registers).  P goes over the scores it came from.
             float2 sum2 = make_float2(0.f, 0.f);
             const float2 neg_m2 = make_float2(-m_ref, -m_ref), scale2 = make_float2(scale_log2, scale_log2);
             const float2* sf2 = reinterpret_cast<const float2*>(sf);
 #pragma unroll
-            for (int c = 0; c < BN / 8; ++c) {
-                float e[8];
+            for (int c = 0; c < BN / 32; ++c) {
+                uint32_t pk[16];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 x = PLANE ? __fadd2_rn(sf2[c * 4 + j], neg_m2) : __ffma2_rn(sf2[c * 4 + j], scale2, neg_m2);
-                    e[2 * j] = fast_exp2(x.x);
-                    e[2 * j + 1] = fast_exp2(x.y);
-                    sum2 = __fadd2_rn(sum2, make_float2(e[2 * j], e[2 * j + 1]));
+                for (int j = 0; j < 16; ++j) {
+                    const float2 x = PLANE ? __fadd2_rn(sf2[c * 16 + j], neg_m2) : __ffma2_rn(sf2[c * 16 + j], scale2, neg_m2);
+                    const float2 e = make_float2(fast_exp2(x.x), fast_exp2(x.y));
+                    sum2 = __fadd2_rn(sum2, e);
+                    pk[j] = pack_bf16(e.x, e.y);
                 }
-                uint4 v;
-                v.x = pack_bf16(e[0], e[1]); v.y = pack_bf16(e[2], e[3]); v.z = pack_bf16(e[4], e[5]); v.w = pack_bf16(e[6], e[7]);
-                *reinterpret_cast<uint4*>(pb + sw128_offset(row, c)) = v;
+                tmem_st16(tmem_base + s * BN + lane_sel + c * 16, pk);
             }
-            l_sum = l_sum * factor + (sum2.x + sum2.y);
-            fence_async_smem();
+            l_sum = l_sum * mine + (sum2.x + sum2.y);
+            tmem_wait_st();
             tc_fence_before();
-            mbar_arrive(p_full + s);
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(p_full + s);
+                if constexpr (CARRY) {
+                    tma_store_wait_read<0>();   // the logits have left: the stage may be refilled
+                    mbar_arrive(y_empty + ys);
+                }
+            }
+            if (PLANE) {
+                if ((ys += 2) >= L::YST) { ys -= L::YST; ypar ^= 1; }
+            }
         }
-        if constexpr (EMIT || CARRY) {
+        if constexpr (CARRY) {
             if (lane == 0) tma_store_wait_all<0>();
         }
-        if constexpr (EMIT) {
-        } else if (ok && mbar_wait(pv_done + ((nt - 1) & 1), ((nt - 1) >> 1) & 1, abort_flag)) {
+        // The row's sum: both warpgroups' shares on the last reference maximum, through the Q tile, which nobody reads any more once
+        // the last P.V has run.  Every softmax warp comes to the barrier, one whose wait ran out as well.
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_full, 0, abort_flag));
+        float* l_x = reinterpret_cast<float*>(sQ);
+        if (ok) l_x[wg * BM + row] = l_sum * fast_exp2(m_ref - *m_row);
+        asm volatile("barrier.cta.sync 1, 256;" ::: "memory");
+        if (ok) {
             tc_fence_after();
-            const float inv_l = 1.f / l_sum;
-            __nv_bfloat16* orow = p.o + b * p.o_sb + (int64_t)qi * p.o_sn + h * p.o_sh;
+            const float inv_l = 1.f / (l_x[row] + l_x[BM + row]);
+            __nv_bfloat16* orow = p.o + b * p.o_sb + (int64_t)qi * p.o_sn + h * p.o_sh + wg * (D / 2);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < D / 2 / 32; ++c) {
                 uint32_t orr[32];
-                tmem_ld32(tmem_O + lane_sel + c * 32, orr);
+                tmem_ld32(tmem_O + lane_sel + wg * (D / 2) + c * 32, orr);
                 tmem_wait_ld();
                 if (qi < p.N) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
+                    for (int k = 0; k < 4; ++k) {
                         uint4 v;
-                        v.x = pack_bf16(__uint_as_float(orr[q * 8 + 0]) * inv_l, __uint_as_float(orr[q * 8 + 1]) * inv_l);
-                        v.y = pack_bf16(__uint_as_float(orr[q * 8 + 2]) * inv_l, __uint_as_float(orr[q * 8 + 3]) * inv_l);
-                        v.z = pack_bf16(__uint_as_float(orr[q * 8 + 4]) * inv_l, __uint_as_float(orr[q * 8 + 5]) * inv_l);
-                        v.w = pack_bf16(__uint_as_float(orr[q * 8 + 6]) * inv_l, __uint_as_float(orr[q * 8 + 7]) * inv_l);
-                        *reinterpret_cast<uint4*>(orow + c * 32 + q * 8) = v;
+                        v.x = pack_bf16(__uint_as_float(orr[k * 8 + 0]) * inv_l, __uint_as_float(orr[k * 8 + 1]) * inv_l);
+                        v.y = pack_bf16(__uint_as_float(orr[k * 8 + 2]) * inv_l, __uint_as_float(orr[k * 8 + 3]) * inv_l);
+                        v.z = pack_bf16(__uint_as_float(orr[k * 8 + 4]) * inv_l, __uint_as_float(orr[k * 8 + 5]) * inv_l);
+                        v.w = pack_bf16(__uint_as_float(orr[k * 8 + 6]) * inv_l, __uint_as_float(orr[k * 8 + 7]) * inv_l);
+                        *reinterpret_cast<uint4*>(orow + c * 32 + k * 8) = v;
                     }
                 }
             }
@@ -497,7 +518,7 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
         while (clock64() - t0 < 4000000ll) __nanosleep(1000);
         __syncthreads();
     }
-    if (warp == 5) {
+    if (warp == kSoftmaxWarps + 1) {
         __syncwarp();
         tc_fence_after();
         tmem_dealloc(tmem_base, L::TMEM_COLS);
@@ -565,7 +586,7 @@ cudaError_t launch_tc_flash(const TcFlashArgs& a, cudaStream_t stream) {
         // emit: one epilogue warp's 32 rows x 64 columns per copy; attention: the CTA's 128 rows x 64 columns
         const uint32_t box[5] = {(uint32_t)BN, 1, a.emit_plane ? 32u : (uint32_t)BM, 1, 1};
         if (!make_tensor_map_bf16(&tmY, a.emit_plane ? a.emit_plane : a.plane, 5, dims, str, box, true)) return cudaErrorInvalidValue;
-        if (a.carry) {   // the logits leave one epilogue warp's 32 rows at a time
+        if (a.carry) {   // the logits leave one softmax warp's 32 rows at a time
             if (a.emit_plane || !a.plane) return cudaErrorInvalidValue;
             const uint32_t cbox[5] = {(uint32_t)BN, 1, 32u, 1, 1};
             if (!make_tensor_map_bf16(&tmC, a.carry, 5, dims, str, cbox, true)) return cudaErrorInvalidValue;

@@ -454,3 +454,39 @@ def test_single_links_of_several_waves_take_the_link_kernel(B, N, Hq, Hkv, m, ac
         got = lb.lisa_attn_shared_prefill_carry(q0, k0, dl[k], dev(t[f"v{k + 1}"]), scores, first=k == 0, keep=k == 0)
         assert_close(got.float().cpu().numpy(), ref[k], "bf16", "one link a call, layer %d" % (k + 1))
     assert lb.lisa_check() == lb.OK
+
+
+@pytest.mark.parametrize("N", [1, 64, 65, 129, 193, 384])
+@pytest.mark.parametrize("form", ["anchor", "plane", "carry"])
+def test_attention_whose_maxima_keep_growing(N, form):
+    """Scores that rise along the keys by 3 every 16, and fall by 2 every 40 on top: nearly every tile moves the reference maximum of its rows
+    (the accumulator is rescaled, and one warpgroup's sum meets a reference the other has set).  Scores up to 72 are rounded where the kernels
+    round them: Q.K (or Q'.K') in fp32 from bf16 products, exact here; so the stated bar holds."""
+    j = torch.arange(N)
+    a = (j // 16 * 3 - j % 40 // 20 * 2).float()                       # whole numbers below 256: exact in bf16
+    v = synth.as_dtype(synth.normal("v", (1, N, 32, 128), 5), "bf16")
+    r = 16
+    if form == "anchor":
+        q, k = torch.zeros(1, N, 32, 128), torch.zeros(1, N, 32, 128)
+        q[..., 0], k[..., 0] = 1.0, a[None, :, None]
+        scale = 128 ** -0.5
+        q = q * 8.0                                                    # score = a / sqrt(2)
+        s = (8.0 * scale * a).double()
+        got = lb.lisa_attn_anchor(dev(q.bfloat16()), dev(k.bfloat16()), dev(v))
+    else:
+        z = synth.as_dtype(synth.normal("q", (1, N, 32, 128), 6), "bf16")
+        qp, kp = torch.zeros(1, N, 32, r), torch.zeros(1, N, 32, r)
+        qp[..., 0], kp[..., 0] = 4.0, a[None, :, None]                 # score = a, with an aligner of zero weights
+        s = a.double()
+        link = lb.Link(dev(qp.bfloat16()), dev(kp.bfloat16()), torch.zeros(32, 64, dtype=torch.bfloat16, device="cuda"),
+                       torch.zeros(64, 32, dtype=torch.bfloat16, device="cuda"))
+        if form == "plane":
+            got = lb.lisa_attn_shared_prefill(dev(z), dev(z), [link], dev(v))
+        else:
+            scores = torch.empty(lb.lisa_prefill_scores_bytes(1, N, 32), dtype=torch.uint8, device="cuda")
+            got = lb.lisa_attn_shared_prefill_carry(dev(z), dev(z), link, dev(v), scores, first=True, keep=True)
+    torch.cuda.synchronize()
+    assert lb.lisa_check() == lb.OK
+    p = torch.softmax(s[None, :].expand(N, N).masked_fill(torch.ones(N, N, dtype=torch.bool).triu(1), float("-inf")), -1)
+    ref = torch.einsum("ij,bjhd->bihd", p, v.double())
+    assert_close(got.float().cpu().numpy(), ref.numpy(), "bf16", form)
