@@ -341,7 +341,7 @@ static lisa_status_t shared_prefill_impl(const lisa_shared_prefill_args* a, lisa
     if (!g_force_general.load() && a->d == 128 && a->chain_len == 0) {
         TcFlashArgs f{a->B, a->N, a->Hq, a->Hkv, 128, a->q0, a->k0, a->v, a->o, 1.0f / sqrtf((float)a->d), nullptr, 0, 0,
                       0, (a->N + 127) / 128};
-        f.chained = (int64_t)a->B * a->Hq * f.qt_count <= 2 * (int64_t)sm_count();
+        f.chained = true;
         if (tc_flash_supported(f)) {
             cudaError_t e = launch_tc_flash(f, s);
             return e == cudaSuccess ? LISA_OK : cuda_fail(e);

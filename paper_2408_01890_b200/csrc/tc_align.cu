@@ -65,7 +65,6 @@ __global__ void __launch_bounds__(NT, MIN_CTAS)
 tc_align_kernel(const __grid_constant__ AlignParams p) {
     extern __shared__ __align__(16) uint8_t smem[];
     const int c = p.chain;
-    chain_release();
     uint8_t* sW = smem;                               // per link: W1 fragments, W2 fragments, b1[64], b2[32]
     uint8_t* sScr = sW + c * LINK_BYTES;              // per warp: STAGES buffers of c planes x [32 heads][64 B]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -79,6 +78,7 @@ tc_align_kernel(const __grid_constant__ AlignParams p) {
     }
     __syncthreads();
     chain_wait();   // from here on: the planes, which earlier kernels of the stream produce
+    chain_release();   // (not earlier: what follows may read what came before this call without a wait of its own)
 
     // Parameter fields of the main loop, read once into registers: behind the asm statements (memory clobbers) the
     // compiler would re-read them from the parameter bank every time, the per-link ones through a run-time index.

@@ -37,10 +37,13 @@ struct PackJobs {
 // A CTA packs kPackPos positions of one sequence: the rows of H x r values are read as they lie (one warp per position) into shared
 // memory and leave as whole 128-byte rows.  Bound by HBM where it runs alone; beside a flash kernel, by the shared memory that leaves free.
 constexpr int kPackPos = 8, kPackThreads = kPackPos * 32;
-__global__ void __launch_bounds__(kPackThreads) pack_lowrank_kernel(const __grid_constant__ PackJobs jobs, int B, int N) {
+// behind: launched in a programmatic chain right behind a kernel of the same call that releases its successors after its own wait, and
+// writes nothing that is read here.  What came before the call is then complete when this kernel starts, so it runs beside that kernel
+// and waits for it at its own end only (so that completion stays transitive).
+__global__ void __launch_bounds__(kPackThreads) pack_lowrank_kernel(const __grid_constant__ PackJobs jobs, int B, int N, int behind) {
     __shared__ __align__(16) __nv_bfloat16 rows[kPackPos][kMaxHeads * kMaxRank];
     chain_release();
-    chain_wait();
+    if (!behind) chain_wait();
     const TView src = jobs.src[blockIdx.y];
     const int H = jobs.H[blockIdx.y], r = jobs.r[blockIdx.y], n0 = blockIdx.x * kPackPos;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, vals = H * r;
@@ -73,6 +76,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_lowrank_kernel(const __grid
         }
         __syncthreads();
     }
+    if (behind) chain_wait();
 }
 
 // Optional per-phase timing of the tensor-core prefill (lisa_prefill_phase_timing): CUDA events recorded on the
@@ -208,7 +212,7 @@ size_t tc_carry_bytes(int B, int N, int Hq) {
 
 namespace {
 // The packing of Q'/K' feeds only the kernels that come after the first emit (the attention kernel; the emits of the
-// differences of deeper chains), so it runs beside that emit on a stream of the library's own: forked from the
+// differences of deeper chains), so in calls of several waves it runs beside that emit on a stream of the library's own: forked from the
 // caller's stream with one event and joined with another before its first consumer.  One stream and one event pair
 // per device, created on first use; the fork and the join are each enqueued under a lock, so calls from several host
 // threads cannot pair one call's wait with another call's record.
@@ -339,11 +343,29 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
     char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(ws) + 1023) & ~(uintptr_t)1023);
     const int c = a.chain_len;
     cudaError_t e;
+    const bool concat = concat_chain(a);
+    const bool one_wave = (int64_t)a.B * a.Hq * ((a.N + kTile - 1) / kTile) <= 2 * (int64_t)sm_count();   // of CTAs, all resident at once
+    Wave waves[1024];
+    int nw = plan_waves(a.B, a.N, a.Hq, cy ? 1 : plane_count(a), waves, 1024, cy != nullptr && !concat);
+    // A host-memory call whose prompt fits fewer than four waves is cut into four strips of query tiles all the same (they
+    // run one after the other in the planes laid out for the larger waves): its time is the copies', and strips let the
+    // copies in, the compute and the copies out overlap.
+    if (ho && !all_layers && nw < 4 && !g_pt.on) {
+        const int n_qt = (a.N + kTile - 1) / kTile, per = (n_qt + 3) / 4;
+        if (n_qt >= 4) {
+            nw = 0;
+            for (int qt = 0; qt < n_qt; qt += per) waves[nw++] = Wave{qt, std::min(per, n_qt - qt)};
+        }
+    }
+    // A call of one wave goes out as a programmatic chain on the caller's stream, set-up of each kernel under the tail of the one before,
+    // and Q', K' are packed beside its first kernel (as chains of CTAs resident at once did, with a fork to a stream for the packing and back
+    // in each call: a prompt of 197 tokens through an anchor and three layers 71.6 -> 62.9 us, host 70 -> 46; one layer of 2048 tokens
+    // 167 -> 162, 2 x 1777 tokens of 40 heads through three layers 737 -> 724).  Otherwise they are packed beside the first emit on a stream of their own (and on the
+    // caller's, before everything, while the per-kernel timing is on).
+    const bool chained = nw == 1 && !ho && !g_pt.on;
     SideStream* side = nullptr;
-    // one wave of CTAs that are resident at once: the call's kernels go out as a programmatic chain
-    const bool one_wave = (int64_t)a.B * a.Hq * ((a.N + kTile - 1) / kTile) <= 2 * (int64_t)sm_count(), small = one_wave && !ho;
-    {
-        PhaseMark mark(0, s);
+    bool packed = false;
+    auto launch_pack = [&](bool chain, int behind, cudaStream_t ps) -> cudaError_t {
         PackJobs jobs{};
         for (int k = 0; k < c; ++k) {
             jobs.src[2 * k] = make_view(a.links[k].qp); jobs.dst[2 * k] = reinterpret_cast<__nv_bfloat16*>(base + l.qp_off[k]);
@@ -351,42 +373,34 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
             jobs.src[2 * k + 1] = make_view(a.links[k].kp); jobs.dst[2 * k + 1] = reinterpret_cast<__nv_bfloat16*>(base + l.kp_off[k]);
             jobs.H[2 * k + 1] = a.Hkv; jobs.r[2 * k + 1] = a.links[k].r;
         }
-        const dim3 grid((a.N + kPackPos - 1) / kPackPos, 2 * c, std::min(a.B, 65535));
-        // beside the first emit, unless the per-kernel timing is on (then every kernel is timed on the caller's stream)
+        packed = true;
+        count_launches(1);
+        return launch_kernel(chain, pack_lowrank_kernel, dim3((a.N + kPackPos - 1) / kPackPos, 2 * c, std::min(a.B, 65535)), dim3(kPackThreads), 0, ps,
+                             jobs, a.B, a.N, behind);
+    };
+    if (!chained) {
+        PhaseMark mark(0, s);
         if (!g_pt.on) {
             std::lock_guard<std::mutex> lock(g_side_mutex);
             side = side_stream();
             if (side) {
                 if ((e = cudaEventRecord(side->fork, s)) != cudaSuccess) return e;
                 if ((e = cudaStreamWaitEvent(side->stream, side->fork, 0)) != cudaSuccess) return e;
-                pack_lowrank_kernel<<<grid, kPackThreads, 0, side->stream>>>(jobs, a.B, a.N);
-                if ((e = cudaGetLastError()) != cudaSuccess) return e;
+                if ((e = launch_pack(false, 0, side->stream)) != cudaSuccess) return e;
                 if ((e = cudaEventRecord(side->join, side->stream)) != cudaSuccess) return e;
             }
         }
-        if (!side && (e = launch_kernel(false, pack_lowrank_kernel, grid, dim3(kPackThreads), 0, s, jobs, a.B, a.N)) != cudaSuccess) return e;
-        count_launches(1);
+        if (!side && (e = launch_pack(false, 0, s)) != cudaSuccess) return e;
     }
     bool joined = side == nullptr;
+    // behind a kernel of the call (first = false), or before all of them where the first reads the packed rows; see pack_lowrank_kernel
+    auto pack_behind = [&](bool first) -> cudaError_t { return packed ? cudaSuccess : launch_pack(true, first ? 0 : 1, s); };
     auto join_pack = [&]() -> cudaError_t {   // before the first kernel that reads the packed Q'/K'
         if (joined) return cudaSuccess;
         joined = true;
         std::lock_guard<std::mutex> lock(g_side_mutex);
         return cudaStreamWaitEvent(s, side->join, 0);
     };
-    const bool concat = concat_chain(a);
-    Wave waves[1024];
-    int nw = plan_waves(a.B, a.N, a.Hq, cy ? 1 : plane_count(a), waves, 1024, cy != nullptr && !concat);
-    // A host-memory call whose prompt fits fewer than four waves is cut into four strips of query tiles all the same (they
-    // run one after the other in the planes laid out for the larger waves): its time is the copies', and strips let the
-    // copies in, the compute and the copies out overlap.
-    if (ho && side && !all_layers && nw < 4) {
-        const int n_qt = (a.N + kTile - 1) / kTile, per = (n_qt + 3) / 4;
-        if (n_qt >= 4) {
-            nw = 0;
-            for (int qt = 0; qt < n_qt; qt += per) waves[nw++] = Wave{qt, std::min(per, n_qt - qt)};
-        }
-    }
     // Several waves in flight (see kWaveSets): wave w runs on stream w % sets (0 = the caller's) with plane set w % sets.
     // All of it is forked from and joined back into the caller's stream inside this call, under the lock that keeps
     // another host thread's call from interleaving its event records with these waits.
@@ -415,7 +429,7 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
         // 1. anchor scores and the differences of the links below the top one
         TcFlashArgs fw{a.B, a.N, a.Hq, a.Hkv, 128, a.q0, a.k0, a.v, a.o, 1.f / sqrtf((float)a.d), nullptr, l.plane_rows, l.plane_cols,
                              wv.begin, wv.count};                 // the wave's own planes
-        fw.chained = small;
+        fw.chained = chained;
         TcFlashArgs f = fw;                                       // the plane of the running scores
         f.plane_rows = x_rows; f.plane_cols = x_cols; f.plane_row0 = row0;
         char* const x_plane = cy ? plane_base : base + po[0];
@@ -423,9 +437,10 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
         if (!cy || cy->first) {
             PhaseMark mark(1, st);
             if ((e = launch_tc_flash(f, st)) != cudaSuccess) return e;
+            if (chained && (e = pack_behind(false)) != cudaSuccess) return e;
         }
         for (int k = 0; k + (concat ? 0 : 1) < c; ++k) {   // the concatenating form also needs the top link's difference as a plane
-            if ((e = join_pack()) != cudaSuccess) return e;
+            if ((e = chained ? pack_behind(true) : join_pack()) != cudaSuccess) return e;
             PhaseMark mark(1, st);
             TcFlashArgs fd = fw;
             fd.kd = kPadRank;
@@ -445,7 +460,7 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
                                    &a.links[k], (k + 1 < c || (cy && cy->keep)) ? 0 : -1, (all_layers || k == c - 1) ? 1 : -1, row0,
                                    l.plane_rows, l.plane_cols, -1};
                 PhaseMark mark(2, st);
-                ac.chained = small;
+                ac.chained = chained;
                 if ((e = launch_tc_align_link(ac, st)) != cudaSuccess) return e;
             }
             // 3c. softmax and .V on the finished scores: the attention kernel's own difference is switched off (scale 0)
@@ -477,8 +492,9 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
                                    k + 1 < c ? base + po[k + 1] : nullptr, &a.links[k], k + 1 < c ? 1 : -1,
                                    (all_layers || k == c - 1) ? 0 : -1, row0};
                 PhaseMark mark(2, st);
-                al.chained = small;
+                al.chained = chained;
                 if ((e = launch_tc_align_link(al, st)) != cudaSuccess) return e;
+                if (chained && (e = pack_behind(false)) != cudaSuccess) return e;
             }
         }
         // 2. the FFN chain over the head axis, in place
@@ -489,10 +505,11 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
         al.links = a.links;
         al.row0 = row0;
         al.store_all = all_layers;
-        al.chained = small;
+        al.chained = chained;
         if (!per_link) {
             PhaseMark mark(2, st);
             if ((e = launch_tc_align(al, st)) != cudaSuccess) return e;
+            if (chained && (e = pack_behind(false)) != cudaSuccess) return e;
         }
         // 3. each layer's own difference, softmax and .V
         if ((e = join_pack()) != cudaSuccess) return e;

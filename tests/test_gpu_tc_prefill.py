@@ -490,3 +490,37 @@ def test_attention_whose_maxima_keep_growing(N, form):
     p = torch.softmax(s[None, :].expand(N, N).masked_fill(torch.ones(N, N, dtype=torch.bool).triu(1), float("-inf")), -1)
     ref = torch.einsum("ij,bjhd->bihd", p, v.double())
     assert_close(got.float().cpu().numpy(), ref.numpy(), "bf16", form)
+
+
+@pytest.mark.parametrize("N", [50, 197, 1300])
+@pytest.mark.parametrize("Hq,integrate", [(32, lb.INTEGRATE_ADD), (40, lb.INTEGRATE_ADD), (32, lb.INTEGRATE_CONCAT)])
+def test_a_programmatic_chain_equals_its_kernels_one_by_one(Hq, integrate, N):
+    """A carried chain of two layers, a fresh scores buffer and workspace for each of three inputs, called back to back: every output as with the
+    per-kernel timing on, which takes the chain apart (packing first, every kernel behind the one before)."""
+    m, h_in = 64, Hq * (2 if integrate == lb.INTEGRATE_CONCAT else 1)
+
+    def inputs(seed):
+        n = lambda name, *shape: dev(synth.as_dtype(synth.normal(name, shape, seed), "bf16"))  # noqa: E731
+        w = lambda name, *shape: dev(synth.as_dtype(synth.normal(name, shape, seed, std=shape[0] ** -0.5), "bf16"))  # noqa: E731
+        return n("q", 1, N, Hq, 128), n("k", 1, N, Hq, 128), [
+            (n("v%d" % k, 1, N, Hq, 128), lb.Link(n("qp%d" % k, 1, N, Hq, 21), n("kp%d" % k, 1, N, Hq, 21), w("w1%d" % k, h_in, m), w("w2%d" % k, m, Hq),
+                                                  integrate=integrate)) for k in range(2)]
+
+    def run(all_in):
+        outs = []
+        for q, k, layers in all_in:
+            scores = torch.empty(lb.lisa_prefill_scores_bytes(1, N, Hq), dtype=torch.uint8, device="cuda")
+            for i, (v, link) in enumerate(layers):
+                outs.append(lb.lisa_attn_shared_prefill_carry(q, k, link, v, scores, first=i == 0, keep=i == 0))
+        torch.cuda.synchronize()
+        assert lb.lisa_check() == lb.OK
+        return outs
+
+    all_in = [inputs(s) for s in (1, 2, 3)]
+    lb.lisa_prefill_phase_timing(True)
+    try:
+        ref = run(all_in)
+    finally:
+        lb.lisa_prefill_phase_timing(False)
+    for _ in range(3):
+        assert all(torch.equal(x, y) for x, y in zip(run(all_in), ref))
