@@ -460,12 +460,26 @@ bool three_per_sm(int64_t ctas) {
     return 1.3 * (double)((ctas + 3 * sms - 1) / (3 * sms)) < (double)((ctas + 2 * sms - 1) / (2 * sms));
 }
 
+// Ragged batches whose grid is not resident at once have their chunks dealt to the CTAs (decode_item).  A smaller grid leaves an SM at most
+// one CTA with work or two whichever way; there the count costs more than it gives (paper's default layer, 16 sequences of up to 1500: 70.5 us
+// dealt, 66.8 not; 16 of up to 2900 of the 8B shape: an anchor and three layers 148 us dealt, 168 not; 16 of up to 3000, 40 heads: 80 and 92).
+// A much larger grid evens itself out (100 of up to 3000, 2400 CTAs: 131 us dealt, 125 not; a uniform 7B-shaped batch whose lengths are given,
+// 544 CTAs: 0.3 % slower dealt).
+bool deal_chunks(const DecodeParams& p, int64_t ctas) {
+    const int64_t sms = sm_count();
+    return p.seq_lens && p.B > 1 && p.B <= kDenseMaxB && ctas > 2 * sms && ctas <= 3 * sms;
+}
+
 template <int HQ, int HG, int CH, int M_C, int ENG>
 cudaError_t launch_shared_fast(DecodeParams& p, cudaStream_t s) {
     const int64_t ctas = (int64_t)p.n_chunks * (HQ / HG) * p.B;
-    auto kernel = shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2>;
+    p.dense = deal_chunks(p, ctas);
+    auto kernel = p.dense ? shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2, true> : shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2, false>;
+    // (a ragged batch, whose lengths the host does not know, only where the build suits it with all of its chunks and with nine sixteenths of
+    // them, which lengths spread over [L / 8, L] leave: 16 sequences of up to 2900 positions 168 -> 148 us with the dealt chunks)
     if constexpr (ENG == kEngTf32 && CH == 128)
-        if (three_per_sm(ctas)) kernel = shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3>;
+        if (three_per_sm(ctas) && (!p.dense || three_per_sm((ctas * 9 + 15) / 16)))
+            kernel = p.dense ? shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3, true> : shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3, false>;
     const size_t smem = shared_fast_layout(HQ, HG, CH, ENG, p.m, HQ / p.Hkv).total;
     p.prefetch = ctas <= 2 * (int64_t)sm_count();   // a grid that is resident at once
     cudaError_t e = allow_smem(kernel, smem);
@@ -591,9 +605,12 @@ cudaError_t launch_anchor_decode(const lisa_anchor_args& a, void* ws, cudaStream
         while (kv % 2 == 0 && chunks * (p.Hkv / kv) < want) kv /= 2;
         p.heads = kv * G;
         set_chunk(p, chunk_length(p.B, p.Hq, a.L, p.Hkv / kv), ws);
-        p.prefetch = (int64_t)p.n_chunks * p.B * (p.Hkv / kv) <= 2 * want;   // a grid that is resident at once
+        const int64_t ctas = (int64_t)p.n_chunks * p.B * (p.Hkv / kv);
+        p.prefetch = ctas <= 2 * want;   // a grid that is resident at once
+        p.dense = deal_chunks(p, ctas);
         const size_t smem = anchor_fast_smem(p.heads, p.chunk, G);
-        auto kernel = p.chunk == 128 ? anchor_decode_fast_kernel<128> : p.chunk == 64 ? anchor_decode_fast_kernel<64> : anchor_decode_fast_kernel<32>;
+        auto kernel = p.dense ? (p.chunk == 128 ? anchor_decode_fast_kernel<128, true> : p.chunk == 64 ? anchor_decode_fast_kernel<64, true> : anchor_decode_fast_kernel<32, true>)
+                              : (p.chunk == 128 ? anchor_decode_fast_kernel<128, false> : p.chunk == 64 ? anchor_decode_fast_kernel<64, false> : anchor_decode_fast_kernel<32, false>);
         if ((e = allow_smem(kernel, smem)) != cudaSuccess) return e;
         e = launch_chained(kernel, dim3(p.n_chunks, p.Hkv / kv, p.B), dim3(kDecodeThreads), smem, s, p);
     } else {

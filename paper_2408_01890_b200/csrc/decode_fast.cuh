@@ -259,8 +259,8 @@ __device__ __forceinline__ void pv_chunk(const DecodeParams& p, const float* s_s
 
 // The caches of this CTA's chunk on their way into L2, before the wait for the preceding kernel: a hint (the length may be read before
 // an earlier kernel has set it), and L2 is the point of coherence, so a new token's row that is still being written is read right later.
-__device__ __forceinline__ void prefetch_chunk(const DecodeParams& p, int b, int kv0, int n_kv, int j0, int ch, bool standard) {
-    const int hint = min(decode_length(p, b), p.L_cap) - j0;
+__device__ __forceinline__ void prefetch_chunk(const DecodeParams& p, int kv0, int n_kv, int ch, bool standard) {
+    const int b = blockIdx.z, j0 = blockIdx.x * ch, hint = min(decode_length(p, b), p.L_cap) - j0;
     if (hint <= 0 || !p.prefetch) return;
     const int nrows = min(ch, hint), tid = threadIdx.x;
     const size_t row0 = ((size_t)b * p.Hkv + kv0) * p.L_cap + j0;
@@ -284,17 +284,17 @@ inline size_t anchor_fast_smem(int HG, int ch, int G) {
     return sizeof(float) * ((size_t)HG * ch + (size_t)row_parts(HG / gv, ch, gv) * HG * 128);
 }
 
-template <int CH>
+template <int CH, bool DENSE>
 __global__ void __launch_bounds__(kDecodeThreads, 2) anchor_decode_fast_kernel(const __grid_constant__ DecodeParams p) {
     extern __shared__ __align__(16) float smem[];
-    const int b = blockIdx.z, chunk = blockIdx.x, tid = threadIdx.x;
-    const int HG = p.heads, h0 = blockIdx.y * HG, G = p.Hq / p.Hkv, kv0 = h0 / G, j0 = chunk * CH, gv = kv_group(G);
+    const int tid = threadIdx.x;
+    const int HG = p.heads, h0 = blockIdx.y * HG, G = p.Hq / p.Hkv, kv0 = h0 / G, gv = kv_group(G);
     chain_release();
-    prefetch_chunk(p, b, kv0, HG / G, j0, CH, true);
+    if constexpr (!DENSE) prefetch_chunk(p, kv0, HG / G, CH, true);
     chain_wait();
-    const int L = decode_length(p, b);
-    if (j0 >= L) return;
-    const int nrows = min(CH, L - j0);
+    int b, chunk, L;
+    if (!decode_item<CH, DENSE>(p, b, chunk, L)) return;
+    const int j0 = chunk * CH, nrows = min(CH, L - j0);
     float* s_s = smem;
     float* q_s = s_s + HG * CH;
     float* red = q_s + HG * 128;
@@ -439,16 +439,16 @@ __host__ __device__ inline SharedFastLayout shared_fast_layout(int HQ, int HG, i
 
 // CTAS: CTAs per SM the kernel is compiled for.  Three hide the FFN phase (no loads in flight from the CTA that is in it) better than
 // two, at 80 instead of 128 registers; which one a launch takes depends on how its grid fills the waves.
-template <int HQ, int HG, int CH, int M_C, int ENG, int CTAS>
+template <int HQ, int HG, int CH, int M_C, int ENG, int CTAS, bool DENSE>
 __global__ void __launch_bounds__(kDecodeThreads, CTAS) shared_decode_fast_kernel(const __grid_constant__ DecodeParams p) {
     static_assert(ENG == kEngTf32 ? M_C > 0 : HG == HQ, "the split forms run with all heads");
     constexpr int HS = 128 / CH, NT2 = HG / 8;
     extern __shared__ __align__(16) uint8_t smem_b[];
-    const int b = blockIdx.z, chunk = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int h0 = blockIdx.y * HG, G = HQ / p.Hkv, kv0 = h0 / G, j0 = chunk * CH;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int h0 = blockIdx.y * HG, G = HQ / p.Hkv, kv0 = h0 / G;
     const int m = ENG == kEngTf32 ? M_C : p.m;
     chain_release();
-    prefetch_chunk(p, b, kv0, HG / G, j0, CH, false);
+    if constexpr (!DENSE) prefetch_chunk(p, kv0, HG / G, CH, false);
     const SharedFastLayout lay = shared_fast_layout(HQ, HG, CH, ENG, m, G);
     float* s_s = reinterpret_cast<float*>(smem_b);
     float* y_s = reinterpret_cast<float*>(smem_b + lay.y);
@@ -501,9 +501,9 @@ __global__ void __launch_bounds__(kDecodeThreads, CTAS) shared_decode_fast_kerne
     for (int e = tid; e < (ENG == kEngTf32 ? m : mp); e += kDecodeThreads) b1_s[e] = e < m ? ldw(p.b1, e, p.w_dtype) : 0.f;
     for (int e = tid; e < HG; e += kDecodeThreads) b2_s[e] = ldw(p.b2, h0 + e, p.w_dtype);
     chain_wait();   // from here on: lengths, Q', the caches and the score row, which earlier kernels of the stream produce
-    const int L = decode_length(p, b);
-    if (j0 >= L) return;
-    const int nrows = min(CH, L - j0);
+    int b, chunk, L;
+    if (!decode_item<CH, DENSE>(p, b, chunk, L)) return;
+    const int j0 = chunk * CH, nrows = min(CH, L - j0);
     for (int e = tid; e < HG * p.r; e += kDecodeThreads) {
         const int h = e / p.r, x = e - h * p.r;
         qp_s[h * kMaxRank + x] = ld_elem(p.qp.ptr, b * p.qp.sb + (h0 + h) * p.qp.sh + x, p.qp.dtype);

@@ -326,3 +326,24 @@ def test_multi_layer_cache_handle_matches_per_layer_caches():
     with pytest.raises(lb.LisaError):
         whole.append(3, dev(t["kp"]), dev(t["v"]))               # no such layer
     assert lb.lisa_check() == lb.OK
+
+
+@pytest.mark.parametrize("Hq,Hkv,m,integrate,B,L", [(32, 8, 64, lb.INTEGRATE_ADD, 66, 600), (40, 40, 80, lb.INTEGRATE_ADD, 34, 1150),
+                                                     (32, 32, 128, lb.INTEGRATE_CONCAT, 34, 1100)])
+def test_ragged_batches_whose_chunks_are_dealt(Hq, Hkv, m, integrate, B, L):
+    """Grids of 297..444 CTAs (on 148 SMs) of a ragged batch: the chunks that hold positions are numbered on the device.  Lengths on and around
+    the chunk's edges, sequences past the first 32 and 64; then the standard layer of the same lengths."""
+    lens = np.random.default_rng(B).integers(1, L + 1, B).astype(np.int32)
+    lens[[0, 1, 2, 3, 31, 32, 33, B - 1]] = [1, 127, 128, 129, L, 256, 1, L - 1]
+    w = synth.Workload("dealt", "bf16", B, L, Hq, Hkv, 128, 21, m, "relu", 1, True)
+    run_shared_decode(w, B, L, lens=lens, seed=3, integrate=integrate)
+    if Hkv == 8:
+        t = synth.decode_inputs(w, 3, B=B, L=L)
+        cache = lb.KVCacheLayer(lb.CACHE_STANDARD, B, Hkv, (L + 7) // 8 * 8, 128)
+        lb.lisa_kvcache_append(cache, dev(t["k"]), dev(t["v"]))
+        row = torch.full((B, Hq, (L + 7) // 8 * 8), -7.0, dtype=torch.float32, device="cuda")
+        out = lb.lisa_attn_anchor(dev(t["q0"]), cache=cache, L=L, seq_lens=torch.from_numpy(lens).cuda(), out_scores=row)
+        O, R = oracle.decode_anchor(f64(t["q0"])[:, 0], f64(t["k"]), f64(t["v"]), lens)
+        assert_close(out[:, 0].float().cpu().numpy(), O, "bf16", "standard O")
+        for b in range(B):
+            assert_close(row.cpu().numpy()[b, :, :lens[b]], R[b, :, :lens[b]], "bf16", "standard row")
