@@ -78,7 +78,7 @@ size_t decode_workspace(int B, int Hq, int d, int L);
 size_t shared_decode_smem(int Hq, int m, int integrate);   // dynamic shared memory the shared-layer decode kernel asks for
 
 // Tensor-core flash kernel (head width 128, bf16): O = softmax_causal(QA.KA^T * scale [+ plane]) . V for query tiles
-// [qt_begin, qt_begin + qt_count).  qa [B,N,Hq,kd], ka [B,N,Hkv,kd] with kd in {64,128}; plane (optional) holds
+// [qt_begin, qt_begin + qt_count).  qa [B,N,Hq,kd], ka [B,N,Hkv,kd] with kd in {32,128}; plane (optional) holds
 // bf16 blocked [rows/128][cols/64][128][B*Hq][64] pre-computed scores for query rows qt_begin*128 onwards.
 struct TcFlashArgs {
     int B, N, Hq, Hkv, kd;

@@ -14,13 +14,15 @@
 //
 // Warp roles: warps 0-3 and 4-7 softmax/epilogue (thread = query row = TMEM lane; the two warpgroups take the key tiles in turn), warp 8
 // TMA producer, warp 9 issuer of the score MMAs and TMEM owner, warp 10 issuer of the P.V MMAs (warp 11 only completes the warpgroup).
-// P stays in tensor memory, over the scores it came from, as the A operand of P.V: a K stage is free again as soon as its score MMA has
-// run, a Y stage once its rows are read, a V stage and a score buffer after the P.V MMA.
+// A K stage is free again as soon as its score MMA has run, a Y stage once its rows are read, a V stage after the P.V MMA; where P lies, see
+// Smem::P_SMEM.
 // Sizing: a softmax warp spends as long on waits (tensor memory, barriers, the next scores behind P.V) as on its 64 exponentials a row (16
 // lanes a cycle and SM: 512 cycles a tile), so an SM partition needs four of them in different phases: TWO CTAs share an SM (64-key tiles
 // keep a CTA at 112 KB of shared memory and 256 tensor-memory columns), each with two warpgroups on alternate tiles.  One warpgroup
 // per CTA took 1010 cycles a tile and SM, two warpgroups on halves of the same tile as long (in step, they wait for the same unit at the
-// same time), alternate tiles 845 (attention with plane, 2048 tokens of 32 heads 51 -> 47 us, 4 x 8192 tokens 3.6 -> 3.1 ms).
+// same time), alternate tiles 845.  A row's reference maximum is handed on behind the exponentials, which keeps the two warpgroups of a CTA
+// from coming to theirs together.  Attention with plane, 2048 tokens of 32 heads 56 -> 51 us timed alone (of which 3 are the first loads of
+// 296 CTAs at a time, 22 MB, and 8 the tail); 2 x 1777 of 40 heads, with and without write-back 241 -> 228; 4 x 8192 3.6 -> 3.1 ms without.
 // Every wait is bounded; on expiry the CTA records it in the status word, drains and exits.
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -65,8 +67,14 @@ struct Smem {
     static constexpr bool PLANE = MODE == MODE_ATTN_PLANE || MODE == MODE_ATTN_CARRY;
     static constexpr bool EMIT = MODE == MODE_EMIT;
     static constexpr bool CARRY = MODE == MODE_ATTN_CARRY;
-    static constexpr int KST = KD == 128 ? 3 : 2;  // K ring depth (V: two stages)
-    static constexpr int YST = PLANE ? 3 : 0;      // Y ring depth
+    // Where P lies: over the scores it came from, in tensor memory, as a tensor-memory operand of P.V, or in shared memory.  Over the scores,
+    // S(t + 2) has to wait for P(t).V(t), 1300 of a warpgroup's 3700 cycles a tile; in shared memory it need not, but there is room for that
+    // only beside a plane that is not written back (a written one has its logits over Y until the copy engine has read them: four stages).
+    static constexpr bool P_SMEM = MODE == MODE_ATTN_PLANE;
+    static constexpr int KST = EMIT || KD == 128 ? 3 : 2;  // K ring depth
+    static constexpr int VST = 2;                  // V ring depth
+    static constexpr int RB = KD == 128 ? 128 : 64;   // bytes of a row of a Q or K tile: 64 of the 128 columns, or all 32
+    static constexpr int YST = !PLANE ? 0 : P_SMEM ? 2 : 4;   // Y ring depth
     static constexpr int Q_BYTES = BM * KD * 2;
     static constexpr int K_BYTES = BN * KD * 2;
     static constexpr int V_BYTES = EMIT ? 0 : BN * D * 2;
@@ -75,11 +83,13 @@ struct Smem {
     static constexpr int OFF_Q = 0;
     static constexpr int OFF_K = OFF_Q + Q_BYTES;
     static constexpr int OFF_V = OFF_K + KST * K_BYTES;
-    static constexpr int OFF_Y = OFF_V + 2 * V_BYTES;
-    static constexpr int OFF_STG = OFF_Y + YST * Y_BYTES;
+    static constexpr int OFF_Y = OFF_V + VST * V_BYTES;
+    static constexpr int P_BYTES = P_SMEM ? BM * BN * 2 : 0;
+    static constexpr int OFF_P = OFF_Y + YST * Y_BYTES;
+    static constexpr int OFF_STG = OFF_P + 2 * P_BYTES;
     static constexpr int OFF_M = OFF_STG + STG_BYTES;      // reference maximum of each row: [128] fp32
     static constexpr int OFF_BAR = OFF_M + (EMIT ? 0 : BM * 4);
-    static constexpr int TOTAL = OFF_BAR + 288;
+    static constexpr int TOTAL = OFF_BAR + 320;
     static constexpr uint32_t TMEM_COLS = EMIT ? 128 : 256;   // S[2]: [0,128), O: [128,256)
     static_assert(TOTAL <= 115712, "two CTAs must fit one SM's shared memory");
 };
@@ -103,22 +113,24 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
     uint8_t* sK = smem + L::OFF_K;
     uint8_t* sV = smem + L::OFF_V;
     uint8_t* sY = smem + L::OFF_Y;
+    uint8_t* sP = smem + L::OFF_P;
     uint8_t* sStg = smem + L::OFF_STG;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);
     uint64_t* q_full = bars + 0;
     uint64_t* k_full = bars + 1;    // [KST <= 3]
     uint64_t* k_empty = bars + 4;   // [KST <= 3]
-    uint64_t* v_full = bars + 7;    // [2]
-    uint64_t* y_full = bars + 9;    // [YST <= 3]
-    uint64_t* y_empty = bars + 12;  // [YST <= 3] Y rows read (carry: and the logits that went over them stored)
-    uint64_t* s_full = bars + 15;   // [2] score buffer written by the MMA
-    uint64_t* s_free = bars + 17;   // [2] emit: score buffer copied to registers (attention: free with pv_done)
-    uint64_t* p_full = bars + 19;   // [2] P in tensor memory
-    uint64_t* pv_done = bars + 21;  // [2] P.V has run: its V stage and its score buffer, which held P, are free
-    uint64_t* m_set = bars + 23;    // [2][4] the rows of a quarter have their reference maximum for a tile
-    uint64_t* o_full = bars + 31;   // the last P.V has run (a barrier of its own: pv_done tells only neighbouring phases apart)
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 32);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 33);
+    uint64_t* v_full = bars + 7;    // [VST <= 2]
+    uint64_t* y_full = bars + 9;    // [YST <= 4]
+    uint64_t* y_empty = bars + 13;  // [YST <= 4] Y rows read (carry: and the logits that went over them stored)
+    uint64_t* s_full = bars + 17;   // [2] score buffer written by the MMA
+    uint64_t* s_free = bars + 19;   // [2] emit, P_SMEM: score buffer copied to registers (else free with pv_done)
+    uint64_t* p_full = bars + 21;   // [2] P is there
+    uint64_t* pv_done = bars + 23;  // [2] P.V has run: the place of P is free
+    uint64_t* m_set = bars + 25;    // [2][4] the rows of a quarter have their reference maximum for a tile
+    uint64_t* v_empty = bars + 33;  // [VST] P.V of the tile in the stage has run
+    uint64_t* o_full = bars + 35;   // the last P.V has run (a barrier of its own: pv_done tells only neighbouring phases apart)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 36);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 37);
 
     const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
     // blockIdx.x (the fastest-dispatched index) runs over (batch, head), blockIdx.y over query tiles from the last one
@@ -137,10 +149,10 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
         mbar_init(q_full, 1);
         for (int i = 0; i < KST; ++i) { mbar_init(k_full + i, 1); mbar_init(k_empty + i, 1); }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(v_full + i, 1);
             mbar_init(s_full + i, 1); mbar_init(s_free + i, 4);
             mbar_init(p_full + i, 4); mbar_init(pv_done + i, 1);
         }
+        for (int i = 0; i < L::VST; ++i) { mbar_init(v_full + i, 1); mbar_init(v_empty + i, 1); }
         for (int i = 0; i < L::YST; ++i) { mbar_init(y_full + i, 1); mbar_init(y_empty + i, 4); }
         for (int i = 0; i < 8; ++i) mbar_init(m_set + i, 1);
         mbar_init(o_full, 1);
@@ -166,18 +178,18 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
         // ------------------------------ TMA producer ------------------------------
         // Round t brings K(t) and Y(t), then V(t - 1): V is needed a softmax pass later than the others, and asked for in its own round
         // its stage, which waits for the P.V two tiles before, would hold up the Y of the next.
-        constexpr int NQ = KD / 64, NK = KD / 64, NV = EMIT ? 0 : D / 64;
+        constexpr int NQ = KD * 2 / L::RB, NK = NQ, NV = EMIT ? 0 : D / 64;
         if (elect_one()) {
             tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK);
             if (!EMIT) tma_prefetch_desc(&tmV);
             if (PLANE) tma_prefetch_desc(&tmY);
             mbar_expect_tx(q_full, L::Q_BYTES);
 #pragma unroll
-            for (int i = 0; i < NQ; ++i) tma_load_4d(sQ + i * (BM * 128), &tmQ, q_full, i * 64, h, q0, b);
+            for (int i = 0; i < NQ; ++i) tma_load_4d(sQ + i * (BM * L::RB), &tmQ, q_full, i * 64, h, q0, b);
         }
         __syncwarp();
-        int ks = 0, ys = 0;              // K and Y stage of tile t
-        uint32_t kpar = 1, ypar = 1;     // parity to wait for on their "empty" barriers (first pass: passes at once)
+        int ks = 0, ys = 0, vs = 0;      // K and Y stage of tile t, V stage of tile t - 1
+        uint32_t kpar = 1, ypar = 1, vpar = 1;     // parity to wait for on their "empty" barriers (first pass: passes at once)
         for (int t = 0; t < nt + (EMIT ? 0 : 1); ++t) {
             bool okp = true;
             if (t < nt) {
@@ -186,7 +198,7 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                 if (elect_one()) {
                     mbar_expect_tx(k_full + ks, L::K_BYTES);
 #pragma unroll
-                    for (int i = 0; i < NK; ++i) tma_load_4d(sK + ks * L::K_BYTES + i * (BN * 128), &tmK, k_full + ks, i * 64, g, t * BN, b);
+                    for (int i = 0; i < NK; ++i) tma_load_4d(sK + ks * L::K_BYTES + i * (BN * L::RB), &tmK, k_full + ks, i * 64, g, t * BN, b);
                 }
                 __syncwarp();
                 if constexpr (PLANE) {
@@ -201,15 +213,15 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
             }
             if constexpr (!EMIT) {
                 if (t > 0) {
-                    const int tv = t - 1, s2 = tv & 1;
-                    okp = mbar_wait(pv_done + s2, ((tv >> 1) & 1) ^ 1, abort_flag);
+                    okp = mbar_wait(v_empty + vs, vpar, abort_flag);
                     if (!__all_sync(0xffffffffu, okp)) break;
                     if (elect_one()) {
-                        mbar_expect_tx(v_full + s2, L::V_BYTES);
+                        mbar_expect_tx(v_full + vs, L::V_BYTES);
 #pragma unroll
-                        for (int i = 0; i < NV; ++i) tma_load_4d(sV + s2 * L::V_BYTES + i * (BN * 128), &tmV, v_full + s2, i * 64, g, tv * BN, b);
+                        for (int i = 0; i < NV; ++i) tma_load_4d(sV + vs * L::V_BYTES + i * (BN * 128), &tmV, v_full + vs, i * 64, g, (t - 1) * BN, b);
                     }
                     __syncwarp();
+                    if (++vs == L::VST) { vs = 0; vpar ^= 1; }
                 }
             }
             // The V and Y stages can be refilled at most two softmax passes before they are needed, under load less than a trip to HBM.
@@ -239,11 +251,11 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
         auto desc_off = [](uint64_t d, uint32_t bytes) -> uint64_t {
             return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4));
         };
-        const uint64_t dq0 = umma_desc_sw128(smem_u32(sQ), 16, 1024);
-        const uint64_t dk0 = umma_desc_sw128(smem_u32(sK), 16, 1024);
-        // scores of tile t into buffer t&1; needs K(t) loaded and (t >= 2) the buffer: P(t-2), which lies there, multiplied (emit: the
-        // scores read)
-        uint64_t* buf_free = EMIT ? s_free : pv_done;
+        const uint64_t dq0 = KD == 128 ? umma_desc_sw128(smem_u32(sQ), 16, 1024) : umma_desc_sw64(smem_u32(sQ));
+        const uint64_t dk0 = KD == 128 ? umma_desc_sw128(smem_u32(sK), 16, 1024) : umma_desc_sw64(smem_u32(sK));
+        // scores of tile t into buffer t&1; needs K(t) loaded and (t >= 2) the buffer: the scores of t-2 read, or P(t-2), which lies there,
+        // multiplied
+        uint64_t* buf_free = EMIT || L::P_SMEM ? s_free : pv_done;
         int sk = 0;
         uint32_t kpar = 0;
         bool ok = __all_sync(0xffffffffu, mbar_wait(q_full, 0, abort_flag));
@@ -258,7 +270,7 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
 #pragma unroll
                 for (int ks = 0; ks < KD / 16; ++ks) {
                     if (ks < ksteps)
-                        umma_ss(dst, desc_off(dq0, (ks >> 2) * (BM * 128) + (ks & 3) * 32), desc_off(dk, (ks >> 2) * (BN * 128) + (ks & 3) * 32), IDESC_QK, ks > 0);
+                        umma_ss(dst, desc_off(dq0, (ks >> 2) * (BM * L::RB) + (ks & 3) * 32), desc_off(dk, (ks >> 2) * (BN * L::RB) + (ks & 3) * 32), IDESC_QK, ks > 0);
                 }
                 umma_commit(s_full + s);
                 if (t + KST < nt) umma_commit(k_empty + sk);  // nobody waits for the last ones: do not arm them
@@ -274,23 +286,29 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                 return (d & 0xffffffff00000000ull) | (uint32_t)((uint32_t)d + (bytes >> 4));
             };
             const uint64_t dv0 = umma_desc_sw128(smem_u32(sV), BN * 128, 1024);
+            const uint64_t dp0 = umma_desc_sw128(smem_u32(sP), 16, 1024);
             bool ok = true;
+            int vs = 0;
+            uint32_t vpar = 0;
             for (int t = 0; ok && t < nt; ++t) {
                 const int s = t & 1;
-                ok = mbar_wait(v_full + s, (t >> 1) & 1, abort_flag) && mbar_wait(p_full + s, (t >> 1) & 1, abort_flag);
+                ok = mbar_wait(v_full + vs, vpar, abort_flag) && mbar_wait(p_full + s, (t >> 1) & 1, abort_flag);
                 if (!(ok = __all_sync(0xffffffffu, ok))) break;
                 tc_fence_after();
-                const uint64_t dv = desc_off(dv0, s * L::V_BYTES);
+                const uint64_t dv = desc_off(dv0, vs * L::V_BYTES);
                 if (elect_one()) {
 #pragma unroll
                     for (int ks = 0; ks < BN / 16; ++ks) {
-                        // P: two keys a column; V: 16 keys = two 8-row groups, the next 64 d-columns BN * 128 bytes further on
-                        umma_ts(tmem_O, tmem_base + s * BN + ks * 8, desc_off(dv, ks * 2048), IDESC_PV, (t > 0) || (ks > 0));
+                        // P: two keys a column, or K-major, 64 keys per 128-byte row; V: 16 keys = two 8-row groups, the next 64 d-columns BN * 128 bytes further on
+                        if constexpr (L::P_SMEM) umma_ss(tmem_O, desc_off(dp0, s * L::P_BYTES + ks * 32), desc_off(dv, ks * 2048), IDESC_PV, (t > 0) || (ks > 0));
+                        else umma_ts(tmem_O, tmem_base + s * BN + ks * 8, desc_off(dv, ks * 2048), IDESC_PV, (t > 0) || (ks > 0));
                     }
                     umma_commit(pv_done + s);
+                    if (t + L::VST < nt) umma_commit(v_empty + vs);
                     if (t + 1 == nt) umma_commit(o_full);
                 }
                 __syncwarp();
+                if (++vs == L::VST) { vs = 0; vpar ^= 1; }
             }
         }
     }
@@ -358,6 +376,11 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                 if (!(ok = __all_sync(0xffffffffu, mbar_wait(y_full + ys, ypar, abort_flag)))) break;
                 uint8_t* yb = sY + ys * L::Y_BYTES;
                 tmem_wait_ld();
+                if constexpr (L::P_SMEM) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(s_free + s);
+                }
 #pragma unroll
                 for (int c = 0; c < BN / 8; ++c) {
                     const uint4 y = *reinterpret_cast<const uint4*>(yb + sw128_offset(row, c));
@@ -423,8 +446,8 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                 m_new = fmaxf(m_new, m_t);
                 *m_row = m_new;
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(m_set + wg * 4 + q);
+            // P(t - 2) has been multiplied: its place is free, and p_full, whose phases the P.V warp tells apart by parity alone, cannot run ahead
+            if (L::P_SMEM && t >= 2 && !(ok = __all_sync(0xffffffffu, mbar_wait(pv_done + s, ((t - 2) >> 1) & 1, abort_flag)))) break;
             const float mine = fast_exp2(m_ref - m_new);   // this warpgroup's sum so far: 1 unless the reference has moved since
             m_ref = m_new;
             if (t > 0 && rescale) {
@@ -445,7 +468,7 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                 }
             }
             // The fp32 arithmetic around the exponentials runs two values per instruction (packed fp32 pairs; the scores of a thread sit in
-            // consecutive registers).  P goes over the scores it came from.
+            // consecutive registers).
             float2 sum2 = make_float2(0.f, 0.f);
             const float2 neg_m2 = make_float2(-m_ref, -m_ref), scale2 = make_float2(scale_log2, scale_log2);
             const float2* sf2 = reinterpret_cast<const float2*>(sf);
@@ -459,11 +482,20 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
                     sum2 = __fadd2_rn(sum2, e);
                     pk[j] = pack_bf16(e.x, e.y);
                 }
-                tmem_st16(tmem_base + s * BN + lane_sel + c * 16, pk);
+                if constexpr (L::P_SMEM) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        *reinterpret_cast<uint4*>(sP + s * L::P_BYTES + sw128_offset(row, c * 4 + j)) = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+                } else {
+                    tmem_st16(tmem_base + s * BN + lane_sel + c * 16, pk);
+                }
             }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(m_set + wg * 4 + q);
             l_sum = l_sum * mine + (sum2.x + sum2.y);
-            tmem_wait_st();
+            tmem_wait_st();   // (P, or a rescaled accumulator)
             tc_fence_before();
+            if constexpr (L::P_SMEM) fence_async_smem();
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(p_full + s);
@@ -555,16 +587,17 @@ bool tma_ok(const lisa_tensor& t) {
     return t.dtype == LISA_BF16 && (reinterpret_cast<uintptr_t>(t.ptr) & 15u) == 0 && t.stride_b % 8 == 0 && t.stride_n % 8 == 0 &&
            t.stride_h % 8 == 0 && t.stride_b > 0 && t.stride_n > 0 && t.stride_h > 0;
 }
+// boxes of 64 columns, or of all 32
 bool map_bnhx(CUtensorMap* m, const lisa_tensor& t, int B, int N, int H, int X, int rows) {
     const uint64_t dims[4] = {(uint64_t)X, (uint64_t)H, (uint64_t)N, (uint64_t)B};
     const uint64_t str[3] = {(uint64_t)t.stride_h * 2, (uint64_t)t.stride_n * 2, (uint64_t)t.stride_b * 2};
-    const uint32_t box[4] = {64, 1, (uint32_t)rows, 1};
-    return make_tensor_map_bf16(m, t.ptr, 4, dims, str, box);
+    const uint32_t box[4] = {(uint32_t)std::min(X, 64), 1, (uint32_t)rows, 1};
+    return make_tensor_map_bf16(m, t.ptr, 4, dims, str, box, false, X == 32 ? 64 : 128);
 }
 }  // namespace
 
 bool tc_flash_supported(const TcFlashArgs& a) {
-    if (!((a.kd == 128 || a.kd == 64) && tma_ok(a.qa) && tma_ok(a.ka) && a.Hq % a.Hkv == 0)) return false;
+    if (!((a.kd == 128 || a.kd == 32) && tma_ok(a.qa) && tma_ok(a.ka) && a.Hq % a.Hkv == 0)) return false;
     return a.emit_plane ? true : (tma_ok(a.v) && tma_ok(a.o));
 }
 
@@ -620,11 +653,10 @@ cudaError_t launch_tc_flash(const TcFlashArgs& a, cudaStream_t stream) {
     } while (0)
     if (a.emit_plane) {
         if (a.kd == 128) LISA_LAUNCH_FLASH(128, MODE_EMIT);
-        else LISA_LAUNCH_FLASH(64, MODE_EMIT);
+        else LISA_LAUNCH_FLASH(32, MODE_EMIT);
     } else if (a.kd == 128 && !a.plane) LISA_LAUNCH_FLASH(128, MODE_ATTN);
-    else if (a.kd == 64 && a.plane && a.carry) LISA_LAUNCH_FLASH(64, MODE_ATTN_CARRY);
-    else if (a.kd == 64 && a.plane) LISA_LAUNCH_FLASH(64, MODE_ATTN_PLANE);
-    else if (a.kd == 64 && !a.plane) LISA_LAUNCH_FLASH(64, MODE_ATTN);
+    else if (a.kd == 32 && a.plane && a.carry) LISA_LAUNCH_FLASH(32, MODE_ATTN_CARRY);
+    else if (a.kd == 32 && a.plane) LISA_LAUNCH_FLASH(32, MODE_ATTN_PLANE);
     else return cudaErrorInvalidValue;  // 128-wide scores plus a plane do not fit shared memory
 #undef LISA_LAUNCH_FLASH
     count_launches(1);

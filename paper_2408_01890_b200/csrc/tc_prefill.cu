@@ -18,7 +18,7 @@ namespace lisa {
 namespace {
 
 constexpr int kTile = 128;
-constexpr int kPadRank = 64;
+constexpr int kPadRank = 32;   // low ranks are at most this (tc_shared_prefill_supported)
 constexpr int kMaxPackLinks = kMaxChain;   // links whose Q', K' one call packs
 // A wave takes query tiles until its head-partitioned kernels have at least kWaveCtasPerSm CTAs per SM (with
 // fewer, the grids do not fill the GPU and launch and tail costs dominate) and then further tiles while the causal
@@ -35,7 +35,7 @@ struct PackJobs {
 };
 
 // A CTA packs kPackPos positions of one sequence: the rows of H x r values are read as they lie (one warp per position) into shared
-// memory and leave as whole 128-byte rows.  Bound by HBM where it runs alone; beside a flash kernel, by the shared memory that leaves free.
+// memory and leave as whole 64-byte rows.  Bound by HBM where it runs alone; beside a flash kernel, by the shared memory that leaves free.
 constexpr int kPackPos = 8, kPackThreads = kPackPos * 32;
 // behind: launched in a programmatic chain right behind a kernel of the same call that releases its successors after its own wait, and
 // writes nothing that is read here.  What came before the call is then complete when this kernel starts, so it runs beside that kernel
@@ -197,7 +197,7 @@ bool tc_shared_prefill_supported(const lisa_shared_prefill_args& a) {
         !tc_align_link_supported(a.Hq, a.links, a.chain_len))
         return false;
     for (int k = 0; k < a.chain_len; ++k)
-        if (a.links[k].qp.dtype != LISA_BF16 || a.links[k].kp.dtype != LISA_BF16 || a.links[k].r > 32) return false;
+        if (a.links[k].qp.dtype != LISA_BF16 || a.links[k].kp.dtype != LISA_BF16 || a.links[k].r > kPadRank) return false;
     TcFlashArgs f{a.B, a.N, a.Hq, a.Hkv, 128, a.q0, a.k0, a.v, a.o, 1.f, nullptr, 0, 0, 0, 1};
     return tc_flash_supported(f);
 }

@@ -524,3 +524,10 @@ def test_a_programmatic_chain_equals_its_kernels_one_by_one(Hq, integrate, N):
         lb.lisa_prefill_phase_timing(False)
     for _ in range(3):
         assert all(torch.equal(x, y) for x, y in zip(run(all_in), ref))
+
+
+@pytest.mark.parametrize("r", [1, 15, 16, 17, 31, 32])
+def test_low_ranks_at_the_edges_of_their_padding(r):
+    """Q' and K' are packed into rows of 32, of which whole groups of 16 are multiplied: with an emitted difference (chain of two) and without."""
+    run_tc_shared(1, 200, 8, 1, "relu", seed=r, r=r)
+    run_tc_shared(2, 130, 32, 2, "silu", seed=r, r=r)
