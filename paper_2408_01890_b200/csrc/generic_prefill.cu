@@ -7,9 +7,9 @@
 // dtype and shape in the supported range runs here; the tensor-core kernels cover the fast cases.
 //
 // A small prompt is bound by the latency of one CTA, so every phase spreads over all threads with its loads in flight together: the dot
-// products over (head, key, part of the row), the FFN over keys (weights in shared memory; 2, 4 or 8 heads in registers), the softmax over heads, the
-// product with V over (head, column) and, where these are few, ranges of keys.  4 heads of 32, N 128: 31 us with a thread per key
-// doing all of it, 10 now.
+// products over (head, key, part of the row), the FFN over keys and hidden units (weights in shared memory; 2, 4 or 8 heads in registers), the softmax over heads, the
+// product with V over (head, column) and, where these are few, ranges of keys.  4 heads of 32, N 128, the standard layer and a shared one back to
+// back: 22.4 us with four loads of a thread in flight, a thread to a position's FFN and V's loads behind the softmax, 17.5 now.
 #include "common.cuh"
 
 namespace lisa {
@@ -59,24 +59,28 @@ __device__ __forceinline__ float ld(const TView& t, int64_t i) {
 }
 
 // out[h][jj] = scale * (q[h] . row of key jj in KV head h / G) for the chunk's nk keys: neighbouring lanes take neighbouring V values of a
-// row (V values are 16 bytes, or one where rows do not start on 16 bytes), four rows of a lane are in flight, shuffles add up a row.
-template <int DT, int V>
+// row (V values are 16 bytes, or one where rows do not start on 16 bytes), eight rows of a lane are in flight, shuffles add up a row.  Rows are
+// numbered key by key, so that a chunk of few keys takes few rounds (with a head count known at run time: four, head by head, which spares the
+// divisions: 6 heads of 64, 300 positions 115 us, 162 the other way).
+template <int DT, int V, int HQ>
 __device__ __forceinline__ void dots(float* out, const float* q, int q_ld, const TView& t, int64_t at, int Hq, int G, int nk, int n, float scale) {
-    constexpr int U = 4;
+    constexpr int U = HQ ? 8 : 4;
     const int lanes = (n + V - 1) / V;
     const int lpr = lanes <= 1 ? 1 : lanes >= 32 ? 32 : 1 << (32 - __clz(lanes - 1));   // lanes per row
-    const int sub = threadIdx.x & (lpr - 1), grp = threadIdx.x / lpr, groups = blockDim.x / lpr, total = Hq * kChunk;
+    const int sub = threadIdx.x & (lpr - 1), grp = threadIdx.x / lpr, groups = blockDim.x / lpr, total = Hq * (HQ ? nk : kChunk);
     for (int r0 = 0; r0 < total; r0 += U * groups) {
         float part[U];
         int64_t row[U];
         const float* qh[U];
         bool ok[U];
+        int o[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int rr = r0 + u * groups + grp, h = rr / kChunk, jj = rr % kChunk;
+            const int rr = r0 + u * groups + grp, jj = HQ ? rr / Hq : rr % kChunk, h = HQ ? rr - jj * Hq : rr / kChunk;
             ok[u] = rr < total && jj < nk;
             row[u] = at + jj * t.sn + (G == 1 ? h : h / G) * t.sh;
             qh[u] = q + h * q_ld;
+            o[u] = h * kChunk + jj;
             part[u] = 0.f;
         }
         for (int x = sub * V; x < n; x += lpr * V) {   // (once, unless rows of more than 32 values are read one by one)
@@ -120,14 +124,14 @@ __device__ __forceinline__ void dots(float* out, const float* q, int q_ld, const
         if (sub == 0)
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (ok[u]) out[r0 + u * groups + grp] = part[u] * scale;
+                if (ok[u]) out[o[u]] = part[u] * scale;
     }
 }
-template <int DT>
+template <int DT, int HQ>
 __device__ __forceinline__ void dots_any(float* out, const float* q, int q_ld, const TView& t, int64_t at, int Hq, int G, int nk, int n, float scale, int vec) {
-    if (DT == 0 && vec && n % 4 == 0) dots<DT, DT == 0 ? 4 : 1>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
-    else if (DT == 1 && vec && n % 8 == 0) dots<DT, DT == 1 ? 8 : 1>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
-    else dots<DT, 1>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
+    if (DT == 0 && vec && n % 4 == 0) dots<DT, DT == 0 ? 4 : 1, HQ>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
+    else if (DT == 1 && vec && n % 8 == 0) dots<DT, DT == 1 ? 8 : 1, HQ>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
+    else dots<DT, 1, HQ>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
 }
 
 // A link's FFN weights: fp32 in shared memory (SM; w1, b1, w2, b2 one after the other), or where the model keeps them.
@@ -143,13 +147,15 @@ struct Weights {
 };
 
 // Sec. 5.1 at one position: a <- Integrate(Align(a), dl); a and dl are columns of shared memory, one head every kChunk floats.  HQ > 0: that
-// many heads, in registers.
+// many heads, in registers, and the hidden units over `parts` neighbouring lanes (all lanes of the warp come here; lanes without a
+// position of their own write nothing).
 template <int HQ, bool SM>
-__device__ __forceinline__ void align_integrate(float* a, const float* dl, int n_heads, const Weights<SM>& w) {
+__device__ __forceinline__ void align_integrate(float* a, const float* dl, int n_heads, const Weights<SM>& w, int part, int parts, bool write) {
     const int Hq = HQ ? HQ : n_heads;
     const LinkDev& lk = w.l;
     if (lk.integrate == LISA_INTEGRATE_PLUS) {
-        for (int g = 0; g < Hq; ++g) a[g * kChunk] += dl[g * kChunk];
+        if (write)
+            for (int g = 0; g < Hq; ++g) a[g * kChunk] += dl[g * kChunk];
         return;
     }
     const int m = lk.m;
@@ -160,11 +166,11 @@ __device__ __forceinline__ void align_integrate(float* a, const float* dl, int n
 #pragma unroll(HQ ? HQ : 1)
     for (int h = 0; h < Hq; ++h) {
         x[h] = a[h * kChunk];
-        y[h] = two ? w.b2(h) : 0.f;
+        y[h] = two && part == 0 ? w.b2(h) : 0.f;
     }
     auto units = [&](auto activate) {
 #pragma unroll(HQ ? 4 : 1)
-        for (int u = 0; u < m; ++u) {
+        for (int u = part; u < m; u += parts) {
             float s = w.b1(u);
 #pragma unroll(HQ ? HQ : 4)
             for (int h = 0; h < Hq; ++h) s = fmaf(x[h], w.w1(h * m + u), s);
@@ -186,6 +192,12 @@ __device__ __forceinline__ void align_integrate(float* a, const float* dl, int n
     const float floor = act == LISA_ACT_RELU ? 0.f : -INFINITY;
     if (act == LISA_ACT_SILU) units([](float s) { return act_apply(s, LISA_ACT_SILU); });
     else units([floor](float s) { return fmaxf(s, floor); });
+    if constexpr (HQ > 0) {
+        for (int off = parts >> 1; off > 0; off >>= 1)
+#pragma unroll
+            for (int g = 0; g < HQ; ++g) y[g] += __shfl_xor_sync(0xffffffffu, y[g], off);
+    }
+    if (!write) return;
 #pragma unroll(HQ ? HQ : 1)
     for (int g = 0; g < Hq; ++g) a[g * kChunk] = lk.integrate == LISA_INTEGRATE_ADD ? y[g] + dl[g * kChunk] : y[g];
 }
@@ -243,15 +255,28 @@ __global__ void __launch_bounds__(kMaxThreads) generic_prefill_kernel(const __gr
     const int cols = Hq * d, splits = cols < kThreads ? min(kThreads / cols, max(1, Hq * kChunk / cols)) : 1;
     for (int j0 = 0; j0 <= i; j0 += kChunk) {
         const int nk = min(kChunk, i + 1 - j0);
-        dots_any<DT>(s_s, q0_s, d, p.k0, b * p.k0.sb + (int64_t)j0 * p.k0.sn, Hq, G, nk, d, inv_sqrt_d, p.vec_k0);
+        dots_any<DT, HQ>(s_s, q0_s, d, p.k0, b * p.k0.sb + (int64_t)j0 * p.k0.sn, Hq, G, nk, d, inv_sqrt_d, p.vec_k0);
+        // where a thread has one column and a short range of keys, its values of V come now, under the phases before the product
+        constexpr int VA = 32;
+        const int v_part = tid / cols, v_col = tid - v_part * cols, v0 = nk * v_part / splits, v1 = nk * (v_part + 1) / splits;
+        const bool ahead = HQ > 0 && splits > 1 && (nk + splits - 1) / splits <= VA;
+        float va[VA];
+        if (ahead && v_part < splits) {
+            const int h = v_col / d;
+            const int64_t vb = b * p.v.sb + (int64_t)(j0 + v0) * p.v.sn + (h / G) * p.v.sh + (v_col - h * d);
+#pragma unroll
+            for (int q = 0; q < VA; ++q) va[q] = v0 + q < v1 ? ld<DT>(p.v, vb + (int64_t)q * p.v.sn) : 0.f;
+        }
         for (int k = 0; k < p.c; ++k) {
             const LinkDev& lk = p.links[k];
-            dots_any<DT>(d_s, qp_s + k * Hq * kMaxRank, kMaxRank, lk.kp, b * lk.kp.sb + (int64_t)j0 * lk.kp.sn, Hq, G, nk, lk.r, rsqrtf((float)lk.r), p.vec_kp[k]);
+            dots_any<DT, HQ>(d_s, qp_s + k * Hq * kMaxRank, kMaxRank, lk.kp, b * lk.kp.sb + (int64_t)j0 * lk.kp.sn, Hq, G, nk, lk.r, rsqrtf((float)lk.r), p.vec_kp[k]);
             __syncthreads();
             const int h_in = (lk.integrate == LISA_INTEGRATE_CONCAT ? 2 : 1) * Hq;
-            if (tid < nk) {
-                if (p.w_off[k] >= 0) align_integrate<HQ>(s_s + tid, d_s + tid, Hq, Weights<true>(smem + p.w_off[k], lk, h_in, Hq));
-                else align_integrate<HQ>(s_s + tid, d_s + tid, Hq, Weights<false>(nullptr, lk, h_in, Hq));
+            if (HQ > 0 || tid < nk) {
+                const int parts = HQ > 0 ? kThreads / kChunk : 1, pos = tid / parts, part = tid - pos * parts;
+                const bool write = part == 0 && pos < nk;
+                if (p.w_off[k] >= 0) align_integrate<HQ>(s_s + pos, d_s + pos, Hq, Weights<true>(smem + p.w_off[k], lk, h_in, Hq), part, parts, write);
+                else align_integrate<HQ>(s_s + pos, d_s + pos, Hq, Weights<false>(nullptr, lk, h_in, Hq), part, parts, write);
             }
             __syncthreads();
         }
@@ -286,7 +311,16 @@ __global__ void __launch_bounds__(kMaxThreads) generic_prefill_kernel(const __gr
             }
         }
         __syncthreads();
-        for (int e = tid; e < cols * splits; e += kThreads) {
+        if (ahead) {
+            if (v_part < splits) {
+                const float* e_s = s_s + v_col / d * kChunk + v0;
+                float acc = 0.f;
+#pragma unroll
+                for (int q = 0; q < VA; ++q)
+                    if (v0 + q < v1) acc = fmaf(e_s[q], va[q], acc);
+                d_s[tid] = acc;
+            }
+        } else for (int e = tid; e < cols * splits; e += kThreads) {
             const int part = e / cols, col = e % cols, h = col / d, x = col % d;
             const int k0 = nk * part / splits, k1 = nk * (part + 1) / splits;
             const int64_t vb = b * p.v.sb + (int64_t)j0 * p.v.sn + (h / G) * p.v.sh + x;

@@ -106,3 +106,14 @@ def test_host_variant_matches_device_variant():
     arena = torch.empty(lb.lisa_host_arena_bytes(q0, k0, hl, v, out), dtype=torch.uint8, device="cuda")
     lb.lisa_attn_shared_prefill_host(q0, k0, hl, v, out, arena)
     assert torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,r,m,N", [(2, 1, 32, 5, 5, 1), (2, 2, 128, 8, 7, 37), (4, 2, 32, 8, 16, 130), (4, 4, 64, 12, 3, 300), (8, 8, 32, 7, 33, 17),
+                                             (8, 1, 64, 4, 32, 129)])
+@pytest.mark.parametrize("integrate,layers", [(lb.INTEGRATE_ADD, 2), (lb.INTEGRATE_CONCAT, 2), (lb.INTEGRATE_ADD, 1), (lb.INTEGRATE_PLUS, 2)])
+def test_fp32_head_counts_in_registers(Hq, Hkv, d, r, m, N, integrate, layers):
+    """Two, four and eight heads: hidden units over two and four lanes of a position (fewer units than lanes, odd counts), rows numbered key by key,
+    V ahead of the product (one column a thread, up to 32 keys) and not."""
+    w = synth.Workload("regs", "f32", 1, N, Hq, Hkv, d, r, m, "silu", 2)
+    run_prefill_case(w, seed=N, integrate=integrate, ffn_layers=layers, bias=True, chain=2)
+    run_prefill_case(w, seed=N, chain=0)
