@@ -504,9 +504,21 @@ __global__ void __launch_bounds__(kDecodeThreads, CTAS) shared_decode_fast_kerne
     int b, chunk, L;
     if (!decode_item<CH, DENSE>(p, b, chunk, L)) return;
     const int j0 = chunk * CH, nrows = min(CH, L - j0);
-    for (int e = tid; e < HG * p.r; e += kDecodeThreads) {
-        const int h = e / p.r, x = e - h * p.r;
-        qp_s[h * kMaxRank + x] = ld_elem(p.qp.ptr, b * p.qp.sb + (h0 + h) * p.qp.sh + x, p.qp.dtype);
+    {   // at most HG * kMaxRank values: all loads in flight together
+        constexpr int NQ = HG * kMaxRank / kDecodeThreads;
+        auto fetch = [&](const auto* q) {
+            q += b * p.qp.sb + h0 * p.qp.sh;
+            float v[NQ];
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) {
+                const int e = tid + i * kDecodeThreads, h = e / kMaxRank, x = e % kMaxRank;
+                v[i] = x < p.r ? (float)q[h * p.qp.sh + x] : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < NQ; ++i) qp_s[tid + i * kDecodeThreads] = v[i];
+        };
+        if (p.qp.dtype == LISA_BF16) fetch(reinterpret_cast<const __nv_bfloat16*>(p.qp.ptr));
+        else fetch(reinterpret_cast<const float*>(p.qp.ptr));
     }
     __syncthreads();
     {
