@@ -480,6 +480,16 @@ bool deal_chunks(const DecodeParams& p, int64_t ctas) {
     return p.seq_lens && p.B > 1 && p.B <= kDenseMaxB && ctas > 2 * sms && ctas <= 3 * sms;
 }
 
+// KV heads whose V the CTAs of a grid that is resident at once ask into L2 behind their K or K' (k_row bytes a position and head); -1: the grid
+// is not resident.  All of a chunk at once (paper's default model, 8 x 1111: 146 MB for the anchor layer, 85 for a shared one) stands in the
+// queue for HBM before the score rows and K', and the anchor's is more than L2 holds; V is needed last: anchor and two shared layers
+// 108.6 -> 102.8 us, the same with 24, 32, 36 and 48 MB, 107.5 with 110.  Small batches (1 x 333, 7B-shaped: 7 MB a layer) ask for all.
+constexpr int64_t kPrefetchBytes = (int64_t)48 << 20;
+int plan_prefetch(const DecodeParams& p, int64_t ctas, int n_kv, int k_row) {
+    if (ctas > 2 * (int64_t)sm_count()) return -1;
+    return (int)std::max<int64_t>(0, (kPrefetchBytes / (ctas * p.chunk) - (int64_t)n_kv * k_row) / 256);
+}
+
 template <int HQ, int HG, int CH, int M_C, int ENG>
 cudaError_t launch_shared_fast(DecodeParams& p, cudaStream_t s) {
     const int64_t ctas = (int64_t)p.n_chunks * (HQ / HG) * p.B;
@@ -491,7 +501,7 @@ cudaError_t launch_shared_fast(DecodeParams& p, cudaStream_t s) {
         if (three_per_sm(ctas) && (!p.dense || three_per_sm((ctas * 9 + 15) / 16)))
             kernel = p.dense ? shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3, true> : shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3, false>;
     const size_t smem = shared_fast_layout(HQ, HG, CH, ENG, p.m, HQ / p.Hkv).total;
-    p.prefetch = ctas <= 2 * (int64_t)sm_count();   // a grid that is resident at once
+    p.prefetch = plan_prefetch(p, ctas, HG / (HQ / p.Hkv), p.r * 2);
     cudaError_t e = allow_smem(kernel, smem);
     return e != cudaSuccess ? e : launch_chained(kernel, dim3(p.n_chunks, HQ / HG, p.B), dim3(kDecodeThreads), smem, s, p);
 }
@@ -616,7 +626,7 @@ cudaError_t launch_anchor_decode(const lisa_anchor_args& a, void* ws, cudaStream
         p.heads = kv * G;
         set_chunk(p, chunk_length(p.B, p.Hq, a.L, p.Hkv / kv), ws);
         const int64_t ctas = (int64_t)p.n_chunks * p.B * (p.Hkv / kv);
-        p.prefetch = ctas <= 2 * want;   // a grid that is resident at once
+        p.prefetch = plan_prefetch(p, ctas, kv, 256);
         p.dense = deal_chunks(p, ctas);
         const size_t smem = anchor_fast_smem(p.heads, p.chunk, G);
         auto kernel = p.dense ? (p.chunk == 128 ? anchor_decode_fast_kernel<128, true> : p.chunk == 64 ? anchor_decode_fast_kernel<64, true> : anchor_decode_fast_kernel<32, true>)

@@ -11,7 +11,7 @@ struct DecodeParams {
     int B, Hq, Hkv, d, L_cap, L_uniform, n_chunks;
     int chunk;              // cached positions per chunk: 128, or 64 or 32 in the kernels for small batches
     int heads;              // query heads per CTA where the heads are divided over CTAs
-    int prefetch;           // a CTA asks its part of the caches into L2 when it starts
+    int prefetch;           // a CTA asks its K or K' and V of this many of its KV heads into L2 when it starts; -1: nothing
     int dense;              // ragged batches: the chunks that hold positions are dealt to the CTAs in order (see decode_item)
     const int32_t* seq_lens;
     // shared layer

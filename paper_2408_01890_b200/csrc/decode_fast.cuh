@@ -261,7 +261,7 @@ __device__ __forceinline__ void pv_chunk(const DecodeParams& p, const float* s_s
 // an earlier kernel has set it), and L2 is the point of coherence, so a new token's row that is still being written is read right later.
 __device__ __forceinline__ void prefetch_chunk(const DecodeParams& p, int kv0, int n_kv, int ch, bool standard) {
     const int b = blockIdx.z, j0 = blockIdx.x * ch, hint = min(decode_length(p, b), p.L_cap) - j0;
-    if (hint <= 0 || !p.prefetch) return;
+    if (hint <= 0 || p.prefetch < 0) return;
     const int nrows = min(ch, hint), tid = threadIdx.x;
     const size_t row0 = ((size_t)b * p.Hkv + kv0) * p.L_cap + j0;
     auto bulk = [](const void* q, uint32_t bytes) { asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(q), "r"(bytes) : "memory"); };
@@ -273,7 +273,7 @@ __device__ __forceinline__ void prefetch_chunk(const DecodeParams& p, int kv0, i
         for (int e = tid; e < n_kv * p.r * lines; e += kDecodeThreads)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (size_t)(e / lines) * p.L_cap + e % lines * 64) : "memory");
     }
-    if (tid < n_kv) bulk(reinterpret_cast<const uint4*>(p.vcache) + (row0 + (size_t)tid * p.L_cap) * 16, nrows * 256);
+    if (tid < min(n_kv, p.prefetch)) bulk(reinterpret_cast<const uint4*>(p.vcache) + (row0 + (size_t)tid * p.L_cap) * 16, nrows * 256);
 }
 
 // ---------------------------------------------------------------------------------------------
