@@ -374,10 +374,13 @@ __global__ void __launch_bounds__(kThreads, 2) anchor_decode_chunk_kernel(const 
 
 // Merge the per-chunk (m, l, o) partials of one (b, h): o = sum_c e^{m_c - M} o_c / sum_c e^{m_c - M} l_c.  Bound by latency: every
 // warp forms M and the denominator by itself (the chunks' m and l come from L2), its lanes take four columns each, the warps
-// different chunks, and one exchange through shared memory adds their sums; a thread's first eight partial outputs come with the maxima, not
+// different chunks, and one exchange through shared memory adds their sums; a thread's first U partial outputs come with the maxima, not
 // behind them (with the chunk kernels' q' loads in flight together: one layer of the paper's default model, 8 x 1111, 38.9 -> 35.2 us;
 // 7B-shaped, 1 x 333, 12.0 -> 11.2; 13B-shaped, 64 x 4096, 518 -> 515).
+// U outputs, as many as a thread has where the contexts are short: with eight a CTA takes twice the registers, and the grid of a large batch
+// more than one wave (38 sequences of 180 positions, anchor and three layers: 101 us with one or two, 107 with eight).
 constexpr int kMergeThreads = 128;
+template <int U>
 __global__ void __launch_bounds__(kMergeThreads) decode_merge_kernel(const __grid_constant__ DecodeParams p) {
     __shared__ float4 s_o[kMergeThreads];
     const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
@@ -386,7 +389,6 @@ __global__ void __launch_bounds__(kMergeThreads) decode_merge_kernel(const __gri
     const int nc = (decode_length(p, b) + p.chunk - 1) / p.chunk;
     const size_t base = (size_t)b * p.n_chunks * p.Hq + h;
     const int lpr = p.d / 4, x = tid % lpr, c0 = tid / lpr, cstep = kMergeThreads / lpr;   // lanes per partial output, this thread's chunks
-    constexpr int U = 8;
     const float4* po = reinterpret_cast<const float4*>(p.ws_o + base * p.d) + x;
     const size_t step = (size_t)p.Hq * lpr;
     float4 first[U];
@@ -474,10 +476,11 @@ bool three_per_sm(int64_t ctas) {
 // one CTA with work or two whichever way; there the count costs more than it gives (paper's default layer, 16 sequences of up to 1500: 70.5 us
 // dealt, 66.8 not; 16 of up to 2900 of the 8B shape: an anchor and three layers 148 us dealt, 168 not; 16 of up to 3000, 40 heads: 80 and 92).
 // A much larger grid evens itself out (100 of up to 3000, 2400 CTAs: 131 us dealt, 125 not; a uniform 7B-shaped batch whose lengths are given,
-// 544 CTAs: 0.3 % slower dealt).
+// 544 CTAs: 0.3 % slower dealt).  With fewer than four chunks to the longest sequence nearly every CTA has positions (63 of up to 99, 40 heads,
+// an anchor and three layers: 140 us dealt, 118 not).
 bool deal_chunks(const DecodeParams& p, int64_t ctas) {
     const int64_t sms = sm_count();
-    return p.seq_lens && p.B > 1 && p.B <= kDenseMaxB && ctas > 2 * sms && ctas <= 3 * sms;
+    return p.seq_lens && p.B > 1 && p.B <= kDenseMaxB && p.n_chunks >= 4 && ctas > 2 * sms && ctas <= 3 * sms;
 }
 
 // KV heads whose V the CTAs of a grid that is resident at once ask into L2 behind their K or K' (k_row bytes a position and head); -1: the grid
@@ -552,7 +555,9 @@ cudaError_t shared_fast(DecodeParams& p, void* ws, cudaStream_t s, bool* taken) 
 }
 
 cudaError_t launch_merge(const DecodeParams& p, cudaStream_t s) {
-    const cudaError_t e = launch_chained(decode_merge_kernel, dim3(p.Hq, p.B), dim3(kMergeThreads), 0, s, p);
+    const int each = kMergeThreads * 4 / p.d;   // chunks that the CTA's threads take side by side
+    auto kernel = p.n_chunks <= each ? decode_merge_kernel<1> : p.n_chunks <= 2 * each ? decode_merge_kernel<2> : decode_merge_kernel<8>;
+    const cudaError_t e = launch_chained(kernel, dim3(p.Hq, p.B), dim3(kMergeThreads), 0, s, p);
     count_launches(2);
     return e;
 }
