@@ -499,7 +499,8 @@ cudaError_t launch_shared_fast(DecodeParams& p, cudaStream_t s) {
     p.dense = deal_chunks(p, ctas);
     auto kernel = p.dense ? shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2, true> : shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2, false>;
     // (a ragged batch, whose lengths the host does not know, only where the build suits it with all of its chunks and with nine sixteenths of
-    // them, which lengths spread over [L / 8, L] leave: 16 sequences of up to 2900 positions 168 -> 148 us with the dealt chunks)
+    // them, which lengths spread over [L / 8, L] leave: 16 sequences of up to 2900 positions 168 -> 148 us with the dealt chunks; given lengths
+    // that are all alike pay for it, 13 x 3079 148 -> 164)
     if constexpr (ENG == kEngTf32 && CH == 128)
         if (three_per_sm(ctas) && (!p.dense || three_per_sm((ctas * 9 + 15) / 16)))
             kernel = p.dense ? shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3, true> : shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3, false>;
