@@ -14,6 +14,7 @@
 // bf16 caches of head width 128 (32 or 40 heads for a shared layer) run on the kernels of decode_fast.cuh; the kernels here
 // take every other head count, width, type and Integrate mode.
 #include <algorithm>
+#include <climits>
 
 #include "decode_fast.cuh"
 
@@ -472,12 +473,13 @@ bool three_per_sm(int64_t ctas) {
     return 1.3 * (double)((ctas + 3 * sms - 1) / (3 * sms)) < (double)((ctas + 2 * sms - 1) / (2 * sms));
 }
 
-// Ragged batches whose grid is not resident at once have their chunks dealt to the CTAs (decode_item).  A smaller grid leaves an SM at most
-// one CTA with work or two whichever way; there the count costs more than it gives (paper's default layer, 16 sequences of up to 1500: 70.5 us
-// dealt, 66.8 not; 16 of up to 2900 of the 8B shape: an anchor and three layers 148 us dealt, 168 not; 16 of up to 3000, 40 heads: 80 and 92).
-// A much larger grid evens itself out (100 of up to 3000, 2400 CTAs: 131 us dealt, 125 not; a uniform 7B-shaped batch whose lengths are given,
-// 544 CTAs: 0.3 % slower dealt).  With fewer than four chunks to the longest sequence nearly every CTA has positions (63 of up to 99, 40 heads,
-// an anchor and three layers: 140 us dealt, 118 not).
+// Batches with given lengths whose grid is not resident at once have their chunks dealt to the CTAs (decode_item).  A smaller grid leaves an SM
+// at most one CTA with work or two whichever way; there the count costs more than it gives (paper's default layer, 16 sequences of up to 1500:
+// 70.5 us dealt, 66.8 not; 16 of up to 2900 of the 8B shape: an anchor and three layers 148 us dealt, 168 not; 16 of up to 3000, 40 heads: 80 and 92).
+// A larger grid evens itself out (spread over [L / 8, L], 100 sequences of up to 1150, 900 CTAs: 306 us dealt, 289 not; 30 of up to 1900, 450 CTAs:
+// 145 and 144) unless most sequences are short (four fifths at L / 8: 172 and 176, 125 and 133), and loses 1 to 5 % where they are all long.  With
+// fewer than four chunks to the longest sequence nearly every CTA has positions (63 of up to 99, 40 heads, an anchor and three layers: 140 us dealt,
+// 118 not).
 bool deal_chunks(const DecodeParams& p, int64_t ctas) {
     const int64_t sms = sm_count();
     return p.seq_lens && p.B > 1 && p.B <= kDenseMaxB && p.n_chunks >= 4 && ctas > 2 * sms && ctas <= 3 * sms;
@@ -496,18 +498,39 @@ int plan_prefetch(const DecodeParams& p, int64_t ctas, int n_kv, int k_row) {
 template <int HQ, int HG, int CH, int M_C, int ENG>
 cudaError_t launch_shared_fast(DecodeParams& p, cudaStream_t s) {
     const int64_t ctas = (int64_t)p.n_chunks * (HQ / HG) * p.B;
-    p.dense = deal_chunks(p, ctas);
-    auto kernel = p.dense ? shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2, true> : shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2, false>;
-    // (a ragged batch, whose lengths the host does not know, only where the build suits it with all of its chunks and with nine sixteenths of
-    // them, which lengths spread over [L / 8, L] leave: 16 sequences of up to 2900 positions 168 -> 148 us with the dealt chunks; given lengths
-    // that are all alike pay for it, 13 x 3079 148 -> 164)
-    if constexpr (ENG == kEngTf32 && CH == 128)
-        if (three_per_sm(ctas) && (!p.dense || three_per_sm((ctas * 9 + 15) / 16)))
-            kernel = p.dense ? shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3, true> : shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3, false>;
     const size_t smem = shared_fast_layout(HQ, HG, CH, ENG, p.m, HQ / p.Hkv).total;
     p.prefetch = plan_prefetch(p, ctas, HG / (HQ / p.Hkv), p.r * 2);
-    cudaError_t e = allow_smem(kernel, smem);
-    return e != cudaSuccess ? e : launch_chained(kernel, dim3(p.n_chunks, HQ / HG, p.B), dim3(kDecodeThreads), smem, s, p);
+    auto launch = [&](auto kernel, dim3 grid) -> cudaError_t {
+        const cudaError_t e = allow_smem(kernel, smem);
+        return e != cudaSuccess ? e : launch_chained(kernel, grid, dim3(kDecodeThreads), smem, s, p);
+    };
+    const dim3 grid(p.n_chunks, HQ / HG, p.B);
+    if constexpr (CH == 128) {   // (chunks are shorter only where the grid stays below deal_chunks' range, see chunk_length)
+        const bool dealt = deal_chunks(p, ctas);
+        p.least = 0;
+        p.most = INT_MAX;
+        if constexpr (ENG == kEngTf32) {
+            const bool three = three_per_sm(ctas);
+            if (three && !dealt) return launch(shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3, false>, grid);
+            if (three) {
+                // Which build suits a dealt batch depends on how many chunks hold positions, which only the device knows: both are launched, and
+                // the one that the count is not for leaves at once.  Two CTAs per SM as long as that is one wave, three beyond (an anchor and three
+                // shared layers, us, with both | two per SM alone | three alone | grid coordinates, lengths all alike and spread over [L / 8, L]:
+                // 13 x 3079 with 8 KV heads 181 | 204 | 177 | 187 and 140 | 130 | 150 | 163; 12 x 3500 with 40 heads 453 | 520 | 440 | 454 and
+                // 291 | 286 | 350 | 346).
+                const int one_wave = 2 * sm_count() / (HQ / HG);
+                p.least = one_wave + 1;
+                const cudaError_t e = launch(shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 3, true>, grid);
+                if (e != cudaSuccess) return e;
+                count_launches(1);
+                p.least = 0;
+                p.most = one_wave;
+                return launch(shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2, true>, dim3(one_wave, HQ / HG));
+            }
+        }
+        if (dealt) return launch(shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2, true>, grid);
+    }
+    return launch(shared_decode_fast_kernel<HQ, HG, CH, M_C, ENG, 2, false>, grid);
 }
 
 // The fast kernels' share of the shared layers; *taken says whether the call is one of them.
@@ -633,10 +656,14 @@ cudaError_t launch_anchor_decode(const lisa_anchor_args& a, void* ws, cudaStream
         set_chunk(p, chunk_length(p.B, p.Hq, a.L, p.Hkv / kv), ws);
         const int64_t ctas = (int64_t)p.n_chunks * p.B * (p.Hkv / kv);
         p.prefetch = plan_prefetch(p, ctas, kv, 256);
-        p.dense = deal_chunks(p, ctas);
+        const bool dealt = deal_chunks(p, ctas);   // (only with whole chunks, see launch_shared_fast)
+        p.least = 0;
+        p.most = INT_MAX;
         const size_t smem = anchor_fast_smem(p.heads, p.chunk, G);
-        auto kernel = p.dense ? (p.chunk == 128 ? anchor_decode_fast_kernel<128, true> : p.chunk == 64 ? anchor_decode_fast_kernel<64, true> : anchor_decode_fast_kernel<32, true>)
-                              : (p.chunk == 128 ? anchor_decode_fast_kernel<128, false> : p.chunk == 64 ? anchor_decode_fast_kernel<64, false> : anchor_decode_fast_kernel<32, false>);
+        auto kernel = dealt          ? anchor_decode_fast_kernel<128, true>
+                      : p.chunk == 128 ? anchor_decode_fast_kernel<128, false>
+                      : p.chunk == 64  ? anchor_decode_fast_kernel<64, false>
+                                       : anchor_decode_fast_kernel<32, false>;
         if ((e = allow_smem(kernel, smem)) != cudaSuccess) return e;
         e = launch_chained(kernel, dim3(p.n_chunks, p.Hkv / kv, p.B), dim3(kDecodeThreads), smem, s, p);
     } else {

@@ -12,7 +12,7 @@ struct DecodeParams {
     int chunk;              // cached positions per chunk: 128, or 64 or 32 in the kernels for small batches
     int heads;              // query heads per CTA where the heads are divided over CTAs
     int prefetch;           // a CTA asks its K or K' and V of this many of its KV heads into L2 when it starts; -1: nothing
-    int dense;              // ragged batches: the chunks that hold positions are dealt to the CTAs in order (see decode_item)
+    int least, most;        // dealt chunks (see decode_item): the launch does its work only if least..most of them hold positions (see launch_shared_fast)
     const int32_t* seq_lens;
     // shared layer
     const void* prev;       // fp32, or bf16 when row_bf16
@@ -83,7 +83,7 @@ __device__ __forceinline__ int decode_length(const DecodeParams& p, int b) {
 // A CTA's sequence, chunk and context length; false if there is none for it.  Uniform batches: the grid's coordinates.  Ragged ones: the
 // chunks that hold positions, numbered over all sequences, go to the first CTAs of the grid, which the hardware spreads evenly; with
 // the grid's coordinates those without a chunk leave at once and the others pile up (16 sequences of up to 2900 positions: 210 CTAs with
-// work on 112 of 148 SMs, three on 27 of them).  Every warp counts for itself, 32 sequences at a time.
+// work on 112 of 148 SMs, three on 27 of them).  Every warp counts for itself, 32 sequences at a time, all lengths in flight together.
 constexpr int kDenseMaxB = 128;
 template <int CH, bool DENSE>
 __device__ __forceinline__ bool decode_item(const DecodeParams& p, int& b, int& chunk, int& L) {
@@ -93,10 +93,19 @@ __device__ __forceinline__ bool decode_item(const DecodeParams& p, int& b, int& 
         L = decode_length(p, b);
         return chunk * CH < L;
     }
-    const int lane = threadIdx.x & 31;
-    int left = blockIdx.z * gridDim.x + blockIdx.x;                   // chunks before this CTA's, from sequence b0 on
-    for (int b0 = 0; b0 < p.B; b0 += 32) {
-        const int len = b0 + lane < p.B ? max(0, min(p.seq_lens[b0 + lane], p.L_uniform)) : 0, n = (len + CH - 1) / CH;
+    const int lane = threadIdx.x & 31, at = blockIdx.z * gridDim.x + blockIdx.x;
+    int len[kDenseMaxB / 32];
+#pragma unroll
+    for (int q = 0; q < kDenseMaxB / 32; ++q) {
+        const int s = q * 32 + lane;
+        len[q] = s < p.B ? max(0, min(p.seq_lens[s], p.L_uniform)) : 0;
+    }
+    int count = 0;                                                    // chunks of the sequences before 32 q, in the end of all
+    bool found = false;
+#pragma unroll
+    for (int q = 0; q < kDenseMaxB / 32; ++q) {
+        if (q * 32 >= p.B) break;
+        const int n = (len[q] + CH - 1) / CH, left = at - count;
         int upto = n;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -104,16 +113,16 @@ __device__ __forceinline__ bool decode_item(const DecodeParams& p, int& b, int& 
             if (lane >= o) upto += v;
         }
         const uint32_t above = __ballot_sync(0xffffffffu, upto > left);
-        if (above) {
+        if (above && !found) {
             const int src = __ffs(above) - 1;
-            b = __shfl_sync(0xffffffffu, b0 + src, 0);   // (uniform, as the compiler sees it)
+            b = __shfl_sync(0xffffffffu, q * 32 + src, 0);   // (uniform, as the compiler sees it)
             chunk = __shfl_sync(0xffffffffu, left - (upto - n), src);
-            L = __shfl_sync(0xffffffffu, len, src);
-            return true;
+            L = __shfl_sync(0xffffffffu, len[q], src);
+            found = true;
         }
-        left -= __shfl_sync(0xffffffffu, upto, 31);
+        count += __shfl_sync(0xffffffffu, upto, 31);
     }
-    return false;
+    return found && count >= p.least && count <= p.most;
 }
 
 }  // namespace lisa

@@ -70,13 +70,42 @@ def test_shared_decode_shapes(Hq, Hkv, d, r, m, L):
     run_shared_decode(w, 2, L, lens=None, seed=5, L_cap=(L + 7) // 8 * 8 + 64)
 
 
-@pytest.mark.parametrize("Hq,Hkv,m,B,L", [(32, 8, 64, 10, 4200), (40, 40, 80, 12, 3500)])
+def sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+@pytest.mark.parametrize("Hq,Hkv,m,B,L", [(32, 8, 64, 10, 4200), (40, 40, 80, 12, 3500), (32, 32, 64, 50, 385)])
 def test_shared_decode_three_ctas_per_sm(Hq, Hkv, m, B, L):
-    """Grids of 297..444 chunk CTAs (on 148 SMs) take the build of the chunk kernel that runs three CTAs per SM; ragged
-    lengths, against the oracle like every other shape."""
+    """Grids of 297..444 chunk CTAs (on 148 SMs) take the build of the chunk kernel that runs three CTAs per SM: all sequences of the
+    call's length (by grid coordinates; the last chunk is partial), then ragged lengths (dealt), against the oracle like every other shape.
+    The last shape runs with sixteen heads to a CTA."""
     w = synth.Workload("dthree", "bf16", B, L, Hq, Hkv, 128, 21, m, "relu", 1, True)
+    run_shared_decode(w, B, L, lens=None, seed=5)
     lens = [L if b % 3 == 0 else (1 + (b * 977) % L) for b in range(B)]
     run_shared_decode(w, B, L, lens=lens, seed=6)
+
+
+@pytest.mark.parametrize("Hq,Hkv,m,L", [(32, 8, 64, 3201), (40, 40, 80, 2625)])
+@pytest.mark.parametrize("more", ["all", 1, 0])
+def test_the_count_of_a_dealt_batch_picks_its_build(Hq, Hkv, m, L, more):
+    """Given lengths, a grid of two to three CTAs per SM: with one chunk that holds positions more than two per SM, up to all of them, the
+    build for three per SM does the work, with no more than two per SM the other.  Both are launched (and the merge): lengths are on the device."""
+    nc, slots = (L + 127) // 128, 2 * sms()
+    B = slots // nc + 2
+    assert slots < B * nc <= 3 * sms() and B <= 32
+    if more == "all":
+        lens = [L] * B
+    else:   # every sequence keeps a chunk; the first ones give up whole chunks until slots + more are left
+        spare, lens = B * nc - slots - more, []
+        for b in range(B):
+            cut = min(spare, nc - 1)
+            spare -= cut
+            lens.append(L - 128 * cut)
+        assert sum((x + 127) // 128 for x in lens) == slots + more and min(lens) >= 1
+    w = synth.Workload("dpair", "bf16", B, L, Hq, Hkv, 128, 21, m, "relu", 1, True)
+    n0 = lb.lisa_kernel_launches()
+    run_shared_decode(w, B, L, lens=lens, seed=7)
+    assert lb.lisa_kernel_launches() - n0 == 1 + 2 * 3   # the append, two calls
 
 
 @pytest.mark.parametrize("Hq,Hkv,m,act,integrate,B,L", [
@@ -329,10 +358,10 @@ def test_multi_layer_cache_handle_matches_per_layer_caches():
 
 
 @pytest.mark.parametrize("Hq,Hkv,m,integrate,B,L", [(32, 8, 64, lb.INTEGRATE_ADD, 66, 600), (40, 40, 80, lb.INTEGRATE_ADD, 34, 1150),
-                                                     (32, 32, 128, lb.INTEGRATE_CONCAT, 34, 1100)])
+                                                     (32, 32, 128, lb.INTEGRATE_CONCAT, 34, 1100), (32, 8, 72, lb.INTEGRATE_ADD, 34, 1100)])
 def test_ragged_batches_whose_chunks_are_dealt(Hq, Hkv, m, integrate, B, L):
     """Grids of 297..444 CTAs (on 148 SMs) of a ragged batch: the chunks that hold positions are numbered on the device.  Lengths on and around
-    the chunk's edges, sequences past the first 32 and 64; then the standard layer of the same lengths."""
+    the chunk's edges, sequences past the first 32 and 64; the aligners on tf32 and on bf16 terms; then the standard layer of the same lengths."""
     lens = np.random.default_rng(B).integers(1, L + 1, B).astype(np.int32)
     lens[[0, 1, 2, 3, 31, 32, 33, B - 1]] = [1, 127, 128, 129, L, 256, 1, L - 1]
     w = synth.Workload("dealt", "bf16", B, L, Hq, Hkv, 128, 21, m, "relu", 1, True)
