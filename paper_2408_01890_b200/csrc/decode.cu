@@ -378,8 +378,10 @@ __global__ void __launch_bounds__(kThreads, 2) anchor_decode_chunk_kernel(const 
 // different chunks, and one exchange through shared memory adds their sums; a thread's first U partial outputs come with the maxima, not
 // behind them (with the chunk kernels' q' loads in flight together: one layer of the paper's default model, 8 x 1111, 38.9 -> 35.2 us;
 // 7B-shaped, 1 x 333, 12.0 -> 11.2; 13B-shaped, 64 x 4096, 518 -> 515).
-// U outputs, as many as a thread has where the contexts are short: with eight a CTA takes twice the registers, and the grid of a large batch
-// more than one wave (38 sequences of 180 positions, anchor and three layers: 101 us with one or two, 107 with eight).
+// U outputs, as many as a thread has where the contexts are short (38 sequences of 180 positions, anchor and three layers: 101 us with one or two,
+// 107 with eight), and no more than leave the grid resident at once: with eight an SM holds 8 CTAs of 64 registers a thread, with two 10, with
+// one 12 (anchor and three layers of 8 KV heads, us, with eight | one: 100 sequences of up to 1150 positions, four fifths of them short, 182 | 172;
+// all of 1150 422 | 416; 60 of 1250, 40 heads 841 | 838; 40 of 1000, where two are resident and one is not needed, with two | one 187 | 190).
 constexpr int kMergeThreads = 128;
 template <int U>
 __global__ void __launch_bounds__(kMergeThreads) decode_merge_kernel(const __grid_constant__ DecodeParams p) {
@@ -580,7 +582,10 @@ cudaError_t shared_fast(DecodeParams& p, void* ws, cudaStream_t s, bool* taken) 
 
 cudaError_t launch_merge(const DecodeParams& p, cudaStream_t s) {
     const int each = kMergeThreads * 4 / p.d;   // chunks that the CTA's threads take side by side
-    auto kernel = p.n_chunks <= each ? decode_merge_kernel<1> : p.n_chunks <= 2 * each ? decode_merge_kernel<2> : decode_merge_kernel<8>;
+    const int64_t ctas = (int64_t)p.Hq * p.B, sms = sm_count();
+    auto kernel = p.n_chunks <= each || ctas > 10 * sms      ? decode_merge_kernel<1>
+                  : p.n_chunks <= 2 * each || ctas > 8 * sms ? decode_merge_kernel<2>
+                                                             : decode_merge_kernel<8>;
     const cudaError_t e = launch_chained(kernel, dim3(p.Hq, p.B), dim3(kMergeThreads), 0, s, p);
     count_launches(2);
     return e;

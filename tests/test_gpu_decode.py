@@ -85,6 +85,15 @@ def test_shared_decode_three_ctas_per_sm(Hq, Hkv, m, B, L):
     run_shared_decode(w, B, L, lens=lens, seed=6)
 
 
+@pytest.mark.parametrize("per_sm,L", [(8, 1100), (10, 1100), (10, 700)])
+def test_merges_of_grids_around_the_resident_ones(per_sm, L):
+    """The merge holds eight, two or one partial outputs of a thread ahead, by how many of its CTAs an SM holds: batches just beyond eight
+    and ten CTAs per SM, with more chunks than are held ahead and sequences of every number of chunks."""
+    B = per_sm * sms() // 32 + 1
+    w = synth.Workload("dmerge", "bf16", B, L, 32, 8, 128, 21, 64, "relu", 1, True)
+    run_shared_decode(w, B, L, lens=[max(1, L * (b + 1) // B) for b in range(B)], seed=11)
+
+
 @pytest.mark.parametrize("Hq,Hkv,m,L", [(32, 8, 64, 3201), (40, 40, 80, 2625)])
 @pytest.mark.parametrize("more", ["all", 1, 0])
 def test_the_count_of_a_dealt_batch_picks_its_build(Hq, Hkv, m, L, more):
