@@ -35,15 +35,12 @@ struct PackJobs {
 };
 
 // A CTA packs kPackPos positions of one sequence: the rows of H x r values are read as they lie (one warp per position) into shared
-// memory and leave as whole 64-byte rows.  Bound by HBM where it runs alone; beside a flash kernel, by the shared memory that leaves free.
+// memory and leave as whole 64-byte rows.  Bound by HBM.
 constexpr int kPackPos = 8, kPackThreads = kPackPos * 32;
-// behind: launched in a programmatic chain right behind a kernel of the same call that releases its successors after its own wait, and
-// writes nothing that is read here.  What came before the call is then complete when this kernel starts, so it runs beside that kernel
-// and waits for it at its own end only (so that completion stays transitive).
-__global__ void __launch_bounds__(kPackThreads) pack_lowrank_kernel(const __grid_constant__ PackJobs jobs, int B, int N, int behind) {
+__global__ void __launch_bounds__(kPackThreads) pack_lowrank_kernel(const __grid_constant__ PackJobs jobs, int B, int N) {
     __shared__ __align__(16) __nv_bfloat16 rows[kPackPos][kMaxHeads * kMaxRank];
     chain_release();
-    if (!behind) chain_wait();
+    chain_wait();
     const TView src = jobs.src[blockIdx.y];
     const int H = jobs.H[blockIdx.y], r = jobs.r[blockIdx.y], n0 = blockIdx.x * kPackPos;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, vals = H * r;
@@ -76,7 +73,6 @@ __global__ void __launch_bounds__(kPackThreads) pack_lowrank_kernel(const __grid
         }
         __syncthreads();
     }
-    if (behind) chain_wait();
 }
 
 // Optional per-phase timing of the tensor-core prefill (lisa_prefill_phase_timing): CUDA events recorded on the
@@ -357,15 +353,16 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
             for (int qt = 0; qt < n_qt; qt += per) waves[nw++] = Wave{qt, std::min(per, n_qt - qt)};
         }
     }
-    // A call of one wave goes out as a programmatic chain on the caller's stream, set-up of each kernel under the tail of the one before,
-    // and Q', K' are packed beside its first kernel (as chains of CTAs resident at once did, with a fork to a stream for the packing and back
-    // in each call: a prompt of 197 tokens through an anchor and three layers 71.6 -> 62.9 us, host 70 -> 46; one layer of 2048 tokens
-    // 167 -> 162, 2 x 1777 tokens of 40 heads through three layers 737 -> 724).  Otherwise they are packed beside the first emit on a stream of their own (and on the
+    // A call of one wave goes out as a programmatic chain on the caller's stream, set-up of each kernel under the tail of the one before, the
+    // packing of Q', K' among them: a fork to a stream for the packing and back costs as much GPU time and more of the host's (a prompt of 197 tokens
+    // through an anchor and three layers 71.6 us, host 70, against 70.5, host 46; one layer of 2048 tokens about 170 either way).  The packing
+    // waits like every kernel of the chain: without a wait of its own, beside the kernel it follows, 62.4 us, but then what the kernels in front of the
+    // call wrote into Q', K' is not certain to be seen.  Otherwise they are packed beside the first emit on a stream of their own (and on the
     // caller's, before everything, while the per-kernel timing is on).
     const bool chained = nw == 1 && !ho && !g_pt.on;
     SideStream* side = nullptr;
     bool packed = false;
-    auto launch_pack = [&](bool chain, int behind, cudaStream_t ps) -> cudaError_t {
+    auto launch_pack = [&](bool chain, cudaStream_t ps) -> cudaError_t {
         PackJobs jobs{};
         for (int k = 0; k < c; ++k) {
             jobs.src[2 * k] = make_view(a.links[k].qp); jobs.dst[2 * k] = reinterpret_cast<__nv_bfloat16*>(base + l.qp_off[k]);
@@ -376,7 +373,7 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
         packed = true;
         count_launches(1);
         return launch_kernel(chain, pack_lowrank_kernel, dim3((a.N + kPackPos - 1) / kPackPos, 2 * c, std::min(a.B, 65535)), dim3(kPackThreads), 0, ps,
-                             jobs, a.B, a.N, behind);
+                             jobs, a.B, a.N);
     };
     if (!chained) {
         PhaseMark mark(0, s);
@@ -386,15 +383,14 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
             if (side) {
                 if ((e = cudaEventRecord(side->fork, s)) != cudaSuccess) return e;
                 if ((e = cudaStreamWaitEvent(side->stream, side->fork, 0)) != cudaSuccess) return e;
-                if ((e = launch_pack(false, 0, side->stream)) != cudaSuccess) return e;
+                if ((e = launch_pack(false, side->stream)) != cudaSuccess) return e;
                 if ((e = cudaEventRecord(side->join, side->stream)) != cudaSuccess) return e;
             }
         }
-        if (!side && (e = launch_pack(false, 0, s)) != cudaSuccess) return e;
+        if (!side && (e = launch_pack(false, s)) != cudaSuccess) return e;
     }
     bool joined = side == nullptr;
-    // behind a kernel of the call (first = false), or before all of them where the first reads the packed rows; see pack_lowrank_kernel
-    auto pack_behind = [&](bool first) -> cudaError_t { return packed ? cudaSuccess : launch_pack(true, first ? 0 : 1, s); };
+    auto pack_chained = [&]() -> cudaError_t { return packed ? cudaSuccess : launch_pack(true, s); };
     auto join_pack = [&]() -> cudaError_t {   // before the first kernel that reads the packed Q'/K'
         if (joined) return cudaSuccess;
         joined = true;
@@ -437,10 +433,10 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
         if (!cy || cy->first) {
             PhaseMark mark(1, st);
             if ((e = launch_tc_flash(f, st)) != cudaSuccess) return e;
-            if (chained && (e = pack_behind(false)) != cudaSuccess) return e;
+            if (chained && (e = pack_chained()) != cudaSuccess) return e;
         }
         for (int k = 0; k + (concat ? 0 : 1) < c; ++k) {   // the concatenating form also needs the top link's difference as a plane
-            if ((e = chained ? pack_behind(true) : join_pack()) != cudaSuccess) return e;
+            if ((e = chained ? pack_chained() : join_pack()) != cudaSuccess) return e;
             PhaseMark mark(1, st);
             TcFlashArgs fd = fw;
             fd.kd = kPadRank;
@@ -494,7 +490,7 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
                 PhaseMark mark(2, st);
                 al.chained = chained;
                 if ((e = launch_tc_align_link(al, st)) != cudaSuccess) return e;
-                if (chained && (e = pack_behind(false)) != cudaSuccess) return e;
+                if (chained && (e = pack_chained()) != cudaSuccess) return e;
             }
         }
         // 2. the FFN chain over the head axis, in place
@@ -509,7 +505,7 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
         if (!per_link) {
             PhaseMark mark(2, st);
             if ((e = launch_tc_align(al, st)) != cudaSuccess) return e;
-            if (chained && (e = pack_behind(false)) != cudaSuccess) return e;
+            if (chained && (e = pack_chained()) != cudaSuccess) return e;
         }
         // 3. each layer's own difference, softmax and .V
         if ((e = join_pack()) != cudaSuccess) return e;

@@ -526,6 +526,55 @@ def test_a_programmatic_chain_equals_its_kernels_one_by_one(Hq, integrate, N):
         assert all(torch.equal(x, y) for x, y in zip(run(all_in), ref))
 
 
+@pytest.mark.parametrize("by", ["project", "copy"])
+@pytest.mark.parametrize("Hq,integrate,N", [(32, lb.INTEGRATE_ADD, 197), (32, lb.INTEGRATE_CONCAT, 333), (40, lb.INTEGRATE_ADD, 333)])
+def test_inputs_rewritten_right_before_a_chained_call(Hq, integrate, N, by):
+    """A serving loop's buffers: Q', K', V (a projection, or copies), the cache append and the aligner's weights are written into the same
+    tensors for every layer and prompt, by the kernels right in front of the carried call, first layer and later ones, one workspace for all.
+    Every output as with the per-kernel timing on, which takes the chain apart."""
+    m, h_in, r, passes = 64, Hq * (2 if integrate == lb.INTEGRATE_CONCAT else 1), 21, 6
+    g = torch.Generator(device="cuda").manual_seed(N)
+    n = lambda *shape, std=1.0: torch.randn(shape, generator=g, device="cuda").mul_(std).bfloat16()  # noqa: E731
+    q0, k0, h = n(1, N, Hq, 128), n(1, N, Hq, 128), n(1, N, 256)
+    w_in = [n(256, Hq * (2 * r + 128), std=256 ** -0.5) for _ in range(passes)]
+    new = [(n(1, N, Hq, r), n(1, N, Hq, r), n(1, N, Hq, 128)) for _ in range(passes)]
+    ffn = [(n(h_in, m, std=h_in ** -0.5), n(m, Hq, std=m ** -0.5)) for _ in range(passes)]
+    qp, kp, v = (torch.zeros_like(x) for x in new[0])
+    w1, w2 = (torch.zeros_like(x) for x in ffn[0])
+    cache = lb.KVCacheLayer(lb.CACHE_SHARED, 1, Hq, (N + 71) // 8 * 8, 128, r, dtype=torch.bfloat16)
+    scores = torch.empty(lb.lisa_prefill_scores_bytes(1, N, Hq), dtype=torch.uint8, device="cuda")
+    link = lb.Link(qp, kp, w1, w2, integrate=integrate)
+    ws = lb.prefill_carry_workspace(q0, k0, link, v, torch.empty_like(q0), scores)
+
+    def run():
+        outs = [torch.empty_like(q0) for _ in range(passes)]
+        for i in range(passes):
+            if by == "project":
+                lb.lisa_project(h, w_in[i], [qp, kp, v])
+            else:
+                for dst, src in zip((v, kp, qp), reversed(new[i])):
+                    dst.copy_(src)
+            if i % 2:
+                lb.lisa_kvcache_append(cache, kp, v)
+            for dst, src in zip((w2, w1), reversed(ffn[i])):
+                dst.copy_(src)
+            if i % 3 == 2:   # the weights' copies are not the last kernels in front of the call
+                lb.lisa_kvcache_append(cache, kp, v)
+            lb.lisa_attn_shared_prefill_carry(q0, k0, link, v, scores, first=i % 3 == 0, keep=i % 3 < 2, out=outs[i], workspace=ws)
+        torch.cuda.synchronize()
+        assert lb.lisa_check() == lb.OK
+        return outs
+
+    lb.lisa_prefill_phase_timing(True)
+    try:
+        ref = run()
+    finally:
+        lb.lisa_prefill_phase_timing(False)
+    assert not any(torch.equal(ref[i], ref[i + 1]) for i in range(passes - 1))
+    for _ in range(5):
+        assert all(torch.equal(x, y) for x, y in zip(run(), ref))
+
+
 @pytest.mark.parametrize("r", [1, 15, 16, 17, 31, 32])
 def test_low_ranks_at_the_edges_of_their_padding(r):
     """Q' and K' are packed into rows of 32, of which whole groups of 16 are multiplied: with an emitted difference (chain of two) and without."""

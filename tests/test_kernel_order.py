@@ -37,3 +37,15 @@ def test_successors_are_released_after_the_tensor_memory_is_held(body):
     released = body.index("chain_release()")
     barrier = body.index("__syncthreads()", body.index("tmem_alloc("))
     assert released > barrier, "chain_release() comes before the barrier behind tmem_alloc()"
+
+
+WAITING = [(n, b) for n, b in kernels() if "chain_release()" in b or "chain_wait()" in b]
+
+
+@pytest.mark.parametrize("body", [pytest.param(b, id=n) for n, b in WAITING])
+def test_kernels_of_a_chain_wait_whatever_their_arguments(body):
+    """What earlier kernels wrote is visible to a kernel behind its own wait only: one wait, at the top level of the kernel."""
+    assert len(re.findall(r"chain_wait\(\)", body)) == 1
+    at = body.index("chain_wait()")
+    assert body[:at].count("{") - body[:at].count("}") == 1, "the wait is inside a block"
+    assert body[:at].rstrip()[-1] in ";}", "the wait hangs on a condition"
