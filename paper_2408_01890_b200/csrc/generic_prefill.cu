@@ -8,8 +8,8 @@
 //
 // A small prompt is bound by the latency of one CTA, so every phase spreads over all threads with its loads in flight together: the dot
 // products over (head, key, part of the row), the FFN over keys and hidden units (weights in shared memory; 2, 4 or 8 heads in registers), the softmax over heads, the
-// product with V over (head, column) and, where these are few, ranges of keys.  4 heads of 32, N 128, the standard layer and a shared one back to
-// back: 22.4 us with four loads of a thread in flight, a thread to a position's FFN and V's loads behind the softmax, 17.5 now.
+// product with V over (head, column) and, where these are few, ranges of keys.  How far that goes without costing resident CTAs depends on the
+// grid and the type, see kOverHeads below.  4 heads of 32, N 128, fp32, the standard layer and a shared one back to back 17.6 us (22.7 as kOverHeads).
 #include "common.cuh"
 
 namespace lisa {
@@ -58,16 +58,33 @@ __device__ __forceinline__ float ld(const TView& t, int64_t i) {
     else return ld_elem(t.ptr, i, t.dtype);
 }
 
+// How a CTA's phases are laid out.
+//   kOverHeads  rows of K numbered head by head, four of a lane in flight; a thread to a position's FFN.  Every bf16 or mixed call, and head counts
+//               known at run time.
+//   kWide       rows numbered key by key, eight of a lane in flight; hidden units over the lanes a position has to spare; V ahead of the product.
+//               Twice the registers: one CTA of 512 threads to an SM, two of 256.
+//   kResident   as kWide with four rows of a lane and V behind the softmax: 64 registers, twice the CTAs.
+// fp32 takes kWide where one CTA per SM is all there is, and for one prompt of up to three rows per SM, whose later CTAs are the short rows;
+// elsewhere kResident.  One link, heads of 32, us, kOverHeads | kWide | kResident:
+//   fp32, 4 heads   128 rows 12.1 | 10.2 | -     400 44.8 | 37.9 | 46.5    2 x 80 12.0 | 16.9 | 11.8    2 x 1000 223 | 310 | 230
+//   fp32, 8 heads   128 rows 16.0 | 16.2 | -     400 67.7 | 67.2 | 86.6    2 x 80 22.3 | 20.3 | 16.7    2 x 1000 525 | 535 | 435
+//   bf16, 4 heads   128 rows 11.1 | 12.7 | -     400 38.9 | 38.3 | 47.0    2 x 80 11.0 | 18.1 | 11.6    2 x 1000 189 | 293 | 224
+//   bf16, 8 heads   128 rows 14.9 | 18.6 | -     400 57.4 | 79.0 | 117     2 x 80 19.8 | 21.7 | 19.3    2 x 1000 445 | 638 | 573
+// (Prompts between lose up to 14 % to kOverHeads at 4 heads of 32, 148 rows 15.0 | 16.9 and 296 rows 28.8 | 32.9 | 30.4, and gain as much at heads of
+// 64, 200 rows 28.8 | 22.1 | 27.4; 2 heads 400 rows 24.0 | 26.8 | 28.3, 2 x 1000 180 | 211 | 135.)
+constexpr int kOverHeads = 0, kWide = 1, kResident = 2;
+
 // out[h][jj] = scale * (q[h] . row of key jj in KV head h / G) for the chunk's nk keys: neighbouring lanes take neighbouring V values of a
-// row (V values are 16 bytes, or one where rows do not start on 16 bytes), eight rows of a lane are in flight, shuffles add up a row.  Rows are
-// numbered key by key, so that a chunk of few keys takes few rounds (with a head count known at run time: four, head by head, which spares the
-// divisions: 6 heads of 64, 300 positions 115 us, 162 the other way).
-template <int DT, int V, int HQ>
+// row (V values are 16 bytes, or one where rows do not start on 16 bytes), several rows of a lane are in flight, shuffles add up a row.  Numbered
+// key by key, a chunk of few keys takes few rounds; head by head spares the divisions where the head count is known at run time (6 heads of
+// 64, 300 positions 115 us, 162 the other way).
+template <int DT, int V, int HQ, int FORM>
 __device__ __forceinline__ void dots(float* out, const float* q, int q_ld, const TView& t, int64_t at, int Hq, int G, int nk, int n, float scale) {
-    constexpr int U = HQ ? 8 : 4;
+    constexpr bool KEYS = FORM != kOverHeads;
+    constexpr int U = FORM == kWide ? 8 : 4;
     const int lanes = (n + V - 1) / V;
     const int lpr = lanes <= 1 ? 1 : lanes >= 32 ? 32 : 1 << (32 - __clz(lanes - 1));   // lanes per row
-    const int sub = threadIdx.x & (lpr - 1), grp = threadIdx.x / lpr, groups = blockDim.x / lpr, total = Hq * (HQ ? nk : kChunk);
+    const int sub = threadIdx.x & (lpr - 1), grp = threadIdx.x / lpr, groups = blockDim.x / lpr, total = Hq * (KEYS ? nk : kChunk);
     for (int r0 = 0; r0 < total; r0 += U * groups) {
         float part[U];
         int64_t row[U];
@@ -76,7 +93,7 @@ __device__ __forceinline__ void dots(float* out, const float* q, int q_ld, const
         int o[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int rr = r0 + u * groups + grp, jj = HQ ? rr / Hq : rr % kChunk, h = HQ ? rr - jj * Hq : rr / kChunk;
+            const int rr = r0 + u * groups + grp, jj = KEYS ? rr / Hq : rr % kChunk, h = KEYS ? rr - jj * Hq : rr / kChunk;
             ok[u] = rr < total && jj < nk;
             row[u] = at + jj * t.sn + (G == 1 ? h : h / G) * t.sh;
             qh[u] = q + h * q_ld;
@@ -127,11 +144,11 @@ __device__ __forceinline__ void dots(float* out, const float* q, int q_ld, const
                 if (ok[u]) out[o[u]] = part[u] * scale;
     }
 }
-template <int DT, int HQ>
+template <int DT, int HQ, int FORM>
 __device__ __forceinline__ void dots_any(float* out, const float* q, int q_ld, const TView& t, int64_t at, int Hq, int G, int nk, int n, float scale, int vec) {
-    if (DT == 0 && vec && n % 4 == 0) dots<DT, DT == 0 ? 4 : 1, HQ>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
-    else if (DT == 1 && vec && n % 8 == 0) dots<DT, DT == 1 ? 8 : 1, HQ>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
-    else dots<DT, 1, HQ>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
+    if (DT == 0 && vec && n % 4 == 0) dots<DT, DT == 0 ? 4 : 1, HQ, FORM>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
+    else if (DT == 1 && vec && n % 8 == 0) dots<DT, DT == 1 ? 8 : 1, HQ, FORM>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
+    else dots<DT, 1, HQ, FORM>(out, q, q_ld, t, at, Hq, G, nk, n, scale);
 }
 
 // A link's FFN weights: fp32 in shared memory (SM; w1, b1, w2, b2 one after the other), or where the model keeps them.
@@ -202,8 +219,8 @@ __device__ __forceinline__ void align_integrate(float* a, const float* dl, int n
     for (int g = 0; g < Hq; ++g) a[g * kChunk] = lk.integrate == LISA_INTEGRATE_ADD ? y[g] + dl[g * kChunk] : y[g];
 }
 
-template <int DT, int HQ>
-__global__ void __launch_bounds__(kMaxThreads) generic_prefill_kernel(const __grid_constant__ PrefillParams p) {
+template <int DT, int HQ, int FORM>
+__global__ void __launch_bounds__(kMaxThreads, FORM == kResident ? 2 : 0) generic_prefill_kernel(const __grid_constant__ PrefillParams p) {
     extern __shared__ __align__(16) float smem[];
     const int b = blockIdx.y, i = (int)(gridDim.x - 1 - blockIdx.x), tid = threadIdx.x;   // the longest rows first
     const int Hq = HQ ? HQ : p.Hq, d = p.d, G = Hq / p.Hkv;
@@ -255,11 +272,11 @@ __global__ void __launch_bounds__(kMaxThreads) generic_prefill_kernel(const __gr
     const int cols = Hq * d, splits = cols < kThreads ? min(kThreads / cols, max(1, Hq * kChunk / cols)) : 1;
     for (int j0 = 0; j0 <= i; j0 += kChunk) {
         const int nk = min(kChunk, i + 1 - j0);
-        dots_any<DT, HQ>(s_s, q0_s, d, p.k0, b * p.k0.sb + (int64_t)j0 * p.k0.sn, Hq, G, nk, d, inv_sqrt_d, p.vec_k0);
+        dots_any<DT, HQ, FORM>(s_s, q0_s, d, p.k0, b * p.k0.sb + (int64_t)j0 * p.k0.sn, Hq, G, nk, d, inv_sqrt_d, p.vec_k0);
         // where a thread has one column and a short range of keys, its values of V come now, under the phases before the product
         constexpr int VA = 32;
         const int v_part = tid / cols, v_col = tid - v_part * cols, v0 = nk * v_part / splits, v1 = nk * (v_part + 1) / splits;
-        const bool ahead = HQ > 0 && splits > 1 && (nk + splits - 1) / splits <= VA;
+        const bool ahead = FORM == kWide && splits > 1 && (nk + splits - 1) / splits <= VA;
         float va[VA];
         if (ahead && v_part < splits) {
             const int h = v_col / d;
@@ -269,11 +286,11 @@ __global__ void __launch_bounds__(kMaxThreads) generic_prefill_kernel(const __gr
         }
         for (int k = 0; k < p.c; ++k) {
             const LinkDev& lk = p.links[k];
-            dots_any<DT, HQ>(d_s, qp_s + k * Hq * kMaxRank, kMaxRank, lk.kp, b * lk.kp.sb + (int64_t)j0 * lk.kp.sn, Hq, G, nk, lk.r, rsqrtf((float)lk.r), p.vec_kp[k]);
+            dots_any<DT, HQ, FORM>(d_s, qp_s + k * Hq * kMaxRank, kMaxRank, lk.kp, b * lk.kp.sb + (int64_t)j0 * lk.kp.sn, Hq, G, nk, lk.r, rsqrtf((float)lk.r), p.vec_kp[k]);
             __syncthreads();
             const int h_in = (lk.integrate == LISA_INTEGRATE_CONCAT ? 2 : 1) * Hq;
-            if (HQ > 0 || tid < nk) {
-                const int parts = HQ > 0 ? kThreads / kChunk : 1, pos = tid / parts, part = tid - pos * parts;
+            if (FORM != kOverHeads || tid < nk) {
+                const int parts = FORM != kOverHeads ? kThreads / kChunk : 1, pos = tid / parts, part = tid - pos * parts;
                 const bool write = part == 0 && pos < nk;
                 if (p.w_off[k] >= 0) align_integrate<HQ>(s_s + pos, d_s + pos, Hq, Weights<true>(smem + p.w_off[k], lk, h_in, Hq), part, parts, write);
                 else align_integrate<HQ>(s_s + pos, d_s + pos, Hq, Weights<false>(nullptr, lk, h_in, Hq), part, parts, write);
@@ -356,12 +373,12 @@ bool vec_rows(const lisa_tensor& t) {
 // Head counts a compile-time constant keeps a position's scores in registers for; every other count runs the loops over local memory.
 // One link, heads of 32, fp32, 128 positions: 2 heads 8.9 us (loops 10.3), 4 heads 11.9 (13.0), 8 heads 15.9 (21.9); two
 // sequences of 1000, 8 heads: 525 (720).  Counts of tiny test and draft models; beyond eight, larger models are the tensor-core kernels'.
-template <int DT>
+template <int DT, int FORM>
 void* pick(int Hq) {
-    return Hq == 2   ? reinterpret_cast<void*>(generic_prefill_kernel<DT, 2>)
-           : Hq == 4 ? reinterpret_cast<void*>(generic_prefill_kernel<DT, 4>)
-           : Hq == 8 ? reinterpret_cast<void*>(generic_prefill_kernel<DT, 8>)
-                     : reinterpret_cast<void*>(generic_prefill_kernel<DT, 0>);
+    return Hq == 2   ? reinterpret_cast<void*>(generic_prefill_kernel<DT, 2, FORM>)
+           : Hq == 4 ? reinterpret_cast<void*>(generic_prefill_kernel<DT, 4, FORM>)
+           : Hq == 8 ? reinterpret_cast<void*>(generic_prefill_kernel<DT, 8, FORM>)
+                     : reinterpret_cast<void*>(generic_prefill_kernel<DT, 0, kOverHeads>);
 }
 
 }  // namespace
@@ -387,11 +404,13 @@ cudaError_t launch_generic_prefill(const lisa_shared_prefill_args& a, cudaStream
         const size_t room = floats > kMaxSmemFloats / 2 - 512 ? kMaxSmemFloats : kMaxSmemFloats / 2 - 512;
         if (floats + n <= room) { p.w_off[k] = (int)floats; p.w_floats[k] = (int)n; floats += n; }
     }
-    const void* kernel = !same ? pick<2>(a.Hq) : dt == LISA_BF16 ? pick<1>(a.Hq) : pick<0>(a.Hq);
+    const int64_t rows = (int64_t)a.N * a.B, sms = sm_count();
+    const bool wide = rows <= sms || (a.B == 1 && rows <= 3 * sms);
+    const void* kernel = !same ? pick<2, kOverHeads>(a.Hq) : dt == LISA_BF16 ? pick<1, kOverHeads>(a.Hq) : wide ? pick<0, kWide>(a.Hq) : pick<0, kResident>(a.Hq);
     const size_t smem = floats * sizeof(float);
     cudaError_t e = allow_smem(kernel, smem);
     if (e != cudaSuccess) return e;
-    const int threads = (int64_t)a.N * a.B <= 2 * (int64_t)sm_count() ? kMaxThreads : kMaxThreads / 2;
+    const int threads = rows <= 2 * sms ? kMaxThreads : kMaxThreads / 2;
     e = launch_chained(reinterpret_cast<void (*)(PrefillParams)>(const_cast<void*>(kernel)), dim3(a.N, a.B), dim3(threads), smem, s, p);
     count_launches(1);
     return e;

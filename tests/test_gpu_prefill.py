@@ -117,3 +117,15 @@ def test_fp32_head_counts_in_registers(Hq, Hkv, d, r, m, N, integrate, layers):
     w = synth.Workload("regs", "f32", 1, N, Hq, Hkv, d, r, m, "silu", 2)
     run_prefill_case(w, seed=N, integrate=integrate, ffn_layers=layers, bias=True, chain=2)
     run_prefill_case(w, seed=N, chain=0)
+
+
+@pytest.mark.parametrize("Hq,Hkv,d", [(2, 2, 64), (4, 4, 32), (4, 1, 64), (8, 8, 32)])
+@pytest.mark.parametrize("per_sm,more", [(1, 0), (1, 1), (2, 0), (2, 1), (3, 1)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_head_counts_in_registers_around_the_resident_grids(Hq, Hkv, d, per_sm, more, dtype):
+    """One CTA to a row: grids of one, two and three CTAs per SM, and one row more, where the build or the number of threads changes."""
+    N = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + more
+    w = synth.Workload("rows", dtype, 1, N, Hq, Hkv, d, 8, 4 * Hq, "relu", 1)
+    run_prefill_case(w, seed=N, chain=1)
+    if per_sm == 1:   # as many rows in two sequences
+        run_prefill_case(dataclasses.replace(w, B=2, N=(N + 1) // 2), seed=N, chain=1)
