@@ -80,7 +80,9 @@ typedef struct lisa_tensor {
  *   w2 [m, Hq], b2 [Hq] or NULL                       (ffn_layers == 2)
  *   ffn_layers == 1: y = W1^T x + b1 with m == Hq, no activation, w2/b2 ignored (the LiSA_SL variant)
  *   integrate == PLUS: all four ignored.
- * For a two-layer FFN: y = W2^T act(W1^T x + b1) + b2. */
+ * For a two-layer FFN: y = W2^T act(W1^T x + b1) + b2.
+ * Weights are constants of a model: a decode call may read them before the kernels in front of it in the stream have finished.
+ * A program that writes them on the device waits for that (a synchronisation, or an event) before it decodes with them. */
 typedef struct lisa_link {
     lisa_tensor qp; /* Q' [B, N, Hq, r]   (decode: [B, 1, Hq, r], the new token's) */
     lisa_tensor kp; /* K' [B, N, Hkv, r]  (decode: ignored, K' is read from the cache) */

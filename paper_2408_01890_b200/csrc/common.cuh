@@ -138,8 +138,10 @@ cudaError_t launch_tc_align_link(const TcAlignLinkArgs& a, cudaStream_t s);
 
 // Programmatic dependent launch for chains of short kernels (the decode step: append, chunk, merge, layer after layer):
 // a kernel launched with launch_chained may start while its predecessor in the stream is still running; it must call
-// chain_wait() before it touches anything an earlier kernel wrote or still reads (what it does before -- staging constant
-// weights -- overlaps the predecessor's tail), and calls chain_release() early so that its own successor can be set up.
+// chain_wait() before it touches anything an earlier kernel wrote or still reads, and calls chain_release() early so that its own
+// successor can be set up.  That it started says nothing about the kernels before: their writes are visible behind its own wait only, also
+// where a kernel between them has waited.  Set-up of its own comes before, and in the shared layers' decode kernels the aligner's weights, which the
+// interface takes for constants of the model (behind the wait: one sequence 148.4 -> 151.8 us, paper's default model 104.7 -> 109.9).
 // chain_wait() returns once the predecessor has completed and its writes are visible; as every kernel of such a chain
 // waits before it finishes, completion is transitive.  In a kernel launched the ordinary way both are no-ops.
 // A kernel that allocates tensor memory calls chain_release() behind the __syncthreads() that follows its allocation.  The successor may

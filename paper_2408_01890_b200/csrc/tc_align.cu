@@ -69,6 +69,9 @@ tc_align_kernel(const __grid_constant__ AlignParams p) {
     uint8_t* sScr = sW + c * LINK_BYTES;              // per warp: STAGES buffers of c planes x [32 heads][64 B]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+    // the weights come behind the wait: the kernel right in front of the call may have written them
+    chain_wait();
+    chain_release();
     // ---- one-time set-up: weights as ready-made B fragments (fp16, the last link's W2/b2 times log2 e) ----
     for (int k = 0; k < c; ++k) {
         // the last link's log2(e) is folded into its W2 and b2, except where every link's output leaves (store_all with
@@ -77,8 +80,6 @@ tc_align_kernel(const __grid_constant__ AlignParams p) {
         stage_link_fragments(sW + k * LINK_BYTES, p.w1[k], p.b1[k], p.w2[k], p.b2[k], p.w_dtype[k], p.kind[k], out_scale, tid, NT);
     }
     __syncthreads();
-    chain_wait();   // from here on: the planes, which earlier kernels of the stream produce
-    chain_release();   // (not earlier: what follows may read what came before this call without a wait of its own)
 
     // Parameter fields of the main loop, read once into registers: behind the asm statements (memory clobbers) the
     // compiler would re-read them from the parameter bank every time, the per-link ones through a run-time index.

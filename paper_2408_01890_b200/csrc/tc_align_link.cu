@@ -201,6 +201,18 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
     const int per = (p.total + (int)gridDim.x - 1) / (int)gridDim.x;
     const int t_begin = min(p.total, (int)blockIdx.x * per), n_tiles = min(p.total, t_begin + per) - t_begin;
 
+    // barriers and tensor memory are set up under the tail of the kernel before this one; not the weights, which it may have written
+    for (int e = tid; e < S::ZERO / 16; e += S::THREADS)
+        *reinterpret_cast<uint4*>(smem + stages * stage_bytes + e * 16) = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) {
+        for (int i = 0; i < stages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, (!CONCAT && has_d) ? 1 + 4 * S::TW : 1); }
+        for (int i = 0; i < BUFS; ++i) { mbar_init(s_full + i, 1); mbar_init(h_full + i, 4 * S::TW); mbar_init(o_full + i, 1); mbar_init(b_free + i, 4 * S::TW); }
+        *abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp == 0) tmem_alloc(tmem_slot, 512);
+    chain_wait();
+
     // ---- weights as fp16 B operands; inputs beyond the heads and hidden units beyond m are zero ----
     auto first = [&](int k, int n) -> float {      // [inputs][hidden]
         if (k >= S::H_IN) return 0.f;
@@ -231,20 +243,10 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
         b1h[e] = (kind != KIND_FFN || 2 * e >= m) ? 0u : pack_f16(ldw(p.b1, 2 * e, wd), 2 * e + 1 < m ? ldw(p.b1, 2 * e + 1, wd) : 0.f);
     for (int e = tid; e < HK; e += S::THREADS)
         b2[e] = e >= NH ? 0.f : (kind == KIND_FFN ? ldw(p.b2, e, wd) : (kind == KIND_SINGLE ? ldw(p.b1, e, wd) : 0.f));
-    for (int e = tid; e < S::ZERO / 16; e += S::THREADS)
-        *reinterpret_cast<uint4*>(smem + stages * stage_bytes + e * 16) = make_uint4(0u, 0u, 0u, 0u);
-    if (tid == 0) {
-        for (int i = 0; i < stages; ++i) { mbar_init(full + i, 1); mbar_init(empty + i, (!CONCAT && has_d) ? 1 + 4 * S::TW : 1); }
-        for (int i = 0; i < BUFS; ++i) { mbar_init(s_full + i, 1); mbar_init(h_full + i, 4 * S::TW); mbar_init(o_full + i, 1); mbar_init(b_free + i, 4 * S::TW); }
-        *abort_flag = 0;
-        fence_barrier_init();
-    }
-    if (warp == 0) tmem_alloc(tmem_slot, 512);
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    chain_wait();
     chain_release();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 

@@ -21,7 +21,7 @@
 // keep a CTA at 112 KB of shared memory and 256 tensor-memory columns), each with two warpgroups on alternate tiles.  One warpgroup
 // per CTA took 1010 cycles a tile and SM, two warpgroups on halves of the same tile as long (in step, they wait for the same unit at the
 // same time), alternate tiles 845.  A row's reference maximum is handed on behind the exponentials, which keeps the two warpgroups of a CTA
-// from coming to theirs together.  Attention with plane, 2048 tokens of 32 heads 56 -> 51 us timed alone (of which 3 are the first loads of
+// from coming to theirs together.  Attention with plane, 2048 tokens of 32 heads 53.6 -> 51.6 us captured cold (of which 3 are the first loads of
 // 296 CTAs at a time, 22 MB, and 8 the tail); 2 x 1777 of 40 heads, with and without write-back 241 -> 228; 4 x 8192 3.6 -> 3.1 ms without.
 // Every wait is bounded; on expiry the CTA records it in the status word, drains and exits.
 #include "common.cuh"
@@ -163,8 +163,7 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // What comes before -- barriers, tensor memory -- overlaps the tail of the kernel before this one.  The release comes second, so that a
-    // kernel further down the chain starts only after everything that preceded the call, weights it reads before its own wait included.
+    // What comes before -- barriers, tensor memory -- overlaps the tail of the kernel before this one.
     chain_wait();
     chain_release();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);

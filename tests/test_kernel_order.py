@@ -49,3 +49,11 @@ def test_kernels_of_a_chain_wait_whatever_their_arguments(body):
     at = body.index("chain_wait()")
     assert body[:at].count("{") - body[:at].count("}") == 1, "the wait is inside a block"
     assert body[:at].rstrip()[-1] in ";}", "the wait hangs on a condition"
+
+
+@pytest.mark.parametrize("name,inputs", [("pack_lowrank_kernel", ("jobs.",)), ("tc_align_kernel", ("p.w", "p.b", "planes")),
+                                         ("tc_align_link_kernel", ("p.w1", "p.b1", "p.w2", "p.b2"))])
+def test_prefill_kernels_wait_before_they_read(name, inputs):
+    """Q', K' and the weights as well: the kernel right in front of the call may have written them."""
+    body = next(b for n, b in WAITING if n.endswith(":" + name))
+    assert not [x for x in inputs if x in body[:body.index("chain_wait()")]]
