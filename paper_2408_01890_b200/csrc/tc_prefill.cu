@@ -35,39 +35,53 @@ struct PackJobs {
 };
 
 // A CTA packs kPackPos positions of one sequence: the rows of H x r values are read as they lie (one warp per position) into shared
-// memory and leave as whole 64-byte rows.  Bound by HBM.
-constexpr int kPackPos = 8, kPackThreads = kPackPos * 32;
+// memory and leave as whole 64-byte rows, whose 16-byte pieces a thread shifts together from five words (r may be odd, a head's values then
+// start in the middle of one).  Bound by the latency of its loads, so a warp has all of a row's in flight as 16-byte vectors; rows lie 1028
+// words apart, so that the pieces of eight positions come from different banks (with 16-bit reads of rows 1024 words apart the packing took
+// twice as long).
+constexpr int kPackPos = 8, kPackThreads = kPackPos * 32, kPackRow = kMaxHeads * kMaxRank + 8;
 __global__ void __launch_bounds__(kPackThreads) pack_lowrank_kernel(const __grid_constant__ PackJobs jobs, int B, int N) {
-    __shared__ __align__(16) __nv_bfloat16 rows[kPackPos][kMaxHeads * kMaxRank];
+    __shared__ __align__(16) __nv_bfloat16 rows[kPackPos * kPackRow];
     chain_release();
     chain_wait();
     const TView src = jobs.src[blockIdx.y];
     const int H = jobs.H[blockIdx.y], r = jobs.r[blockIdx.y], n0 = blockIdx.x * kPackPos;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, vals = H * r;
+    __nv_bfloat16* mine = rows + warp * kPackRow;
     for (int b = blockIdx.z; b < B; b += gridDim.z) {
         if (n0 + warp < N) {
             const __nv_bfloat16* sp = reinterpret_cast<const __nv_bfloat16*>(src.ptr) + b * src.sb + (int64_t)(n0 + warp) * src.sn;
-            if (src.sh == r && (vals & 1) == 0 && (reinterpret_cast<uintptr_t>(sp) & 3u) == 0) {
+            if (src.sh == r && (vals & 7) == 0 && (reinterpret_cast<uintptr_t>(sp) & 15u) == 0) {
+                const uint4* wp = reinterpret_cast<const uint4*>(sp);
+#pragma unroll 4
+                for (int e = lane; e < vals / 8; e += 32) reinterpret_cast<uint4*>(mine)[e] = wp[e];
+            } else if (src.sh == r && (vals & 1) == 0 && (reinterpret_cast<uintptr_t>(sp) & 3u) == 0) {
                 const uint32_t* wp = reinterpret_cast<const uint32_t*>(sp);
 #pragma unroll 8
-                for (int e = lane; e < vals / 2; e += 32) reinterpret_cast<uint32_t*>(rows[warp])[e] = wp[e];
+                for (int e = lane; e < vals / 2; e += 32) reinterpret_cast<uint32_t*>(mine)[e] = wp[e];
             } else {
-                for (int e = lane; e < vals; e += 32) rows[warp][e] = sp[(e / r) * src.sh + e % r];
+                for (int e = lane; e < vals; e += 32) mine[e] = sp[(e / r) * src.sh + e % r];
             }
         }
         __syncthreads();
         __nv_bfloat16* dst = jobs.dst[blockIdx.y] + ((int64_t)b * H * N + n0) * kPadRank;
         constexpr int CH = kPadRank / 8;   // 16-byte pieces of a row
         for (int e = threadIdx.x; e < H * kPackPos * CH; e += kPackThreads) {
-            const int c = e % CH, n = e / CH % kPackPos, h = e / (CH * kPackPos);
+            const int c = e % CH, n = e / CH % kPackPos, h = e / (CH * kPackPos), left = r - c * 8;   // values of the piece
             if (n0 + n >= N) continue;
             uint32_t w[4] = {0u, 0u, 0u, 0u};
+            if (left > 0) {
+                const int at = h * r + c * 8;
+                const uint32_t* v = reinterpret_cast<const uint32_t*>(rows + n * kPackRow) + (at >> 1);
+                const uint32_t shift = (at & 1) * 16;
+                uint32_t x[5];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int x = c * 8 + 2 * j;
-                const uint16_t* v = reinterpret_cast<const uint16_t*>(rows[n]) + h * r + x;
-                if (x < r) w[j] = v[0];
-                if (x + 1 < r) w[j] |= (uint32_t)v[1] << 16;
+                for (int j = 0; j < 5; ++j) x[j] = v[j];   // (past a piece's end: the row's padding at most, masked below)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    w[j] = __funnelshift_r(x[j], x[j + 1], shift);
+                    if (left < 2 * j + 2) w[j] = left < 2 * j + 1 ? 0u : w[j] & 0xffffu;
+                }
             }
             *reinterpret_cast<uint4*>(dst + ((int64_t)h * N + n) * kPadRank + c * 8) = make_uint4(w[0], w[1], w[2], w[3]);
         }
