@@ -52,7 +52,6 @@ struct FlashParams {
     int* status;
     int plane_row0;  // first query row held by the plane workspace (rows are stored relative to it)
     int qt_begin;    // this launch covers query tiles [qt_begin, qt_begin + gridDim.y)
-    int head_major;  // grid is (query tiles, batch x heads) instead of (batch x heads, query tiles)
     int ksteps;      // 16-wide k-steps of the score MMA actually issued (<= KD/16; the rest is zero padding)
     float scale;     // MODE_EMIT: scores are multiplied by this before rounding to fp16
 };
@@ -133,13 +132,11 @@ tc_flash_kernel(const __grid_constant__ FlashParams p, const __grid_constant__ C
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 37);
 
     const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
-    // blockIdx.x (the fastest-dispatched index) runs over (batch, head), blockIdx.y over query tiles from the last one
-    // down: every CTA of the heaviest tile is handed out before any lighter one, so the SMs finish close together
-    // With keys and values too large for L2 to hold for all heads at once, the order is turned round: blockIdx.x runs over the
-    // query tiles of one (batch, head), heaviest first, blockIdx.y over (batch, head), so that the CTAs resident at any time
-    // share the K and V tiles of a few heads instead of re-reading every head's for each query tile.
-    const int qt = p.qt_begin + (p.head_major ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)gridDim.y - 1 - (int)blockIdx.y);
-    const int bh = p.head_major ? (int)blockIdx.y : (int)blockIdx.x;
+    // blockIdx.x (the fastest-dispatched index) runs over a group of (batch, head) pairs, blockIdx.y over query tiles from the last one
+    // down: every CTA of a group's heaviest tile is handed out before any lighter one, so the SMs finish close together.  blockIdx.z runs
+    // over the groups: see launch_tc_flash.
+    const int qt = p.qt_begin + (int)gridDim.y - 1 - (int)blockIdx.y;
+    const int bh = (int)(blockIdx.z * gridDim.x + blockIdx.x);
     const int h = bh % p.Hq, b = bh / p.Hq;
     const int g = h / (p.Hq / p.Hkv);
     const int q0 = qt * BM;
@@ -638,11 +635,22 @@ cudaError_t launch_tc_flash(const TcFlashArgs& a, cudaStream_t stream) {
     p.scale = a.scale;
 
     if (a.qt_count < 1 || a.qt_count > 65535) return cudaErrorInvalidValue;
-    // K and V of all (batch, KV head) pairs against half of a 126 MB L2 (the other half for everything else that streams)
-    const int64_t kv_bytes = (int64_t)a.B * a.Hkv * a.N * (a.kd + (a.emit_plane ? 0 : D)) * 2;
-    p.head_major = kv_bytes > ((int64_t)63 << 20) && (int64_t)a.Hq * a.B <= 65535 && a.qt_count > 1;
-    dim3 grid(a.Hq * a.B, a.qt_count);
-    if (p.head_major) grid = dim3(a.qt_count, a.Hq * a.B);
+    // (batch, head) pairs that the CTAs handed out one after the other share out: as many as have their K and V in half of a 126 MB L2 (the other
+    // half for everything else that streams), so that the ~300 CTAs resident at a time re-read them from there for every query tile.  As
+    // many, because the heads of a position lie side by side in a plane, whose lines the CTAs of neighbouring heads then write at about the
+    // same time, and because a grid ends with the lightest tiles of its last group only.  One pair at a time, as it was beyond 63 MB | this, us:
+    // write-back at 4 x 8192 tokens of 32 / 8 heads 4171 | 3452, 2 x 4096 of 32 / 32 heads 509 | 434, attention over 2 x 1777 of 40 heads 109 | 88.
+    const int64_t kv_head = (int64_t)a.N * (a.kd + (a.emit_plane ? 0 : D)) * 2;
+    int group = a.B * a.Hq;
+    if (a.qt_count > 1)
+        while (group > 1 && ((group + a.Hq / a.Hkv - 1) / (a.Hq / a.Hkv)) * kv_head > ((int64_t)63 << 20)) {
+            int d = 2;   // smallest factor: batches first, then heads
+            const int over = group > a.Hq ? group / a.Hq : group;
+            while (over % d) ++d;
+            group /= d;
+        }
+    if (a.B * a.Hq / group > 65535) group = a.B * a.Hq;
+    const dim3 grid(group, a.qt_count, a.B * a.Hq / group);
     cudaError_t e;
 #define LISA_LAUNCH_FLASH(KD_, PL_)                                                                                       \
     do {                                                                                                                   \
