@@ -357,6 +357,14 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
     const bool one_wave = (int64_t)a.B * a.Hq * ((a.N + kTile - 1) / kTile) <= 2 * (int64_t)sm_count();   // of CTAs, all resident at once
     Wave waves[1024];
     int nw = plan_waves(a.B, a.N, a.Hq, cy ? 1 : plane_count(a), waves, 1024, cy != nullptr && !concat);
+    // Carried scores need no planes of a wave's own: the whole prompt is one wave, whose kernels run one after the other as a programmatic
+    // chain.  Each of them is bound by memory (aligner 6.2 of 6.55 TB/s at 4 x 8192 tokens of 32 heads) or fills the GPU, so that waves side by side
+    // only added their tails: an anchor and its chain, in waves | in one, 4 x 8192 of the 8B shape 23260 | 22980 us, 1 x 8192 4232 | 4119, 2 x 4096
+    // of the 7B shape 2426 | 2329, 4 x 2500 of 40 heads 2653 | 2537.
+    if (cy && !concat && !ho) {
+        waves[0] = Wave{0, (a.N + kTile - 1) / kTile};
+        nw = 1;
+    }
     // A host-memory call whose prompt fits fewer than four waves is cut into four strips of query tiles all the same (they
     // run one after the other in the planes laid out for the larger waves): its time is the copies', and strips let the
     // copies in, the compute and the copies out overlap.
