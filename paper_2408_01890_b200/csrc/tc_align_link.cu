@@ -211,6 +211,11 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
         fence_barrier_init();
     }
     if (warp == 0) tmem_alloc(tmem_slot, 512);
+    if (warp == 16 && elect_one()) {
+        tma_prefetch_desc(&tmX); tma_prefetch_desc(&tmXs);
+        if (has_d) { tma_prefetch_desc(&tmD); tma_prefetch_desc(&tmDs); }
+    }
+    __syncwarp();
     chain_wait();
 
     // ---- weights as fp16 B operands; inputs beyond the heads and hidden units beyond m are zero ----
@@ -258,8 +263,6 @@ tc_align_link_kernel(const __grid_constant__ LinkParams p, const __grid_constant
             if (n_tiles > 0) cu.seek(p, t_begin);
             int s = 0;
             uint32_t par = 1;
-            tma_prefetch_desc(&tmX);
-            if (has_d) tma_prefetch_desc(&tmD);
             for (int i = 0; i < n_tiles; ++i) {
                 if (!mbar_wait(empty + s, par, abort_flag)) break;
                 mbar_expect_tx(full + s, (has_d ? 2 : 1) * TILE);
