@@ -580,3 +580,42 @@ def test_low_ranks_at_the_edges_of_their_padding(r):
     """Q' and K' are packed into rows of 32, of which whole groups of 16 are multiplied: with an emitted difference (chain of two) and without."""
     run_tc_shared(1, 200, 8, 1, "relu", seed=r, r=r)
     run_tc_shared(2, 130, 32, 2, "silu", seed=r, r=r)
+
+
+@pytest.mark.parametrize("r,Hkv", [(21, 32), (21, 4), (20, 8), (1, 1), (7, 2), (32, 32)])
+def test_low_ranks_are_packed_alike_wherever_their_rows_start(r, Hkv):
+    """Rows of Q' and K' that start on 16, 4 and 2 bytes, heads with a stride of their own, a row of values that is no whole number of
+    16-byte units: the outputs of the dense tensors, bit for bit.  N is no multiple of the eight positions a CTA packs."""
+    w = synth.Workload("tc_pack", "bf16", 2, 203, 32, Hkv, 128, r, 64, "relu", 1)
+    t = synth.prefill_inputs(w, r)
+    q0, k0, v, w1, w2 = (dev(t[n]) for n in ("q0", "k0", "v1", "w1_1", "w2_1"))
+
+    def run(qp, kp):
+        out = lb.lisa_attn_shared_prefill(q0, k0, [lb.Link(qp, kp, w1, w2, act=lb.ACT_RELU)], v)
+        torch.cuda.synchronize()
+        assert lb.lisa_check() == lb.OK
+        return out
+
+    def strided(x, more, head):
+        B, N, H, n = x.shape
+        row = H * head + more
+        y = torch.zeros(B * N * row + 8, dtype=x.dtype, device="cuda").as_strided((B, N, H, n), (N * row, row, head, 1))
+        return y.copy_(x)
+
+    qp, kp = dev(t["qp1"]), dev(t["kp1"])
+    ref = run(qp, kp)
+    for more, head in ((8, r), (2, r), (1, r), (0, r + 3)):
+        assert torch.equal(run(strided(qp, more, head), strided(kp, more, head)), ref), (more, head)
+
+
+@pytest.mark.parametrize("B,N,Hq,Hkv", [(6, 4096, 32, 32), (3, 5000, 40, 40), (5, 7000, 32, 8)])
+def test_attention_whose_keys_and_values_exceed_l2(B, N, Hq, Hkv):
+    """Past 63 MB of K and V the (batch, head) pairs are handed out in groups (whole batches, then parts of one, by the factors of both counts):
+    every pair and query tile is computed once, whatever the order.  A sequence alone is handed out in other groups; its outputs are the same bytes."""
+    g = torch.Generator(device="cuda").manual_seed(B)
+    q, k, v = (torch.randn((B, N, h, 128), generator=g, device="cuda", dtype=torch.bfloat16) for h in (Hq, Hkv, Hkv))
+    got = torch.full_like(q, float("nan"))
+    lb.lisa_attn_anchor(q, k, v, out=got)
+    for b in range(B):
+        assert torch.equal(lb.lisa_attn_anchor(q[b:b + 1], k[b:b + 1], v[b:b + 1]), got[b:b + 1])
+    assert lb.lisa_check() == lb.OK
