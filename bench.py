@@ -39,11 +39,11 @@ CFG2_POSITIONS_HEADS = 2098176 * 32
 PREFILL_TRAFFIC_PER_PH = {"emit_scores": (40335360 + 84761344) / CFG2_POSITIONS_HEADS,
                           "align": (138465792 + 84176384) / CFG2_POSITIONS_HEADS,
                           "attention": (175657216 + 3785216) / CFG2_POSITIONS_HEADS}
-# The kernels of a carried layer, captured on the first wave (query rows 0..3199) of the headline chain at B 1, N 4096:
+# The kernels of a carried layer, captured on the first layer of the headline chain at B 1, N 4096:
 # the one-link aligner in place on the scores buffer and the attention kernel that writes its logits back.
-CARRY_POSITIONS_HEADS = 3200 * 3201 // 2 * 32
-CARRY_TRAFFIC_PER_PH = {"align": (334301440 + 284014080) / CARRY_POSITIONS_HEADS,
-                        "attention_keep": (362388992 + 310542592) / CARRY_POSITIONS_HEADS}
+CARRY_POSITIONS_HEADS = 4096 * 4097 // 2 * 32
+CARRY_TRAFFIC_PER_PH = {"align": (545329920 + 494662400) / CARRY_POSITIONS_HEADS,
+                        "attention_keep": (586332160 + 531177472) / CARRY_POSITIONS_HEADS}
 DECODE_TRAFFIC_PER_SEQ = (593891584 + 5096704) / 12  # shared decode chunk kernel, captured at 12 sequences; scales with the batch
 PROJECT_TRAFFIC = 249444608 + 161213184             # projection kernel at the benchmark's own size
 
