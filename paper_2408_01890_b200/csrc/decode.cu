@@ -670,16 +670,11 @@ cudaError_t launch_anchor_decode(const lisa_anchor_args& a, void* ws, cudaStream
         const bool dealt = deal_chunks(p, ctas);   // (only with whole chunks, see launch_shared_fast)
         p.least = 0;
         p.most = INT_MAX;
-        // Scores on the tensor cores where heads share a KV head, and where the grid is resident at once and a CTA's latency counts (paper's default
-        // model, 8 x 1111, 102.1 -> 97.8 us; one sequence of 333 145.4 -> 142.8; 10 x 700 of 40 heads 66.3 -> 66.9).  A grid that streams rows of
-        // one head each is faster with qk_stream, whose loads take whole rows: a step of 32 x 2176 of the 7B shape 715, 751 on the tensor cores.
-        const bool mma = dealt || p.prefetch >= 0 || G > 1;
-        const size_t smem = anchor_fast_smem(p.heads, p.chunk, G, mma);
-        auto kernel = dealt            ? anchor_decode_fast_kernel<128, true, true>
-                      : !mma           ? anchor_decode_fast_kernel<128, false, false>
-                      : p.chunk == 128 ? anchor_decode_fast_kernel<128, false, true>
-                      : p.chunk == 64  ? anchor_decode_fast_kernel<64, false, true>
-                                       : anchor_decode_fast_kernel<32, false, true>;
+        const size_t smem = anchor_fast_smem(p.heads, p.chunk, G);
+        auto kernel = dealt          ? anchor_decode_fast_kernel<128, true>
+                      : p.chunk == 128 ? anchor_decode_fast_kernel<128, false>
+                      : p.chunk == 64  ? anchor_decode_fast_kernel<64, false>
+                                       : anchor_decode_fast_kernel<32, false>;
         if ((e = allow_smem(kernel, smem)) != cudaSuccess) return e;
         e = launch_chained(kernel, dim3(p.n_chunks, p.Hkv / kv, p.B), dim3(kDecodeThreads), smem, s, p);
     } else {

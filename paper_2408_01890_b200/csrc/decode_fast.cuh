@@ -202,85 +202,6 @@ __device__ __forceinline__ void qk_stream(const Rows& r, int nv, int vper, const
     stream_rows<CH, U>(r, nv, vper, row_parts(nv, CH, GV), body, [](int, int) {});
 }
 
-// d += a (16x16, row) . b (16x8, col), bf16 in, fp32 accumulate
-__device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// The same on mma m16n8k16, rows of K as M and the GV heads that share them as N (bf16 operands as they are cached, products exact, sums in
-// fp32); q: the group's first query row, heads q_sh apart.  Which of the 128 dimensions is which k index is free as long as both operands
-// agree, so a lane's 16-byte loads are its fragments as they stand: lane (g, t) = (lane / 4, lane % 4) takes the pieces t, t + 4, t + 8, t + 12 of
-// rows g and g + 8 of a batch of 16, and the same pieces of head g's query.  qk_stream spends some fifteen instructions a row and head and
-// its share of a butterfly of shuffles, so that with several heads to a KV head the scores of a chunk take as long as its loads.
-// An anchor and one shared layer of the 8B shape, us, FMAs | this: 12 x 3500 100.0 | 91.5, 32 x 4096 221 | 208, 16 ragged of up to 2900 (four layers)
-// 142.0 | 134.5.
-template <int CH, int GV>
-__device__ __forceinline__ void qk_mma(const Rows& r, int nv, int vper, const __nv_bfloat16* q, int64_t q_sh, float* s_s, int ld, float scale) {
-    constexpr int NB = CH / 16;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int ps = nv >= kDecodeWarps ? 1 : min(kDecodeWarps / nv, NB);   // ranges of rows where there are fewer heads than warps
-    const int part = ps > 1 ? warp / nv : 0, first = ps > 1 ? warp % nv : warp;
-    if (first >= nv || part >= ps) return;
-    const int nb_all = (r.nrows + 15) / 16, b0 = nb_all * part / ps, b1 = nb_all * (part + 1) / ps;
-    if (b0 == b1) return;
-    auto load = [&](uint4 (*k)[4], int v, int bt) {
-        const uint4* p = r.base + (size_t)(v / vper) * r.head_stride + (bt * 16 + g) * 16 + t;
-        const int left = r.nrows - bt * 16 - g;
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) k[i][j] = ld_stream16_or_zero(p + i * 128 + j * 4, i * 8 < left);
-    };
-    uint4 ka[2][4], kb[2][4], qf[4];
-    int lv = first, lb = b0;      // next batch to load
-    auto load_next = [&](uint4 (*k)[4]) {
-        if (lv < nv) {
-            load(k, lv, lb);
-            if (++lb == b1) { lb = b0; lv += ps > 1 ? nv : kDecodeWarps; }
-        }
-    };
-    auto query = [&](int v) {
-        const uint4* p = reinterpret_cast<const uint4*>(q + (v * GV + g) * q_sh) + t;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) qf[j] = g < GV ? p[j * 4] : make_uint4(0u, 0u, 0u, 0u);
-    };
-    auto body = [&](const uint4 (*k)[4], int v, int bt) {
-        float d[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t lo[4] = {k[0][j].x, k[1][j].x, k[0][j].y, k[1][j].y}, hi[4] = {k[0][j].z, k[1][j].z, k[0][j].w, k[1][j].w};
-            mma_bf16(d, lo, qf[j].x, qf[j].y);
-            mma_bf16(d, hi, qf[j].z, qf[j].w);
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {   // rows g (+ 8), heads 2t (+ 1)
-            const int head = 2 * t + (e & 1);
-            if (head < GV) s_s[(v * GV + head) * ld + bt * 16 + g + (e >> 1) * 8] = d[e] * scale;
-        }
-    };
-    load_next(ka);
-    query(first);
-    int v = first, bt = b0;
-    auto next = [&]() {   // the head and batch behind the one just done; false behind the last
-        if (++bt < b1) return true;
-        bt = b0;
-        v += ps > 1 ? nv : kDecodeWarps;
-        if (v >= nv) return false;
-        query(v);
-        return true;
-    };
-    while (true) {
-        load_next(kb);
-        body(ka, v, bt);
-        if (!next()) break;
-        load_next(ka);
-        body(kb, v, bt);
-        if (!next()) break;
-    }
-}
-
 // Softmax of a chunk per head, in place: s_s[head][CH] scores (add_s), plus HS partial sums y_s[hs][head][CH] where y_s is given,
 // become exponentials; the finished scores go to the row of the next layer, maximum and sum to the workspace.
 template <int CH, int HS>
@@ -356,14 +277,14 @@ __device__ __forceinline__ void prefetch_chunk(const DecodeParams& p, int kv0, i
 }
 
 // ---------------------------------------------------------------------------------------------
-// Standard layer.  Shared memory: scores [HG][CH], queries fp32 [HG][128] (not with MMA), position ranges of P.V.
+// Standard layer.  Shared memory: scores [HG][CH], queries fp32 [HG][128], position ranges of P.V.
 // ---------------------------------------------------------------------------------------------
-inline size_t anchor_fast_smem(int HG, int ch, int G, bool mma) {
+inline size_t anchor_fast_smem(int HG, int ch, int G) {
     const int gv = kv_group(G);
-    return sizeof(float) * ((size_t)HG * ch + (size_t)(row_parts(HG / gv, ch, gv) - mma) * HG * 128);
+    return sizeof(float) * ((size_t)HG * ch + (size_t)row_parts(HG / gv, ch, gv) * HG * 128);
 }
 
-template <int CH, bool DENSE, bool MMA>
+template <int CH, bool DENSE>
 __global__ void __launch_bounds__(kDecodeThreads, 2) anchor_decode_fast_kernel(const __grid_constant__ DecodeParams p) {
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x;
@@ -376,30 +297,21 @@ __global__ void __launch_bounds__(kDecodeThreads, 2) anchor_decode_fast_kernel(c
     const int j0 = chunk * CH, nrows = min(CH, L - j0);
     float* s_s = smem;
     float* q_s = s_s + HG * CH;
-    float* red = MMA ? q_s : q_s + HG * 128;
-    const __nv_bfloat16* q = reinterpret_cast<const __nv_bfloat16*>(p.q.ptr) + b * p.q.sb + h0 * p.q.sh;
-    if constexpr (!MMA) {
-        for (int e = tid; e < HG * 16; e += kDecodeThreads) {
-            const int h = e >> 4, x = e & 15;
-            float f[8];
-            bf16x8_to_f32(*reinterpret_cast<const uint4*>(q + h * p.q.sh + x * 8), f);
-            float4* dst = reinterpret_cast<float4*>(q_s + h * 128 + x * 8);
-            dst[0] = make_float4(f[0], f[1], f[2], f[3]);
-            dst[1] = make_float4(f[4], f[5], f[6], f[7]);
-        }
-        __syncthreads();
+    float* red = q_s + HG * 128;
+    for (int e = tid; e < HG * 16; e += kDecodeThreads) {
+        const int h = e >> 4, x = e & 15;
+        float f[8];
+        bf16x8_to_f32(*reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.q.ptr) + b * p.q.sb + (h0 + h) * p.q.sh + x * 8), f);
+        float4* dst = reinterpret_cast<float4*>(q_s + h * 128 + x * 8);
+        dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+        dst[1] = make_float4(f[4], f[5], f[6], f[7]);
     }
+    __syncthreads();
     const Rows rows{reinterpret_cast<const uint4*>(p.kcache) + (((size_t)b * p.Hkv + kv0) * p.L_cap + j0) * 16, (size_t)p.L_cap * 16, nrows};
     const float scale = rsqrtf(128.f);
-    if constexpr (MMA) {
-        if (gv == 1) qk_mma<CH, 1>(rows, HG, G, q, p.q.sh, s_s, CH, scale);
-        else if (gv == 2) qk_mma<CH, 2>(rows, HG / 2, G / 2, q, p.q.sh, s_s, CH, scale);
-        else qk_mma<CH, 4>(rows, HG / 4, G / 4, q, p.q.sh, s_s, CH, scale);
-    } else {
-        if (gv == 1) qk_stream<CH, 1>(rows, HG, G, q_s, s_s, CH, scale);
-        else if (gv == 2) qk_stream<CH, 2>(rows, HG / 2, G / 2, q_s, s_s, CH, scale);
-        else qk_stream<CH, 4>(rows, HG / 4, G / 4, q_s, s_s, CH, scale);
-    }
+    if (gv == 1) qk_stream<CH, 1>(rows, HG, G, q_s, s_s, CH, scale);
+    else if (gv == 2) qk_stream<CH, 2>(rows, HG / 2, G / 2, q_s, s_s, CH, scale);
+    else qk_stream<CH, 4>(rows, HG / 4, G / 4, q_s, s_s, CH, scale);
     __syncthreads();
     const size_t part = ((size_t)b * p.n_chunks + chunk) * p.Hq + h0;
     finish_scores<CH, 1>(p, s_s, nullptr, true, HG, h0, b, j0, nrows, part);
@@ -468,6 +380,12 @@ __device__ __forceinline__ uint32_t to_tf32(float x) {
 // d += a (16x8, row) . b (8x8, col), tf32 in, fp32 accumulate
 __device__ __forceinline__ void mma_tf32(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// d += a (16x16, row) . b (16x8, col), bf16 in, fp32 accumulate
+__device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
