@@ -387,13 +387,9 @@ template <int U>
 __global__ void __launch_bounds__(kMergeThreads) decode_merge_kernel(const __grid_constant__ DecodeParams p) {
     __shared__ float4 s_o[kMergeThreads];
     const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
-    // The successor of a step's last kernel is the projection through W_O, which asks its first slices of W into L2 as soon as it is there.  Beside a
-    // chunk kernel that waits for its own loads that is too early, so it is let in behind the wait; a grid that streams its caches for some
-    // rounds has the time (one sequence 148.7 -> 145.6 us, paper's default model 104.4 -> 102.7; a step of 32 sequences 715 -> 718, hence the
-    // condition).
-    if (p.prefetch < 0) chain_release();
+    if (!p.late_release) chain_release();
     chain_wait();
-    chain_release();
+    if (p.late_release) chain_release();
     const int nc = (decode_length(p, b) + p.chunk - 1) / p.chunk;
     const size_t base = (size_t)b * p.n_chunks * p.Hq + h;
     const int lpr = p.d / 4, x = tid % lpr, c0 = tid / lpr, cstep = kMergeThreads / lpr;   // lanes per partial output, this thread's chunks
@@ -585,7 +581,20 @@ cudaError_t shared_fast(DecodeParams& p, void* ws, cudaStream_t s, bool* taken) 
     return launch_shared_fast<HQ, HQ, 32, 0, kEngConcat>(p, s);
 }
 
-cudaError_t launch_merge(const DecodeParams& p, cudaStream_t s) {
+// Whether the merge lets its successor in behind its wait instead of at its start.  The kernels behind it ask their caches and weights into L2
+// and stage the aligner when they start.  With few positions in the batch there is little to stream, and that early start only stands in the way of
+// a chunk kernel that waits for its own loads; with more, or with merges enough to fill the SMs behind the chunks, it is worth its while.  An anchor
+// and three layers, us, released early | late: one sequence of 640 positions 53.1 | 46.5 (7B-shaped), 52.6 | 48.4 (8B), 56.2 | 49.6 (13B), 78.0 | 72.2
+// (paper's default), 5 x 200 54.0 | 50.6, 55.2 | 51.3, 55.6 | 55.1 and 88.4 | 86.9; beyond the lines 8 x 700 89.0 | 95.6 (7B), 20 x 700 102 | 112 (8B),
+// 6 x 700 93.0 | 97.8 (13B), 1 x 2500 70.2 | 72.4 (7B), and 8 x 100 and 20 x 30 of the paper's default 72.9 | 81.2 and 83.5 | 87.2, although
+// 20 x 30 of the others gains (53.9 | 49.5, 53.6 | 51.3, 56.1 | 53.7).
+constexpr int kLatePositions = 1024;
+bool merge_releases_late(const DecodeParams& p) {
+    return (int64_t)p.B * p.L_uniform <= kLatePositions && 2 * (int64_t)p.Hq * p.B <= 3 * (int64_t)sm_count();
+}
+
+cudaError_t launch_merge(DecodeParams& p, cudaStream_t s) {
+    p.late_release = merge_releases_late(p);
     const int each = kMergeThreads * 4 / p.d;   // chunks that the CTA's threads take side by side
     const int64_t ctas = (int64_t)p.Hq * p.B, sms = sm_count();
     auto kernel = p.n_chunks <= each || ctas > 10 * sms      ? decode_merge_kernel<1>
@@ -633,7 +642,6 @@ cudaError_t launch_shared_decode(const lisa_shared_decode_args& a, void* ws, cud
     else if (p.Hq == 32) e = shared_fast<32, 64>(p, ws, s, &taken);
     if (!taken) {
         set_chunk(p, kChunk, ws);
-        p.prefetch = -1;
         const size_t smem = shared_decode_smem(p.Hq, p.m, p.integrate);
         auto kernel = p.row_bf16 ? shared_decode_chunk_kernel<true> : shared_decode_chunk_kernel<false>;
         if ((e = allow_smem(kernel, smem)) != cudaSuccess) return e;
@@ -679,7 +687,6 @@ cudaError_t launch_anchor_decode(const lisa_anchor_args& a, void* ws, cudaStream
         e = launch_chained(kernel, dim3(p.n_chunks, p.Hkv / kv, p.B), dim3(kDecodeThreads), smem, s, p);
     } else {
         set_chunk(p, kChunk, ws);
-        p.prefetch = -1;
         const size_t smem = sizeof(float) * ((size_t)p.Hq * kChunk + (size_t)p.Hq * p.d);
         if ((e = allow_smem(anchor_decode_chunk_kernel, smem)) != cudaSuccess) return e;
         e = launch_chained(anchor_decode_chunk_kernel, dim3(p.n_chunks, p.B), dim3(kThreads), smem, s, p);

@@ -12,6 +12,7 @@ struct DecodeParams {
     int chunk;              // cached positions per chunk: 128, or 64 or 32 in the kernels for small batches
     int heads;              // query heads per CTA where the heads are divided over CTAs
     int prefetch;           // a CTA asks its K or K' and V of this many of its KV heads into L2 when it starts; -1: nothing
+    int late_release;       // the merge lets its successor in behind its wait, not at its start (see merge_releases_late)
     int least, most;        // dealt chunks (see decode_item): the launch does its work only if least..most of them hold positions (see launch_shared_fast)
     const int32_t* seq_lens;
     // shared layer

@@ -385,3 +385,53 @@ def test_ragged_batches_whose_chunks_are_dealt(Hq, Hkv, m, integrate, B, L):
         assert_close(out[:, 0].float().cpu().numpy(), O, "bf16", "standard O")
         for b in range(B):
             assert_close(row.cpu().numpy()[b, :, :lens[b]], R[b, :, :lens[b]], "bf16", "standard row")
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,m,B,L", [
+    (32, 8, 128, 64, 4, 256), (32, 8, 128, 64, 4, 257),        # 1024 positions and more
+    (32, 32, 128, 64, 6, 60), (32, 32, 128, 64, 7, 60),        # 192 and 224 merges on 148 SMs: one and a half times as many lie between
+    (40, 40, 128, 80, 5, 128), (40, 40, 128, 80, 6, 128),
+    (8, 2, 64, 16, 3, 300), (8, 2, 64, 16, 4, 300)])           # the general chunk kernels
+def test_layers_enqueued_behind_one_another_equal_layers_one_by_one(Hq, Hkv, d, m, B, L):
+    """Where the merge lets the kernels behind it in at its start and where behind its wait: append, standard layer, append, shared layers with one
+    workspace and no wait between them give the bytes of the same calls with the GPU waited for after each, and the last layer is the oracle's."""
+    w = synth.Workload("behind", "bf16", B, L, Hq, Hkv, d, 21, m, "relu", 1, True)
+    t = synth.decode_inputs(w, 5, B=B, L=L)
+    L_cap = (L + 15) // 8 * 8
+    ws = torch.empty(lb.decode_workspace_bytes(B, Hq, d, L), dtype=torch.uint8, device="cuda")
+    before = torch.full((B,), L - 1, dtype=torch.int32, device="cuda")
+    x = {k: dev(v) for k, v in t.items()}
+
+    def step(wait):
+        def done(y=None):
+            if wait:
+                torch.cuda.synchronize()
+            return y
+        st = lb.KVCacheLayer(lb.CACHE_STANDARD, B, Hkv, L_cap, d)
+        sh = [lb.KVCacheLayer(lb.CACHE_SHARED, B, Hkv, L_cap, d, w.r) for _ in range(2)]
+        rows = [torch.zeros((B, Hq, L_cap), dtype=torch.float32, device="cuda") for _ in range(2)]
+        for cache, k in [(st, "k")] + [(c, "kp") for c in sh]:
+            lb.lisa_kvcache_append(cache, x[k][:, :L - 1].contiguous(), x["v"][:, :L - 1].contiguous())
+        new = {k: x[k][:, L - 1:].contiguous() for k in ("k", "kp", "v")}
+        torch.cuda.synchronize()
+        outs = []
+        done(lb.lisa_kvcache_append(st, new["k"], new["v"], before))
+        outs.append(done(lb.lisa_attn_anchor(x["q0"], cache=st, L=L, out_scores=rows[0], workspace=ws)))
+        for i in range(2):
+            done(lb.lisa_kvcache_append(sh[i], new["kp"], new["v"], before))
+            link = lb.Link(x["qp"], None, x["w1"], x["w2"], act=lb.ACT_RELU)
+            outs.append(done(lb.lisa_attn_shared_decode(rows[i], link, sh[i], L=L, out_scores=rows[1] if i == 0 else None, workspace=ws)))
+        torch.cuda.synchronize()
+        return outs + rows
+
+    ref = step(True)
+    for _ in range(3):
+        assert all(torch.equal(a, b) for a, b in zip(step(False), ref))
+    lens = np.full((B,), L, dtype=np.int32)
+    O0, R0 = oracle.decode_anchor(f64(t["q0"])[:, 0], f64(t["k"]), f64(t["v"]), lens)
+    assert_close(ref[0][:, 0].float().cpu().numpy(), O0, "bf16", "standard O")
+    olink = oracle.Link(None, None, f64(t["w1"]), f64(t["w2"]), r=w.r, act=oracle.ACT_RELU)
+    for i in range(2):
+        O, R = oracle.decode_shared(R0 if i == 0 else ref[4][:, :, :L].cpu().numpy().astype(np.float64), f64(t["qp"])[:, 0], f64(t["kp"]), f64(t["v"]), olink, lens)
+        assert_close(ref[1 + i][:, 0].float().cpu().numpy(), O, "bf16", "shared O %d" % i)
+    assert lb.lisa_check() == lb.OK
