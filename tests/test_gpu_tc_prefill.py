@@ -321,11 +321,31 @@ def test_carried_scores_concatenating_integrate(B, N, Hkv, chain, m, act, layers
         assert_close(got.float().cpu().numpy(), ref, "bf16", "carried scores, concatenating integrate, layer %d of %d" % (k + 1, chain))
 
 
+def test_carried_scores_concatenating_integrate_in_two_waves():
+    """B = 4, N = 1600: the plane of the difference exceeds one wave's budget, so the eleven first query tiles and the two last ones go out as two waves
+    on two streams, each with a plane of its own, over one scores buffer.  Launches: pack, and per wave [A_0,] the difference, align, attention."""
+    B, N, chain = 4, 1600, 2
+    t = concat_inputs(B, N, 8, chain, 64, "relu", 2, 20, 19, True)
+    dl, ol = make_links(t, chain, "relu", lb.INTEGRATE_CONCAT, 2, True)
+    scores = torch.full((lb.lisa_prefill_scores_bytes(B, N, 32),), 0xFF, dtype=torch.uint8, device="cuda")
+    q0, k0 = dev(t["q0"]), dev(t["k0"])
+    ri = np.concatenate([np.arange(0, 1408, 97), np.arange(1407, 1411), np.arange(1535, 1538), np.arange(N - 3, N)]).astype(np.int32)
+    rb = np.full(ri.shape, B - 1, dtype=np.int32)
+    for k in range(chain):
+        n0 = lb.lisa_kernel_launches()
+        got = lb.lisa_attn_shared_prefill_carry(q0, k0, dl[k], dev(t[f"v{k + 1}"]), scores, first=k == 0, keep=k + 1 < chain)
+        torch.cuda.synchronize()
+        assert lb.lisa_kernel_launches() - n0 == (9 if k == 0 else 7)
+        assert lb.lisa_check() == lb.OK
+        ref = oracle.prefill_rows(f64(t["q0"]), f64(t["k0"]), f64(t[f"v{k + 1}"]), ol[:k + 1], rb, ri)
+        assert_close(got[B - 1, torch.from_numpy(ri).long().cuda()].float().cpu().numpy(), ref, "bf16", "concatenating integrate, two waves, layer %d" % (k + 1))
+
+
 def test_carried_scores_several_waves_from_device_and_host_memory():
-    """B = 4, N = 1600: the prompt's scores exceed one wave's budget, so the layers run as two waves on two streams; the
-    host-memory call then also brings q0, k0, v in and takes o out wave by wave.  Both must give bit-identical outputs
-    (same kernels on the same data), and sampled rows (first and last tile, 32 random rows per sequence) must match the
-    oracle at every depth."""
+    """B = 4, N = 1600: carried scores from device memory are one wave on the caller's stream whatever the prompt's size; the host-memory call
+    goes strip by strip on several streams, brings q0, k0, v in and takes o out.  Both must give bit-identical outputs (same kernels on the same data),
+    and sampled rows (first and last tile, 32 random rows per sequence) must match the oracle at every depth.  The recomputing calls, whose planes
+    exceed one wave's budget, are several waves from either memory."""
     B, N, Hq, Hkv, chain = 4, 1600, 32, 8, 2
     t = link_inputs(B, N, Hq, Hkv, chain, 64, "relu", 2, 21, 43, False)
     dl, ol = make_links(t, chain, "relu")
@@ -352,7 +372,7 @@ def test_carried_scores_several_waves_from_device_and_host_memory():
         assert torch.equal(out_h, got.cpu())
         ref = oracle.prefill_rows(f64(t["q0"]), f64(t["k0"]), f64(t[f"v{k + 1}"]), ol[:k + 1], rb, ri)
         sel = got[torch.from_numpy(rb).long().cuda(), torch.from_numpy(ri).long().cuda()].float().cpu().numpy()
-        assert_close(sel, ref, "bf16", "carried scores over two waves, layer %d" % (k + 1))
+        assert_close(sel, ref, "bf16", "carried scores, whole prompt and strips, layer %d" % (k + 1))
     # the recomputing call at depth 2 through the host-memory entry point (inputs and output streamed per wave as well)
     hlinks = [lb.Link(pin[f"qp{j}"], pin[f"kp{j}"], pin[f"w1_{j}"], pin[f"w2_{j}"], act=lb.ACT_RELU) for j in (1, 2)]
     out_h = torch.empty_like(t["q0"]).pin_memory()
@@ -362,7 +382,7 @@ def test_carried_scores_several_waves_from_device_and_host_memory():
     torch.cuda.synchronize()
     assert torch.equal(out_h, got2.cpu())
     sel = got2[torch.from_numpy(rb).long().cuda(), torch.from_numpy(ri).long().cuda()].float().cpu().numpy()
-    assert_close(sel, ref, "bf16", "recomputed over two waves, depth 2")
+    assert_close(sel, ref, "bf16", "recomputed in several waves, depth 2")
     assert lb.lisa_check() == lb.OK
 
 
@@ -405,8 +425,8 @@ def test_carried_scores_single_layer_keeps_nothing():
 
 
 def test_small_prompt_chain_replayed_from_a_graph():
-    """A prompt whose kernels are launched as a programmatic chain, with the packing on a stream of its own: captured and replayed, the
-    results are those of the plain calls."""
+    """A prompt whose kernels are launched as a programmatic chain, the packing among them: captured and replayed, the results are those of the
+    plain calls."""
     B, N, Hkv, chain = 1, 200, 8, 2
     w = synth.Workload("graph", "bf16", B, N, 32, Hkv, 128, 21, 64, "relu", chain)
     t = synth.prefill_inputs(w, 12)
@@ -492,8 +512,11 @@ def test_attention_whose_maxima_keep_growing(N, form):
     assert_close(got.float().cpu().numpy(), ref.numpy(), "bf16", form)
 
 
-@pytest.mark.parametrize("N", [50, 197, 1300])
-@pytest.mark.parametrize("Hq,integrate", [(32, lb.INTEGRATE_ADD), (40, lb.INTEGRATE_ADD), (32, lb.INTEGRATE_CONCAT)])
+CHAIN_FORMS = [(32, lb.INTEGRATE_ADD), (40, lb.INTEGRATE_ADD), (32, lb.INTEGRATE_CONCAT)]
+
+
+# (4500 tokens: 1152 CTAs of a head-partitioned kernel, nearly four rounds, in one programmatic chain)
+@pytest.mark.parametrize("Hq,integrate,N", [(*form, N) for form in CHAIN_FORMS for N in (50, 197, 1300)] + [(32, lb.INTEGRATE_ADD, 4500)])
 def test_a_programmatic_chain_equals_its_kernels_one_by_one(Hq, integrate, N):
     """A carried chain of two layers, a fresh scores buffer and workspace for each of three inputs, called back to back: every output as with the
     per-kernel timing on, which takes the chain apart (packing first, every kernel behind the one before)."""
@@ -610,12 +633,20 @@ def test_low_ranks_are_packed_alike_wherever_their_rows_start(r, Hkv):
 
 @pytest.mark.parametrize("B,N,Hq,Hkv", [(6, 4096, 32, 32), (3, 5000, 40, 40), (5, 7000, 32, 8)])
 def test_attention_whose_keys_and_values_exceed_l2(B, N, Hq, Hkv):
-    """Past 63 MB of K and V the (batch, head) pairs are handed out in groups (whole batches, then parts of one, by the factors of both counts):
-    every pair and query tile is computed once, whatever the order.  A sequence alone is handed out in other groups; its outputs are the same bytes."""
+    """Past 63 MB of K and V the (batch, head) pairs are handed out in groups (whole batches, then parts of one): every pair and query tile is computed
+    once, whatever the order.  The heads of a few KV heads at a time, of all sequences, whose K and V fit: one group, heads and sequences side by side;
+    the same bytes.  Rows of the first and last tiles of the last sequence, all heads of it, are the oracle's."""
     g = torch.Generator(device="cuda").manual_seed(B)
     q, k, v = (torch.randn((B, N, h, 128), generator=g, device="cuda", dtype=torch.bfloat16) for h in (Hq, Hkv, Hkv))
     got = torch.full_like(q, float("nan"))
     lb.lisa_attn_anchor(q, k, v, out=got)
-    for b in range(B):
-        assert torch.equal(lb.lisa_attn_anchor(q[b:b + 1], k[b:b + 1], v[b:b + 1]), got[b:b + 1])
+    G, at_once = Hq // Hkv, (63 << 20) // (B * N * 512)
+    assert 1 <= at_once < Hkv
+    for a in range(0, Hkv, at_once):
+        b = min(a + at_once, Hkv)
+        part = lb.lisa_attn_anchor(q[:, :, a * G:b * G], k[:, :, a:b], v[:, :, a:b])
+        assert torch.equal(part, got[:, :, a * G:b * G]), (a, b)
     assert lb.lisa_check() == lb.OK
+    rows = np.array([0, 1, 63, 64, 127, 128, N - 130, N - 65, N - 1], dtype=np.int32)
+    ref = oracle.prefill_rows(*(f64(x[B - 1:].cpu()) for x in (q, k, v)), [], np.zeros_like(rows), rows)
+    assert_close(got[B - 1, torch.from_numpy(rows).long().cuda()].float().cpu().numpy(), ref, "bf16", "rows of the last sequence")
