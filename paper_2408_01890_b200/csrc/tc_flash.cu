@@ -644,11 +644,14 @@ cudaError_t launch_tc_flash(const TcFlashArgs& a, cudaStream_t stream) {
     p.scale = a.scale;
 
     if (a.qt_count < 1 || a.qt_count > 65535) return cudaErrorInvalidValue;
-    // (batch, head) pairs that the CTAs handed out one after the other share out: as many as have their K and V in half of a 126 MB L2 (the other
-    // half for everything else that streams), so that the ~300 CTAs resident at a time re-read them from there for every query tile.  As
-    // many, because the heads of a position lie side by side in a plane, whose lines the CTAs of neighbouring heads then write at about the
-    // same time, and because a grid ends with the lightest tiles of its last group only.  One pair at a time, as it was beyond 63 MB | this, us:
-    // write-back at 4 x 8192 tokens of 32 / 8 heads 4171 | 3452, 2 x 4096 of 32 / 32 heads 509 | 434, attention over 2 x 1777 of 40 heads 109 | 88.
+    // (batch, head) pairs that the CTAs are handed out for one after the other, in groups whose K and V fit half of a 126 MB L2 (the other half for
+    // everything else that streams), so that the ~300 CTAs resident at a time re-read them from there for every query tile.  All pairs where they
+    // fit; else all divided by the smallest prime factor of the batch count until they do, sequence by sequence from there, then by those of the
+    // heads: equal groups, so a batch of 13 goes from all at once to one sequence.  Larger ones are better, because the heads of a position lie side
+    // by side in a plane, whose lines the CTAs of neighbouring heads then write at about the same time, and because a grid ends with the lightest
+    // tiles of its last group only.  One pair at a time, as it was beyond 63 MB | this, us: write-back at 4 x 8192 tokens of 32 / 8 heads
+    // 4171 | 3452, 2 x 4096 of 32 / 32 heads 509 | 434, attention over 2 x 1777 of 40 heads 109 | 88; an anchor and one carried layer, prime
+    // batches: 13 x 2048 of 32 / 8 heads 2552 | 2496, 61 x 1200 4997 | 4813, 7 x 1500 of 40 heads 1201 | 1157.
     const int64_t kv_head = (int64_t)a.N * (a.kd + (a.emit_plane ? 0 : D)) * 2;
     int group = a.B * a.Hq;
     if (a.qt_count > 1)

@@ -36,9 +36,10 @@ struct PackJobs {
 
 // A CTA packs kPackPos positions of one sequence: the rows of H x r values are read as they lie (one warp per position) into shared
 // memory and leave as whole 64-byte rows, whose 16-byte pieces a thread shifts together from five words (r may be odd, a head's values then
-// start in the middle of one).  Bound by the latency of its loads, so a warp has all of a row's in flight as 16-byte vectors; rows lie 1028
-// words apart, so that the pieces of eight positions come from different banks (with 16-bit reads of rows 1024 words apart the packing took
-// twice as long).
+// start in the middle of one).  Bound by the latency of its loads, so a warp has all of a row's in flight as 16-byte vectors.  Rows lie 1028
+// words apart: the same piece of eight positions comes from eight groups of four banks.  A warp reads the three or four pieces of eight positions at
+// once, 4 words apart, so that a read still meets three or four in a bank (with 16-bit reads of rows 1024 words apart, where all eight positions
+// met, the packing took twice as long).
 constexpr int kPackPos = 8, kPackThreads = kPackPos * 32, kPackRow = kMaxHeads * kMaxRank + 8;
 __global__ void __launch_bounds__(kPackThreads) pack_lowrank_kernel(const __grid_constant__ PackJobs jobs, int B, int N) {
     __shared__ __align__(16) __nv_bfloat16 rows[kPackPos * kPackRow];
@@ -158,9 +159,10 @@ bool concat_chain(const lisa_shared_prefill_args& a) { return a.chain_len > 0 &&
 int plane_count(const lisa_shared_prefill_args& a) { return a.chain_len + (concat_chain(a) ? 1 : 0); }
 
 // Waves are independent of one another, and the three kernels of a wave stress different things (the emit kernel only
-// writes HBM, the attention kernel mostly reads it, the aligner is bound by its MMA rate), so up to kWaveSets waves are
-// in flight at a time, each on a stream and a set of planes of its own: wave w uses set w % sets, and set reuse is
-// ordered by the stream the set belongs to.
+// writes HBM, the attention kernel mostly reads it, the aligner of a recomputed chain, which takes all its links at once, is bound by its MMA rate),
+// so up to kWaveSets waves are in flight at a time, each on a stream and a set of planes of its own: wave w uses set w % sets, and set reuse is
+// ordered by the stream the set belongs to.  Calls that carry their scores from device memory have no waves, the concatenating Integrate's excepted
+// (see launch_tc_shared_prefill_chain).
 constexpr int kWaveSets = 3;
 
 struct Layout {
@@ -356,14 +358,15 @@ cudaError_t launch_tc_shared_prefill_chain(const lisa_shared_prefill_args& a, co
     const bool concat = concat_chain(a);
     const bool one_wave = (int64_t)a.B * a.Hq * ((a.N + kTile - 1) / kTile) <= 2 * (int64_t)sm_count();   // of CTAs, all resident at once
     Wave waves[1024];
-    int nw = plan_waves(a.B, a.N, a.Hq, cy ? 1 : plane_count(a), waves, 1024, cy != nullptr && !concat);
+    int nw = 0;
     // Carried scores need no planes of a wave's own: the whole prompt is one wave, whose kernels run one after the other as a programmatic
     // chain.  Each of them is bound by memory (aligner 6.2 of 6.55 TB/s at 4 x 8192 tokens of 32 heads) or fills the GPU, so that waves side by side
     // only added their tails: an anchor and its chain, in waves | in one, 4 x 8192 of the 8B shape 23260 | 22980 us, 1 x 8192 4232 | 4119, 2 x 4096
     // of the 7B shape 2426 | 2329, 4 x 2500 of 40 heads 2653 | 2537.
     if (cy && !concat && !ho) {
-        waves[0] = Wave{0, (a.N + kTile - 1) / kTile};
-        nw = 1;
+        waves[nw++] = Wave{0, (a.N + kTile - 1) / kTile};
+    } else {
+        nw = plan_waves(a.B, a.N, a.Hq, cy ? 1 : plane_count(a), waves, 1024, cy != nullptr && !concat);
     }
     // A host-memory call whose prompt fits fewer than four waves is cut into four strips of query tiles all the same (they
     // run one after the other in the planes laid out for the larger waves): its time is the copies', and strips let the
